@@ -10,6 +10,7 @@
 
 #include "common.cuh"
 #include "conv_simt.cuh"
+#include "conv_f32.cuh"
 #include "conv_tc.cuh"
 #include "conv_stem.cuh"
 #include "conv_halo.cuh"
@@ -34,8 +35,8 @@ thread_local std::string g_cuda_err;
 
 constexpr int kBranchMaxBatch = 32;   // shortcut layers run on the branch stream up to this batch size
 
-enum KernelKind { KK_SIMT = 0, KK_TC = 1, KK_DW = 2, KK_POOL = 3, KK_TC_GATHER = 4 };
-const char* kKernelNames[] = {"conv_igemm_simt", "conv_igemm_tcgen05", "dwconv", "maxpool", "conv_igemm_tcgen05_gather"};
+enum KernelKind { KK_SIMT = 0, KK_TC = 1, KK_DW = 2, KK_POOL = 3, KK_TC_GATHER = 4, KK_F32 = 5 };
+const char* kKernelNames[] = {"conv_igemm_simt", "conv_igemm_tcgen05", "dwconv", "maxpool", "conv_igemm_tcgen05_gather", "conv_igemm_f64mma"};
 
 struct LayerPlan {
   ee_layer_desc_t d;
@@ -48,6 +49,7 @@ struct LayerPlan {
   float* scale_dev = nullptr;
   float* bias_dev = nullptr;
   TcLayer tc;  // tensor-core plan (valid iff kind == KK_TC or KK_TC_GATHER)
+  F32Plan f32; // tile and K cut of a dense convolution of the fp32 model (kind == KK_F32)
   // Kernel variant per batch size, index 0..max_batch (TcVariant; empty = TCV_AUTO everywhere).  The analogue of the
   // paper's per-(layer, batch) look-up table that configures the array for the active batch (Section III-C): the
   // variant may change with the batch, the layer's K ranges (tc.splits) may not.
@@ -245,9 +247,20 @@ ee_status_t launch_layer(ee_model* m, const LayerPlan& L, const void* src, const
   constexpr int V = Elem<T>::kVec;
   switch (L.kind) {
     case KK_SIMT: {
-      dim3 grid(cdiv((long)B * L.out_h * L.out_w, kSimtBM), cdiv(L.d.cout, kSimtBN));
-      conv_igemm_simt_kernel<T><<<grid, kSimtThreads, 0, st>>>((const T*)src, (const T*)L.w_dev, L.scale_dev, L.bias_dev,
-                                                                 (const T*)res, (T*)dst, g);
+      if constexpr (sizeof(T) == 2) {
+        dim3 grid(cdiv((long)B * L.out_h * L.out_w, kSimtBM), cdiv(L.d.cout, kSimtBN));
+        conv_igemm_simt_kernel<<<grid, kSimtThreads, 0, st>>>((const bf16*)src, (const bf16*)L.w_dev, L.scale_dev, L.bias_dev, (const bf16*)res,
+                                                              (bf16*)dst, g);
+      } else {
+        return EE_ERR_INTERNAL;
+      }
+      break;
+    }
+    case KK_F32: {
+      if constexpr (sizeof(T) == 4)
+        EE_CUDA(f32_launch(L.f32, (const float*)src, (const float*)L.w_dev, L.scale_dev, L.bias_dev, (const float*)res, (float*)dst, g, st));
+      else
+        return EE_ERR_INTERNAL;
       break;
     }
     case KK_TC: {
@@ -766,6 +779,7 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
   if (rc == EE_OK) rc = halo_context_init();
   if (rc == EE_OK) rc = pair_context_init();
   if (rc == EE_OK) rc = dw_context_init();
+  if (rc == EE_OK) rc = f32_context_init();
   if (rc == EE_OK && hc_context_init() != cudaSuccess) rc = EE_ERR_CUDA;
   if (rc != EE_OK) return fail(rc);
 
@@ -1001,6 +1015,9 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
         L.tc.splits = 1, L.tc.kb_per = kp / kTcBK;
         L.tc.g_h = L.in_h, L.tc.g_w = L.in_w, L.tc.g_cin = d.cin, L.tc.g_kh = d.kh, L.tc.g_kw = d.kw;
         L.tc.g_stride = d.stride, L.tc.g_pad = d.pad, L.tc.g_runp = runp;
+      } else if (desc->dtype == EE_F32) {
+        L.kind = KK_F32;
+        L.f32 = f32_plan((long)desc->max_batch * L.out_h * L.out_w, d.cout, d.kh * d.kw * d.cin, m->tc.sm_count);
       } else {
         L.kind = KK_SIMT;
       }
@@ -1062,7 +1079,7 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
       for (int i = 0; i < sd.n_layers; ++i) {
         LayerPlan& L = sp.layers[i];
         const size_t in_sz = (size_t)L.in_h * L.in_w * L.d.cin, res_sz = L.res_slot == -2 ? 0 : (size_t)L.out_h * L.out_w * L.d.cout;
-        const bool rev = L.kind != KK_SIMT && !(res_sz > in_sz ? dir_of(L.res_slot) : dir_of(L.src_slot));   // the CUDA-core kernel walks forward
+        const bool rev = L.kind != KK_SIMT && L.kind != KK_F32 && !(res_sz > in_sz ? dir_of(L.res_slot) : dir_of(L.src_slot));   // the CUDA-core and fp64 kernels walk forward
         L.tc.rev = rev;
         if (L.src_slot < 0 || L.res_slot == -1) in_rev = rev;
         if (L.src_slot >= 0) slot_rev[L.src_slot] = rev;

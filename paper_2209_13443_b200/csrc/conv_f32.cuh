@@ -1,0 +1,274 @@
+// Convolutions of the fp32 model: implicit GEMM on the double-precision matrix instruction.
+//
+// The fp32 model multiplies floats exactly and sums in fp64 (see Accum in common.cuh), so its bound is the fp64 rate
+// (one DFMA per lane and two clocks) for large maps and, for the small maps this model is used on, latency: a layer
+// has few output tiles and a long K, e.g. 24 x 512 outputs over K = 4608.  Both are answered by mma.m16n8k16.f64 (2048
+// FMAs per instruction; operands converted from float once per fragment instead of once per product) and by cutting
+// K: the 8 warps of a CTA are KG groups that take every KG-th 16-wide K step of a tile, and a cluster of Z CTAs cuts
+// the K range of the tile once more.  Partial tiles (fp64) are added in ascending group order in each CTA and then in
+// ascending CTA order through distributed shared memory; every CTA of the cluster finishes a share of the tile.
+// Z, KG and the tile depend on the layer and max_batch only, so a sample's sums are grouped the same way in any batch.
+//
+// Measured on B200: the ResNet-50-shaped fp32 model at 64 x 64, batch 6 (K up to 4608, 12 to 1536 rows): see f32_plan.
+#pragma once
+#include "common.cuh"
+#include "conv_simt.cuh"
+
+namespace ee {
+
+constexpr int kF32Threads = 256;
+
+template <int WM, int WN, int KG, int MF, int NF>
+struct F32Tile {   // WM x WN warps per K group, each MF x NF fragments of 16 x 8
+  static constexpr int kBM = WM * MF * 16, kBN = WN * NF * 8, kKS = 16 * KG;   // output tile; K per ring stage
+  static constexpr int kStages = KG == 8 ? 3 : 4;
+  static constexpr int kRow = kKS + 4;                     // floats per shared-memory row: 4 mod 32 (20 mod 32 for KG = 1) spreads a fragment's 8 rows over all banks
+  static constexpr int kStageFloats = (kBM + kBN) * kRow;
+  static constexpr int kPRow = kBN + 2;                    // doubles per row of a partial tile
+  static constexpr int kRing = kStages * kStageFloats * 4, kPart = KG * kBM * kPRow * 8;
+  static constexpr int kBytes = kRing > kPart ? kRing : kPart;
+  static_assert(WM * WN * KG == 8, "8 warps");
+  static_assert(kBytes <= 227 * 1024, "exceeds the shared memory of an SM");
+};
+
+__device__ __forceinline__ void mma_f64(double* c, const double* a, const double* b) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f64.f64.f64.f64 {%0, %1, %2, %3}, {%4, %5, %6, %7, %8, %9, %10, %11}, {%12, %13, %14, %15}, {%0, %1, %2, %3};"
+      : "+d"(c[0]), "+d"(c[1]), "+d"(c[2]), "+d"(c[3])
+      : "d"(a[0]), "d"(a[1]), "d"(a[2]), "d"(a[3]), "d"(a[4]), "d"(a[5]), "d"(a[6]), "d"(a[7]), "d"(b[0]), "d"(b[1]), "d"(b[2]), "d"(b[3]));
+}
+template <int BYTES>   // 16 or 4; `in` false fills zeros
+__device__ __forceinline__ void cp_async_zfill(uint32_t dst, const void* src, bool in) {
+  if constexpr (BYTES == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ double ld_cluster_f64(uint32_t addr, uint32_t rank) {
+  uint32_t a;
+  double v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+  return v;
+}
+
+// V: floats per copy (4 when Cin is a multiple of 4 and the pointers are 16-byte aligned, else 1).  k_per: K range of a CTA.
+template <int WM, int WN, int KG, int MF, int NF, int V>
+__global__ void __launch_bounds__(kF32Threads)
+conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ w, const float* __restrict__ scale,
+                         const float* __restrict__ bias, const float* __restrict__ residual, float* __restrict__ y, ConvGeom g, int k_per) {
+  using S = F32Tile<WM, WN, KG, MF, NF>;
+  constexpr int BM = S::kBM, BN = S::kBN, KS = S::kKS, ROW = S::kRow, STAGES = S::kStages;
+  constexpr int UNITS = KS / V;                       // copies per row and stage
+  constexpr int STEP = kF32Threads / UNITS;           // rows covered by one pass of the CTA
+  constexpr int RA = (BM + STEP - 1) / STEP, RB = (BN + STEP - 1) / STEP;
+  extern __shared__ __align__(16) uint8_t f32_smem[];
+  float* ring = reinterpret_cast<float*>(f32_smem);
+  const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(f32_smem);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int M = g.B * g.Ho * g.Wo, N = g.Cout, K = g.kh * g.kw * g.Cin;
+  const int m0 = (int)blockIdx.x * BM, n0 = (int)blockIdx.y * BN;
+  const int z = (int)blockIdx.z, Z = (int)gridDim.z;
+  const int k_begin = z * k_per, k_end = min(K, k_begin + k_per);
+  const int steps = max(0, (k_end - k_begin + KS - 1) / KS);
+
+  const int ku = tid % UNITS, r0 = tid / UNITS;       // this thread copies column ku of rows r0, r0 + STEP, ...
+  const float* a_base[RA];
+  int a_h[RA], a_w[RA];
+#pragma unroll
+  for (int i = 0; i < RA; ++i) {
+    const int r = r0 + i * STEP, m = m0 + r;
+    const bool in = r < BM && m < M;
+    const int mm = in ? m : 0;
+    const int wo = mm % g.Wo, q = mm / g.Wo, ho = q % g.Ho, b = q / g.Ho;
+    a_base[i] = x + (size_t)b * g.H * g.W * g.Cin;
+    a_h[i] = in ? ho * g.stride - g.pad : -(1 << 20);   // far outside the image: zeros
+    a_w[i] = wo * g.stride - g.pad_w;
+  }
+  auto load = [&](int step) {
+    if (step < steps) {
+      const uint32_t st = ring_s + (uint32_t)((step % STAGES) * S::kStageFloats) * 4u;
+      const int k = k_begin + step * KS + ku * V;
+      const bool kin = k < k_end;
+      const int tap = k / g.Cin, ci = k - tap * g.Cin, r = tap / g.kw, s = tap - r * g.kw;
+#pragma unroll
+      for (int i = 0; i < RA; ++i) {
+        const int row = r0 + i * STEP;
+        if (BM % STEP == 0 || row < BM) {
+          const int hi = a_h[i] + r, wi = a_w[i] + s;
+          const bool in = kin && hi >= 0 && hi < g.H && wi >= 0 && wi < g.W;
+          cp_async_zfill<V * 4>(st + (uint32_t)(row * ROW + ku * V) * 4u, in ? a_base[i] + ((size_t)hi * g.W + wi) * g.Cin + ci : x, in);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < RB; ++i) {
+        const int row = r0 + i * STEP, n = n0 + row;
+        if (BN % STEP == 0 || row < BN) {
+          const bool in = kin && n < N;
+          cp_async_zfill<V * 4>(st + (uint32_t)((BM + row) * ROW + ku * V) * 4u, in ? w + (size_t)n * K + k : w, in);
+        }
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int kg = warp / (WM * WN), wmn = warp % (WM * WN), wm = wmn / WN, wn = wmn % WN;
+  const int fr = lane >> 2, fk = lane & 3;            // fragment row (column of B) and K position of this lane
+  double acc[MF][NF][4];
+#pragma unroll
+  for (int i = 0; i < MF; ++i)
+#pragma unroll
+    for (int j = 0; j < NF; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.0;
+#pragma unroll
+  for (int s = 0; s < STAGES - 1; ++s) load(s);
+  for (int step = 0; step < steps; ++step) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+    __syncthreads();                                  // this stage has landed for all; the stage refilled below was read one step ago
+    load(step + STAGES - 1);
+    const float* as = ring + (step % STAGES) * S::kStageFloats + (wm * MF * 16 + fr) * ROW + kg * 16 + fk;
+    const float* bs = ring + (step % STAGES) * S::kStageFloats + (BM + wn * NF * 8 + fr) * ROW + kg * 16 + fk;
+    double b[NF][4];
+#pragma unroll
+    for (int j = 0; j < NF; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) b[j][e] = (double)bs[j * 8 * ROW + 4 * e];
+#pragma unroll
+    for (int i = 0; i < MF; ++i) {
+      double a[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) a[e] = (double)as[(i * 16 + 8 * (e & 1)) * ROW + 4 * (e >> 1)];
+#pragma unroll
+      for (int j = 0; j < NF; ++j) mma_f64(acc[i][j], a, b[j]);
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  // partial tiles: [KG][BM][kPRow] doubles over the drained ring
+  double* part = reinterpret_cast<double*>(f32_smem);
+  {
+    double* p = part + ((size_t)kg * BM + wm * MF * 16 + fr) * S::kPRow + wn * NF * 8 + 2 * fk;
+#pragma unroll
+    for (int i = 0; i < MF; ++i)
+#pragma unroll
+      for (int j = 0; j < NF; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          *reinterpret_cast<double2*>(p + (i * 16 + 8 * h) * S::kPRow + j * 8) = make_double2(acc[i][j][2 * h], acc[i][j][2 * h + 1]);
+  }
+  __syncthreads();
+  if (Z > 1) {
+    if (KG > 1) {
+      for (int idx = tid; idx < BM * BN; idx += kF32Threads) {
+        const int o = (idx / BN) * S::kPRow + idx % BN;
+        double v = part[o];
+#pragma unroll
+        for (int q = 1; q < KG; ++q) v += part[q * BM * S::kPRow + o];
+        part[o] = v;
+      }
+    }
+    asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+  }
+  const uint32_t part_s = ring_s;
+  const int share = BM * BN / Z;                      // Z is 1, 2, 4 or 8: divides every tile
+  for (int idx = z * share + tid; idx < (z + 1) * share; idx += kF32Threads) {
+    const int r = idx / BN, c = idx % BN, m = m0 + r, n = n0 + c;
+    if (m >= M || n >= N) continue;
+    const int o = r * S::kPRow + c;
+    double v = 0.0;
+    if (Z > 1) {
+      for (int q = 0; q < Z; ++q) v += ld_cluster_f64(part_s + (uint32_t)o * 8u, (uint32_t)q);
+    } else {
+#pragma unroll
+      for (int q = 0; q < KG; ++q) v += part[q * BM * S::kPRow + o];
+    }
+    v = (double)(scale ? scale[n] : 1.f) * v + (double)(bias ? bias[n] : 0.f);
+    if (residual) v += (double)residual[(size_t)m * N + n];
+    y[(size_t)m * N + n] = (float)apply_act(v, g.act);
+  }
+  if (Z > 1) asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");   // peers may still read this CTA's partials
+}
+
+// ----------------------------------------------------------------------------- host side
+
+struct F32Plan {
+  int tile = 0;    // 0: 64 x 32, one K group; 1: 64 x 64, two; 2: 32 x 32, eight; 3: 16 x 32, eight
+  int z = 1;       // CTAs of a cluster that share a tile's K
+};
+
+// Tile and cluster size of a layer, from its geometry and max_batch.  Short K (stems on 3 channels): one K group, a ring
+// stage is 16 wide and nothing is padded to 128.  Grids of two waves of 64 x 64 tiles: that tile reads its operands least.
+// Everything else has idle SMs: small tiles, eight K groups, and as many CTAs per tile (up to 8) as keep the grid within
+// two CTAs per SM while every CTA still has two ring stages of K.
+inline F32Plan f32_plan(long m_max, int n, int k, int sms) {
+  F32Plan p;
+  if (k < 128) return p;
+  if ((long)cdiv(m_max, 64) * cdiv(n, 64) >= 2L * sms) {
+    p.tile = 1;
+    return p;
+  }
+  p.tile = m_max <= 16 ? 3 : 2;
+  const long tiles = (long)cdiv(m_max, p.tile == 3 ? 16 : 32) * cdiv(n, 32);
+  while (p.z < 8 && tiles * p.z * 2 <= 2L * sms && k >= p.z * 2 * 256) p.z *= 2;
+  return p;
+}
+
+template <int WM, int WN, int KG, int MF, int NF, int V>
+inline cudaError_t f32_launch_t(const F32Plan& p, const float* x, const float* w, const float* scale, const float* bias, const float* residual,
+                                float* y, const ConvGeom& g, cudaStream_t st) {
+  using S = F32Tile<WM, WN, KG, MF, NF>;
+  const int K = g.kh * g.kw * g.Cin;
+  const int k_per = cdiv(cdiv(K, S::kKS), p.z) * S::kKS;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cdiv((long)g.B * g.Ho * g.Wo, S::kBM), cdiv(g.Cout, S::kBN), p.z);
+  cfg.blockDim = dim3(kF32Threads);
+  cfg.dynamicSmemBytes = S::kBytes;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = p.z;
+  cfg.attrs = attr;
+  cfg.numAttrs = p.z > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, conv_igemm_f64mma_kernel<WM, WN, KG, MF, NF, V>, x, w, scale, bias, residual, y, g, k_per);
+}
+
+template <int V>
+inline cudaError_t f32_launch_v(const F32Plan& p, const float* x, const float* w, const float* scale, const float* bias, const float* residual,
+                                float* y, const ConvGeom& g, cudaStream_t st) {
+  switch (p.tile) {
+    case 1: return f32_launch_t<2, 2, 2, 2, 4, V>(p, x, w, scale, bias, residual, y, g, st);
+    case 2: return f32_launch_t<1, 1, 8, 2, 4, V>(p, x, w, scale, bias, residual, y, g, st);
+    case 3: return f32_launch_t<1, 1, 8, 1, 4, V>(p, x, w, scale, bias, residual, y, g, st);
+    default: return f32_launch_t<4, 2, 1, 1, 2, V>(p, x, w, scale, bias, residual, y, g, st);
+  }
+}
+
+inline cudaError_t f32_launch(const F32Plan& p, const float* x, const float* w, const float* scale, const float* bias, const float* residual,
+                              float* y, const ConvGeom& g, cudaStream_t st) {
+  const bool vec = g.Cin % 4 == 0 && (((uintptr_t)x | (uintptr_t)w) & 15) == 0;
+  return vec ? f32_launch_v<4>(p, x, w, scale, bias, residual, y, g, st) : f32_launch_v<1>(p, x, w, scale, bias, residual, y, g, st);
+}
+
+inline ee_status_t f32_context_init() {
+  cudaError_t e = cudaSuccess;
+  auto set = [&](auto kernel, int bytes) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  };
+  set(conv_igemm_f64mma_kernel<4, 2, 1, 1, 2, 4>, F32Tile<4, 2, 1, 1, 2>::kBytes);
+  set(conv_igemm_f64mma_kernel<4, 2, 1, 1, 2, 1>, F32Tile<4, 2, 1, 1, 2>::kBytes);
+  set(conv_igemm_f64mma_kernel<2, 2, 2, 2, 4, 4>, F32Tile<2, 2, 2, 2, 4>::kBytes);
+  set(conv_igemm_f64mma_kernel<2, 2, 2, 2, 4, 1>, F32Tile<2, 2, 2, 2, 4>::kBytes);
+  set(conv_igemm_f64mma_kernel<1, 1, 8, 2, 4, 4>, F32Tile<1, 1, 8, 2, 4>::kBytes);
+  set(conv_igemm_f64mma_kernel<1, 1, 8, 2, 4, 1>, F32Tile<1, 1, 8, 2, 4>::kBytes);
+  set(conv_igemm_f64mma_kernel<1, 1, 8, 1, 4, 4>, F32Tile<1, 1, 8, 1, 4>::kBytes);
+  set(conv_igemm_f64mma_kernel<1, 1, 8, 1, 4, 1>, F32Tile<1, 1, 8, 1, 4>::kBytes);
+  return e == cudaSuccess ? EE_OK : EE_ERR_CUDA;
+}
+
+}  // namespace ee

@@ -1,10 +1,10 @@
-// CUDA-core convolution kernels: fp32 implicit GEMM (the fp32 model path, and layers whose
-// channel counts no tensor-core tile covers, e.g. a 3-channel stem), depthwise 3x3 and max-pool.
+// CUDA-core convolution kernels: fp32 implicit GEMM (layers of bf16 models whose channel counts no
+// tensor-core tile covers), depthwise 3x3 and max-pool.
 //
 // The convolution is the product of the implicit Toeplitz matrix A [M = B*Ho*Wo][K = kh*kw*Cin]
 // with the weight matrix W [N = Cout][K] (paper Section II-C); A is never materialised.
-// Every output sums its K terms in ascending k (fp32 FMAs for bf16 models, fp64 for the fp32 model: see Accum),
-// independent of the batch size, so a sample's result does not depend on which batch it rides in.
+// Every output sums its K terms in ascending k, independent of the batch size, so a sample's result does not depend on
+// which batch it rides in.
 #pragma once
 #include "common.cuh"
 
@@ -16,10 +16,9 @@ struct ConvGeom {
 
 constexpr int kSimtBM = 64, kSimtBN = 64, kSimtBK = 16, kSimtThreads = 256, kSimtPad = 4;
 
-template <typename T>
 __global__ void __launch_bounds__(kSimtThreads)
-conv_igemm_simt_kernel(const T* __restrict__ x, const T* __restrict__ w, const float* __restrict__ scale,
-                       const float* __restrict__ bias, const T* __restrict__ residual, T* __restrict__ y, ConvGeom g) {
+conv_igemm_simt_kernel(const bf16* __restrict__ x, const bf16* __restrict__ w, const float* __restrict__ scale,
+                       const float* __restrict__ bias, const bf16* __restrict__ residual, bf16* __restrict__ y, ConvGeom g) {
   __shared__ __align__(16) float As[kSimtBK][kSimtBM + kSimtPad];
   __shared__ __align__(16) float Bs[kSimtBK][kSimtBN + kSimtPad];
   const int t = threadIdx.x;
@@ -50,12 +49,11 @@ conv_igemm_simt_kernel(const T* __restrict__ x, const T* __restrict__ w, const f
   }
 
   const int tx = t & 15, ty = t >> 4;
-  typedef typename Accum<T>::type A;
-  A acc[4][4];
+  float acc[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = (A)0;
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
 
   for (int k0 = 0; k0 < K; k0 += kSimtBK) {
     const int k = k0 + kk;
@@ -72,14 +70,14 @@ conv_igemm_simt_kernel(const T* __restrict__ x, const T* __restrict__ w, const f
       float v = 0.f;
       if (kin && a_base[i] >= 0) {
         const int hi = a_hi0[i] + r, wi = a_wi0[i] + s;
-        if (hi >= 0 && hi < g.H && wi >= 0 && wi < g.W) v = Elem<T>::ld(x + ((a_base[i] + (long)hi * g.W + wi) * g.Cin + ci));
+        if (hi >= 0 && hi < g.H && wi >= 0 && wi < g.W) v = Elem<bf16>::ld(x + ((a_base[i] + (long)hi * g.W + wi) * g.Cin + ci));
       }
       As[kk][rb + 16 * i] = v;
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int n = n0 + rb + 16 * i;
-      Bs[kk][rb + 16 * i] = (kin && n < N) ? Elem<T>::ld(w + (long)n * K + k) : 0.f;
+      Bs[kk][rb + 16 * i] = (kin && n < N) ? Elem<bf16>::ld(w + (long)n * K + k) : 0.f;
     }
     __syncthreads();
 #pragma unroll
@@ -103,9 +101,9 @@ conv_igemm_simt_kernel(const T* __restrict__ x, const T* __restrict__ w, const f
     for (int j = 0; j < 4; ++j) {
       const int n = n0 + tx * 4 + j;
       if (n >= N) continue;
-      A v = (A)(scale ? scale[n] : 1.f) * acc[i][j] + (A)(bias ? bias[n] : 0.f);   // float: one FMA; double: exact product, one add
-      if (residual) v += (A)Elem<T>::ld(residual + m * N + n);
-      Elem<T>::st(y + m * N + n, (float)apply_act(v, g.act));
+      float v = (scale ? scale[n] : 1.f) * acc[i][j] + (bias ? bias[n] : 0.f);
+      if (residual) v += Elem<bf16>::ld(residual + m * N + n);
+      Elem<bf16>::st(y + m * N + n, apply_act(v, g.act));
     }
   }
 }

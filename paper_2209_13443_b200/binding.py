@@ -225,7 +225,7 @@ class EEModel:
             _check(self._L.ee_model_create(C.byref(desc), _stream(stream), C.byref(h)), "ee_model_create")
         self._h = h
         self._keep = []
-        self._outs_key, self._outs_arr = None, None
+        self._outs, self._outs_arr = (), None
         self.table = None
         if apply_tables:
             self.table = apply_table(self, spec)
@@ -266,12 +266,11 @@ class EEModel:
         """ee_run_until_exit: every stage from ``first_stage`` on, each on the survivors of the one before, until the
         batch is empty or the last stage has been launched.  ``outs`` holds one StageBuffers per stage of the model.
         Returns the batch each stage ran on (0 for stages not reached)."""
-        key = tuple(id(o) for o in outs)
-        if self._outs_key != key:       # the array of ee_stage_out_t is built once per set of buffers
-            arr = (StageOut * self.n_stages)()
+        if len(outs) != len(self._outs) or any(a is not b for a, b in zip(outs, self._outs)):
+            arr = (StageOut * self.n_stages)()   # built once per set of buffers, which are held: an id may return with other buffers
             for s, o in enumerate(outs):
                 arr[s] = o.as_struct()
-            self._outs_key, self._outs_arr = key, arr
+            self._outs, self._outs_arr = tuple(outs), arr
         base = workspace.data_ptr()
         aligned = (base + 255) // 256 * 256
         sin = StageIn(_ptr(features), _ptr(ids), int(batch), _ptr(logit_shift), _ptr(shift_class))

@@ -335,7 +335,7 @@ ee_status_t launch_layer(ee_model* m, const LayerPlan& L, const void* src, const
 template <typename T>
 ee_status_t launch_head(ee_model* m, StagePlan& sp, const void* x, int B, int hw, const float* shift,
                         const int32_t* shift_cls, char* scratch, const ee_stage_in_t* in_ids, const ee_stage_out_t* out,
-                        cudaStream_t st, bool timed, const float* gap_part = nullptr, int gap_g = 0) {
+                        cudaStream_t st, bool timed, int32_t* host_count = nullptr, const float* gap_part = nullptr, int gap_g = 0) {
   const int C = sp.out_c, K = sp.n_classes;
   HeadLayout h = head_layout(m->max_batch, C, K);
   unsigned* cnt = (unsigned*)(scratch + h.off_cnt);
@@ -344,7 +344,7 @@ ee_status_t launch_head(ee_model* m, StagePlan& sp, const void* x, int B, int hw
   if constexpr (sizeof(T) == 2) {
     if (m->fused_head && hc_supported(C, K, x, sp.fc_w)) {
       DecideArgs da{shift, shift_cls, sp.threshold, sp.always_exit, out->conf, out->pred, out->exit_mask,
-                    in_ids ? in_ids->ids : nullptr, out->survivor_idx, out->ids_out, out->n_surv_dev, nullptr, m->head_done + (&sp - m->stages.data())};
+                    in_ids ? in_ids->ids : nullptr, out->survivor_idx, out->ids_out, out->n_surv_dev, nullptr, m->head_done + (&sp - m->stages.data()), host_count};
       EE_CUDA(hc_launch((const bf16*)x, hw, C, (const bf16*)sp.fc_w, sp.fc_b, B, K, z, da, st));
       if (timed) record(m, sp, st, "head_gap_fc_softmax_scan");
       return EE_OK;
@@ -385,17 +385,12 @@ ee_status_t launch_head(ee_model* m, StagePlan& sp, const void* x, int B, int hw
     EE_CUDA(launch_pdl(gap_kernel<T, 1>, ggrid, dim3(kGapThreads), st, (const T*)x, hw, C, lanes, gap, cnt, n_zero, sp.gap_rev ? 1 : 0));
   if (timed) record(m, sp, st, "head_gap");
   DecideArgs da{shift, shift_cls, sp.threshold, sp.always_exit, out->conf, out->pred, out->exit_mask,
-                in_ids ? in_ids->ids : nullptr, out->survivor_idx, out->ids_out, out->n_surv_dev, cnt, cnt + m->max_batch};
-  const int fs = fc_tile_samples(B);
-  dim3 fgrid(cdiv(K, kFcClasses), cdiv(B, fs));
-  const bool fal = C % V == 0 && ((uintptr_t)sp.fc_w & 15) == 0;
-  auto fc_launch = [&](auto kernel) {
-    return launch_pdl(kernel, fgrid, dim3(kFcThreads), st, (const float*)gap, (const T*)sp.fc_w, (const float*)sp.fc_b, B, C, K, z, da);
-  };
-  if (fs == 4)
-    EE_CUDA(fal ? fc_launch(fc_kernel<T, true, 4>) : fc_launch(fc_kernel<T, false, 4>));
+                in_ids ? in_ids->ids : nullptr, out->survivor_idx, out->ids_out, out->n_surv_dev, cnt, cnt + m->max_batch, host_count};
+  if (fc_cluster_supported(B, C, K, (int)sizeof(T), sp.fc_w))
+    EE_CUDA(fc_cluster_launch<T>(gap, (const T*)sp.fc_w, sp.fc_b, B, C, K, out->logits, da, st));
   else
-    EE_CUDA(fal ? fc_launch(fc_kernel<T, true, 8>) : fc_launch(fc_kernel<T, false, 8>));
+    EE_CUDA(launch_pdl(fc_kernel<T>, dim3(cdiv(K, kFcClasses), cdiv(B, kFcSamples)), dim3(kFcThreads), st, (const float*)gap, (const T*)sp.fc_w,
+                       (const float*)sp.fc_b, B, C, K, z, da));
   if (timed) record(m, sp, st, "head_fc_softmax_scan");
   return EE_OK;
 }
@@ -405,8 +400,7 @@ ee_status_t gather_launch_t(const void* feat, size_t bytes_per_sample, const int
                             void* out, bool rev, cudaStream_t st) {
   const size_t vecs = bytes_per_sample / sizeof(V);
   dim3 grid(cdiv((long)vecs, kCopyThreads * kCopyUnroll), max_rows);
-  gather_rows_kernel<V><<<grid, kCopyThreads, 0, st>>>((const V*)feat, vecs, idx, n_dev, (V*)out, rev ? 1 : 0);
-  EE_CUDA(cudaGetLastError());
+  EE_CUDA(launch_pdl(gather_rows_kernel<V>, grid, dim3(kCopyThreads), st, (const V*)feat, vecs, idx, n_dev, (V*)out, rev ? 1 : 0));
   return EE_OK;
 }
 
@@ -432,8 +426,7 @@ ee_status_t append_launch_t(const void* src, void* dst, size_t bytes, const int3
                             cudaStream_t st) {
   const size_t vecs = bytes / sizeof(V);
   const int grid = (int)std::min<size_t>((vecs + kCopyThreads - 1) / kCopyThreads, 148 * 16);
-  append_rows_kernel<V><<<grid, kCopyThreads, 0, st>>>((const V*)src, (V*)dst, vecs, ids_src, ids_dst, n_ids);
-  EE_CUDA(cudaGetLastError());
+  EE_CUDA(launch_pdl(append_rows_kernel<V>, dim3(grid), dim3(kCopyThreads), st, (const V*)src, (V*)dst, vecs, ids_src, ids_dst, n_ids));
   return EE_OK;
 }
 
@@ -485,8 +478,19 @@ ee_status_t launch_segment(ee_model* m, StagePlan& sp, const StagePlan::Segment&
   return EE_OK;
 }
 
-// Everything one stage launches, in stream order (also the body of a captured graph).
-ee_status_t enqueue_stage(ee_model* m, StagePlan& sp, const ee_stage_in_t* in, char* ws, const ee_stage_out_t* out, cudaStream_t st) {
+// Device address of the pinned count word, so that the scan can store the survivor count there itself: a copy behind it
+// (a forked branch of the graph) reached the host about 5 us later.  nullptr: no word, or memory the device cannot
+// address; then the count is copied.
+int32_t* count_word(const ee_stage_out_t* out) {
+  void* p = nullptr;
+  if (!out->n_surv_host || cudaHostGetDevicePointer(&p, out->n_surv_host, 0) == cudaSuccess) return (int32_t*)p;
+  cudaGetLastError();
+  return nullptr;
+}
+
+// Everything one stage launches, in stream order (also the body of a captured graph).  host_count: count_word(out).
+ee_status_t enqueue_stage(ee_model* m, StagePlan& sp, const ee_stage_in_t* in, char* ws, const ee_stage_out_t* out, int32_t* host_count,
+                          cudaStream_t st) {
   const int B = in->batch;
   sp.ev_used = 0;
   record(m, sp, st, "begin");
@@ -539,12 +543,12 @@ ee_status_t enqueue_stage(ee_model* m, StagePlan& sp, const ee_stage_in_t* in, c
   const void* so = ws + sp.slot_off[sp.out_slot];
   const int hw = sp.out_h * sp.out_w;
   ee_status_t s = m->dtype == EE_BF16
-                      ? launch_head<bf16>(m, sp, so, B, hw, in->logit_shift, in->shift_class, ws + sp.head_off, in, out, st, true, gpart, sp.gap_g)
-                      : launch_head<float>(m, sp, so, B, hw, in->logit_shift, in->shift_class, ws + sp.head_off, in, out, st, true);
+                      ? launch_head<bf16>(m, sp, so, B, hw, in->logit_shift, in->shift_class, ws + sp.head_off, in, out, st, true, host_count, gpart, sp.gap_g)
+                      : launch_head<float>(m, sp, so, B, hw, in->logit_shift, in->shift_class, ws + sp.head_off, in, out, st, true, host_count);
   if (s != EE_OK) return s;
-  // B_exit goes to the host as soon as the decisions are taken: the copy runs on a side branch (also when the stage
-  // is captured into a graph) while the survivors' features are gathered, and rejoins the stream behind the gather.
-  const bool fork = out->n_surv_host && !sp.always_exit;
+  // Where the scan could not store the count in the host's word itself, a copy on a side branch (also when the stage is
+  // captured into a graph) takes it there while the survivors' features are gathered, and rejoins the stream behind the gather.
+  const bool copy = out->n_surv_host && !host_count, fork = copy && !sp.always_exit;
   if (fork) {
     EE_CUDA(cudaEventRecord(m->ev_fork, st));
     EE_CUDA(cudaStreamWaitEvent(m->side, m->ev_fork, 0));
@@ -558,7 +562,7 @@ ee_status_t enqueue_stage(ee_model* m, StagePlan& sp, const ee_stage_in_t* in, c
   }
   if (fork)
     EE_CUDA(cudaStreamWaitEvent(st, m->ev_join, 0));
-  else if (out->n_surv_host)
+  else if (copy)
     EE_CUDA(cudaMemcpyAsync(out->n_surv_host, out->n_surv_dev, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   return EE_OK;
 }
@@ -588,8 +592,6 @@ bool same_chain(const ee_model::ChainGraph& c, int first, const ee_stage_in_t* i
   return true;
 }
 
-ee_status_t enqueue_stage(ee_model* m, StagePlan& sp, const ee_stage_in_t* in, char* ws, const ee_stage_out_t* out, cudaStream_t st);
-
 ee_status_t build_chain(ee_model* m, int first, const ee_stage_in_t* in, char* ws, const ee_stage_out_t* outs, ee_model::ChainGraph* out) {
   const int n_stages = (int)m->stages.size();
   cudaGraph_t g = nullptr;
@@ -613,8 +615,10 @@ ee_status_t build_chain(ee_model* m, int first, const ee_stage_in_t* in, char* w
   }
   // the first stage, at the caller's batch
   cudaGraph_t sub = nullptr;
+  std::vector<int32_t*> word(n_stages);
+  for (int s = first; s < n_stages; ++s) word[s] = count_word(&outs[s]);
   if (cudaStreamBeginCapture(m->cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return fail(EE_ERR_CUDA);
-  ee_status_t es = enqueue_stage(m, m->stages[first], in, ws, &outs[first], m->cap);
+  ee_status_t es = enqueue_stage(m, m->stages[first], in, ws, &outs[first], word[first], m->cap);
   cudaError_t ce = cudaStreamEndCapture(m->cap, &sub);
   if (es != EE_OK || ce != cudaSuccess || !sub) {
     if (sub) cudaGraphDestroy(sub);
@@ -650,7 +654,7 @@ ee_status_t build_chain(ee_model* m, int first, const ee_stage_in_t* in, char* w
       cur.batch = b;
       cudaGraph_t body = np.conditional.phGraph_out[b];
       if (cudaStreamBeginCaptureToGraph(m->cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return fail(EE_ERR_CUDA);
-      es = enqueue_stage(m, m->stages[s], &cur, ws, &outs[s], m->cap);
+      es = enqueue_stage(m, m->stages[s], &cur, ws, &outs[s], word[s], m->cap);
       cudaGraph_t ended = nullptr;
       ce = cudaStreamEndCapture(m->cap, &ended);
       if (es != EE_OK || ce != cudaSuccess) return fail(es != EE_OK ? es : EE_ERR_CUDA);
@@ -780,7 +784,7 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
   if (rc == EE_OK) rc = pair_context_init();
   if (rc == EE_OK) rc = dw_context_init();
   if (rc == EE_OK) rc = f32_context_init();
-  if (rc == EE_OK && hc_context_init() != cudaSuccess) rc = EE_ERR_CUDA;
+  if (rc == EE_OK && (hc_context_init() != cudaSuccess || fc_context_init() != cudaSuccess)) rc = EE_ERR_CUDA;
   if (rc != EE_OK) return fail(rc);
 
   int h = desc->in_h, w = desc->in_w, c = desc->in_c;
@@ -1248,10 +1252,16 @@ ee_status_t ee_stage_run(ee_model_t* m, int stage, const ee_stage_in_t* in, void
   // Replay path: the whole stage (every layer, the head, the gather, the count copy) as one CUDA graph, captured the
   // first time this exact call (same buffers, same batch) is seen on a capturable stream.  It removes the host cost
   // of ~25 launches per stage and most of the launch latency between the small kernels of a small batch.
+  // The legacy default stream cannot be captured, but a graph captured on the model's own stream launches into it like
+  // into any other (a program that never chose a stream pays one launch per stage instead of one per kernel: 16 kernels of
+  // the tiny model's pass, 325 us of host time).
   const bool legacy = st == nullptr || st == cudaStreamLegacy || st == cudaStreamPerThread;
-  if (m->graphs && !m->timing && !legacy) {
+  const cudaStream_t cap = legacy ? m->cap : st;
+  if (m->graphs && !m->timing) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) {
+    const cudaError_t qe = cudaStreamIsCapturing(st, &cs);
+    if (qe != cudaSuccess) cudaGetLastError();   // another stream of the program is being captured: plain launches
+    if (qe == cudaSuccess && cs == cudaStreamCaptureStatusNone) {
       StageCallKey key;
       key.in = *in;
       key.out = *out;
@@ -1261,10 +1271,11 @@ ee_status_t ee_stage_run(ee_model_t* m, int stage, const ee_stage_in_t* in, void
           EE_CUDA(cudaGraphLaunch(g.exec, st));
           return EE_OK;
         }
-      if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-        ee_status_t es = enqueue_stage(m, sp, in, (char*)workspace, out, st);
+      int32_t* const word = count_word(out);
+      if (cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+        ee_status_t es = enqueue_stage(m, sp, in, (char*)workspace, out, word, cap);
         cudaGraph_t graph = nullptr;
-        cudaError_t ce = cudaStreamEndCapture(st, &graph);
+        cudaError_t ce = cudaStreamEndCapture(cap, &graph);
         cudaGraphExec_t exec = nullptr;
         if (es == EE_OK && ce == cudaSuccess && graph && cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess) {
           cudaGraphDestroy(graph);
@@ -1293,7 +1304,7 @@ ee_status_t ee_stage_run(ee_model_t* m, int stage, const ee_stage_in_t* in, void
       }
     }
   }
-  return enqueue_stage(m, sp, in, (char*)workspace, out, st);
+  return enqueue_stage(m, sp, in, (char*)workspace, out, count_word(out), st);
 }
 
 ee_status_t ee_layer_run(ee_model_t* m, int stage, int layer, const void* input, const void* residual, int batch, void* output,

@@ -185,6 +185,7 @@ struct DecideArgs {  // everything the exit decision needs besides the logits
   int32_t* n_surv;
   unsigned* tile_done;  // per sample tile: CTAs of the FC kernel that have written its logits; zero between launches
   unsigned* done;       // sample tiles whose exit decisions are written; zero between launches
+  volatile int32_t* n_surv_host;   // optional: device address of a pinned host word that receives the count (exit_scan)
 };
 
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc, int src_bytes) {  // bytes past src_bytes are zero-filled
@@ -297,64 +298,337 @@ __device__ __forceinline__ void exit_scan(int B, const DecideArgs& d) {
     base += pass_total;
     __syncthreads();
   }
-  if (tid == 0) d.n_surv[0] = base;
+  if (tid == 0) {
+    d.n_surv[0] = base;
+    if (d.n_surv_host) *d.n_surv_host = base;   // B_exit goes to the scheduler: the host polls this word
+  }
 }
 
-constexpr int kFcWarps = 8, kFcClassesPerWarp = 2, kFcChunk = 128;
-constexpr int kFcClasses = kFcWarps * kFcClassesPerWarp;
-constexpr int kFcThreads = kFcWarps * 32;
-
-// z[b][k] = bfc[k] + sum_c wfc[k][c] * gap[b][c].  CTA (x, y) owns 16 classes (two per warp) of the S samples of
-// tile y (S = 8, or 4 for batches of at most 16: one warp per sample in the exit decision, shorter chains; the tile
-// height changes no sum) and walks the channels 128 at a time: the tile's pooled values and the classes' weights of a
-// chunk arrive in shared memory through cp.async, two chunks ahead of the arithmetic (ALIGNED; rows that are not whole 16-byte
-// vectors take plain loads, one chunk at a time).  Per (b, k): every lane adds its four channels of each chunk in
-// ascending order, then a shuffle tree; the order does not depend on the batch size or the sample's position.
+// The FC layer, softmax top-1, threshold and survivor scan of a batch of pooled vectors, in clusters of CL CTAs: one
+// cluster per tile of S samples, z[b][k] = bfc[k] + sum_c wfc[k][c] * gap[b][c].
 //
-// No CTA waits for another.  The CTA that completes a sample tile's logits (a counter per tile) takes that tile's
-// exit decisions: softmax top-1 and threshold.  The CTA that completes the last tile's decisions (a second
-// counter) runs the stable scan of the survivors over the whole batch and leaves all counters at zero.
-// Launched with programmatic stream serialization.
-template <typename T, bool ALIGNED, int S>
+// The layer is a few MFLOP over at most a few MB of weights, so nothing but latency bounds it.  Every wait on another
+// SM through global memory costs about a microsecond, so a tile's CTAs exchange what the decision needs through
+// distributed shared memory (one cluster barrier), and the weights, which no kernel writes, are on their way into
+// shared memory before the kernel waits for the pooled vectors.
+//   1. The classes are cut into 16 blocks of kb (a multiple of 8), CTA r owns 16 / CL of them.  A warp takes groups of eight
+//      classes: its weights stream through a ring of its own, [8 classes][512 bytes of channels] per slot, filled by
+//      cp.async kFcRing - 1 slots ahead; no barrier but __syncwarp inside the loop.  A lane adds its 16 bytes of channels
+//      of every slot in ascending order, then a halving butterfly (distances 16, 8, ..., 1) forms all 8 S sums at once:
+//      the tree of a sum does not depend on S, so a logit is the same bits in any batch.
+//   2. Per (sample, block): maximum, lowest argmax and sum of exp(z - max) go into the leader CTA's shared memory.
+//   3. The leader adds the 16 triples in a fixed order: conf = 1 / sum_r s_r exp(m_r - m), exit = always || conf >= thr (NaN
+//      never exits).  With several tiles the leader that finishes last runs the stable scan over the batch.
+// No wait spins.  Launched with programmatic stream serialization.  Measured on B200 (pooling kernel + this kernel, one
+// graph): see fc_shape.
+constexpr int kFcMaxSmem = 226 * 1024;   // dynamic; the scan's static arrays come on top
+constexpr int kFcThreads = 256, kFcRing = 4, kFcBlocks = 16, kFcRows = 8, kFcSlot = kFcRows * 512;
+
+__device__ __forceinline__ uint32_t hc_cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t hc_map(const void* smem_ptr, uint32_t rank) {   // the same variable in CTA `rank` of the cluster
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(smem_ptr)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void hc_st_f32(uint32_t cluster_addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ void hc_cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void hc_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+struct FcShape {
+  int S, CL;     // samples per tile, CTAs per cluster
+  int kb;        // classes per block
+  int Cp;        // channels rounded up to whole ring slots
+};
+// Samples per tile: few, so that a CTA's arithmetic stays below the time its weights need and the tiles fill the GPU.  Cluster: 64 classes per CTA while few tiles leave SMs idle (16 CTAs need the non-portable
+// size), 128 otherwise; fewer CTAs for few classes.  Neither changes a sum.
+inline FcShape fc_shape(int B, int C, int K, int elem_bytes) {
+  FcShape f;
+  f.S = B <= 4 ? 1 : B <= 16 ? 2 : 4;
+  const int tiles = (B + f.S - 1) / f.S;
+  f.CL = 1;
+  while (f.CL < (tiles <= 4 ? 16 : 8) && f.CL * 64 < K) f.CL *= 2;
+  f.kb = ((K + kFcBlocks - 1) / kFcBlocks + kFcRows - 1) / kFcRows * kFcRows;
+  const int chunk = 512 / elem_bytes;
+  f.Cp = (C + chunk - 1) / chunk * chunk;
+  return f;
+}
+inline size_t fc_smem_bytes(const FcShape& f) {
+  return (size_t)(kFcThreads / 32) * kFcRing * kFcSlot + (size_t)f.S * f.Cp * 4 + (size_t)f.S * (kFcBlocks / f.CL) * f.kb * 4 +
+         (size_t)kFcBlocks * f.S * 16;
+}
+// C in whole 16-byte vectors of both operands, shared memory for the pooled tile and the logits of a CTA.
+inline bool fc_cluster_supported(int B, int C, int K, int elem_bytes, const void* wfc) {
+  return C % (16 / elem_bytes) == 0 && ((uintptr_t)wfc & 15) == 0 && fc_smem_bytes(fc_shape(B, C, K, elem_bytes)) <= (size_t)kFcMaxSmem;
+}
+
+__device__ __forceinline__ void fc_fma2(float (&a)[2], float w0, float w1, float g0, float g1) {   // two independent FMAs, one instruction
+  asm("{\n .reg .b64 w, g, a;\n mov.b64 w, {%2, %3};\n mov.b64 g, {%4, %5};\n mov.b64 a, {%0, %1};\n fma.rn.f32x2 a, w, g, a;\n"
+      " mov.b64 {%0, %1}, a;\n}"
+      : "+f"(a[0]), "+f"(a[1])
+      : "f"(w0), "f"(w1), "f"(g0), "f"(g1));
+}
+__device__ __forceinline__ void fc_fma2(double (&a)[2], float w0, float w1, float g0, float g1) {
+  a[0] = acc_fma(w0, g0, a[0]);
+  a[1] = acc_fma(w1, g1, a[1]);
+}
+
+template <typename T, int S>
+__global__ void __launch_bounds__(kFcThreads)
+fc_cluster_kernel(const float* __restrict__ gap, const T* __restrict__ wfc, const float* __restrict__ bfc, int B, int C, int K, float* z,
+                  DecideArgs d, FcShape f) {
+  typedef typename Accum<T>::type A;                        // fp64 sums for the fp32 model
+  constexpr int VEC = 16 / (int)sizeof(T), CHUNK = 32 * VEC, NV = kFcRows * S;
+  extern __shared__ __align__(16) uint8_t fc_smem[];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint8_t* ring = fc_smem + (size_t)warp * kFcRing * kFcSlot;                             // this warp's slots
+  float* gs = reinterpret_cast<float*>(fc_smem + (size_t)(kFcThreads / 32) * kFcRing * kFcSlot);   // [S][Cp] pooled vectors
+  const int my_blocks = kFcBlocks / f.CL, kc = my_blocks * f.kb;
+  float* zs = gs + (size_t)S * f.Cp;                                                      // [S][kc] this CTA's logits
+  float* part = zs + (size_t)S * kc;                                                      // [16][S][4] (leader): max, argmax, sum
+  const uint32_t rank = hc_cluster_rank();
+  const int tile = (int)blockIdx.x / f.CL, tiles = (int)gridDim.x / f.CL, b0 = tile * S;
+  const int k0 = (int)rank * kc;
+  const int nchunk = f.Cp / CHUNK, ngroups = max(0, min(kc, K - k0) + kFcRows - 1) / kFcRows;
+  const int T_w = warp < ngroups ? ((ngroups - 1 - warp) / (kFcThreads / 32) + 1) * nchunk : 0;   // ring slots this warp consumes
+
+  if (f.CL > 1) hc_cluster_arrive();   // #1: every CTA of the cluster runs (waited for before the first remote store)
+  auto load = [&](int t) {
+    if (t < T_w) {
+      const int g = warp + (t / nchunk) * (kFcThreads / 32), c = (t % nchunk) * CHUNK + lane * VEC;
+      uint8_t* dst = ring + (size_t)(t % kFcRing) * kFcSlot + lane * 16;
+#pragma unroll
+      for (int r = 0; r < kFcRows; ++r) {
+        const int k = k0 + g * kFcRows + r;
+        const bool in = k < K && c < C;
+        cp_async16(dst + r * 512, in ? wfc + (size_t)k * C + c : wfc, in ? 16 : 0);
+      }
+    }
+    cp_async_commit();
+  };
+#pragma unroll
+  for (int t = 0; t < kFcRing - 1; ++t) load(t);
+  pdl_wait();
+  pdl_launch_dependents();
+  for (int i = tid; i < S * (f.Cp / 4); i += kFcThreads) {
+    const int s = i / (f.Cp / 4), c = (i % (f.Cp / 4)) * 4;
+    const bool in = b0 + s < B && c < C;
+    cp_async16(gs + (size_t)s * f.Cp + c, in ? gap + (size_t)(b0 + s) * C + c : gap, in ? 16 : 0);
+  }
+  cp_async_commit();
+  cp_async_wait<0>();
+  __syncthreads();
+
+  A acc[kFcRows][S][2];   // even and odd channels
+#pragma unroll
+  for (int q = 0; q < kFcRows; ++q)
+#pragma unroll
+    for (int s = 0; s < S; ++s) acc[q][s][0] = acc[q][s][1] = (A)0;
+  for (int t = 0; t < T_w; ++t) {
+    cp_async_wait<kFcRing - 2>();
+    __syncwarp();           // slot t has landed for every lane; the slot refilled below was read one step ago
+    load(t + kFcRing - 1);
+    const int ch = t % nchunk;
+    const uint8_t* slot = ring + (size_t)(t % kFcRing) * kFcSlot + lane * 16;
+    float gv[S][VEC];
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+#pragma unroll
+      for (int e = 0; e < VEC; e += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(gs + (size_t)s * f.Cp + ch * CHUNK + lane * VEC + e);
+        gv[s][e] = v.x, gv[s][e + 1] = v.y, gv[s][e + 2] = v.z, gv[s][e + 3] = v.w;
+      }
+#pragma unroll
+    for (int q = 0; q < kFcRows; ++q) {
+      Vec16<T> w;
+      w.load(reinterpret_cast<const T*>(slot + q * 512));
+#pragma unroll
+      for (int s = 0; s < S; ++s)
+#pragma unroll
+        for (int e = 0; e < VEC; e += 2) fc_fma2(acc[q][s], w.v[e], w.v[e + 1], gv[s][e], gv[s][e + 1]);
+    }
+    if (ch == nchunk - 1) {   // the group's sums are complete: all 8 S of them in one halving butterfly
+      A v[NV];
+#pragma unroll
+      for (int q = 0; q < kFcRows; ++q)
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+          v[s * kFcRows + q] = acc[q][s][0] + acc[q][s][1];
+          acc[q][s][0] = acc[q][s][1] = (A)0;
+        }
+      int n = NV;             // values a lane still holds (a compile-time constant after unrolling)
+#pragma unroll
+      for (int dd = 16; dd >= 1; dd >>= 1) {
+        if (n > 1) {
+          const bool up = (lane & dd) != 0;
+#pragma unroll
+          for (int i = 0; i < NV / 2; ++i)
+            if (i < n / 2) {
+              const A send = up ? v[i] : v[i + n / 2], keep = up ? v[i + n / 2] : v[i];
+              v[i] = keep + __shfl_xor_sync(0xffffffffu, send, dd);
+            }
+          n /= 2;
+        } else {
+          v[0] += __shfl_xor_sync(0xffffffffu, v[0], dd);
+        }
+      }
+      constexpr int LEFT = NV > 32 ? NV / 32 : 1, REP = NV < 32 ? 32 / NV : 1;   // values per lane, lanes per value
+#pragma unroll
+      for (int j = 0; j < LEFT; ++j) {
+        const int idx = (lane / REP) * LEFT + j, s = idx / kFcRows, kl = (warp + (t / nchunk) * (kFcThreads / 32)) * kFcRows + idx % kFcRows;
+        if (lane % REP == 0) zs[s * kc + kl] = (float)(v[j] + (A)((bfc && k0 + kl < K) ? bfc[k0 + kl] : 0.f));
+      }
+    }
+  }
+  cp_async_wait<0>();
+  __syncthreads();
+
+  // ---- 2. one warp per (block, sample)
+  if (f.CL > 1) hc_cluster_wait();   // #1
+  for (int it = warp; it < my_blocks * S; it += kFcThreads / 32) {
+    const int s = it % S, bl = it / S, b = b0 + s, kf = k0 + bl * f.kb;
+    const int nk = max(0, min(f.kb, K - kf));
+    float m = -INFINITY, sum = 0.f;
+    int arg = 0x7fffffff;
+    if (b < B) {
+      const int cls = (d.shift && d.shift_cls) ? d.shift_cls[b] : -1;
+      float* zb = zs + s * kc + bl * f.kb;
+      if (lane == 0 && cls >= kf && cls < kf + nk) zb[cls - kf] += d.shift[b];
+      __syncwarp();
+      for (int j = lane; j < nk; j += 32) {
+        const float v = zb[j];
+        if (z) z[(size_t)b * K + kf + j] = v;
+        if (v > m) m = v, arg = kf + j;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float om = __shfl_xor_sync(0xffffffffu, m, o);
+        const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
+        if (om > m || (om == m && oa < arg)) m = om, arg = oa;
+      }
+      for (int j = lane; j < nk; j += 32) sum += expf(zb[j] - m);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    }
+    if (lane == 0) {
+      float* mine = part + ((size_t)((int)rank * my_blocks + bl) * S + s) * 4;
+      hc_st_f32(hc_map(mine, 0), m);
+      hc_st_f32(hc_map(mine + 1, 0), __int_as_float(arg));
+      hc_st_f32(hc_map(mine + 2, 0), sum);
+    }
+  }
+  if (f.CL > 1) {
+    hc_cluster_arrive();   // #2: the leader holds every block's triple
+    hc_cluster_wait();
+    if (rank != 0) return;
+  } else {
+    __syncthreads();
+  }
+  // ---- 3. decision: one warp per sample, lane r holds block r
+  if (warp < S && b0 + warp < B) {
+    const int s = warp, b = b0 + s;
+    float mr = -INFINITY, sr = 0.f;
+    int arg = 0x7fffffff;
+    if (lane < kFcBlocks) {
+      const float* t3 = part + ((size_t)lane * S + s) * 4;
+      mr = t3[0], arg = __float_as_int(t3[1]), sr = t3[2];
+    }
+    float m = mr;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float om = __shfl_xor_sync(0xffffffffu, m, o);
+      const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
+      if (om > m || (om == m && oa < arg)) m = om, arg = oa;
+    }
+    float tot = sr * (lane < kFcBlocks ? expf(mr - m) : 0.f);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    if (lane == 0) {
+      const float cf = 1.0f / tot;
+      if (d.conf) d.conf[b] = cf;
+      if (d.pred) d.pred[b] = arg == 0x7fffffff ? 0 : arg;
+      d.mask[b] = (uint8_t)((d.always_exit || cf >= d.thr) ? 1 : 0);
+    }
+  }
+  __threadfence();
+  __syncthreads();
+  if (tiles > 1) {         // the leader that finishes last scans
+    int* flag = reinterpret_cast<int*>(part);
+    if (tid == 0) *flag = atomicAdd(d.done, 1u) == (unsigned)(tiles - 1) ? 1 : 0;
+    __syncthreads();
+    if (!*flag) return;
+    __threadfence();
+    if (tid == 0) *d.done = 0;
+  }
+  exit_scan<kFcThreads>(B, d);
+}
+
+template <typename T, int S>
+inline cudaError_t fc_cluster_launch_t(const float* gap, const T* wfc, const float* bfc, int B, int C, int K, float* z, const DecideArgs& d,
+                                       const FcShape& f, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((B + S - 1) / S * f.CL));
+  cfg.blockDim = dim3(kFcThreads);
+  cfg.dynamicSmemBytes = fc_smem_bytes(f);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = f.CL;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, fc_cluster_kernel<T, S>, gap, wfc, bfc, B, C, K, z, d, f);
+}
+// d.done must be zero when the kernel starts and is zero again when it ends.
+template <typename T>
+inline cudaError_t fc_cluster_launch(const float* gap, const T* wfc, const float* bfc, int B, int C, int K, float* z, const DecideArgs& d,
+                                     cudaStream_t st) {
+  const FcShape f = fc_shape(B, C, K, (int)sizeof(T));
+  switch (f.S) {
+    case 1: return fc_cluster_launch_t<T, 1>(gap, wfc, bfc, B, C, K, z, d, f, st);
+    case 2: return fc_cluster_launch_t<T, 2>(gap, wfc, bfc, B, C, K, z, d, f, st);
+    default: return fc_cluster_launch_t<T, 4>(gap, wfc, bfc, B, C, K, z, d, f, st);
+  }
+}
+template <typename T, int S>
+inline cudaError_t fc_cluster_attr() {
+  cudaError_t e = cudaFuncSetAttribute(fc_cluster_kernel<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFcMaxSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(fc_cluster_kernel<T, S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  return e;
+}
+inline cudaError_t fc_context_init() {
+  cudaError_t e = cudaSuccess;
+  for (cudaError_t r : {fc_cluster_attr<bf16, 1>(), fc_cluster_attr<bf16, 2>(), fc_cluster_attr<bf16, 4>(), fc_cluster_attr<float, 1>(),
+                        fc_cluster_attr<float, 2>(), fc_cluster_attr<float, 4>()})
+    if (e == cudaSuccess) e = r;
+  return e;
+}
+
+// The same layer for any C, K and alignment (channels that are not whole 16-byte vectors, very many classes): CTA (x, y)
+// owns 16 classes (two per warp) of eight samples and walks the channels 128 at a time with plain loads.  The CTA that
+// completes a sample tile's logits (a counter per tile) takes that tile's exit decisions; the CTA that completes the last
+// tile's decisions runs the scan and leaves all counters at zero.
+constexpr int kFcWarps = 8, kFcClassesPerWarp = 2, kFcChunk = 128, kFcSamples = 8;
+constexpr int kFcClasses = kFcWarps * kFcClassesPerWarp;
+
+template <typename T>
 __global__ void __launch_bounds__(kFcThreads)
 fc_kernel(const float* __restrict__ gap, const T* __restrict__ wfc, const float* __restrict__ bfc, int B, int C, int K, float* z,
           DecideArgs d) {
-  constexpr int STAGES = ALIGNED ? (sizeof(T) == 2 ? 3 : 2) : 1;
-  constexpr int PER = kFcChunk / 32;  // channels per lane per chunk (4)
-  __shared__ __align__(16) float gs[STAGES][S][kFcChunk];
-  __shared__ __align__(16) T wsm[STAGES][kFcClasses][kFcChunk];
+  constexpr int PER = kFcChunk / 32, S = kFcSamples;  // channels per lane per chunk (4)
+  __shared__ __align__(16) float gs[S][kFcChunk];
+  __shared__ __align__(16) T wsm[kFcClasses][kFcChunk];
   __shared__ bool last_flag;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int k0 = blockIdx.x * kFcClasses, b0 = blockIdx.y * S;
   const int nchunk = (C + kFcChunk - 1) / kFcChunk;
-
-  auto stage_load = [&](int chunk, int buf) {
-    const int c0 = chunk * kFcChunk;
-    if constexpr (ALIGNED) {
-      constexpr int WV = 16 / (int)sizeof(T);       // weight elements per 16-byte vector
-      constexpr int WPC = kFcChunk / WV;            // vectors per class
-      for (int i = tid; i < S * (kFcChunk / 4); i += kFcThreads) {
-        const int sidx = i / (kFcChunk / 4), c = (i % (kFcChunk / 4)) * 4;
-        const bool in = b0 + sidx < B && c0 + c < C;
-        cp_async16(&gs[buf][sidx][c], in ? gap + (size_t)(b0 + sidx) * C + c0 + c : gap, in ? 16 : 0);
-      }
-      for (int i = tid; i < kFcClasses * WPC; i += kFcThreads) {
-        const int cls = i / WPC, c = (i % WPC) * WV;
-        const bool in = k0 + cls < K && c0 + c < C;
-        cp_async16(&wsm[buf][cls][c], in ? wfc + (size_t)(k0 + cls) * C + c0 + c : wfc, in ? 16 : 0);
-      }
-    } else {
-      for (int i = tid; i < S * kFcChunk; i += kFcThreads) {
-        const int sidx = i / kFcChunk, c = i % kFcChunk;
-        gs[buf][sidx][c] = (b0 + sidx < B && c0 + c < C) ? gap[(size_t)(b0 + sidx) * C + c0 + c] : 0.f;
-      }
-      for (int i = tid; i < kFcClasses * kFcChunk; i += kFcThreads) {
-        const int cls = i / kFcChunk, c = i % kFcChunk;
-        Elem<T>::st(&wsm[buf][cls][c], (k0 + cls < K && c0 + c < C) ? Elem<T>::ld(wfc + (size_t)(k0 + cls) * C + c0 + c) : 0.f);
-      }
-    }
-  };
-
   pdl_wait();
   pdl_launch_dependents();
   typedef typename Accum<T>::type A;   // fp64 sums for the fp32 model
@@ -363,34 +637,26 @@ fc_kernel(const float* __restrict__ gap, const T* __restrict__ wfc, const float*
   for (int q = 0; q < kFcClassesPerWarp; ++q)
 #pragma unroll
     for (int s2 = 0; s2 < S; ++s2) acc[q][s2] = (A)0;
-  if constexpr (ALIGNED) {
-#pragma unroll
-    for (int s0 = 0; s0 < STAGES - 1; ++s0) {
-      if (s0 < nchunk) stage_load(s0, s0);
-      cp_async_commit();   // one group per chunk, possibly empty: the wait below counts groups
-    }
-  }
   for (int chunk = 0; chunk < nchunk; ++chunk) {
-    const int buf = chunk % STAGES;
-    if constexpr (ALIGNED) {
-      cp_async_wait<STAGES - 2>();
-      __syncthreads();   // chunk landed for every thread; the buffer refilled below was read one iteration ago
-      const int next = chunk + STAGES - 1;
-      if (next < nchunk) stage_load(next, next % STAGES);
-      cp_async_commit();
-    } else {
-      __syncthreads();
-      stage_load(chunk, 0);
-      __syncthreads();
+    const int c0 = chunk * kFcChunk;
+    __syncthreads();
+    for (int i = tid; i < S * kFcChunk; i += kFcThreads) {
+      const int sidx = i / kFcChunk, c = i % kFcChunk;
+      gs[sidx][c] = (b0 + sidx < B && c0 + c < C) ? gap[(size_t)(b0 + sidx) * C + c0 + c] : 0.f;
     }
+    for (int i = tid; i < kFcClasses * kFcChunk; i += kFcThreads) {
+      const int cls = i / kFcChunk, c = i % kFcChunk;
+      Elem<T>::st(&wsm[cls][c], (k0 + cls < K && c0 + c < C) ? Elem<T>::ld(wfc + (size_t)(k0 + cls) * C + c0 + c) : 0.f);
+    }
+    __syncthreads();
     float wv[kFcClassesPerWarp][PER];
 #pragma unroll
     for (int q = 0; q < kFcClassesPerWarp; ++q)
 #pragma unroll
-      for (int e = 0; e < PER; ++e) wv[q][e] = Elem<T>::ld(&wsm[buf][warp * kFcClassesPerWarp + q][lane * PER + e]);
+      for (int e = 0; e < PER; ++e) wv[q][e] = Elem<T>::ld(&wsm[warp * kFcClassesPerWarp + q][lane * PER + e]);
 #pragma unroll
     for (int s2 = 0; s2 < S; ++s2) {
-      const float4 g = *reinterpret_cast<const float4*>(&gs[buf][s2][lane * PER]);
+      const float4 g = *reinterpret_cast<const float4*>(&gs[s2][lane * PER]);
       const float gv[PER] = {g.x, g.y, g.z, g.w};
 #pragma unroll
       for (int q = 0; q < kFcClassesPerWarp; ++q)
@@ -430,9 +696,6 @@ fc_kernel(const float* __restrict__ gap, const T* __restrict__ wfc, const float*
   exit_scan<kFcThreads>(B, d);
 }
 
-// Samples per FC tile for a batch.
-inline int fc_tile_samples(int B) { return B <= 16 ? 4 : 8; }
-
 // ----------------------------------------------------------------------------- the whole exit head in one launch
 //
 // bf16 models: global average pool, FC, softmax top-1, threshold and the survivor scan as ONE kernel of 8-CTA
@@ -452,22 +715,6 @@ inline int fc_tile_samples(int B) { return B <= 16 ? 4 : 8; }
 // No wait in this kernel spins: cluster barriers and cp.async groups only.  Launched with programmatic stream
 // serialization.
 constexpr int kHcCluster = 8, kHcThreads = 256, kHcRing = 4, kHcBlockClasses = 64, kHcBlockCh = 256, kHcMaxKc = 128;
-
-__device__ __forceinline__ uint32_t hc_cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t hc_map(const void* smem_ptr, uint32_t rank) {   // the same variable in CTA `rank` of the cluster
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(smem_ptr)), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void hc_st_f32(uint32_t cluster_addr, float v) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
-}
-__device__ __forceinline__ void hc_cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void hc_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 struct HcShape {   // functions of the head's shape (C, K) only
   int Cp;          // C rounded up to whole 256-channel blocks
@@ -752,6 +999,8 @@ template <typename V>
 __global__ void __launch_bounds__(kCopyThreads)
 gather_rows_kernel(const V* __restrict__ src, size_t vecs_per_row, const int32_t* __restrict__ surv_idx,
                    const int32_t* __restrict__ n_surv, V* __restrict__ dst, int rev) {
+  pdl_wait();
+  pdl_launch_dependents();
   const int j = rev ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;   // rev: last row first, each row from its end
   const unsigned bx = rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
   if (j >= *n_surv) return;
@@ -776,6 +1025,8 @@ template <typename V>
 __global__ void __launch_bounds__(kCopyThreads)
 append_rows_kernel(const V* __restrict__ src, V* __restrict__ dst, size_t n, const int32_t* __restrict__ ids_src,
                    int32_t* __restrict__ ids_dst, int n_ids) {
+  pdl_wait();
+  pdl_launch_dependents();
   const size_t stride = (size_t)gridDim.x * kCopyThreads;
   for (size_t v = (size_t)blockIdx.x * kCopyThreads + threadIdx.x; v < n; v += stride) dst[v] = __ldcs(src + v);
   if (ids_src && ids_dst && blockIdx.x == 0)

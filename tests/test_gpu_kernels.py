@@ -6,6 +6,8 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("needs a CUDA device", allow_module_level=True)
 
+from oracle import ee_oracle as eo
+from paper_2209_13443_b200 import binding as eb
 from paper_2209_13443_b200 import workloads as wl
 from tests import util
 
@@ -35,3 +37,75 @@ def test_fp32_convolution_tiles_and_k_cuts(geom):
         util.check_stage(spec, g, util.oracle_stage(spec, 0, x), f"f32 {geom} B={B}", elementwise=True)
         alone[B] = g["features_out"][0]
     assert np.array_equal(alone[1], alone[5])     # the cut of K does not depend on the batch
+
+
+# exit heads: dtype, B, HW, C, K: every tile height and cluster size, channels that leave a ring slot ragged, class blocks
+# that are short or empty, classes past one block per CTA, C the cluster kernel does not take
+HEADS = [("bf16", 3, 4, 520, 1000), ("bf16", 13, 9, 8, 17), ("bf16", 64, 2, 2048, 1000), ("bf16", 17, 3, 264, 129), ("bf16", 5, 5, 256, 5000),
+         ("bf16", 7, 6, 20, 33), ("f32", 1, 4, 132, 70), ("f32", 33, 2, 64, 10), ("f32", 6, 4, 2048, 100), ("f32", 9, 3, 7, 12)]
+
+
+@pytest.mark.parametrize("case", HEADS)
+def test_fc_cluster_tiles_against_the_oracle_and_alone(case):
+    dtype, B, HW, C, K = case
+    bf16 = dtype == "bf16"
+    rng = wl._rng(B + C + K, 907)
+    fw, fb = wl._head(rng, C, K, 4.0, bf16)
+    layers = [wl._conv(rng, wl.OP_CONV, C, C, 1, 1, 0, wl.ACT_NONE, bf16=bf16)]
+    spec = wl.Model("head", dtype, 1, HW, C, [wl.Stage(layers, K, fw, fb, 0.5, False)], B)
+    m = eb.EEModel(spec)
+    out = eb.StageBuffers(m, 0)
+    scratch = torch.empty(m.exit_head_scratch_bytes(0) + 256, dtype=torch.uint8, device="cuda")
+    x = wl.random_features((B, HW, C), seed=3, bf16=bf16)
+    shift = (np.arange(B) % 3 == 0).astype(np.float32) * 12.0
+    cls = (np.arange(B) * 7 % K).astype(np.int32)
+    xd, sd, cd = eb.to_device(dtype, x), torch.as_tensor(shift, device="cuda"), torch.as_tensor(cls, device="cuda")
+    for _ in range(2):      # the second call: the counters of the first are back at zero
+        m.exit_head(0, xd, B, HW, out, scratch, sd, cd)
+    torch.cuda.synchronize()
+    z, conf, mask = out.logits[:B].cpu().numpy(), out.conf[:B].cpu().numpy(), out.exit_mask[:B].cpu().numpy()
+    o = eo.exit_head(x, fw, fb, 0.5, False, shift, cls)
+    assert util.rel_err(z, o["z"], dtype, floor=util.LOGIT_FLOOR[dtype]) <= util.TOL[dtype]
+    assert np.max(np.abs(conf - o["conf"])) <= util.TOL[dtype]
+    sure = np.abs(o["conf"] - 0.5) > util.BAND
+    assert np.array_equal(mask[sure], o["exit"][sure])
+    n = int(out.n_surv_dev[0])
+    assert np.array_equal(out.survivor_idx[:n].cpu().numpy(), np.nonzero(mask == 0)[0]) and n == B - int(mask.sum())
+    b = B - 1               # alone: another tile height and cluster size, the same bits
+    m.exit_head(0, xd[b:].contiguous(), 1, HW, out, scratch, sd[b:].contiguous(), cd[b:].contiguous())
+    torch.cuda.synchronize()
+    assert np.array_equal(out.logits[0].cpu().numpy(), z[b]) and float(out.conf[0]) == float(conf[b])
+
+
+def test_stage_replay_on_the_default_stream_is_bit_identical():
+    spec = wl.resnet50_ee(seed=1, in_hw=64, n_classes=100, max_batch=6)
+    run = util.GpuRunner(spec)
+    xd = eb.to_device("bf16", wl.make_input(spec, 5, seed=3))
+    out, snaps = run.bufs[0], []
+    default = torch.cuda.default_stream()
+    for graphs in (False, True, True):
+        run.m.set_graphs(graphs)
+        out.logits.fill_(0)
+        torch.cuda.synchronize()
+        out.arm_count()
+        run.m.stage_run(0, xd, 5, out, run.ws, stream=default)
+        n = out.wait_count()
+        torch.cuda.synchronize()
+        snaps.append((n, out.logits[:5].clone(), out.features_out[:n].clone()))
+    for n, z, f in snaps[1:]:
+        assert n == snaps[0][0] == int(out.n_surv_dev[0]) and torch.equal(z, snaps[0][1]) and torch.equal(f, snaps[0][2])
+
+
+def test_stage_outputs_of_a_new_buffer_set_are_not_those_of_a_dead_one():
+    """run_until_exit keeps the ee_stage_out_t array of the last buffer set; a new set may have the ids of a dead one."""
+    spec = wl.tiny_ee_cnn(seed=0)
+    m = eb.EEModel(spec)
+    ws = m.workspace()
+    x = eb.to_device("f32", wl.make_input(spec, 4, seed=1))
+    for _ in range(4):
+        bufs = [eb.StageBuffers(m, s) for s in range(m.n_stages)]
+        bufs[0].conf.fill_(-1.0)
+        m.run_until_exit(0, x, 4, bufs, ws)
+        torch.cuda.synchronize()
+        assert bool((bufs[0].conf[:4] > 0).all())
+        del bufs

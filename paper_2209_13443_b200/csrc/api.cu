@@ -110,6 +110,8 @@ struct StagePlan {
   int n_classes = 0;
   void* fc_w = nullptr;
   float* fc_b = nullptr;
+  bool fc_cluster = false;   // the cluster FC kernel takes this head; tm_fc: its weights
+  CUtensorMap tm_fc;
   float threshold = 0.f;
   int always_exit = 0;
   bool gap_rev = false, gather_rev = false;   // walk directions of the pooling and gather kernels
@@ -172,6 +174,7 @@ struct ee_model {
   int proj_waves = 0;                  // tiles per SM from which a layer absorbs its projection (measured: a gain at every batch)
   bool gap_fusion = true;              // pooling partials from the last layer's epilogue where that applies
   bool proj_fusion = true;             // projection shortcuts computed inside the layer that adds them, where that applies
+  int fc_room = 1;                     // clusters of the FC kernel that run side by side
   bool fused_head = false;             // bf16 models: pool + FC + decision + scan as one cluster kernel where the shape allows (an option)
   long long wait_cycles = kTcWaitCycles;   // limit of the bounded device-side waits of the pair kernel and the self-test
   int device = -1;           // the GPU the model lives on
@@ -386,8 +389,9 @@ ee_status_t launch_head(ee_model* m, StagePlan& sp, const void* x, int B, int hw
   if (timed) record(m, sp, st, "head_gap");
   DecideArgs da{shift, shift_cls, sp.threshold, sp.always_exit, out->conf, out->pred, out->exit_mask,
                 in_ids ? in_ids->ids : nullptr, out->survivor_idx, out->ids_out, out->n_surv_dev, cnt, cnt + m->max_batch, host_count};
-  if (fc_cluster_supported(B, C, K, (int)sizeof(T), sp.fc_w))
-    EE_CUDA(fc_cluster_launch<T>(gap, (const T*)sp.fc_w, sp.fc_b, B, C, K, out->logits, da, st));
+  if (sp.fc_cluster)
+    EE_CUDA(fc_cluster_launch<T>(fc_shape(B, C, K, (int)sizeof(T), m->fc_room), gap, sp.tm_fc, sp.fc_b, B, C, K, out->logits,
+                                 (float4*)(scratch + h.off_z), da, m->err_flag, st));
   else
     EE_CUDA(launch_pdl(fc_kernel<T>, dim3(cdiv(K, kFcClasses), cdiv(B, kFcSamples)), dim3(kFcThreads), st, (const float*)gap, (const T*)sp.fc_w,
                        (const float*)sp.fc_b, B, C, K, z, da));
@@ -786,6 +790,7 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
   if (rc == EE_OK) rc = f32_context_init();
   if (rc == EE_OK && (hc_context_init() != cudaSuccess || fc_context_init() != cudaSuccess)) rc = EE_ERR_CUDA;
   if (rc != EE_OK) return fail(rc);
+  m->fc_room = fc_room();
 
   int h = desc->in_h, w = desc->in_w, c = desc->in_c;
   bool in_rev = false;   // direction in which the stage input was last walked (by the gather of the stage before)
@@ -1099,6 +1104,12 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
       if (L.kind == KK_TC && !L.tc.gather && !L.tc.halo) m->pair_counter_words = std::max(m->pair_counter_words, pair_counter_words(L.tc, desc->max_batch));
     if ((rc = upload_bytes(m, sd.fc_weight, (size_t)sd.n_classes * sp.out_c * es, ondev, st, &sp.fc_w)) != EE_OK) return fail(rc);
     if ((rc = upload<float>(m, sd.fc_bias, sd.n_classes, ondev, st, &sp.fc_b)) != EE_OK) return fail(rc);
+    sp.fc_cluster = fc_cluster_supported(sp.out_c, sd.n_classes, (int)es, sp.fc_w);
+    if (sp.fc_cluster) {
+      rc = desc->dtype == EE_BF16 ? fc_weight_map<bf16>(m->tc, sp.fc_w, sp.out_c, sd.n_classes, &sp.tm_fc)
+                                  : fc_weight_map<float>(m->tc, sp.fc_w, sp.out_c, sd.n_classes, &sp.tm_fc);
+      if (rc != EE_OK) return fail(rc);
+    }
     h = sp.out_h, w = sp.out_w, c = sp.out_c;
   }
   {

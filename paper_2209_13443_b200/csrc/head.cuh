@@ -11,7 +11,7 @@
 // All reductions run in a fixed order that depends on the layer shape only, never on the
 // batch size or on scheduling, so a sample's logits are bit-identical in any batch.
 #pragma once
-#include "common.cuh"
+#include "conv_tc.cuh"
 
 namespace ee {
 
@@ -304,22 +304,24 @@ __device__ __forceinline__ void exit_scan(int B, const DecideArgs& d) {
   }
 }
 
-// The FC layer, softmax top-1, threshold and survivor scan of a batch of pooled vectors, in clusters of CL CTAs: one
-// cluster per tile of S samples, z[b][k] = bfc[k] + sum_c wfc[k][c] * gap[b][c].
+// The FC layer, softmax top-1, threshold and survivor scan of a batch of pooled vectors: CL CTAs per tile of S samples,
+// z[b][k] = bfc[k] + sum_c wfc[k][c] * gap[b][c].
 //
 // The layer is a few MFLOP over at most a few MB of weights, so nothing but latency bounds it.  Every wait on another
-// SM through global memory costs about a microsecond, so a tile's CTAs exchange what the decision needs through
-// distributed shared memory (one cluster barrier), and the weights, which no kernel writes, are on their way into
+// SM through global memory costs about a microsecond, so a tile's CTAs form a cluster and exchange what the decision
+// needs through distributed shared memory (one cluster barrier), and the weights, which no kernel writes, are on their way into
 // shared memory before the kernel waits for the pooled vectors.
 //   1. The classes are cut into 16 blocks of kb (a multiple of 8), CTA r owns 16 / CL of them.  A warp takes groups of eight
-//      classes: its weights stream through a ring of its own, [8 classes][512 bytes of channels] per slot, filled by
-//      cp.async kFcRing - 1 slots ahead; no barrier but __syncwarp inside the loop.  A lane adds its 16 bytes of channels
+//      classes: its weights stream through a ring of its own, [8 classes][512 bytes of channels] per slot, one TMA box
+//      each (as eight row copies a slot took 1200 clocks), requested kFcRing - 1 slots ahead; no barrier across warps.  A lane adds its 16 bytes of channels
 //      of every slot in ascending order, then a halving butterfly (distances 16, 8, ..., 1) forms all 8 S sums at once:
 //      the tree of a sum does not depend on S, so a logit is the same bits in any batch.
-//   2. Per (sample, block): maximum, lowest argmax and sum of exp(z - max) go into the leader CTA's shared memory.
+//   2. Per (sample, block): maximum, lowest argmax and sum of exp(z - max) go into the leader CTA's shared memory.  More tiles
+//      than clusters fit side by side: no clusters, the triples go through global memory and the CTA that finishes a tile
+//      last is its leader.
 //   3. The leader adds the 16 triples in a fixed order: conf = 1 / sum_r s_r exp(m_r - m), exit = always || conf >= thr (NaN
 //      never exits).  With several tiles the leader that finishes last runs the stable scan over the batch.
-// No wait spins.  Launched with programmatic stream serialization.  Measured on B200 (pooling kernel + this kernel, one
+// Waits on copies are bounded.  Launched with programmatic stream serialization.  Measured on B200 (pooling kernel + this kernel, one
 // graph): see fc_shape.
 constexpr int kFcMaxSmem = 226 * 1024;   // dynamic; the scan's static arrays come on top
 constexpr int kFcThreads = 256, kFcRing = 4, kFcBlocks = 16, kFcRows = 8, kFcSlot = kFcRows * 512;
@@ -341,18 +343,22 @@ __device__ __forceinline__ void hc_cluster_arrive() { asm volatile("barrier.clus
 __device__ __forceinline__ void hc_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 struct FcShape {
-  int S, CL;     // samples per tile, CTAs per cluster
+  int S, CL;     // samples per tile, CTAs per tile
+  int cluster;   // 1: the CTAs of a tile are a cluster; 0: they exchange through global memory (or CL is 1)
   int kb;        // classes per block
   int Cp;        // channels rounded up to whole ring slots
 };
-// Samples per tile: few, so that a CTA's arithmetic stays below the time its weights need and the tiles fill the GPU.  Cluster: 64 classes per CTA while few tiles leave SMs idle (16 CTAs need the non-portable
-// size), 128 otherwise; fewer CTAs for few classes.  Neither changes a sum.
-inline FcShape fc_shape(int B, int C, int K, int elem_bytes) {
+// 64 classes per CTA (clusters of 16 need the non-portable size), fewer CTAs for few classes.  Samples per tile: the fewest
+// whose clusters run side by side (`room16` clusters of 16: not every GPC has 16 SMs), up to 8, as a second wave costs the
+// whole kernel once more; past that the same tiles without clusters, 128 CTAs for 64 samples.  What bounds a CTA is then
+// its FMAs and its shared memory, which every weight crosses twice per tile.  Nothing here changes a sum.
+inline FcShape fc_shape(int B, int C, int K, int elem_bytes, int room16) {
   FcShape f;
-  f.S = B <= 4 ? 1 : B <= 16 ? 2 : 4;
-  const int tiles = (B + f.S - 1) / f.S;
   f.CL = 1;
-  while (f.CL < (tiles <= 4 ? 16 : 8) && f.CL * 64 < K) f.CL *= 2;
+  while (f.CL < 16 && f.CL * 64 < K) f.CL *= 2;
+  const int room = std::max(1, room16 * (16 / f.CL)), most = elem_bytes == 4 ? 4 : 8;   // eight fp64 sums per class do not fit the registers
+  f.S = B <= room ? 1 : B <= 2 * room ? 2 : B <= 4 * room ? 4 : most;
+  f.cluster = f.CL > 1 && ((B + f.S - 1) / f.S <= room || f.CL < 16);
   f.kb = ((K + kFcBlocks - 1) / kFcBlocks + kFcRows - 1) / kFcRows * kFcRows;
   const int chunk = 512 / elem_bytes;
   f.Cp = (C + chunk - 1) / chunk * chunk;
@@ -360,11 +366,14 @@ inline FcShape fc_shape(int B, int C, int K, int elem_bytes) {
 }
 inline size_t fc_smem_bytes(const FcShape& f) {
   return (size_t)(kFcThreads / 32) * kFcRing * kFcSlot + (size_t)f.S * f.Cp * 4 + (size_t)f.S * (kFcBlocks / f.CL) * f.kb * 4 +
-         (size_t)kFcBlocks * f.S * 16;
+         (size_t)kFcBlocks * f.S * 16 + (kFcThreads / 32) * kFcRing * 8;
 }
-// C in whole 16-byte vectors of both operands, shared memory for the pooled tile and the logits of a CTA.
-inline bool fc_cluster_supported(int B, int C, int K, int elem_bytes, const void* wfc) {
-  return C % (16 / elem_bytes) == 0 && ((uintptr_t)wfc & 15) == 0 && fc_smem_bytes(fc_shape(B, C, K, elem_bytes)) <= (size_t)kFcMaxSmem;
+// C in whole 16-byte vectors (a row of the weights is then a multiple of 16 bytes), shared memory for the pooled tile and
+// the logits of a CTA.
+inline bool fc_cluster_supported(int C, int K, int elem_bytes, const void* wfc) {
+  FcShape f = fc_shape(1, C, K, elem_bytes, 1);
+  f.S = elem_bytes == 4 ? 4 : 8;
+  return C % (16 / elem_bytes) == 0 && ((uintptr_t)wfc & 15) == 0 && fc_smem_bytes(f) <= (size_t)kFcMaxSmem;
 }
 
 __device__ __forceinline__ void fc_fma2(float (&a)[2], float w0, float w1, float g0, float g1) {   // two independent FMAs, one instruction
@@ -380,45 +389,55 @@ __device__ __forceinline__ void fc_fma2(double (&a)[2], float w0, float w1, floa
 
 template <typename T, int S>
 __global__ void __launch_bounds__(kFcThreads)
-fc_cluster_kernel(const float* __restrict__ gap, const T* __restrict__ wfc, const float* __restrict__ bfc, int B, int C, int K, float* z,
-                  DecideArgs d, FcShape f) {
+fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restrict__ gap, const float* __restrict__ bfc, int B, int C, int K,
+                  float* z, float4* exchange, DecideArgs d, FcShape f, int* err_flag) {
   typedef typename Accum<T>::type A;                        // fp64 sums for the fp32 model
-  constexpr int VEC = 16 / (int)sizeof(T), CHUNK = 32 * VEC, NV = kFcRows * S;
-  extern __shared__ __align__(16) uint8_t fc_smem[];
+  constexpr int VEC = 16 / (int)sizeof(T), CHUNK = 32 * VEC, NV = kFcRows * S, WARPS = kFcThreads / 32;
+  extern __shared__ __align__(128) uint8_t fc_smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint8_t* ring = fc_smem + (size_t)warp * kFcRing * kFcSlot;                             // this warp's slots
-  float* gs = reinterpret_cast<float*>(fc_smem + (size_t)(kFcThreads / 32) * kFcRing * kFcSlot);   // [S][Cp] pooled vectors
+  float* gs = reinterpret_cast<float*>(fc_smem + (size_t)WARPS * kFcRing * kFcSlot);      // [S][Cp] pooled vectors, see below
   const int my_blocks = kFcBlocks / f.CL, kc = my_blocks * f.kb;
   float* zs = gs + (size_t)S * f.Cp;                                                      // [S][kc] this CTA's logits
   float* part = zs + (size_t)S * kc;                                                      // [16][S][4] (leader): max, argmax, sum
-  const uint32_t rank = hc_cluster_rank();
+  const uint32_t bars = smem_u32(part + kFcBlocks * S * 4) + (uint32_t)(warp * kFcRing * 8);   // this warp's slot barriers
+  const uint32_t rank = blockIdx.x % (unsigned)f.CL;   // also the CTA's rank in its cluster
   const int tile = (int)blockIdx.x / f.CL, tiles = (int)gridDim.x / f.CL, b0 = tile * S;
   const int k0 = (int)rank * kc;
   const int nchunk = f.Cp / CHUNK, ngroups = max(0, min(kc, K - k0) + kFcRows - 1) / kFcRows;
-  const int T_w = warp < ngroups ? ((ngroups - 1 - warp) / (kFcThreads / 32) + 1) * nchunk : 0;   // ring slots this warp consumes
+  const int my_groups = warp < ngroups ? (ngroups - 1 - warp) / WARPS + 1 : 0, slots = my_groups * nchunk;
 
-  if (f.CL > 1) hc_cluster_arrive();   // #1: every CTA of the cluster runs (waited for before the first remote store)
-  auto load = [&](int t) {
-    if (t < T_w) {
-      const int g = warp + (t / nchunk) * (kFcThreads / 32), c = (t % nchunk) * CHUNK + lane * VEC;
-      uint8_t* dst = ring + (size_t)(t % kFcRing) * kFcSlot + lane * 16;
+  if (f.cluster) hc_cluster_arrive();   // #1: every CTA of the cluster runs (waited for before the first remote store)
+  if (lane == 0) {
 #pragma unroll
-      for (int r = 0; r < kFcRows; ++r) {
-        const int k = k0 + g * kFcRows + r;
-        const bool in = k < K && c < C;
-        cp_async16(dst + r * 512, in ? wfc + (size_t)k * C + c : wfc, in ? 16 : 0);
+    for (int i = 0; i < kFcRing; ++i) mbar_init(bars + 8u * i, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncwarp();
+  // slot lt of this warp: classes of group lg, channels of chunk lc; classes past K and channels past C arrive as zeros
+  int lt = 0, lg = warp, lc = 0;
+  auto load = [&]() {
+    if (lt < slots) {
+      if (lane == 0) {
+        const uint32_t bar = bars + 8u * (lt % kFcRing);
+        mbar_expect_tx(bar, kFcSlot);
+        tma_load_2d(smem_u32(ring + (lt % kFcRing) * kFcSlot), &tmW, bar, lc * CHUNK, k0 + lg * kFcRows);
       }
+      if (++lc == nchunk) lc = 0, lg += WARPS;
     }
-    cp_async_commit();
+    ++lt;
   };
 #pragma unroll
-  for (int t = 0; t < kFcRing - 1; ++t) load(t);
+  for (int t = 0; t < kFcRing - 1; ++t) load();
   pdl_wait();
   pdl_launch_dependents();
+  // pooled vectors: within a chunk the float4 `e` of lane l's VEC channels sits at [e][l], so that a warp's reads are 512
+  // consecutive bytes
   for (int i = tid; i < S * (f.Cp / 4); i += kFcThreads) {
-    const int s = i / (f.Cp / 4), c = (i % (f.Cp / 4)) * 4;
+    const int s = i / (f.Cp / 4), c4 = i - s * (f.Cp / 4), c = c4 * 4;
+    const int ch = c / CHUNK, l = (c % CHUNK) / VEC, e = (c % VEC) / 4;
     const bool in = b0 + s < B && c < C;
-    cp_async16(gs + (size_t)s * f.Cp + c, in ? gap + (size_t)(b0 + s) * C + c : gap, in ? 16 : 0);
+    cp_async16(gs + (size_t)s * f.Cp + ch * CHUNK + (e * 32 + l) * 4, in ? gap + (size_t)(b0 + s) * C + c : gap, in ? 16 : 0);
   }
   cp_async_commit();
   cp_async_wait<0>();
@@ -429,29 +448,33 @@ fc_cluster_kernel(const float* __restrict__ gap, const T* __restrict__ wfc, cons
   for (int q = 0; q < kFcRows; ++q)
 #pragma unroll
     for (int s = 0; s < S; ++s) acc[q][s][0] = acc[q][s][1] = (A)0;
-  for (int t = 0; t < T_w; ++t) {
-    cp_async_wait<kFcRing - 2>();
-    __syncwarp();           // slot t has landed for every lane; the slot refilled below was read one step ago
-    load(t + kFcRing - 1);
-    const int ch = t % nchunk;
-    const uint8_t* slot = ring + (size_t)(t % kFcRing) * kFcSlot + lane * 16;
-    float gv[S][VEC];
-#pragma unroll
-    for (int s = 0; s < S; ++s)
-#pragma unroll
-      for (int e = 0; e < VEC; e += 4) {
-        const float4 v = *reinterpret_cast<const float4*>(gs + (size_t)s * f.Cp + ch * CHUNK + lane * VEC + e);
-        gv[s][e] = v.x, gv[s][e + 1] = v.y, gv[s][e + 2] = v.z, gv[s][e + 3] = v.w;
-      }
-#pragma unroll
-    for (int q = 0; q < kFcRows; ++q) {
-      Vec16<T> w;
-      w.load(reinterpret_cast<const T*>(slot + q * 512));
+  int ch = 0, grp = warp;
+  bool ok = true;
+  for (int t = 0; t < slots; ++t) {
+    __syncwarp();           // every lane is done with the slot refilled next
+    if (ok) load();
+    ok = ok && mbar_wait(bars + 8u * (t % kFcRing), (uint32_t)(t / kFcRing) & 1u, err_flag);
+    const uint8_t* slot = ring + (t % kFcRing) * kFcSlot + lane * 16;
+    if (ok) {
+      float gv[S][VEC];
 #pragma unroll
       for (int s = 0; s < S; ++s)
 #pragma unroll
-        for (int e = 0; e < VEC; e += 2) fc_fma2(acc[q][s], w.v[e], w.v[e + 1], gv[s][e], gv[s][e + 1]);
+        for (int e = 0; e < VEC / 4; ++e) {
+          const float4 v = *reinterpret_cast<const float4*>(gs + (size_t)s * f.Cp + ch * CHUNK + (e * 32 + lane) * 4);
+          gv[s][4 * e] = v.x, gv[s][4 * e + 1] = v.y, gv[s][4 * e + 2] = v.z, gv[s][4 * e + 3] = v.w;
+        }
+#pragma unroll
+      for (int q = 0; q < kFcRows; ++q) {
+        Vec16<T> w;
+        w.load(reinterpret_cast<const T*>(slot + q * 512));
+#pragma unroll
+        for (int s = 0; s < S; ++s)
+#pragma unroll
+          for (int e = 0; e < VEC; e += 2) fc_fma2(acc[q][s], w.v[e], w.v[e + 1], gv[s][e], gv[s][e + 1]);
+      }
     }
+    __syncwarp();
     if (ch == nchunk - 1) {   // the group's sums are complete: all 8 S of them in one halving butterfly
       A v[NV];
 #pragma unroll
@@ -480,16 +503,17 @@ fc_cluster_kernel(const float* __restrict__ gap, const T* __restrict__ wfc, cons
       constexpr int LEFT = NV > 32 ? NV / 32 : 1, REP = NV < 32 ? 32 / NV : 1;   // values per lane, lanes per value
 #pragma unroll
       for (int j = 0; j < LEFT; ++j) {
-        const int idx = (lane / REP) * LEFT + j, s = idx / kFcRows, kl = (warp + (t / nchunk) * (kFcThreads / 32)) * kFcRows + idx % kFcRows;
+        const int idx = (lane / REP) * LEFT + j, s = idx / kFcRows, kl = grp * kFcRows + idx % kFcRows;
         if (lane % REP == 0) zs[s * kc + kl] = (float)(v[j] + (A)((bfc && k0 + kl < K) ? bfc[k0 + kl] : 0.f));
       }
+      grp += WARPS;
     }
+    if (++ch == nchunk) ch = 0;
   }
-  cp_async_wait<0>();
   __syncthreads();
 
   // ---- 2. one warp per (block, sample)
-  if (f.CL > 1) hc_cluster_wait();   // #1
+  if (f.cluster) hc_cluster_wait();   // #1
   for (int it = warp; it < my_blocks * S; it += kFcThreads / 32) {
     const int s = it % S, bl = it / S, b = b0 + s, kf = k0 + bl * f.kb;
     const int nk = max(0, min(f.kb, K - kf));
@@ -516,18 +540,34 @@ fc_cluster_kernel(const float* __restrict__ gap, const T* __restrict__ wfc, cons
       for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     }
     if (lane == 0) {
-      float* mine = part + ((size_t)((int)rank * my_blocks + bl) * S + s) * 4;
-      hc_st_f32(hc_map(mine, 0), m);
-      hc_st_f32(hc_map(mine + 1, 0), __int_as_float(arg));
-      hc_st_f32(hc_map(mine + 2, 0), sum);
+      const int at = ((int)rank * my_blocks + bl) * S + s;
+      if (f.cluster || f.CL == 1) {
+        float* mine = part + (size_t)at * 4;
+        hc_st_f32(hc_map(mine, 0), m);
+        hc_st_f32(hc_map(mine + 1, 0), __int_as_float(arg));
+        hc_st_f32(hc_map(mine + 2, 0), sum);
+      } else {
+        __stcg(exchange + (size_t)tile * kFcBlocks * S + at, make_float4(m, __int_as_float(arg), sum, 0.f));
+      }
     }
   }
-  if (f.CL > 1) {
+  if (f.cluster) {
     hc_cluster_arrive();   // #2: the leader holds every block's triple
     hc_cluster_wait();
     if (rank != 0) return;
   } else {
+    if (f.CL > 1) __threadfence();
     __syncthreads();
+    if (f.CL > 1) {
+      int* last = reinterpret_cast<int*>(zs);
+      if (tid == 0) *last = atomicAdd(d.tile_done + tile, 1u) == (unsigned)(f.CL - 1) ? 1 : 0;
+      __syncthreads();
+      if (!*last) return;
+      __threadfence();
+      if (tid == 0) d.tile_done[tile] = 0;
+      for (int i = tid; i < kFcBlocks * S; i += kFcThreads) reinterpret_cast<float4*>(part)[i] = __ldcg(exchange + (size_t)tile * kFcBlocks * S + i);
+      __syncthreads();
+    }
   }
   // ---- 3. decision: one warp per sample, lane r holds block r
   if (warp < S && b0 + warp < B) {
@@ -569,8 +609,8 @@ fc_cluster_kernel(const float* __restrict__ gap, const T* __restrict__ wfc, cons
 }
 
 template <typename T, int S>
-inline cudaError_t fc_cluster_launch_t(const float* gap, const T* wfc, const float* bfc, int B, int C, int K, float* z, const DecideArgs& d,
-                                       const FcShape& f, cudaStream_t st) {
+inline cudaError_t fc_cluster_launch_t(const float* gap, const CUtensorMap& wfc, const float* bfc, int B, int C, int K, float* z,
+                                       float4* exchange, const DecideArgs& d, const FcShape& f, int* err_flag, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((B + S - 1) / S * f.CL));
   cfg.blockDim = dim3(kFcThreads);
@@ -583,19 +623,21 @@ inline cudaError_t fc_cluster_launch_t(const float* gap, const T* wfc, const flo
   attr[1].val.clusterDim.x = f.CL;
   attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, fc_cluster_kernel<T, S>, gap, wfc, bfc, B, C, K, z, d, f);
+  cfg.numAttrs = f.cluster ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, fc_cluster_kernel<T, S>, wfc, gap, bfc, B, C, K, z, exchange, d, f, err_flag);
 }
-// d.done must be zero when the kernel starts and is zero again when it ends.
+// d.done and d.tile_done must be zero when the kernel starts and are zero again when it ends.  exchange: 16 float4 per sample
+// of every tile, less than the batch's logits take wherever it is used (more than 512 classes).
 template <typename T>
-inline cudaError_t fc_cluster_launch(const float* gap, const T* wfc, const float* bfc, int B, int C, int K, float* z, const DecideArgs& d,
-                                     cudaStream_t st) {
-  const FcShape f = fc_shape(B, C, K, (int)sizeof(T));
+inline cudaError_t fc_cluster_launch(const FcShape& f, const float* gap, const CUtensorMap& wfc, const float* bfc, int B, int C, int K, float* z,
+                                     float4* exchange, const DecideArgs& d, int* err_flag, cudaStream_t st) {
   switch (f.S) {
-    case 1: return fc_cluster_launch_t<T, 1>(gap, wfc, bfc, B, C, K, z, d, f, st);
-    case 2: return fc_cluster_launch_t<T, 2>(gap, wfc, bfc, B, C, K, z, d, f, st);
-    default: return fc_cluster_launch_t<T, 4>(gap, wfc, bfc, B, C, K, z, d, f, st);
+    case 1: return fc_cluster_launch_t<T, 1>(gap, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, st);
+    case 2: return fc_cluster_launch_t<T, 2>(gap, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, st);
+    case 4: return fc_cluster_launch_t<T, 4>(gap, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, st);
   }
+  if constexpr (sizeof(T) == 2) return fc_cluster_launch_t<T, 8>(gap, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, st);
+  return cudaErrorInvalidValue;
 }
 template <typename T, int S>
 inline cudaError_t fc_cluster_attr() {
@@ -605,10 +647,42 @@ inline cudaError_t fc_cluster_attr() {
 }
 inline cudaError_t fc_context_init() {
   cudaError_t e = cudaSuccess;
-  for (cudaError_t r : {fc_cluster_attr<bf16, 1>(), fc_cluster_attr<bf16, 2>(), fc_cluster_attr<bf16, 4>(), fc_cluster_attr<float, 1>(),
+  for (cudaError_t r : {fc_cluster_attr<bf16, 1>(), fc_cluster_attr<bf16, 2>(), fc_cluster_attr<bf16, 4>(), fc_cluster_attr<bf16, 8>(), fc_cluster_attr<float, 1>(),
                         fc_cluster_attr<float, 2>(), fc_cluster_attr<float, 4>()})
     if (e == cudaSuccess) e = r;
   return e;
+}
+
+// Clusters of 16 of this kernel that run side by side on the current device (a GPC with fewer than 16 SMs holds none).
+inline int fc_room() {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(16 * 16);
+  cfg.blockDim = dim3(kFcThreads);
+  cfg.dynamicSmemBytes = kFcMaxSmem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 16, attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, fc_cluster_kernel<bf16, 8>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 4;
+  }
+  return std::max(1, n);
+}
+// FC weights [K][C] as boxes of eight classes x 512 bytes of channels.
+template <typename T>
+inline ee_status_t fc_weight_map(const TcContext& c, const void* w, int C, int K, CUtensorMap* out) {
+  const cuuint64_t dims[2] = {(cuuint64_t)C, (cuuint64_t)K};
+  const cuuint64_t strides[1] = {(cuuint64_t)C * sizeof(T)};
+  const cuuint32_t box[2] = {512 / sizeof(T), kFcRows};
+  const cuuint32_t es[2] = {1, 1};
+  return c.encode_tiled(out, sizeof(T) == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(w), dims,
+                        strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+             ? EE_OK
+             : EE_ERR_CUDA;
 }
 
 // The same layer for any C, K and alignment (channels that are not whole 16-byte vectors, very many classes): CTA (x, y)

@@ -38,13 +38,6 @@ constexpr int kDwConsumers = 256;
 constexpr int kDwThreads = 32 + kDwConsumers;
 constexpr int kDwMaxTileBytes = 72 * 1024;
 
-__device__ __forceinline__ void tma_load_4d_tile(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1, int c2, int c3) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-      ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-      : "memory");
-}
-
 // POOL: the same staging for a 3x3 pad-1 window maximum (the max-pool behind a ResNet-style stem): taps outside the
 // image are skipped (the frame's zeros must not win against negative inputs), no weights, no epilogue arithmetic.
 template <int STRIDE, bool POOL>
@@ -84,7 +77,7 @@ dwconv3x3_tma_kernel(const __grid_constant__ CUtensorMap tmX, DwParams p) {
         const int s = j % kDwStages;
         if (!mbar_wait(empty(s), ((uint32_t)(j / kDwStages) & 1u) ^ 1u, p.err_flag)) break;
         mbar_expect_tx(full(s), (uint32_t)p.tile_bytes);
-        tma_load_4d_tile(base + (uint32_t)(s * p.slot_bytes), &tmX, full(s), c0, -1, band * p.RB * STRIDE - 1, b);
+        tma_load_4d(base + (uint32_t)(s * p.slot_bytes), &tmX, full(s), c0, -1, band * p.RB * STRIDE - 1, b);
       }
     }
     return;

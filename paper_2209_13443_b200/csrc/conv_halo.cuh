@@ -52,13 +52,6 @@ struct HaloSmem {
   static_assert(kBytes <= 227 * 1024, "exceeds the shared memory of an SM");
 };
 
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1, int c2, int c3) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-      ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-      : "memory");
-}
-
 // A descriptor may start at any 128-byte row of a swizzled block, not only at a multiple of 1024 bytes: the TMA unit
 // and the tensor core both derive the 16-byte chunk permutation from the shared-memory address itself (address
 // bits 7-9 select the permutation of bits 4-6), so a view shifted by whole rows finds every chunk where the load put
@@ -118,26 +111,29 @@ conv3x3_halo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t block_bytes = (uint32_t)(p.Wp * (p.R + 2) * 128);
+      int s = 0;
+      uint32_t ph = 1;
       for (int j = 0; j < my_tiles; ++j) {
         const int tf = (int)blockIdx.x + j * (int)gridDim.x, t = p.rev ? p.tiles - 1 - tf : tf;
         const int n = t / p.tiles_per_img, h0 = (t - n * p.tiles_per_img) * p.R;
-        const int s = j % kHaloStages;
-        const uint32_t ph = (uint32_t)(j / kHaloStages) & 1u;
-        if (!mbar_wait(a_empty(s), ph ^ 1u, p.err_flag)) break;
+        if (!mbar_wait(a_empty(s), ph, p.err_flag)) break;
         mbar_expect_tx(a_full(s), block_bytes);
         tma_load_4d(base + S::kAOff + (uint32_t)s * kHaloBlockBytes, &tmX, a_full(s), 0, -1, h0 - 1, n);
+        if (++s == kHaloStages) s = 0, ph ^= 1u;
       }
     }
+    __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc = umma_idesc(64);
+      const uint64_t da0 = umma_desc(base + S::kAOff), db0 = umma_desc(base + S::kWOff);
       bool ok = my_tiles > 0 ? mbar_wait(w_bar, 0, p.err_flag) : true;
+      int s = 0;
+      uint32_t ph = 0;
       for (int j = 0; j < my_tiles && ok; ++j) {
         const int b = j & 1;
-        const int s = j % kHaloStages;
-        const uint32_t ph = (uint32_t)(j / kHaloStages) & 1u;
         if (j >= 2) {  // the epilogue must have drained this accumulator (tile j - 2)
           ok = mbar_wait(acc_empty(b), (uint32_t)((j >> 1) - 1) & 1u, p.err_flag);
           if (!ok) break;
@@ -145,20 +141,19 @@ conv3x3_halo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
         ok = mbar_wait(a_full(s), ph, p.err_flag);
         if (!ok) break;
         tc_fence_after();
-        const uint32_t acc = tmem_base + (uint32_t)(b * 64);
-        const uint32_t sa = base + S::kAOff + (uint32_t)s * kHaloBlockBytes;
+        const uint64_t da = da0 + (uint64_t)(s * (kHaloBlockBytes >> 4));
 #pragma unroll
-        for (int tap = 0; tap < kHaloTaps; ++tap) {
-          const uint32_t a_tap = sa + (uint32_t)(((tap / 3) * p.Wp + (tap % 3)) * 128);
-          const uint32_t w_tap = base + S::kWOff + tap * kHaloWTapBytes;
-#pragma unroll
-          for (int k = 0; k < kTcBK / 16; ++k)
-            umma_bf16(acc, umma_desc(a_tap + k * 32), umma_desc(w_tap + k * 32), idesc, (uint32_t)((tap | k) != 0));
+        for (int i = 0; i < kHaloTaps; ++i) {
+          const int tap = i % 3 * 3 + i / 3;   // filter columns outermost: the order of TapWalk
+          umma_block(tmem_base + (uint32_t)(b * 64), da + (uint64_t)(((tap / 3) * p.Wp + (tap % 3)) * 8), db0 + (uint64_t)(tap * (kHaloWTapBytes >> 4)),
+                     idesc, i != 0);
         }
         umma_commit(a_empty(s));    // frees the block once these MMAs have read it
         umma_commit(acc_full(b));
+        if (++s == kHaloStages) s = 0, ph ^= 1u;
       }
     }
+    __syncwarp();
   } else {
     const int et = threadIdx.x - 64;  // 0..127
     if (et < 64) {

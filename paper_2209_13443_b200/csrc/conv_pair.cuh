@@ -32,7 +32,7 @@ constexpr int kPairEpiWarps = 8;
 
 struct PairParams {
   int M, N;             // valid rows (B*Ho*Wo) and Cout
-  int taps, kw;         // kh*kw and kw
+  int taps, kh, kw;     // kh*kw, kh and kw
   int cblocks;          // ceil(Cin / 64)
   int Ho, Wo, stride, pad, pad_w;
   int im2col;           // 0: A is a plain [rows][Cin] matrix, 1: im2col tensor map
@@ -266,22 +266,21 @@ conv_igemm_tcgen05_pair_kernel(const __grid_constant__ PairStageArgs A) {
           auto arm_and_load_w = [&](int kb, int gg) -> bool {
             const int s = gg % kStages;
             const uint32_t ph = (uint32_t)(gg / kStages) & 1u;
-            const int tap = kb / p.cblocks, cb = kb - tap * p.cblocks;
+            const TapWalk t(p.kh, p.kw, p.stride, kb);
             if (!mbar_wait_for(empty_bar(s), ph ^ 1u, err_flag, limit)) return false;
             if (rank == 0) mbar_expect_tx(full_bar(s), (uint32_t)(2 * S::kBBytes + S::kABytes + (peer_rows ? S::kABytes : 0)));
-            tma2_load_3d(base + (uint32_t)s * S::kStage + S::kABytes, tmW, map_to_rank(full_bar(s), 0), cb * kTcBK, tap, nb0);
+            tma2_load_3d(base + (uint32_t)s * S::kStage + S::kABytes, tmW, map_to_rank(full_bar(s), 0), t.cb * kTcBK, t.tap(), nb0);
             return true;
           };
           auto load_a = [&](int kb, int gg) {
             if (!rows) return;
             const int s = gg % kStages;
-            const int tap = kb / p.cblocks, cb = kb - tap * p.cblocks;
+            const TapWalk t(p.kh, p.kw, p.stride, kb);
             const uint32_t sa = base + (uint32_t)s * S::kStage, fb = map_to_rank(full_bar(s), 0);
             if (p.im2col) {
-              const int r = tap / p.kw;
-              tma2_load_im2col_4d(sa, tmA, fb, cb * kTcBK, cw, ch, cn, (uint16_t)(tap - r * p.kw), (uint16_t)r);
+              tma2_load_im2col_4d(sa, tmA, fb, t.cb * kTcBK, cw, ch, cn, (uint16_t)t.s, (uint16_t)t.r);
             } else {
-              tma2_load_2d(sa, tmA, fb, cb * kTcBK, m0);
+              tma2_load_2d(sa, tmA, fb, t.cb * kTcBK, m0);
             }
           };
           int kb = kb_begin;
@@ -612,7 +611,7 @@ inline ee_status_t pair_fill_layer(TcContext& c, const TcLayer& L, int bn, const
   p.M = B * L.out_h * L.out_w;
   p.N = L.cout;
   p.taps = L.kh * L.kw;
-  p.kw = L.kw;
+  p.kh = L.kh, p.kw = L.kw;
   p.cblocks = cdiv(L.cin, kTcBK);
   p.Ho = L.out_h, p.Wo = L.out_w, p.stride = L.stride, p.pad = L.pad, p.pad_w = L.pad_w;
   p.im2col = L.im2col ? 1 : 0;

@@ -183,28 +183,27 @@ conv_stem7x7_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
       });
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc = umma_idesc(64);
+      const uint64_t da0 = umma_desc(base + S::kAOff), db0 = umma_desc(base + S::kWOff);
       if (mbar_wait(w_bar, 0, p.err_flag))
         stem_walk<POOL>(p, [&](int j, int, int, bool, bool, int) {
           const int b = j & 1;
           // the epilogue must have drained this accumulator (row j - 2)
           if (j >= 2 && !mbar_wait(acc_empty(b), (uint32_t)((j >> 1) - 1) & 1u, p.err_flag)) return false;
           tc_fence_after();
-          const uint32_t acc = tmem_base + (uint32_t)(b * 64);
 #pragma unroll
           for (int i = 0; i < kStemKBlocks; ++i) {
             if (!mbar_wait(a_full(i), (uint32_t)j & 1u, p.err_flag)) return false;
             tc_fence_after();
-            const uint32_t sa = base + S::kAOff + i * S::kABytes, sb = base + S::kWOff + i * S::kWBytes;
-#pragma unroll
-            for (int k = 0; k < kTcBK / 16; ++k) umma_bf16(acc, umma_desc(sa + k * 32), umma_desc(sb + k * 32), idesc, (uint32_t)((i | k) != 0));
+            umma_block(tmem_base + (uint32_t)(b * 64), da0 + (uint64_t)(i * (S::kABytes >> 4)), db0 + (uint64_t)(i * (S::kWBytes >> 4)), idesc, i != 0);
             umma_commit(a_empty(i));   // the gather warps may rebuild this K block for the next output row
           }
           umma_commit(acc_full(b));
           return true;
         });
     }
+    __syncwarp();
   } else if (warp < 6) {
     // gather warps: thread r builds row r (output pixel ox = r) of every K block of A
     const int r = (int)threadIdx.x - 64;

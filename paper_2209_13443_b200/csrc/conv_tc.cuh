@@ -11,8 +11,8 @@
 // TMA loads into a ring of shared-memory slots, warp 1 owns the TMEM allocation and issues the MMAs (one thread),
 // the remaining warps run the epilogue: tcgen05.ld of the fp32 accumulator, folded-BN scale/bias, residual add (the
 // residual tile was brought into shared memory by TMA while the main loop ran), activation, one rounding to bf16,
-// then a TMA store of the tile from shared memory.  The K loop visits (tap, channel block) in a fixed order that
-// does not depend on the batch size.  Variants (chosen per launch from the grid size, see tc_launch): shallow or
+// then a TMA store of the tile from shared memory.  The K loop visits (channel block, tap) in a fixed order that
+// does not depend on the batch size (tap_at).  Variants (chosen per launch from the grid size, see tc_launch): shallow or
 // deep ring, cluster split-K with a reduce-scatter through distributed shared memory, gather-mode A operand for
 // 3-channel stems, and a persistent kernel with double-buffered TMEM accumulators for multi-wave 1x1 layers.
 //
@@ -35,7 +35,7 @@ constexpr long long kTcWaitCycles = 4000000000LL;  // ~2 s at boost clock; far b
 
 struct TcParams {
   int M, N;             // valid rows (B*Ho*Wo) and Cout
-  int taps, kw;         // kh*kw and kw
+  int taps, kh, kw;     // kh*kw, kh and kw
   int cblocks;          // ceil(Cin / 64); the TMA unit zero-fills channels past Cin in both operands
   int Ho, Wo, stride, pad, pad_w;   // pad: rows, pad_w: columns
   int im2col;           // 0: A is a plain [rows][Cin] matrix, 1: im2col tensor map
@@ -64,6 +64,34 @@ struct TcParams {
   // pairwise over the rows with distances gap_g/2, ..., 2, 1 - the block sums of gap_blocks_kernel (head.cuh)
   int gap_g;
   float* gap_part;
+};
+
+// Order of a convolution's K blocks, the same in every tensor-core kernel: channel blocks outermost, then filter columns,
+// then filter rows (stride 2: the even rows, then the odd ones), so that consecutive blocks read overlapping input rows
+// (conv_taps.cuh keeps those in shared memory).  Walked by counters: one thread feeds the whole SM, and an integer division
+// by a run-time number is a chain of about 150 clocks in it (two of them per K block were what a K block took).
+struct TapWalk {
+  int kh, kw, step;
+  int r, s, cb;   // filter row and column, channel block
+  __device__ __forceinline__ TapWalk(int kh_, int kw_, int stride, int first) : kh(kh_), kw(kw_), step(stride == 2 ? 2 : 1) {
+    const int taps = kh * kw;
+    cb = first / taps;
+    const int t = first - cb * taps;
+    s = t / kh;
+    const int j = t - s * kh, even = (kh + 1) / 2;
+    r = step == 1 ? j : j < even ? 2 * j : 2 * (j - even) + 1;
+  }
+  __device__ __forceinline__ void next() {
+    r += step;
+    if (r < kh) return;
+    if (step == 2 && (r & 1) == 0 && kh > 1) {
+      r = 1;
+      return;
+    }
+    r = 0;
+    if (++s == kw) s = 0, ++cb;
+  }
+  __device__ __forceinline__ int tap() const { return r * kw + s; }
 };
 
 // ----------------------------------------------------------------------------- PTX wrappers
@@ -98,6 +126,16 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* er
   return true;
 }
 
+// One lane of a converged warp.  A feeding loop runs inside `if (elect_one())`, which tells the compiler that it has one
+// thread: addresses and descriptors live in uniform registers.  With the descriptors stepped instead of rebuilt, no
+// division in the loop and nothing but the barrier test between the blocks, a K block of a 128 x 128 tile takes 267 to 340
+// clocks (257 are its four MMAs) where `if (lane == 0)` took 511, 707 with an im2col coordinate.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}" : "=r"(p));
+  return p != 0;
+}
+
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1) {
   asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
                ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1)
@@ -107,6 +145,12 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm,
   asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
                ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
                : "memory");
+}
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1, int c2, int c3) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+      ::"r"(dst), "l"(tm), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+      : "memory");
 }
 // im2col gather: 128 consecutive output pixels starting at base pixel (w, h, n), channels [c, c+64), filter tap (woff, hoff).
 __device__ __forceinline__ void tma_load_im2col_4d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c, int w, int h, int n,
@@ -140,6 +184,11 @@ __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t da, uint64_t
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
       ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
       : "memory");
+}
+// The four MMAs of a K block: K = 16 each, 32 bytes further into the swizzled rows (2 in the descriptors' address field).
+__device__ __forceinline__ void umma_block(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, bool accumulate) {
+#pragma unroll
+  for (int k = 0; k < kTcBK / 16; ++k) umma_bf16(tmem_d, da + 2 * k, db + 2 * k, idesc, (uint32_t)(accumulate || k != 0));
 }
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -397,7 +446,7 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* tm, uint32_t src
 }
 
 // tmA: activations (2-D tile map or im2col map), tmW: weights [Cin][taps][Cout], tmR / tmO: residual and output as
-// [rows][Cout] matrices with a 64-column x 32-row box (128-byte swizzle).
+// [rows][Cout] matrices with boxes of 64 columns x 128 and 32 rows (128-byte swizzle).
 //
 // SPLIT: the K loop of one output tile is cut into gridDim.z (2 to 8) fixed ranges of p.kb_per K blocks, a
 // property of the layer and never of the batch.  The CTAs of a tile form a thread-block cluster along z.  CTA z owns
@@ -472,26 +521,23 @@ conv_igemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
   // so do the weight tiles of the first ring slots, which no kernel writes.  From the wait on this kernel touches
   // activations, so it needs that kernel's memory; the next kernel in the stream may begin its own prologue now.
   const int w_ahead = min(num_kb, kStages);
-  if (warp == 0 && lane == 0) {
-    for (int i = 0; i < w_ahead; ++i) {   // the slots start out empty
-      const int kb = kb_begin + i;
-      const int tap = kb / p.cblocks, cb = kb - tap * p.cblocks;
+  if (warp == 0 && elect_one()) {
+    TapWalk t(p.kh, p.kw, p.stride, kb_begin);
+    for (int i = 0; i < w_ahead; ++i, t.next()) {   // the slots start out empty
       mbar_expect_tx(full_bar(i), GATHER ? S::kBBytes : S::kStage);
-      tma_load_3d(base + (uint32_t)i * S::kStage + S::kABytes, &tmW, full_bar(i), cb * kTcBK, tap, n0);
+      tma_load_3d(base + (uint32_t)i * S::kStage + S::kABytes, &tmW, full_bar(i), t.cb * kTcBK, t.tap(), n0);
     }
   }
+  __syncwarp();
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       if (RES) {
         mbar_expect_tx(res_bar, S::kIoBytes);
 #pragma unroll
-        for (int h = 0; h < BN / 64; ++h)
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            tma_load_2d(base + S::kIoOff + h * 16384 + q * 4096, &tmR, res_bar, n0 + h * 64, m0 + q * 32);
+        for (int h = 0; h < BN / 64; ++h) tma_load_2d(base + S::kIoOff + h * 16384, &tmR, res_bar, n0 + h * 64, m0);
       }
       int cw = 0, ch = 0, cn = 0;
       if (p.im2col) {
@@ -502,45 +548,47 @@ conv_igemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
         cw = (rem - ho * p.Wo) * p.stride - p.pad_w;
         ch = ho * p.stride - p.pad;
       }
-      for (int i = 0; i < num_kb; ++i) {
-        const int kb = kb_begin + i;
-        const int s = i % kStages;
-        const uint32_t ph = (uint32_t)(i / kStages) & 1u;
-        const int tap = kb / p.cblocks, cb = kb - tap * p.cblocks;
-        const uint32_t sa = base + (uint32_t)s * S::kStage, sb = sa + S::kABytes;
+      TapWalk t(p.kh, p.kw, p.stride, kb_begin);
+      int s = 0;
+      uint32_t ph = 1;
+      for (int i = 0; i < num_kb; ++i, t.next()) {
+        const uint32_t sa = base + (uint32_t)s * S::kStage;
         if (i >= w_ahead) {   // earlier slots: armed and their weight tile requested before the dependency wait
-          if (!mbar_wait(empty_bar(s), ph ^ 1u, p.err_flag)) break;
+          if (!mbar_wait(empty_bar(s), ph, p.err_flag)) break;
           mbar_expect_tx(full_bar(s), GATHER ? S::kBBytes : S::kStage);
-          tma_load_3d(sb, &tmW, full_bar(s), cb * kTcBK, tap, n0);
+          tma_load_3d(sa + S::kABytes, &tmW, full_bar(s), t.cb * kTcBK, t.tap(), n0);
         }
         if (GATHER) {
         } else if (p.im2col) {
-          const int r = tap / p.kw;
-          tma_load_im2col_4d(sa, &tmA, full_bar(s), cb * kTcBK, cw, ch, cn, (uint16_t)(tap - r * p.kw), (uint16_t)r);
+          tma_load_im2col_4d(sa, &tmA, full_bar(s), t.cb * kTcBK, cw, ch, cn, (uint16_t)t.s, (uint16_t)t.r);
         } else {
-          tma_load_2d(sa, &tmA, full_bar(s), cb * kTcBK, m0);
+          tma_load_2d(sa, &tmA, full_bar(s), t.cb * kTcBK, m0);
         }
+        if (++s == kStages) s = 0, ph ^= 1u;
       }
     }
+    __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc = umma_idesc(BN);
+      const uint64_t da0 = umma_desc(base), db0 = umma_desc(base + S::kABytes);
       bool ok = true;
+      int s = 0, ir = 0;           // ring slot; K block within its local range
+      uint32_t ph = 0, acc = tmem_base;
       for (int i = 0; i < num_kb; ++i) {
-        const int s = i % kStages;
-        const uint32_t ph = (uint32_t)(i / kStages) & 1u;
         ok = mbar_wait(full_bar(s), ph, p.err_flag);
         if (!ok) break;
         tc_fence_after();
-        const uint32_t sa = base + (uint32_t)s * S::kStage, sb = sa + S::kABytes;
-        const int r = LOCAL ? i / p.kb_per : 0, ir = i - r * p.kb_per;   // local K range and position inside it
-#pragma unroll
-        for (int k = 0; k < kTcBK / 16; ++k)
-          umma_bf16(tmem_base + (uint32_t)(r * BN), umma_desc(sa + k * 32), umma_desc(sb + k * 32), idesc, (uint32_t)((ir | k) != 0));
+        const uint64_t off = (uint64_t)(s * (S::kStage >> 4));
+        umma_block(acc, da0 + off, db0 + off, idesc, ir != 0);
         umma_commit(empty_bar(s));  // frees the stage once these MMAs have read it
+        ++ir;
+        if (LOCAL && ir == p.kb_per) ir = 0, acc += BN;   // the next local K range has an accumulator of its own
+        if (++s == kStages) s = 0, ph ^= 1u;
       }
       if (ok && num_kb > 0) umma_commit(accum_bar);  // accumulator complete: every MMA has also finished reading the ring
     }
+    __syncwarp();
   } else {
     const int et = threadIdx.x - 64;  // 0..127
     for (int i = et; i < BN; i += 128) {
@@ -768,7 +816,7 @@ conv_igemm_tcgen05_persistent_kernel(const __grid_constant__ CUtensorMap tmA, co
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 8);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int num_kb = p.taps * p.cblocks;
+  const int num_kb = p.cblocks;                // 1x1 layers: one tap
   const int num_kb2 = PROJ ? p.cblocks2 : 0;   // K blocks of the projection (one tap)
   const int n_tiles = (p.N + BN - 1) / BN;
   const int m_tiles = (p.M + kTcBM - 1) / kTcBM;
@@ -809,93 +857,98 @@ conv_igemm_tcgen05_persistent_kernel(const __grid_constant__ CUtensorMap tmA, co
   // weight tiles of the first ring slots (first tile of this CTA) are requested before the dependency wait: no
   // kernel writes them
   const int w_ahead = my_tiles > 0 ? min(num_kb, kStages) : 0;
-  if (warp == 0 && lane == 0) {
-    const int n0 = ((p.rev ? total - 1 - (int)blockIdx.x : (int)blockIdx.x) % n_tiles) * BN;
+  // tiles of this CTA, walked by counters: tile t -> (t / n_tiles, t % n_tiles), + gridDim.x each step (backwards when rev)
+  struct TileWalk {
+    int mt, nt, dm, dn, n_tiles;
+    __device__ __forceinline__ void next() {
+      mt += dm, nt += dn;
+      if (nt >= n_tiles) nt -= n_tiles, ++mt;
+      if (nt < 0) nt += n_tiles, --mt;
+    }
+  };
+  const int t_first = p.rev ? total - 1 - (int)blockIdx.x : (int)blockIdx.x, t_sign = p.rev ? -1 : 1;
+  const TileWalk first_tile{t_first / n_tiles, t_first % n_tiles, t_sign * ((int)gridDim.x / n_tiles), t_sign * ((int)gridDim.x % n_tiles), n_tiles};
+  if (warp == 0 && elect_one()) {
     for (int i = 0; i < w_ahead; ++i) {
-      const int tap = i / p.cblocks, cb = i - tap * p.cblocks;
       mbar_expect_tx(full_bar(i), S::kStage);
-      tma_load_3d(base + (uint32_t)i * S::kStage + S::kABytes, &tmW, full_bar(i), cb * kTcBK, tap, n0);
+      tma_load_3d(base + (uint32_t)i * S::kStage + S::kABytes, &tmW, full_bar(i), i * kTcBK, 0, first_tile.nt * BN);
     }
   }
+  __syncwarp();
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
-    if (lane == 0) {
-      int g = 0;  // K blocks issued so far, across tiles: the ring never drains at a tile boundary
+    if (elect_one()) {
+      int g = 0, s = 0;  // K blocks issued so far, across tiles: the ring never drains at a tile boundary
+      uint32_t ph = 1;
       bool ok = true;
-      for (int j = 0; j < my_tiles && ok; ++j) {
-        const int tf = (int)blockIdx.x + j * (int)gridDim.x, t = p.rev ? total - 1 - tf : tf;
-        const int m0 = (t / n_tiles) * kTcBM, n0 = (t % n_tiles) * BN;
+      TileWalk tw = first_tile;
+      for (int j = 0; j < my_tiles && ok; ++j, tw.next()) {
+        const int m0 = tw.mt * kTcBM, n0 = tw.nt * BN;
         const int b = j & 1;
         if (RES) {
           if (j >= 2) ok = mbar_wait(res_free(b), (uint32_t)((j >> 1) - 1) & 1u, p.err_flag);
           if (!ok) break;
           mbar_expect_tx(res_full(b), S::kIoBytes);
 #pragma unroll
-          for (int h = 0; h < BN / 64; ++h)
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              tma_load_2d(base + S::kROff + b * S::kIoBytes + h * 16384 + q * 4096, &tmR, res_full(b), n0 + h * 64, m0 + q * 32);
+          for (int h = 0; h < BN / 64; ++h) tma_load_2d(base + S::kROff + b * S::kIoBytes + h * 16384, &tmR, res_full(b), n0 + h * 64, m0);
         }
-        int cw = 0, ch = 0, cn = 0;
-        if (p.im2col) {
+        int cw = 0, ch = 0, cn = 0, cw2 = 0, ch2 = 0;
+        if (p.im2col || (PROJ && p.im2col2)) {
           const int hw = p.Ho * p.Wo;
           cn = m0 / hw;
-          const int rem = m0 - cn * hw;
-          const int ho = rem / p.Wo;
-          cw = (rem - ho * p.Wo) * p.stride - p.pad_w;
-          ch = ho * p.stride - p.pad;
+          const int rem = m0 - cn * hw, ho = rem / p.Wo, wo = rem - ho * p.Wo;
+          cw = wo * p.stride - p.pad_w, ch = ho * p.stride - p.pad;
+          if (PROJ) cw2 = wo * p.stride2, ch2 = ho * p.stride2;
         }
         for (int kb = 0; kb < num_kb; ++kb, ++g) {
-          const int s = g % kStages;
-          const uint32_t ph = (uint32_t)(g / kStages) & 1u;
-          const int tap = kb / p.cblocks, cb = kb - tap * p.cblocks;
-          const uint32_t sa = base + (uint32_t)s * S::kStage, sb = sa + S::kABytes;
+          const uint32_t sa = base + (uint32_t)s * S::kStage;
           if (g >= w_ahead) {   // earlier slots were armed before the dependency wait
-            ok = mbar_wait(empty_bar(s), ph ^ 1u, p.err_flag);
+            ok = mbar_wait(empty_bar(s), ph, p.err_flag);
             if (!ok) break;
             mbar_expect_tx(full_bar(s), S::kStage);
-            tma_load_3d(sb, &tmW, full_bar(s), cb * kTcBK, tap, n0);
+            tma_load_3d(sa + S::kABytes, &tmW, full_bar(s), kb * kTcBK, 0, n0);
           }
-          if (p.im2col) {
-            const int r = tap / p.kw;
-            tma_load_im2col_4d(sa, &tmA, full_bar(s), cb * kTcBK, cw, ch, cn, (uint16_t)(tap - r * p.kw), (uint16_t)r);
-          } else {
-            tma_load_2d(sa, &tmA, full_bar(s), cb * kTcBK, m0);
-          }
+          if (p.im2col)
+            tma_load_im2col_4d(sa, &tmA, full_bar(s), kb * kTcBK, cw, ch, cn, (uint16_t)0, (uint16_t)0);
+          else
+            tma_load_2d(sa, &tmA, full_bar(s), kb * kTcBK, m0);
+          if (++s == kStages) s = 0, ph ^= 1u;
         }
         if (PROJ && ok) {   // the projection's K blocks follow in the same ring
-          int cw2 = 0, ch2 = 0, cn2 = 0;
-          if (p.im2col2) {
-            const int hw = p.Ho * p.Wo;
-            cn2 = m0 / hw;
-            const int rem = m0 - cn2 * hw;
-            const int ho = rem / p.Wo;
-            cw2 = (rem - ho * p.Wo) * p.stride2;
-            ch2 = ho * p.stride2;
-          }
           for (int kb = 0; kb < num_kb2; ++kb, ++g) {
-            const int s = g % kStages;
-            const uint32_t ph = (uint32_t)(g / kStages) & 1u;
-            const uint32_t sa = base + (uint32_t)s * S::kStage, sb = sa + S::kABytes;
-            ok = mbar_wait(empty_bar(s), ph ^ 1u, p.err_flag);   // g >= num_kb >= w_ahead: never a pre-armed slot
+            const uint32_t sa = base + (uint32_t)s * S::kStage;
+            ok = mbar_wait(empty_bar(s), ph, p.err_flag);   // g >= num_kb >= w_ahead: never a pre-armed slot
             if (!ok) break;
             mbar_expect_tx(full_bar(s), S::kStage);
-            tma_load_3d(sb, &tmW2, full_bar(s), kb * kTcBK, 0, n0);
+            tma_load_3d(sa + S::kABytes, &tmW2, full_bar(s), kb * kTcBK, 0, n0);
             if (p.im2col2)
-              tma_load_im2col_4d(sa, &tmA2, full_bar(s), kb * kTcBK, cw2, ch2, cn2, (uint16_t)0, (uint16_t)0);
+              tma_load_im2col_4d(sa, &tmA2, full_bar(s), kb * kTcBK, cw2, ch2, cn, (uint16_t)0, (uint16_t)0);
             else
               tma_load_2d(sa, &tmA2, full_bar(s), kb * kTcBK, m0);
+            if (++s == kStages) s = 0, ph ^= 1u;
           }
         }
       }
     }
+    __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc = umma_idesc(BN);
-      int g = 0;
+      const uint64_t da0 = umma_desc(base), db0 = umma_desc(base + S::kABytes);
+      int s = 0;
+      uint32_t ph = 0;
       bool ok = true;
+      auto block = [&](uint32_t acc, bool accumulate) {
+        ok = mbar_wait(full_bar(s), ph, p.err_flag);
+        if (!ok) return;
+        tc_fence_after();
+        const uint64_t off = (uint64_t)(s * (S::kStage >> 4));
+        umma_block(acc, da0 + off, db0 + off, idesc, accumulate);
+        umma_commit(empty_bar(s));
+        if (++s == kStages) s = 0, ph ^= 1u;
+      };
       for (int j = 0; j < my_tiles && ok; ++j) {
         const int b = j & 1;
         if (j >= 2) {  // the epilogue must have drained this accumulator (tile j - 2)
@@ -904,35 +957,13 @@ conv_igemm_tcgen05_persistent_kernel(const __grid_constant__ CUtensorMap tmA, co
           tc_fence_after();
         }
         const uint32_t acc = tmem_base + (uint32_t)(b * kAccs * BN);
-        for (int kb = 0; kb < num_kb; ++kb, ++g) {
-          const int s = g % kStages;
-          const uint32_t ph = (uint32_t)(g / kStages) & 1u;
-          ok = mbar_wait(full_bar(s), ph, p.err_flag);
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t sa = base + (uint32_t)s * S::kStage, sb = sa + S::kABytes;
-#pragma unroll
-          for (int k = 0; k < kTcBK / 16; ++k)
-            umma_bf16(acc, umma_desc(sa + k * 32), umma_desc(sb + k * 32), idesc, (uint32_t)((kb | k) != 0));
-          umma_commit(empty_bar(s));
-        }
-        if (PROJ) {
-          for (int kb = 0; kb < num_kb2 && ok; ++kb, ++g) {
-            const int s = g % kStages;
-            const uint32_t ph = (uint32_t)(g / kStages) & 1u;
-            ok = mbar_wait(full_bar(s), ph, p.err_flag);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t sa = base + (uint32_t)s * S::kStage, sb = sa + S::kABytes;
-#pragma unroll
-            for (int k = 0; k < kTcBK / 16; ++k)
-              umma_bf16(acc + (uint32_t)BN, umma_desc(sa + k * 32), umma_desc(sb + k * 32), idesc, (uint32_t)((kb | k) != 0));
-            umma_commit(empty_bar(s));
-          }
-        }
+        for (int kb = 0; kb < num_kb && ok; ++kb) block(acc, kb != 0);
+        if (PROJ)
+          for (int kb = 0; kb < num_kb2 && ok; ++kb) block(acc + (uint32_t)BN, kb != 0);
         if (ok) umma_commit(acc_full(b));
       }
     }
+    __syncwarp();
   } else {
     const int q = warp & 3;
     const int row = q * 32 + lane;
@@ -942,9 +973,9 @@ conv_igemm_tcgen05_persistent_kernel(const __grid_constant__ CUtensorMap tmA, co
     bool ok = true;
     int sc_n0 = -1;
     bool pending = false;  // lane 0: a bulk store group of this warp may still be reading shared memory
-    for (int j = 0; j < my_tiles; ++j) {
-      const int tf = (int)blockIdx.x + j * (int)gridDim.x, t = p.rev ? total - 1 - tf : tf;
-      const int m0 = (t / n_tiles) * kTcBM, n0 = (t % n_tiles) * BN;
+    TileWalk tw = first_tile;
+    for (int j = 0; j < my_tiles; ++j, tw.next()) {
+      const int m0 = tw.mt * kTcBM, n0 = tw.nt * BN;
       const int b = j & 1;
       if (n0 != sc_n0) {  // consecutive tiles of a CTA usually share the N tile: reload only on change
         __syncwarp();
@@ -1110,6 +1141,12 @@ struct TcContext {
   int sm_count = 148;
 };
 
+struct TapPlan {   // conv_taps.cuh
+  bool on = false;
+  int r = 0, ni = 0, wp = 0;   // output tile: r rows x ni images x wp columns
+  int rows = 0, a_bytes = 0;   // input rows and bytes of one activation block
+};
+
 struct TcLayer {
   int cin = 0, cout = 0, kh = 1, kw = 1, stride = 1, pad = 0, pad_w = 0, act = 0;
   int in_h = 0, in_w = 0, out_h = 0, out_w = 0, max_batch = 0;
@@ -1121,8 +1158,10 @@ struct TcLayer {
   bool gather = false;
   bool stem7 = false;   // the 7x7/2 stem kernel of conv_stem.cuh takes this layer
   bool halo = false;    // the 3x3 halo-block kernel of conv_halo.cuh takes this layer
+  TapPlan tap;          // the tap-view kernel of conv_taps.cuh takes this layer
   int g_h = 0, g_w = 0, g_cin = 0, g_kh = 0, g_kw = 0, g_stride = 1, g_pad = 0, g_runp = 0;
   CUtensorMap tm_w;
+  CUtensorMap tm_w_bn[4];     // the same weights with boxes of 16, 32, 64 and 128 filters (conv_taps.cuh)
   CUtensorMap tm_w_half[2];   // the same weights with boxes of 128 and 64 filters: one CTA's half of a 256- or 128-wide pair tile
   struct Cached {
     const void* ptr;
@@ -1243,6 +1282,12 @@ inline ee_status_t tc_plan_layer(TcContext& c, const ee_layer_desc_t& d, int in_
   CUresult r = c.encode_tiled(&L->tm_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(w_dev), dims, strides, box, es,
                               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  for (int i = 0; i < 4 && r == CUDA_SUCCESS; ++i) {
+    const cuuint32_t bbox[3] = {kTcBK, 1, 16u << i};
+    r = c.encode_tiled(&L->tm_w_bn[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(w_dev), dims, strides, bbox, es,
+                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  }
   for (int i = 0; i < 2 && r == CUDA_SUCCESS; ++i) {
     const cuuint32_t hbox[3] = {kTcBK, 1, (cuuint32_t)(i == 0 ? 128 : 64)};
     r = c.encode_tiled(&L->tm_w_half[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(w_dev), dims, strides, hbox, es,
@@ -1277,6 +1322,16 @@ inline ee_status_t tc_buffer_map(const TcContext& c, const TcLayer& L, const voi
     r = c.encode_tiled(&e.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, es,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  } else if (kind == 6) {
+    // NHWC as (C, W, B, H): a box is tap.rows input rows of tap.ni images and tap.wp columns, every stride-th of each
+    const int st = L.stride;
+    const cuuint64_t dims[4] = {(cuuint64_t)L.cin, (cuuint64_t)L.in_w, (cuuint64_t)batch, (cuuint64_t)L.in_h};
+    const cuuint64_t strides[3] = {(cuuint64_t)L.cin * 2, (cuuint64_t)L.cin * 2 * L.in_w * L.in_h, (cuuint64_t)L.cin * 2 * L.in_w};
+    const cuuint32_t box[4] = {kTcBK, (cuuint32_t)((L.tap.wp - 1) * st + 1), (cuuint32_t)L.tap.ni, (cuuint32_t)((L.tap.rows - 1) * st + 1)};
+    const cuuint32_t es[4] = {1, (cuuint32_t)st, 1, (cuuint32_t)st};
+    r = c.encode_tiled(&e.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, es,
+                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   } else if (kind == 2) {
     // stem input as (W*Cin, H, B): 256 elements of 7 consecutive image rows per load, zero fill outside
     const cuuint64_t dims[3] = {(cuuint64_t)L.g_w * L.g_cin, (cuuint64_t)L.g_h, (cuuint64_t)batch};
@@ -1305,10 +1360,10 @@ inline ee_status_t tc_buffer_map(const TcContext& c, const TcLayer& L, const voi
     r = c.encode_tiled(&e.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, es,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  } else if (kind == 1) {
+  } else if (kind == 1 || kind == 7) {   // output (a warp's 32 rows per store) / residual operand (a whole tile's rows per load)
     const cuuint64_t dims[2] = {(cuuint64_t)L.cout, (cuuint64_t)batch * L.out_h * L.out_w};
     const cuuint64_t strides[1] = {(cuuint64_t)L.cout * 2};
-    const cuuint32_t box[2] = {64, 32};
+    const cuuint32_t box[2] = {64, kind == 1 ? 32u : (cuuint32_t)kTcBM};
     const cuuint32_t es[2] = {1, 1};
     r = c.encode_tiled(&e.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, es,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1443,7 +1498,7 @@ inline ee_status_t tc_launch_proj(TcContext& c, const TcLayer& L, const TcLayer&
   TcParams p = {};
   p.M = B * L.out_h * L.out_w;
   p.N = L.cout;
-  p.taps = 1, p.kw = 1;
+  p.taps = 1, p.kh = 1, p.kw = 1;
   p.cblocks = cdiv(L.cin, kTcBK);
   p.Ho = L.out_h, p.Wo = L.out_w, p.stride = L.stride, p.pad = L.pad, p.pad_w = L.pad_w;
   p.im2col = L.im2col ? 1 : 0;
@@ -1491,7 +1546,7 @@ inline ee_status_t tc_launch(TcContext& c, const TcLayer& L, const void* src, co
   }
   CUtensorMap tmR = tmO;
   if (res) {
-    if ((s = tc_buffer_map(c, L, res, B, 1, &t)) != EE_OK) return s;
+    if ((s = tc_buffer_map(c, L, res, B, 7, &t)) != EE_OK) return s;
     tmR = *t;
   }
   TcParams p = {};
@@ -1499,7 +1554,7 @@ inline ee_status_t tc_launch(TcContext& c, const TcLayer& L, const void* src, co
   p.M = B * L.out_h * L.out_w;
   p.N = L.cout;
   p.taps = L.kh * L.kw;
-  p.kw = L.kw;
+  p.kh = L.kh, p.kw = L.kw;
   p.cblocks = cdiv(L.cin, kTcBK);
   p.Ho = L.out_h, p.Wo = L.out_w, p.stride = L.stride, p.pad = L.pad, p.pad_w = L.pad_w;
   p.im2col = L.im2col ? 1 : 0;

@@ -144,7 +144,7 @@ conv3x3_halo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
         const uint64_t da = da0 + (uint64_t)(s * (kHaloBlockBytes >> 4));
 #pragma unroll
         for (int i = 0; i < kHaloTaps; ++i) {
-          const int tap = i % 3 * 3 + i / 3;   // filter columns outermost: the order of TapWalk
+          const int tap = i % 3 * 3 + i / 3;   // filter columns outermost: the order of tap_at
           umma_block(tmem_base + (uint32_t)(b * 64), da + (uint64_t)(((tap / 3) * p.Wp + (tap % 3)) * 8), db0 + (uint64_t)(tap * (kHaloWTapBytes >> 4)),
                      idesc, i != 0);
         }

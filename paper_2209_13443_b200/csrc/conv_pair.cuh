@@ -266,21 +266,23 @@ conv_igemm_tcgen05_pair_kernel(const __grid_constant__ PairStageArgs A) {
           auto arm_and_load_w = [&](int kb, int gg) -> bool {
             const int s = gg % kStages;
             const uint32_t ph = (uint32_t)(gg / kStages) & 1u;
-            const TapWalk t(p.kh, p.kw, p.stride, kb);
+            const int cb = kb / p.taps;
+            const uint32_t t = tap_at(kb - cb * p.taps, p.kh, p.kw, p.stride);
             if (!mbar_wait_for(empty_bar(s), ph ^ 1u, err_flag, limit)) return false;
             if (rank == 0) mbar_expect_tx(full_bar(s), (uint32_t)(2 * S::kBBytes + S::kABytes + (peer_rows ? S::kABytes : 0)));
-            tma2_load_3d(base + (uint32_t)s * S::kStage + S::kABytes, tmW, map_to_rank(full_bar(s), 0), t.cb * kTcBK, t.tap(), nb0);
+            tma2_load_3d(base + (uint32_t)s * S::kStage + S::kABytes, tmW, map_to_rank(full_bar(s), 0), cb * kTcBK, (int)(t >> 16), nb0);
             return true;
           };
           auto load_a = [&](int kb, int gg) {
             if (!rows) return;
             const int s = gg % kStages;
-            const TapWalk t(p.kh, p.kw, p.stride, kb);
+            const int cb = kb / p.taps;
             const uint32_t sa = base + (uint32_t)s * S::kStage, fb = map_to_rank(full_bar(s), 0);
             if (p.im2col) {
-              tma2_load_im2col_4d(sa, tmA, fb, t.cb * kTcBK, cw, ch, cn, (uint16_t)t.s, (uint16_t)t.r);
+              const uint32_t t = tap_at(kb - cb * p.taps, p.kh, p.kw, p.stride);
+              tma2_load_im2col_4d(sa, tmA, fb, cb * kTcBK, cw, ch, cn, (uint16_t)(t & 255u), (uint16_t)(t >> 8 & 255u));
             } else {
-              tma2_load_2d(sa, tmA, fb, t.cb * kTcBK, m0);
+              tma2_load_2d(sa, tmA, fb, cb * kTcBK, m0);
             }
           };
           int kb = kb_begin;

@@ -12,7 +12,7 @@
 // stride 2 the rows of one parity form a block (tiled map with element strides), two blocks per filter column.
 //
 // The tile width BN (128 ... 16 filters) is picked per launch so that the grid fills the SMs (tap_pick_bn).  It changes no
-// sum: every output adds its K blocks in the order of tap_at, as all kernels of this library do.
+// sum: every output adds its K blocks in the order of tap_at, as in all kernels of this library.
 //
 // Warp roles: warp 0 weights (TMA), warp 1 TMEM and MMA, warps 2-5 epilogue (a thread owns one output pixel and stores its
 // BN channels straight to global memory), warp 6 activations (TMA).  Every wait on an mbarrier is bounded.
@@ -55,6 +55,7 @@ conv_taps_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
   const uint32_t accum_bar = bar0 + 8u * (2 * p.sa + 2 * p.sw);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen + after + 2 * BN * 4 + 8 * (2 * p.sa + 2 * p.sw + 1));
 
+  __shared__ uint32_t tab[kMaxTaps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tile = p.rev ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
   const int n0 = (int)blockIdx.y * BN;
@@ -62,6 +63,7 @@ conv_taps_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
   const int taps = p.kh * p.kw, num_kb = taps * p.cblocks;
   const int parts = p.stride == 1 ? 1 : min(2, p.kh);   // A blocks per filter column
 
+  tap_table_fill(tab, p.kh, p.kw, p.stride);
   if (threadIdx.x == 0) {
     for (int s = 0; s < 2 * (p.sa + p.sw) + 1; ++s) mbar_init(bar0 + 8u * s, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -81,11 +83,13 @@ conv_taps_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_c
     if (elect_one()) {
       int s = 0;
       uint32_t ph = 1;
-      TapWalk t(p.kh, p.kw, p.stride, 0);
-      for (int i = 0; i < num_kb; ++i, t.next()) {
+      int c = 0, t = 0;
+      for (int i = 0; i < num_kb; ++i) {
+        const int tap = (int)(tab[t] >> 16);
         if (i >= p.sw && !mbar_wait(w_empty(s), ph, p.err_flag)) break;
         mbar_expect_tx(w_full(s), kWBytes);
-        tma_load_3d(w_base + (uint32_t)(s * kWBytes), &tmW, w_full(s), t.cb * kTcBK, t.tap(), n0);
+        tma_load_3d(w_base + (uint32_t)(s * kWBytes), &tmW, w_full(s), c, tap, n0);
+        if (++t == taps) t = 0, c += kTcBK;
         if (++s == p.sw) s = 0, ph ^= 1u;
         if (i == min(p.sw, num_kb) - 1) {
           asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -231,7 +235,7 @@ inline int tap_pick_bn(const TcContext& c, const TcLayer& L, int B) {
 template <int BN>
 inline cudaError_t tap_launch_t(dim3 grid, cudaStream_t st, const CUtensorMap& x, const CUtensorMap& w, TapParams p, int sms) {
   // two CTAs per SM when the grid has more tiles than SMs, else a deeper weight ring
-  const int fixed = 2 * BN * 4 + 512 + 1024, room = ((long)grid.x * grid.y > sms ? 113 : 200) * 1024;
+  const int fixed = 2 * BN * 4 + 512 + 1024 + 256, room = ((long)grid.x * grid.y > sms ? 113 : 200) * 1024;
   p.sa = std::min(4, std::max(2, (room - fixed - 4 * BN * 128) / p.a_slot));
   p.sw = std::min(12, std::max(3, (room - fixed - p.sa * p.a_slot) / (BN * 128)));
   cudaLaunchConfig_t cfg = {};

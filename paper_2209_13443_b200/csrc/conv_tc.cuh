@@ -7,9 +7,9 @@
 // K block, zero fill for the padding halo), or reads it as a plain 2-D tile for 1x1 stride-1
 // layers.  Batching appends samples along M, so one weight tile serves every sample of the batch.
 //
-// One CTA computes one 128 x BN output tile (or, in the persistent variant, walks many).  Warp roles: warp 0 issues
-// TMA loads into a ring of shared-memory slots, warp 1 owns the TMEM allocation and issues the MMAs (one thread),
-// the remaining warps run the epilogue: tcgen05.ld of the fp32 accumulator, folded-BN scale/bias, residual add (the
+// One CTA computes one 128 x BN output tile (or, in the persistent variant, walks many).  Warp roles: warp 0 and the last
+// warp issue the TMA loads of weights and activations into a ring of shared-memory slots, warp 1 owns the TMEM allocation and issues the MMAs (one thread),
+// the warps between run the epilogue: tcgen05.ld of the fp32 accumulator, folded-BN scale/bias, residual add (the
 // residual tile was brought into shared memory by TMA while the main loop ran), activation, one rounding to bf16,
 // then a TMA store of the tile from shared memory.  The K loop visits (channel block, tap) in a fixed order that
 // does not depend on the batch size (tap_at).  Variants (chosen per launch from the grid size, see tc_launch): shallow or
@@ -30,7 +30,7 @@ namespace ee {
 
 constexpr int kTcBM = 128;       // output pixels per CTA (= TMEM lanes)
 constexpr int kTcBK = 64;        // bf16 elements per K block: 128 bytes = one swizzle span
-constexpr int kTcThreads = 192;  // producer warp, MMA warp, four epilogue warps
+constexpr int kTcThreads = 224;  // weight producer, MMA warp, four epilogue warps, activation producer
 constexpr long long kTcWaitCycles = 4000000000LL;  // ~2 s at boost clock; far beyond any healthy wait
 
 struct TcParams {
@@ -68,31 +68,18 @@ struct TcParams {
 
 // Order of a convolution's K blocks, the same in every tensor-core kernel: channel blocks outermost, then filter columns,
 // then filter rows (stride 2: the even rows, then the odd ones), so that consecutive blocks read overlapping input rows
-// (conv_taps.cuh keeps those in shared memory).  Walked by counters: one thread feeds the whole SM, and an integer division
-// by a run-time number is a chain of about 150 clocks in it (two of them per K block were what a K block took).
-struct TapWalk {
-  int kh, kw, step;
-  int r, s, cb;   // filter row and column, channel block
-  __device__ __forceinline__ TapWalk(int kh_, int kw_, int stride, int first) : kh(kh_), kw(kw_), step(stride == 2 ? 2 : 1) {
-    const int taps = kh * kw;
-    cb = first / taps;
-    const int t = first - cb * taps;
-    s = t / kh;
-    const int j = t - s * kh, even = (kh + 1) / 2;
-    r = step == 1 ? j : j < even ? 2 * j : 2 * (j - even) + 1;
-  }
-  __device__ __forceinline__ void next() {
-    r += step;
-    if (r < kh) return;
-    if (step == 2 && (r & 1) == 0 && kh > 1) {
-      r = 1;
-      return;
-    }
-    r = 0;
-    if (++s == kw) s = 0, ++cb;
-  }
-  __device__ __forceinline__ int tap() const { return r * kw + s; }
-};
+// (conv_taps.cuh keeps those in shared memory).  Entry i of a channel block, packed: (row * kw + column) << 16 | row << 8 |
+// column.  The feeding loops read the entries from a table in shared memory (tap_table_fill): one thread feeds the whole SM,
+// and in it an integer division by a run-time number is a chain of about 150 clocks, counters with branches still 50.
+constexpr int kMaxTaps = 49;
+__device__ __forceinline__ uint32_t tap_at(int i, int kh, int kw, int stride) {
+  const int s = i / kh, j = i - s * kh, even = (kh + 1) / 2;
+  const int r = stride != 2 ? j : j < even ? 2 * j : 2 * (j - even) + 1;
+  return (uint32_t)((r * kw + s) << 16 | r << 8 | s);
+}
+__device__ __forceinline__ void tap_table_fill(uint32_t* tab, int kh, int kw, int stride) {   // the CTA's first threads
+  if ((int)threadIdx.x < kh * kw) tab[threadIdx.x] = tap_at((int)threadIdx.x, kh, kw, stride);
+}
 
 // ----------------------------------------------------------------------------- PTX wrappers
 
@@ -127,9 +114,10 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* er
 }
 
 // One lane of a converged warp.  A feeding loop runs inside `if (elect_one())`, which tells the compiler that it has one
-// thread: addresses and descriptors live in uniform registers.  With the descriptors stepped instead of rebuilt, no
-// division in the loop and nothing but the barrier test between the blocks, a K block of a 128 x 128 tile takes 267 to 340
-// clocks (257 are its four MMAs) where `if (lane == 0)` took 511, 707 with an im2col coordinate.
+// thread: addresses and descriptors live in uniform registers.  With the descriptors stepped instead of rebuilt, weights
+// and activations requested by a thread each and nothing in a loop but its barrier test, its coordinates and its request, a
+// K block of a 128 x 128 tile takes 267 to 340 clocks (257 are its four MMAs) where one thread behind `if (lane == 0)` took
+// 511, 707 with an im2col coordinate.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}" : "=r"(p));
@@ -435,7 +423,7 @@ struct TcSmem {
   static constexpr int kIoBytes = kTcBM * BN * 2;
   static constexpr int kIoOff = RES ? kTiles : 0;
   static constexpr int kAfter = kTiles + (RES ? kIoBytes : 0);
-  static constexpr int kBytes = kAfter + 2 * BN * 4 + 256 + 1024;  // + scale/bias, barriers, alignment slack
+  static constexpr int kBytes = kAfter + 2 * BN * 4 + 256 + 256 + 1024;  // + scale/bias, barriers, taps, alignment slack
   static_assert(RES || kIoBytes <= kStage, "output staging must fit in ring slot 0");
   static_assert(kBytes <= 227 * 1024, "exceeds the shared memory of an SM");
 };
@@ -481,6 +469,7 @@ conv_igemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
   const uint32_t accum_bar = bar0 + 8u * (2 * kStages);
   const uint32_t res_bar = bar0 + 8u * (2 * kStages + 1);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 2);
+  uint32_t* taps = reinterpret_cast<uint32_t*>(bars + 32);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = (p.rev ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x) * kTcBM, n0 = blockIdx.y * BN;
@@ -491,7 +480,7 @@ conv_igemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
-      mbar_init(full_bar(s), GATHER ? 129 : 1);  // gather: 128 row writers + the weight tile's expect_tx
+      mbar_init(full_bar(s), GATHER ? 129 : 2);  // one expect_tx each of weights and activations; gather: 128 row writers instead
       mbar_init(empty_bar(s), 1);
     }
     mbar_init(accum_bar, 1);
@@ -505,6 +494,7 @@ conv_igemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
     if (RES) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmR) : "memory");
   }
   static_assert(!LOCAL || (!SPLIT && !GATHER), "local K ranges are a mode of the plain one-CTA kernel");
+  tap_table_fill(taps, p.kh, p.kw, p.stride);
   const int n_acc = LOCAL ? max(p.ranges, 1) : 1;   // accumulators of BN fp32 columns
   uint32_t acc_cols = BN;                           // TMEM allocations are powers of two
   if (LOCAL)
@@ -521,50 +511,60 @@ conv_igemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
   // so do the weight tiles of the first ring slots, which no kernel writes.  From the wait on this kernel touches
   // activations, so it needs that kernel's memory; the next kernel in the stream may begin its own prologue now.
   const int w_ahead = min(num_kb, kStages);
+  // ring walk of a producer: its K block (channel block x 64, position in the tap table), slot and phase
+  struct Feed {
+    int c, t, n_taps, s;
+    uint32_t ph;
+    __device__ __forceinline__ void next() {
+      if (++t == n_taps) t = 0, c += kTcBK;
+      if (++s == kStages) s = 0, ph ^= 1u;
+    }
+  };
+  const int cb_first = kb_begin / p.taps;
+  Feed feed{cb_first * kTcBK, kb_begin - cb_first * p.taps, p.taps, 0, 1u};
   if (warp == 0 && elect_one()) {
-    TapWalk t(p.kh, p.kw, p.stride, kb_begin);
-    for (int i = 0; i < w_ahead; ++i, t.next()) {   // the slots start out empty
-      mbar_expect_tx(full_bar(i), GATHER ? S::kBBytes : S::kStage);
-      tma_load_3d(base + (uint32_t)i * S::kStage + S::kABytes, &tmW, full_bar(i), t.cb * kTcBK, t.tap(), n0);
+    for (int i = 0; i < w_ahead; ++i, feed.next()) {   // the slots start out empty
+      mbar_expect_tx(full_bar(i), S::kBBytes);
+      tma_load_3d(base + (uint32_t)i * S::kStage + S::kABytes, &tmW, full_bar(i), feed.c, (int)(taps[feed.t] >> 16), n0);
     }
   }
-  __syncwarp();
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
+    // the elected thread goes on where the prefetch stopped (elect.sync picks the same lane of the same converged warp, and
+    // the walk state of the others is behind: they never issue)
     if (elect_one()) {
+      for (int i = w_ahead; i < num_kb; ++i, feed.next()) {
+        if (!mbar_wait(empty_bar(feed.s), feed.ph, p.err_flag)) break;
+        mbar_expect_tx(full_bar(feed.s), S::kBBytes);
+        tma_load_3d(base + (uint32_t)feed.s * S::kStage + S::kABytes, &tmW, full_bar(feed.s), feed.c, (int)(taps[feed.t] >> 16), n0);
+      }
+    }
+    __syncwarp();
+  } else if (warp == 6) {
+    if (!GATHER && elect_one()) {
       if (RES) {
         mbar_expect_tx(res_bar, S::kIoBytes);
 #pragma unroll
         for (int h = 0; h < BN / 64; ++h) tma_load_2d(base + S::kIoOff + h * 16384, &tmR, res_bar, n0 + h * 64, m0);
       }
-      int cw = 0, ch = 0, cn = 0;
       if (p.im2col) {
-        const int hw = p.Ho * p.Wo;
-        cn = m0 / hw;
-        const int rem = m0 - cn * hw;
-        const int ho = rem / p.Wo;
-        cw = (rem - ho * p.Wo) * p.stride - p.pad_w;
-        ch = ho * p.stride - p.pad;
-      }
-      TapWalk t(p.kh, p.kw, p.stride, kb_begin);
-      int s = 0;
-      uint32_t ph = 1;
-      for (int i = 0; i < num_kb; ++i, t.next()) {
-        const uint32_t sa = base + (uint32_t)s * S::kStage;
-        if (i >= w_ahead) {   // earlier slots: armed and their weight tile requested before the dependency wait
-          if (!mbar_wait(empty_bar(s), ph, p.err_flag)) break;
-          mbar_expect_tx(full_bar(s), GATHER ? S::kBBytes : S::kStage);
-          tma_load_3d(sa + S::kABytes, &tmW, full_bar(s), t.cb * kTcBK, t.tap(), n0);
+        const int hw = p.Ho * p.Wo, cn = m0 / hw, rem = m0 - cn * hw, ho = rem / p.Wo;
+        const int cw = (rem - ho * p.Wo) * p.stride - p.pad_w, ch = ho * p.stride - p.pad;
+        for (int i = 0; i < num_kb; ++i, feed.next()) {
+          const uint32_t t = taps[feed.t];
+          if (i >= kStages && !mbar_wait(empty_bar(feed.s), feed.ph, p.err_flag)) break;
+          mbar_expect_tx(full_bar(feed.s), S::kABytes);
+          tma_load_im2col_4d(base + (uint32_t)feed.s * S::kStage, &tmA, full_bar(feed.s), feed.c, cw, ch, cn, (uint16_t)(t & 255u),
+                             (uint16_t)(t >> 8 & 255u));
         }
-        if (GATHER) {
-        } else if (p.im2col) {
-          tma_load_im2col_4d(sa, &tmA, full_bar(s), t.cb * kTcBK, cw, ch, cn, (uint16_t)t.s, (uint16_t)t.r);
-        } else {
-          tma_load_2d(sa, &tmA, full_bar(s), t.cb * kTcBK, m0);
+      } else {
+        for (int i = 0; i < num_kb; ++i, feed.next()) {
+          if (i >= kStages && !mbar_wait(empty_bar(feed.s), feed.ph, p.err_flag)) break;
+          mbar_expect_tx(full_bar(feed.s), S::kABytes);
+          tma_load_2d(base + (uint32_t)feed.s * S::kStage, &tmA, full_bar(feed.s), feed.c, m0);
         }
-        if (++s == kStages) s = 0, ph ^= 1u;
       }
     }
     __syncwarp();
@@ -703,9 +703,9 @@ conv_igemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
   if (SPLIT) {
     // Every thread of every CTA of the cluster passes both barriers, whatever happened above: the first one before
     // any remote store (epilogue threads took it inside their push loop), the second once all partials have landed.
-    if (warp < 2) asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+    if (warp < 2 || warp == 6) asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
     asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
-    if (warp >= 2) {
+    if (warp >= 2 && warp < 6) {
       // Pull side, all local: this CTA adds the nsplit partials of its rows in ascending range order (the grouping
       // of the sum is fixed by the layer), applies the epilogue and stores.
       constexpr int CH = BN / 4, G = BN / 8;     // 16-byte fp32 chunks and 8-column groups per row
@@ -772,7 +772,7 @@ struct TcPersistSmem {
   // without a residual: a longer ring and two output staging tiles; with one: two residual tiles the producer
   // prefetches (free again as soon as the epilogue has read them) and a single staging tile
   static constexpr int kEpiWarps = BN == 128 ? 8 : 4;   // at BN = 128 two warps share a TMEM lane quarter, one per 64-column half
-  static constexpr int kThreads = 64 + 32 * kEpiWarps;
+  static constexpr int kThreads = 96 + 32 * kEpiWarps;  // weight producer, MMA warp, epilogue warps, activation producer
   static constexpr int kStages = RES ? (BN == 128 ? 3 : 5) : (BN == 128 ? 4 : 7);
   static constexpr int kABytes = kTcBM * kTcBK * 2;
   static constexpr int kBBytes = BN * kTcBK * 2;
@@ -825,7 +825,7 @@ conv_igemm_tcgen05_persistent_kernel(const __grid_constant__ CUtensorMap tmA, co
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
-      mbar_init(full_bar(s), 1);
+      mbar_init(full_bar(s), 2);   // one expect_tx each of weights and activations
       mbar_init(empty_bar(s), 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -870,7 +870,7 @@ conv_igemm_tcgen05_persistent_kernel(const __grid_constant__ CUtensorMap tmA, co
   const TileWalk first_tile{t_first / n_tiles, t_first % n_tiles, t_sign * ((int)gridDim.x / n_tiles), t_sign * ((int)gridDim.x % n_tiles), n_tiles};
   if (warp == 0 && elect_one()) {
     for (int i = 0; i < w_ahead; ++i) {
-      mbar_expect_tx(full_bar(i), S::kStage);
+      mbar_expect_tx(full_bar(i), S::kBBytes);
       tma_load_3d(base + (uint32_t)i * S::kStage + S::kABytes, &tmW, full_bar(i), i * kTcBK, 0, first_tile.nt * BN);
     }
   }
@@ -879,8 +879,37 @@ conv_igemm_tcgen05_persistent_kernel(const __grid_constant__ CUtensorMap tmA, co
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
-    if (elect_one()) {
-      int g = 0, s = 0;  // K blocks issued so far, across tiles: the ring never drains at a tile boundary
+    if (elect_one()) {   // weights; the ring never drains at a tile boundary
+      int g = 0, s = 0;  // K blocks issued so far, across tiles
+      uint32_t ph = 1;
+      bool ok = true;
+      TileWalk tw = first_tile;
+      for (int j = 0; j < my_tiles && ok; ++j, tw.next()) {
+        const int n0 = tw.nt * BN;
+        for (int kb = 0, c = 0; kb < num_kb; ++kb, ++g, c += kTcBK) {
+          if (g >= w_ahead) {   // earlier slots were armed before the dependency wait
+            ok = mbar_wait(empty_bar(s), ph, p.err_flag);
+            if (!ok) break;
+            mbar_expect_tx(full_bar(s), S::kBBytes);
+            tma_load_3d(base + (uint32_t)s * S::kStage + S::kABytes, &tmW, full_bar(s), c, 0, n0);
+          }
+          if (++s == kStages) s = 0, ph ^= 1u;
+        }
+        if (PROJ && ok) {   // the projection's K blocks follow in the same ring
+          for (int kb = 0, c = 0; kb < num_kb2; ++kb, ++g, c += kTcBK) {
+            ok = mbar_wait(empty_bar(s), ph, p.err_flag);   // g >= num_kb >= w_ahead: never a pre-armed slot
+            if (!ok) break;
+            mbar_expect_tx(full_bar(s), S::kBBytes);
+            tma_load_3d(base + (uint32_t)s * S::kStage + S::kABytes, &tmW2, full_bar(s), c, 0, n0);
+            if (++s == kStages) s = 0, ph ^= 1u;
+          }
+        }
+      }
+    }
+    __syncwarp();
+  } else if (warp == 2 + S::kEpiWarps) {
+    if (elect_one()) {   // activations and residual tiles
+      int s = 0;
       uint32_t ph = 1;
       bool ok = true;
       TileWalk tw = first_tile;
@@ -902,31 +931,25 @@ conv_igemm_tcgen05_persistent_kernel(const __grid_constant__ CUtensorMap tmA, co
           cw = wo * p.stride - p.pad_w, ch = ho * p.stride - p.pad;
           if (PROJ) cw2 = wo * p.stride2, ch2 = ho * p.stride2;
         }
-        for (int kb = 0; kb < num_kb; ++kb, ++g) {
-          const uint32_t sa = base + (uint32_t)s * S::kStage;
-          if (g >= w_ahead) {   // earlier slots were armed before the dependency wait
-            ok = mbar_wait(empty_bar(s), ph, p.err_flag);
-            if (!ok) break;
-            mbar_expect_tx(full_bar(s), S::kStage);
-            tma_load_3d(sa + S::kABytes, &tmW, full_bar(s), kb * kTcBK, 0, n0);
-          }
+        for (int kb = 0, c = 0; kb < num_kb; ++kb, c += kTcBK) {
+          ok = mbar_wait(empty_bar(s), ph, p.err_flag);   // the first round passes at once
+          if (!ok) break;
+          mbar_expect_tx(full_bar(s), S::kABytes);
           if (p.im2col)
-            tma_load_im2col_4d(sa, &tmA, full_bar(s), kb * kTcBK, cw, ch, cn, (uint16_t)0, (uint16_t)0);
+            tma_load_im2col_4d(base + (uint32_t)s * S::kStage, &tmA, full_bar(s), c, cw, ch, cn, (uint16_t)0, (uint16_t)0);
           else
-            tma_load_2d(sa, &tmA, full_bar(s), kb * kTcBK, m0);
+            tma_load_2d(base + (uint32_t)s * S::kStage, &tmA, full_bar(s), c, m0);
           if (++s == kStages) s = 0, ph ^= 1u;
         }
-        if (PROJ && ok) {   // the projection's K blocks follow in the same ring
-          for (int kb = 0; kb < num_kb2; ++kb, ++g) {
-            const uint32_t sa = base + (uint32_t)s * S::kStage;
-            ok = mbar_wait(empty_bar(s), ph, p.err_flag);   // g >= num_kb >= w_ahead: never a pre-armed slot
+        if (PROJ && ok) {
+          for (int kb = 0, c = 0; kb < num_kb2; ++kb, c += kTcBK) {
+            ok = mbar_wait(empty_bar(s), ph, p.err_flag);
             if (!ok) break;
-            mbar_expect_tx(full_bar(s), S::kStage);
-            tma_load_3d(sa + S::kABytes, &tmW2, full_bar(s), kb * kTcBK, 0, n0);
+            mbar_expect_tx(full_bar(s), S::kABytes);
             if (p.im2col2)
-              tma_load_im2col_4d(sa, &tmA2, full_bar(s), kb * kTcBK, cw2, ch2, cn, (uint16_t)0, (uint16_t)0);
+              tma_load_im2col_4d(base + (uint32_t)s * S::kStage, &tmA2, full_bar(s), c, cw2, ch2, cn, (uint16_t)0, (uint16_t)0);
             else
-              tma_load_2d(sa, &tmA2, full_bar(s), kb * kTcBK, m0);
+              tma_load_2d(base + (uint32_t)s * S::kStage, &tmA2, full_bar(s), c, m0);
             if (++s == kStages) s = 0, ph ^= 1u;
           }
         }

@@ -14,7 +14,6 @@
 #include "conv_tc.cuh"
 #include "conv_stem.cuh"
 #include "conv_halo.cuh"
-#include "conv_taps.cuh"
 #include "conv_pair.cuh"
 #include "conv_dw.cuh"
 #include "head.cuh"
@@ -276,8 +275,6 @@ ee_status_t launch_layer(ee_model* m, const LayerPlan& L, const void* src, const
         if (pair_v && pair_supported(L.tc, v))
           s = pair_launch(m->tc, L.tc, v, src, res, dst, B, L.scale_dev, L.bias_dev, m->err_flag, partial, partial_bytes, m->pair_counters,
                           m->wait_cycles, st);
-        else if (v == TCV_AUTO && L.tc.tap.on && L.tc.splits == 1 && !L.tc.halo)
-          s = tap_launch(m->tc, L.tc, src, dst, B, L.scale_dev, L.bias_dev, m->err_flag, st);
         else
           s = L.tc.halo ? halo_launch(m->tc, L.tc, src, dst, B, L.scale_dev, L.bias_dev, m->err_flag, st)
                         : tc_launch(m->tc, L.tc, src, res, dst, B, L.scale_dev, L.bias_dev, m->err_flag, st, gap_part, gap_g, range_mode);
@@ -788,7 +785,6 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
   rc = tc_context_init(m->tc);
   if (rc == EE_OK) rc = stem_context_init();
   if (rc == EE_OK) rc = halo_context_init();
-  if (rc == EE_OK) rc = tap_context_init();
   if (rc == EE_OK) rc = pair_context_init();
   if (rc == EE_OK) rc = dw_context_init();
   if (rc == EE_OK) rc = f32_context_init();
@@ -1004,7 +1000,6 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
         }
         if (rc != EE_OK) return fail(rc);
         L.tc.halo = halo_supported(d, L.in_w);
-        if (!L.tc.halo && tap_plan(d, L.out_h, L.out_w, desc->max_batch, &L.tc.tap)) tc_set_splits(L.tc, 1);   // narrow tiles fill the SMs instead
       } else if (desc->dtype == EE_BF16 && d.cout % 8 == 0 && d.kh * d.kw * d.cin <= 1024 && d.pad_w == d.pad) {
         // pixel rows are not 16-byte units (e.g. a 3-channel stem): explicit Toeplitz rows, then the tensor-core GEMM
         L.kind = KK_TC_GATHER;

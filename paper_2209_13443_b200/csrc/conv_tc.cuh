@@ -67,10 +67,9 @@ struct TcParams {
 };
 
 // Order of a convolution's K blocks, the same in every tensor-core kernel: channel blocks outermost, then filter columns,
-// then filter rows (stride 2: the even rows, then the odd ones), so that consecutive blocks read overlapping input rows
-// (conv_taps.cuh keeps those in shared memory).  Entry i of a channel block, packed: (row * kw + column) << 16 | row << 8 |
-// column.  The feeding loops read the entries from a table in shared memory (tap_table_fill): one thread feeds the whole SM,
-// and in it an integer division by a run-time number is a chain of about 150 clocks, counters with branches still 50.
+// then filter rows (stride 2: the even rows, then the odd ones), so that consecutive blocks read overlapping input rows.
+// Entry i of a channel block, packed: (row * kw + column) << 16 | row << 8 | column.  The feeding loops read the entries from
+// a table in shared memory (tap_table_fill): one thread feeds the whole SM, and in it an integer division by a run-time number is a chain of about 150 clocks, counters with branches still 50.
 constexpr int kMaxTaps = 49;
 __device__ __forceinline__ uint32_t tap_at(int i, int kh, int kw, int stride) {
   const int s = i / kh, j = i - s * kh, even = (kh + 1) / 2;
@@ -1164,12 +1163,6 @@ struct TcContext {
   int sm_count = 148;
 };
 
-struct TapPlan {   // conv_taps.cuh
-  bool on = false;
-  int r = 0, ni = 0, wp = 0;   // output tile: r rows x ni images x wp columns
-  int rows = 0, a_bytes = 0;   // input rows and bytes of one activation block
-};
-
 struct TcLayer {
   int cin = 0, cout = 0, kh = 1, kw = 1, stride = 1, pad = 0, pad_w = 0, act = 0;
   int in_h = 0, in_w = 0, out_h = 0, out_w = 0, max_batch = 0;
@@ -1181,10 +1174,9 @@ struct TcLayer {
   bool gather = false;
   bool stem7 = false;   // the 7x7/2 stem kernel of conv_stem.cuh takes this layer
   bool halo = false;    // the 3x3 halo-block kernel of conv_halo.cuh takes this layer
-  TapPlan tap;          // the tap-view kernel of conv_taps.cuh takes this layer
   int g_h = 0, g_w = 0, g_cin = 0, g_kh = 0, g_kw = 0, g_stride = 1, g_pad = 0, g_runp = 0;
   CUtensorMap tm_w;
-  CUtensorMap tm_w_bn[4];     // the same weights with boxes of 16, 32, 64 and 128 filters (conv_taps.cuh)
+  CUtensorMap tm_w_bn[4];     // the same weights with boxes of 16, 32, 64 and 128 filters
   CUtensorMap tm_w_half[2];   // the same weights with boxes of 128 and 64 filters: one CTA's half of a 256- or 128-wide pair tile
   struct Cached {
     const void* ptr;
@@ -1261,9 +1253,8 @@ inline ee_status_t tc_plan_layer(TcContext& c, const ee_layer_desc_t& d, int in_
   L->in_h = in_h, L->in_w = in_w, L->out_h = out_h, L->out_w = out_w, L->max_batch = max_batch;
   L->bn = d.cout > 64 ? 128 : 64;
   L->im2col = !(d.kh == 1 && d.kw == 1 && d.stride == 1 && d.pad == 0 && d.pad_w == 0);
-  // Split-K: a lone CTA cannot pull operands faster than its SM's L2 port (about 126 GB/s: a 32 KB K block of a
-  // 128x128 tile takes 0.26 us in tile mode and 0.36 us in im2col mode, against 0.13 us of MMA time), so a layer
-  // whose grid leaves SMs idle spreads the K range of a tile over a cluster of 2..4 CTAs.  A split costs about
+  // Split-K: a K block of a 128 x 128 tile takes 0.135 us (its MMAs' own rate; 0.10 us at 64 columns), so a long K loop on a
+  // grid that leaves SMs idle spreads over a cluster of 2..4 CTAs per tile.  A split costs about
   // 4.5 us (cluster launch, two cluster barriers, the reduce-scatter), larger clusters gain nothing measurable, and
   // grids of more than two CTAs per SM lose to the unsplit kernel, hence the bounds.  The number of ranges is chosen
   // once per layer by this cost model summed over the batch sizes the model will see (max_batch, 3/4, 1/2 and 1/4
@@ -1273,7 +1264,7 @@ inline ee_status_t tc_plan_layer(TcContext& c, const ee_layer_desc_t& d, int in_
   {
     const int num_kb = d.kh * d.kw * cdiv(d.cin, kTcBK);
     const int n_tiles = cdiv(d.cout, L->bn);
-    const double t_block = (L->im2col ? 0.36 : 0.26) * (16384.0 + L->bn * 128.0) / 32768.0;   // us per K block per SM
+    const double t_block = L->bn == 128 ? 0.135 : 0.10;   // us per K block
     const long tiles_max = (long)cdiv((long)max_batch * out_h * out_w, kTcBM) * n_tiles;
     double best = 0;
     L->splits = 1;
@@ -1285,7 +1276,7 @@ inline ee_status_t tc_plan_layer(TcContext& c, const ee_layer_desc_t& d, int in_
       for (int f = 4; f >= 1; --f) {
         const int b = std::max(1, (max_batch * f + 3) / 4);
         const long tiles = (long)cdiv((long)b * out_h * out_w, kTcBM) * n_tiles;
-        const long share = cdiv(tiles * sp, c.sm_count);   // CTAs that share the L2 port of the busiest SM
+        const long share = cdiv(tiles * sp, c.sm_count);   // CTAs on the busiest SM
         cost += 2.4 + (sp > 1 ? 4.5 : 0.0) + (double)share * per * t_block + 0.8 * cdiv(tiles, c.sm_count);
       }
       if (sp == 1) {
@@ -1342,16 +1333,6 @@ inline ee_status_t tc_buffer_map(const TcContext& c, const TcLayer& L, const voi
     const cuuint64_t strides[3] = {(cuuint64_t)L.cin * 2, (cuuint64_t)L.cin * 2 * L.in_w, (cuuint64_t)L.cin * 2 * L.in_w * L.in_h};
     const cuuint32_t box[4] = {kTcBK, (cuuint32_t)wp, (cuuint32_t)rows, 1};
     const cuuint32_t es[4] = {1, 1, 1, 1};
-    r = c.encode_tiled(&e.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, es,
-                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  } else if (kind == 6) {
-    // NHWC as (C, W, B, H): a box is tap.rows input rows of tap.ni images and tap.wp columns, every stride-th of each
-    const int st = L.stride;
-    const cuuint64_t dims[4] = {(cuuint64_t)L.cin, (cuuint64_t)L.in_w, (cuuint64_t)batch, (cuuint64_t)L.in_h};
-    const cuuint64_t strides[3] = {(cuuint64_t)L.cin * 2, (cuuint64_t)L.cin * 2 * L.in_w * L.in_h, (cuuint64_t)L.cin * 2 * L.in_w};
-    const cuuint32_t box[4] = {kTcBK, (cuuint32_t)((L.tap.wp - 1) * st + 1), (cuuint32_t)L.tap.ni, (cuuint32_t)((L.tap.rows - 1) * st + 1)};
-    const cuuint32_t es[4] = {1, (cuuint32_t)st, 1, (cuuint32_t)st};
     r = c.encode_tiled(&e.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, es,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);

@@ -111,23 +111,23 @@ def test_stage_outputs_of_a_new_buffer_set_are_not_those_of_a_dead_one():
         del bufs
 
 
-# tap-view convolutions: H, W, cin, cout, kh, kw, stride, pad, pad_w, max_batch
+# convolutions with several taps: H, W, cin, cout, kh, kw, stride, pad, pad_w, max_batch
 TAP_GEOMS = [
-    (14, 14, 128, 256, 3, 3, 1, 1, 1, 5),     # 16-column rows, eight rows per tile, ragged last tile
-    (7, 7, 192, 96, 3, 3, 1, 1, 1, 5),        # two images per tile, odd batch, 96 filters
-    (28, 28, 72, 128, 3, 3, 2, 1, 1, 3),      # stride 2: blocks of even and odd rows; ragged channel block
+    (14, 14, 128, 256, 3, 3, 1, 1, 1, 5),     # whole channel blocks, ragged last tile
+    (7, 7, 192, 96, 3, 3, 1, 1, 1, 5),        # a tile over three images, 96 filters
+    (28, 28, 72, 128, 3, 3, 2, 1, 1, 3),      # stride 2: even rows first, then odd ones; ragged channel block
     (9, 13, 64, 40, 3, 3, 2, 1, 1, 3),        # the same, odd sizes, fewer than 64 filters
-    (17, 17, 96, 96, 1, 7, 1, 0, 3, 2),       # one filter row: a block per tap
-    (17, 17, 96, 96, 7, 1, 1, 3, 0, 2),       # one filter column: one block per channel block
-    (6, 70, 64, 16, 3, 3, 1, 1, 1, 2),        # one row of 72 columns per tile (56 rows of the view past its block), 16 filters
-    (3, 128, 16, 24, 5, 3, 1, 2, 1, 1),       # 128 columns, five filter rows
-    (1, 1, 64, 200, 3, 3, 1, 1, 1, 9),        # one pixel per image, 16 images per tile
+    (17, 17, 96, 96, 1, 7, 1, 0, 3, 2),       # one filter row
+    (17, 17, 96, 96, 7, 1, 1, 3, 0, 2),       # one filter column
+    (6, 70, 64, 16, 3, 3, 1, 1, 1, 2),        # rows wider than half a tile, 16 filters
+    (3, 128, 16, 24, 5, 3, 1, 2, 1, 1),       # 24 filters, five filter rows
+    (1, 1, 64, 200, 3, 3, 1, 1, 1, 9),        # one pixel per image
     (11, 11, 64, 72, 5, 5, 2, 2, 2, 4),       # stride 2, three even and two odd rows
 ]
 
 
 @pytest.mark.parametrize("geom", TAP_GEOMS)
-def test_tap_view_convolution(geom):
+def test_convolution_with_several_taps(geom):
     H, W, cin, cout, kh, kw, stride, pad, pad_w, bmax = geom
     rng = wl._rng(sum(geom), 911)
     layer = wl._conv_hw(rng, cin, cout, kh, kw, stride, pad, pad_w, wl.ACT_RELU, bf16=True)
@@ -140,5 +140,5 @@ def test_tap_view_convolution(geom):
         g = run.stage(0, x)
         util.check_stage(spec, g, util.oracle_stage(spec, 0, x), f"{geom} B={B}", elementwise=True)
         first[B] = g["features_out"][0]
-    # the same sums in the im2col kernel (two K ranges or not, any tile width): here its per-tile CTA with one range
+    # the sums do not depend on the batch
     assert np.array_equal(first[1], first[bmax])

@@ -12,6 +12,7 @@
 #include "conv_simt.cuh"
 #include "conv_f32.cuh"
 #include "conv_tc.cuh"
+#include "conv_wave.cuh"
 #include "conv_stem.cuh"
 #include "conv_halo.cuh"
 #include "conv_pair.cuh"
@@ -783,6 +784,7 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
       cudaEventCreateWithFlags(&m->ev_join, cudaEventDisableTiming) != cudaSuccess)
     return fail(EE_ERR_CUDA);
   rc = tc_context_init(m->tc);
+  if (rc == EE_OK) rc = wave_context_init();
   if (rc == EE_OK) rc = stem_context_init();
   if (rc == EE_OK) rc = halo_context_init();
   if (rc == EE_OK) rc = pair_context_init();

@@ -64,6 +64,7 @@ struct TcParams {
   // pairwise over the rows with distances gap_g/2, ..., 2, 1 - the block sums of gap_blocks_kernel (head.cuh)
   int gap_g;
   float* gap_part;
+  int ring;             // operand slots of the one-wave kernel (conv_wave.cuh)
 };
 
 // Order of a convolution's K blocks, the same in every tensor-core kernel: channel blocks outermost, then filter columns,
@@ -89,6 +90,15 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 }
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {   // never suspends the thread
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
 }
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
@@ -294,6 +304,19 @@ __device__ __forceinline__ uint4 epilogue8_act(int act, const float* acc, const 
   if (act == EE_ACT_RELU) return epilogue8<EE_ACT_RELU, RES>(acc, scale, bias, res);
   if (act == EE_ACT_RELU6) return epilogue8<EE_ACT_RELU6, RES>(acc, scale, bias, res);
   return epilogue8<EE_ACT_NONE, RES>(acc, scale, bias, res);
+}
+
+// 32 columns of one pixel, the activation picked once for all of them.
+template <int ACT, bool RES>
+__device__ __forceinline__ void epilogue32_t(const float* v, const float* scale, const float* bias, const uint4* res, uint4* out) {
+#pragma unroll
+  for (int g = 0; g < 4; ++g) out[g] = epilogue8<ACT, RES>(v + g * 8, scale + g * 8, bias + g * 8, RES ? res[g] : make_uint4(0u, 0u, 0u, 0u));
+}
+template <bool RES>
+__device__ __forceinline__ void epilogue32(int act, const float* v, const float* scale, const float* bias, const uint4* res, uint4* out) {
+  if (act == EE_ACT_RELU) epilogue32_t<EE_ACT_RELU, RES>(v, scale, bias, res, out);
+  else if (act == EE_ACT_RELU6) epilogue32_t<EE_ACT_RELU6, RES>(v, scale, bias, res, out);
+  else epilogue32_t<EE_ACT_NONE, RES>(v, scale, bias, res, out);
 }
 
 // Column sums over the 32 rows a warp holds (ov: this lane's row, 64 bf16 columns as eight 16-byte groups), written as
@@ -1176,7 +1199,7 @@ struct TcLayer {
   bool halo = false;    // the 3x3 halo-block kernel of conv_halo.cuh takes this layer
   int g_h = 0, g_w = 0, g_cin = 0, g_kh = 0, g_kw = 0, g_stride = 1, g_pad = 0, g_runp = 0;
   CUtensorMap tm_w;
-  CUtensorMap tm_w_bn[4];     // the same weights with boxes of 16, 32, 64 and 128 filters
+  CUtensorMap tm_w_bn[2];     // the same weights with boxes of 32 and 64 filters
   CUtensorMap tm_w_half[2];   // the same weights with boxes of 128 and 64 filters: one CTA's half of a 256- or 128-wide pair tile
   struct Cached {
     const void* ptr;
@@ -1208,15 +1231,11 @@ inline ee_status_t tc_context_init(TcContext& c) {
   set(conv_igemm_tcgen05_kernel<64, 3, false, false, true>, TcSmem<64, 3, false>::kBytes);
   set(conv_igemm_tcgen05_kernel<128, 3, false, false, true>, TcSmem<128, 3, false>::kBytes);
   set(conv_igemm_tcgen05_kernel<64, 3, false, false, false>, TcSmem<64, 3, false>::kBytes);
-  set(conv_igemm_tcgen05_kernel<64, 6, false, false, false>, TcSmem<64, 6, false>::kBytes);
   set(conv_igemm_tcgen05_kernel<64, 2, true, false, false>, TcSmem<64, 2, true>::kBytes);
-  set(conv_igemm_tcgen05_kernel<64, 5, true, false, false>, TcSmem<64, 5, true>::kBytes);
   set(conv_igemm_tcgen05_kernel<64, 6, false, true, false>, TcSmem<64, 6, false>::kBytes);
   set(conv_igemm_tcgen05_kernel<64, 3, false, true, false>, TcSmem<64, 3, false>::kBytes);
   set(conv_igemm_tcgen05_kernel<128, 3, false, false, false>, TcSmem<128, 3, false>::kBytes);
-  set(conv_igemm_tcgen05_kernel<128, 6, false, false, false>, TcSmem<128, 6, false>::kBytes);
   set(conv_igemm_tcgen05_kernel<128, 2, true, false, false>, TcSmem<128, 2, true>::kBytes);
-  set(conv_igemm_tcgen05_kernel<128, 5, true, false, false>, TcSmem<128, 5, true>::kBytes);
   set(conv_igemm_tcgen05_kernel<128, 6, false, true, false>, TcSmem<128, 6, false>::kBytes);
   set(conv_igemm_tcgen05_kernel<128, 3, false, true, false>, TcSmem<128, 3, false>::kBytes);
   set(conv_igemm_tcgen05_kernel<64, 3, false, false, false, true>, TcSmem<64, 3, false>::kBytes);
@@ -1296,11 +1315,12 @@ inline ee_status_t tc_plan_layer(TcContext& c, const ee_layer_desc_t& d, int in_
   CUresult r = c.encode_tiled(&L->tm_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(w_dev), dims, strides, box, es,
                               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  for (int i = 0; i < 4 && r == CUDA_SUCCESS; ++i) {
-    const cuuint32_t bbox[3] = {kTcBK, 1, 16u << i};
-    r = c.encode_tiled(&L->tm_w_bn[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(w_dev), dims, strides, bbox, es,
-                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  for (int i = 0; i < 2; ++i) {
+    const cuuint32_t nbox[3] = {kTcBK, 1, 32u << i};
+    if (r == CUDA_SUCCESS)
+      r = c.encode_tiled(&L->tm_w_bn[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(w_dev), dims, strides, nbox, es,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   }
   for (int i = 0; i < 2 && r == CUDA_SUCCESS; ++i) {
     const cuuint32_t hbox[3] = {kTcBK, 1, (cuuint32_t)(i == 0 ? 128 : 64)};
@@ -1434,8 +1454,7 @@ inline cudaError_t tc_launch_bn(bool deep, bool res, bool split, dim3 grid, cuda
     return deep ? tc_launch_t<BN, 6, false, false, false, true>(grid, st, a, w, r, o, p) : tc_launch_t<BN, 3, false, false, false, true>(grid, st, a, w, r, o, p);
   }
   if (split) return deep ? tc_launch_t<BN, 6, false, true>(grid, st, a, w, r, o, p) : tc_launch_t<BN, 3, false, true>(grid, st, a, w, r, o, p);
-  if (res) return deep ? tc_launch_t<BN, 5, true, false>(grid, st, a, w, r, o, p) : tc_launch_t<BN, 2, true, false>(grid, st, a, w, r, o, p);
-  return deep ? tc_launch_t<BN, 6, false, false>(grid, st, a, w, r, o, p) : tc_launch_t<BN, 3, false, false>(grid, st, a, w, r, o, p);
+  return res ? tc_launch_t<BN, 2, true, false>(grid, st, a, w, r, o, p) : tc_launch_t<BN, 3, false, false>(grid, st, a, w, r, o, p);
 }
 
 template <int BN, bool RES>
@@ -1486,6 +1505,18 @@ inline bool tc_proj_supported(const TcLayer& L, const TcLayer& P) {
          P.out_h == L.out_h && P.out_w == L.out_w && L.kh * L.kw == 1 && L.splits == 1 && !L.gather && !L.halo;
 }
 
+// Tile width of the one-wave kernel (conv_wave.cuh) for a layer at batch B, 0 = more tiles than SMs: the grid's CTAs then share
+// SMs (or walk tiles on the persistent kernel).  Within one wave the narrower tile is the faster one: more slots for the same
+// round trip of a K block, a shorter epilogue.
+inline int tc_wave_bn(const TcContext& c, const TcLayer& L, int B) {
+  const long mt = cdiv((long)B * L.out_h * L.out_w, kTcBM);
+  for (int bn = 32; bn <= L.bn; bn *= 2)
+    if (mt * cdiv(L.cout, bn) <= c.sm_count) return bn;
+  return 0;
+}
+inline cudaError_t wave_launch(int bn, cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, TcParams p);   // conv_wave.cuh
+inline cudaError_t wave_launch_proj(cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, const CUtensorMap& a2, const CUtensorMap& w2, TcParams p);
+
 // L with the projection P in its launch: src -> L, src2 -> P; P's own output is never written.
 inline ee_status_t tc_launch_proj(TcContext& c, const TcLayer& L, const TcLayer& P, const void* src, const void* src2, void* dst, int B,
                                   const float* scale, const float* bias, const float* scale2, const float* bias2, int* err_flag,
@@ -1516,6 +1547,9 @@ inline ee_status_t tc_launch_proj(TcContext& c, const TcLayer& L, const TcLayer&
   p.cblocks2 = cdiv(P.cin, kTcBK), p.im2col2 = P.im2col ? 1 : 0, p.stride2 = P.stride, p.act2 = P.act;
   p.scale2 = scale2, p.bias2 = bias2;
   p.gap_part = gap_part, p.gap_g = gap_part ? gap_g : 0;
+  // the persistent kernel's long prologue and 128-wide epilogue are for several tiles per SM
+  if (!p.gap_part && tc_wave_bn(c, L, B) == 32)
+    return wave_launch_proj(st, tmA, L.tm_w_bn[0], tmA2, P.tm_w_bn[0], p) == cudaSuccess ? EE_OK : EE_ERR_CUDA;
   const cudaError_t e = L.bn == 128 ? tc_launch_persistent_proj<128>(c.sm_count, st, tmA, L.tm_w, tmO, tmA2, P.tm_w, p)
                                     : tc_launch_persistent_proj<64>(c.sm_count, st, tmA, L.tm_w, tmO, tmA2, P.tm_w, p);
   return e == cudaSuccess ? EE_OK : EE_ERR_CUDA;
@@ -1606,6 +1640,8 @@ inline ee_status_t tc_launch(TcContext& c, const TcLayer& L, const void* src, co
       pe = res ? tc_launch_persistent<64, true>(ctas, st, tmA, L.tm_w, tmR, tmO, p) : tc_launch_persistent<64, false>(ctas, st, tmA, L.tm_w, tmR, tmO, p);
     return pe == cudaSuccess ? EE_OK : EE_ERR_CUDA;
   }
+  if (const int bn = split || local ? 0 : tc_wave_bn(c, L, B))
+    return wave_launch(bn, st, tmA, bn == L.bn ? L.tm_w : L.tm_w_bn[bn / 64], p) == cudaSuccess ? EE_OK : EE_ERR_CUDA;
   cudaError_t e = L.bn == 128 ? tc_launch_bn<128>(deep, tma_res, split, grid, st, tmA, L.tm_w, tmR, tmO, p)
                               : tc_launch_bn<64>(deep, tma_res, split, grid, st, tmA, L.tm_w, tmR, tmO, p);
   return e == cudaSuccess ? EE_OK : EE_ERR_CUDA;

@@ -1,0 +1,276 @@
+// Convolution tiles of grids with at most one tile per SM (small batches, the 14x14 and 7x7 maps): 128 pixels x BN filters per
+// CTA, the narrowest of 32, 64 and 128 whose tiles fit in one wave.
+//
+// Such a layer is a chain of latencies: first operands (600 ns), the K loop of one tile, its epilogue, and about 1 us until the
+// next launch may go on.  What this kernel does about them (clocks measured inside it):
+//  - A K block goes round the ring in about 1900 clocks (its loads 1100, its MMAs and their commit, the feeding thread), so the
+//    K loop's pace is that over the number of slots: all of shared memory is ring when the loop is long, and a narrow tile has
+//    more slots (11 of 20 KB at 32 filters, 6 of 32 KB at 128).
+//  - Weights and activations have two feeding warps each, for the even and the odd blocks: one thread behind both operands spent
+//    400 clocks between a free slot and its second request.
+//  - The MMA thread asks for the next block's barrier before it issues this block's MMAs: the answer is there when it gets to it.
+//  - 32 or 64 columns per epilogue warp (four warps with 128 columns each took 2800 clocks, these take 700 or 1400).  The
+//    residual's rows come to registers while the K loop runs.
+// Bits are those of the other kernels: the same K order, one accumulator per output, one rounding.
+// In a chain of launches, before (128-filter tiles, a feeding thread per operand) -> now, us: 3x3 512 -> 512 on 7x7, batch 1
+// 13.6 -> 10.8, batch 22 14.4 -> 11.3; 3x3 256 -> 256 on 14x14, batch 1 8.4 -> 6.4; 1x1 512 -> 128 on 28x28 4.3 -> 3.0, 128 -> 512 3.7 -> 2.5.
+//
+// PROJ: the residual operand is a 1x1 projection computed into a second accumulator (see the persistent kernel of conv_tc.cuh).
+#pragma once
+#include "conv_tc.cuh"
+
+namespace ee {
+
+template <int BN>
+struct WaveSmem {
+  static constexpr int kEpiWarps = BN == 32 ? 4 : 8;
+  static constexpr int kThreads = 32 * (5 + kEpiWarps);     // warps 0, 1 weights, 2, 3 activations, 4 MMA, then the epilogue
+  static constexpr int kABytes = kTcBM * kTcBK * 2, kBBytes = BN * kTcBK * 2, kSlot = kABytes + kBBytes;
+  static constexpr int kMaxSlots = BN == 32 ? 11 : BN == 64 ? 9 : 6;
+  static_assert(kEpiWarps * 2048 <= kSlot, "output staging: 2 KB per epilogue warp in the drained first slot");
+  static constexpr int bytes(int slots) { return slots * kSlot + 4 * BN * 4 + 256 + 256 + 1024; }   // + scale/bias, barriers, taps, alignment slack
+  static_assert(bytes(kMaxSlots) <= 227 * 1024, "exceeds the shared memory of an SM");
+};
+
+template <int BN, bool PROJ>
+__global__ void __launch_bounds__(WaveSmem<BN>::kThreads, 1)
+conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
+                         const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmW2, TcParams p) {
+  using S = WaveSmem<BN>;
+  constexpr int R = S::kMaxSlots;
+  extern __shared__ uint8_t smem_raw[];
+  const int ring = p.ring;   // slots, <= R
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  uint8_t* gen = smem_raw + (base - raw);
+  float* s_sb = reinterpret_cast<float*>(gen + ring * S::kSlot);      // scale | bias | scale2 | bias2
+  uint64_t* bars = reinterpret_cast<uint64_t*>(gen + ring * S::kSlot + 4 * BN * 4);
+  const uint32_t bar0 = base + (uint32_t)(ring * S::kSlot + 4 * BN * 4);
+  auto full_bar = [&](int s) { return bar0 + 8u * s; };
+  auto empty_bar = [&](int s) { return bar0 + 8u * (R + s); };
+  const uint32_t accum_bar = bar0 + 8u * (2 * R);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * R + 1);
+  uint32_t* taps = reinterpret_cast<uint32_t*>(bars + 32);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int m0 = (p.rev ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x) * kTcBM, n0 = blockIdx.y * BN;
+  const int num_kb1 = p.taps * p.cblocks, num_kb = num_kb1 + (PROJ ? p.cblocks2 : 0);
+  constexpr uint32_t kCols = PROJ ? 2 * BN : BN;   // accumulators, fp32 columns
+
+  if (threadIdx.x < 2 * R + 1) {
+    mbar_init(bar0 + 8u * threadIdx.x, threadIdx.x < R ? 2 : 1);   // full: one expect_tx each of weights and activations
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 5 && lane == 0) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmW) : "memory");
+    if (PROJ) {
+      asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA2) : "memory");
+      asm volatile("prefetch.tensormap [%0];" ::"l"(&tmW2) : "memory");
+    }
+  }
+  tap_table_fill(taps, p.kh, p.kw, p.stride);
+  if (warp == 4) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kCols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  if (warp < 4) {
+    // K blocks h, h + 2, ...: walked by counters (slot and phase, channel block x 64, position in the tap table)
+    const int h = warp & 1, dc = p.taps == 1 ? 2 * kTcBK : 0, dt = p.taps == 1 ? 0 : 2;
+    int i = h, s = h, c = p.taps == 1 ? h * kTcBK : 0, t = p.taps == 1 ? 0 : h;
+    uint32_t ph = 1;
+    auto step = [&] {
+      i += 2, c += dc, t += dt;
+      if (t >= p.taps) t -= p.taps, c += kTcBK;
+      if ((s += 2) >= ring) s -= ring, ph ^= 1u;
+    };
+    if (warp < 2) {
+      if (elect_one()) {
+        // no kernel writes weights: nothing to wait for but a free slot
+        for (; i < num_kb; step()) {
+          if (i >= ring && !mbar_wait(empty_bar(s), ph, p.err_flag)) break;
+          mbar_expect_tx(full_bar(s), S::kBBytes);
+          const uint32_t dst = base + (uint32_t)(s * S::kSlot + S::kABytes);
+          if (PROJ && i >= num_kb1)
+            tma_load_3d(dst, &tmW2, full_bar(s), (i - num_kb1) * kTcBK, 0, n0);
+          else
+            tma_load_3d(dst, &tmW, full_bar(s), c, (int)(taps[t] >> 16), n0);
+        }
+      }
+      __syncwarp();
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    } else {
+      int cw = 0, ch = 0, cn = 0, cw2 = 0, ch2 = 0;
+      if (p.im2col || (PROJ && p.im2col2)) {
+        const int hw = p.Ho * p.Wo;
+        cn = m0 / hw;
+        const int rem = m0 - cn * hw, ho = rem / p.Wo, wo = rem - ho * p.Wo;
+        cw = wo * p.stride - p.pad_w, ch = ho * p.stride - p.pad;
+        if (PROJ) cw2 = wo * p.stride2, ch2 = ho * p.stride2;
+      }
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+      if (elect_one()) {
+        bool ok = true;
+        if (p.im2col) {
+          for (; i < num_kb1; step()) {
+            const uint32_t tap = taps[t];
+            ok = i < ring || mbar_wait(empty_bar(s), ph, p.err_flag);
+            if (!ok) break;
+            mbar_expect_tx(full_bar(s), S::kABytes);
+            tma_load_im2col_4d(base + (uint32_t)(s * S::kSlot), &tmA, full_bar(s), c, cw, ch, cn, (uint16_t)(tap & 255u), (uint16_t)(tap >> 8 & 255u));
+          }
+        } else {
+          for (; i < num_kb1; step()) {
+            ok = i < ring || mbar_wait(empty_bar(s), ph, p.err_flag);
+            if (!ok) break;
+            mbar_expect_tx(full_bar(s), S::kABytes);
+            tma_load_2d(base + (uint32_t)(s * S::kSlot), &tmA, full_bar(s), c, m0);
+          }
+        }
+        if (PROJ) {
+          for (; ok && i < num_kb; step()) {
+            if (i >= ring && !mbar_wait(empty_bar(s), ph, p.err_flag)) break;
+            mbar_expect_tx(full_bar(s), S::kABytes);
+            if (p.im2col2)
+              tma_load_im2col_4d(base + (uint32_t)(s * S::kSlot), &tmA2, full_bar(s), (i - num_kb1) * kTcBK, cw2, ch2, cn, (uint16_t)0, (uint16_t)0);
+            else
+              tma_load_2d(base + (uint32_t)(s * S::kSlot), &tmA2, full_bar(s), (i - num_kb1) * kTcBK, m0);
+          }
+        }
+      }
+      __syncwarp();
+    }
+  } else if (warp == 4) {
+    if (elect_one()) {
+      constexpr uint32_t idesc = umma_idesc(BN);
+      const uint64_t da0 = umma_desc(base), db0 = umma_desc(base + S::kABytes);
+      bool ok = true;
+      int s = 0;
+      uint32_t ph = 0;
+      bool here = mbar_test_wait(full_bar(0), 0);
+      for (int i = 0; i < num_kb; ++i) {
+        if (!here) ok = mbar_wait(full_bar(s), ph, p.err_flag);
+        if (!ok) break;
+        const int cur = s;
+        if (++s == ring) s = 0, ph ^= 1u;
+        here = mbar_test_wait(full_bar(s), ph);   // behind the last block: a phase that nobody waits for
+        const uint64_t off = (uint64_t)(cur * (S::kSlot >> 4));
+        umma_block(tmem_base + (PROJ && i >= num_kb1 ? (uint32_t)BN : 0u), da0 + off, db0 + off, idesc, i != 0 && i != num_kb1);
+        umma_commit(empty_bar(cur));
+      }
+      if (ok) umma_commit(accum_bar);   // everything before it has read its operands as well
+    }
+    __syncwarp();
+  } else {
+    const int et = threadIdx.x - 160;
+    for (int i = et; i < BN; i += 32 * S::kEpiWarps) {
+      const bool in = n0 + i < p.N;
+      s_sb[i] = (p.scale && in) ? p.scale[n0 + i] : 1.f;
+      s_sb[BN + i] = (p.bias && in) ? p.bias[n0 + i] : 0.f;
+      if (PROJ) {
+        s_sb[2 * BN + i] = (p.scale2 && in) ? p.scale2[n0 + i] : 1.f;
+        s_sb[3 * BN + i] = (p.bias2 && in) ? p.bias2[n0 + i] : 0.f;
+      }
+    }
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * S::kEpiWarps) : "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    constexpr int kCover = BN == 128 ? 64 : 32, kSteps = kCover / 32;   // columns of a warp, in steps of 32
+    const int q = warp & 3, half = et >> 7, m = m0 + q * 32 + lane;
+    uint4 r[4 * kSteps];
+#pragma unroll
+    for (int g = 0; g < 4 * kSteps; ++g) {
+      const int n = n0 + half * kCover + g * 8;
+      r[g] = make_uint4(0u, 0u, 0u, 0u);
+      if (!PROJ && p.residual && m < p.M && n < p.N) r[g] = *reinterpret_cast<const uint4*>(p.residual + (size_t)m * p.N + n);
+    }
+    const bool ok = __all_sync(0xffffffffu, mbar_wait(accum_bar, 0, p.err_flag));
+    if (ok) {
+      tc_fence_after();
+      uint8_t* stage = gen + (warp - 5) * 2048;   // 32 rows of 64 bytes, their 16-byte chunks XORed with the row
+#pragma unroll
+      for (int st = 0; st < kSteps; ++st) {
+        const int c0 = half * kCover + st * 32;
+        if (n0 + c0 >= p.N) break;
+        const uint32_t acc = tmem_base + (uint32_t)c0 + ((uint32_t)(q * 32) << 16);
+        float v[32];
+        uint4 o[4];
+        if (PROJ) {   // rounded to bf16 as the projection's own layer would store it
+          float w[32];
+          tmem_ld32_issue(acc, v);
+          tmem_ld32_issue(acc + (uint32_t)BN, w);
+          tmem_ld_wait(v, w);
+          epilogue32<false>(p.act2, w, s_sb + 2 * BN + c0, s_sb + 3 * BN + c0, nullptr, r + 4 * st);
+        } else {
+          tmem_ld32(acc, v);
+        }
+        if (PROJ || p.residual)
+          epilogue32<true>(p.act, v, s_sb + c0, s_sb + BN + c0, r + 4 * st, o);
+        else
+          epilogue32<false>(p.act, v, s_sb + c0, s_sb + BN + c0, nullptr, o);
+        if (st) __syncwarp();
+#pragma unroll
+        for (int g = 0; g < 4; ++g) *reinterpret_cast<uint4*>(stage + lane * 64 + ((g ^ (lane >> 1 & 3)) << 4)) = o[g];
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {   // eight rows per store, four lanes with 64 bytes of each
+          const int row = k * 8 + (lane >> 2), g = lane & 3, mm = m0 + q * 32 + row, n = n0 + c0 + g * 8;
+          const uint4 x = *reinterpret_cast<const uint4*>(stage + row * 64 + ((g ^ (row >> 1 & 3)) << 4));
+          if (mm < p.M && n < p.N) *reinterpret_cast<uint4*>(p.out + (size_t)mm * p.N + n) = x;
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 4) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kCols) : "memory");
+  }
+}
+
+inline ee_status_t wave_context_init() {
+  cudaError_t e = cudaSuccess;
+  auto set = [&](auto kernel, int bytes) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  };
+  set(conv_wave_tcgen05_kernel<32, false>, WaveSmem<32>::bytes(WaveSmem<32>::kMaxSlots));
+  set(conv_wave_tcgen05_kernel<32, true>, WaveSmem<32>::bytes(WaveSmem<32>::kMaxSlots));
+  set(conv_wave_tcgen05_kernel<64, false>, WaveSmem<64>::bytes(WaveSmem<64>::kMaxSlots));
+  set(conv_wave_tcgen05_kernel<128, false>, WaveSmem<128>::bytes(WaveSmem<128>::kMaxSlots));
+  return e == cudaSuccess ? EE_OK : EE_ERR_CUDA;
+}
+
+// Slots: as many as the K loop has blocks for; a short loop leaves room on its SM for the next layer's CTA to set up.
+template <int BN, bool PROJ>
+inline cudaError_t wave_launch_t(cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, const CUtensorMap& a2, const CUtensorMap& w2, TcParams p) {
+  using S = WaveSmem<BN>;
+  p.ring = std::min(S::kMaxSlots, std::max(2, p.taps * p.cblocks + (PROJ ? p.cblocks2 : 0)));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cdiv(p.M, kTcBM), cdiv(p.N, BN));
+  cfg.blockDim = dim3(S::kThreads);
+  cfg.dynamicSmemBytes = S::bytes(p.ring);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, conv_wave_tcgen05_kernel<BN, PROJ>, a, w, a2, w2, p);
+}
+
+inline cudaError_t wave_launch(int bn, cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, TcParams p) {
+  return bn == 32 ? wave_launch_t<32, false>(st, a, w, a, w, p) : bn == 64 ? wave_launch_t<64, false>(st, a, w, a, w, p) : wave_launch_t<128, false>(st, a, w, a, w, p);
+}
+inline cudaError_t wave_launch_proj(cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, const CUtensorMap& a2, const CUtensorMap& w2, TcParams p) {
+  return wave_launch_t<32, true>(st, a, w, a2, w2, p);
+}
+
+}  // namespace ee

@@ -142,3 +142,51 @@ def test_convolution_with_several_taps(geom):
         first[B] = g["features_out"][0]
     # the sums do not depend on the batch
     assert np.array_equal(first[1], first[bmax])
+
+
+# one-wave tiles: H, W, cin, cout, k, stride, residual, batches (32-, 64-, 128-filter tiles, then CTAs that share SMs): one K block,
+# as many as slots and one more, ragged pixels, filters and channels, a tile over several images
+WAVE_GEOMS = [
+    (14, 14, 64, 256, 1, 1, True, (1, 13, 24, 49)), (7, 7, 704, 136, 1, 1, True, (2, 65)), (7, 7, 768, 512, 1, 1, False, (1, 24, 50, 97)),
+    (9, 11, 200, 40, 3, 1, False, (1, 5)), (13, 13, 72, 264, 3, 2, True, (3, 40, 90)), (8, 8, 128, 8, 3, 1, True, (1, 7)),
+]
+
+
+@pytest.mark.parametrize("geom", WAVE_GEOMS)
+def test_one_wave_tiles_against_the_oracle_and_at_every_width(geom):
+    H, W, cin, cout, k, stride, residual, batches = geom
+    spec = util.single_layer_model("bf16", H, W, cin, cout, k, stride, k // 2, wl.ACT_RELU, residual, seed=sum(geom[:6]), max_batch=batches[-1])
+    run = util.GpuRunner(spec)
+    for i in range(len(spec.stages[0].layers)):
+        run.m.set_layer_splits(0, i, 1)
+    first = None
+    for B in batches:
+        x = wl.random_features((batches[-1], H, W, cin), seed=6, bf16=True, relu=False)[:B]
+        g = run.stage(0, x)
+        if first is None:
+            util.check_stage(spec, g, util.oracle_stage(spec, 0, x), f"{geom} B={B}", elementwise=not residual)
+            first = g["features_out"]
+        assert np.array_equal(g["features_out"][: len(first)], first), f"{geom} B={B}"
+
+
+@pytest.mark.parametrize("case", [(7, 7, 64, 40, 128, 1, 1), (14, 14, 128, 520, 96, 2, 2), (5, 9, 320, 256, 704, 1, 3)])
+def test_projection_inside_a_one_wave_tile_gives_the_bits_of_two_layers(case):
+    H, W, mid, wide, cin, stride, B = case
+    rng = wl._rng(H + wide, 917)
+    conv = lambda ci, co, s, act, src, res=wl.NO_RESIDUAL: wl._conv(rng, wl.OP_CONV, ci, co, 1, s, 0, act, bf16=True, input_from=src, residual_from=res)  # noqa: E731
+    layers = [conv(cin, mid, stride, wl.ACT_RELU, wl.FROM_STAGE_INPUT), conv(cin, wide, stride, wl.ACT_NONE, wl.FROM_STAGE_INPUT),
+              conv(mid, wide, 1, wl.ACT_RELU, 0, 1)]
+    fw, fb = wl._head(rng, wide, 5, 1.0, True)
+    spec = wl.Model("proj", "bf16", H, W, cin, [wl.Stage(layers, 5, fw, fb, 2.0, False)], B)
+    run = util.GpuRunner(spec)
+    x = eb.to_device("bf16", wl.random_features((B, H, W, cin), seed=8, bf16=True))
+    got = []
+    for fused in (True, False):
+        run.m.set_proj_fusion(fused)
+        run.bufs[0].features_out.fill_(0)
+        run.m.stage_run(0, x, B, run.bufs[0], run.ws)
+        torch.cuda.synchronize()
+        run.m.check()
+        got.append(run.bufs[0].features_out[:B].clone())
+        assert sum(p["launches"] for p in run.m.plan(0, B)) == (2 if fused else 3)
+    assert torch.equal(*got) and bool(got[0].any())

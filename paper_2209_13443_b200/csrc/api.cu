@@ -285,7 +285,7 @@ ee_status_t launch_layer(ee_model* m, const LayerPlan& L, const void* src, const
     }
     case KK_TC_GATHER: {
       if constexpr (sizeof(T) == 2) {
-        ee_status_t s = L.tc.stem7 ? stem_launch(m->tc, L.tc, src, dst, B, L.scale_dev, L.bias_dev, m->err_flag, st, fuse_pool)
+        ee_status_t s = L.tc.stem ? stem_launch(m->tc, L.tc, src, dst, B, L.scale_dev, L.bias_dev, m->err_flag, st, fuse_pool)
                                    : tc_launch(m->tc, L.tc, src, res, dst, B, L.scale_dev, L.bias_dev, m->err_flag, st);
         if (s != EE_OK) return s;
       } else {
@@ -1005,15 +1005,15 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
       } else if (desc->dtype == EE_BF16 && d.cout % 8 == 0 && d.kh * d.kw * d.cin <= 1024 && d.pad_w == d.pad) {
         // pixel rows are not 16-byte units (e.g. a 3-channel stem): explicit Toeplitz rows, then the tensor-core GEMM
         L.kind = KK_TC_GATHER;
-        const bool stem7 = stem_supported(d, L.in_h, L.in_w, L.out_w) && d.residual_from == EE_NO_RESIDUAL;
+        const bool stem = stem_supported(d, L.out_w) && d.residual_from == EE_NO_RESIDUAL;
         const int run = d.kw * d.cin;
         const int runp = cdiv(run, 8) * 8;
-        const int kp = cdiv(d.kh * runp, kTcBK) * kTcBK;
+        const int kp = stem ? stem_packed_cols(d.kh) : cdiv(d.kh * runp, kTcBK) * kTcBK;
         void* wp = nullptr;
         if (cudaMalloc(&wp, (size_t)d.cout * kp * 2) != cudaSuccess) return fail(EE_ERR_CUDA);
         m->owned.push_back(wp);
-        if (stem7)
-          pack_stem_weights_kernel<<<cdiv((long)d.cout * kp, 256), 256, 0, st>>>((const bf16*)L.w_dev, (bf16*)wp, d.cout);
+        if (stem)
+          stem_pack(d.kh, (const bf16*)L.w_dev, (bf16*)wp, d.cout, st);
         else
           pack_weights_kernel<<<cdiv((long)d.cout * kp, 256), 256, 0, st>>>((const bf16*)L.w_dev, (bf16*)wp, d.cout, d.kh, run, runp, kp);
         if (cudaGetLastError() != cudaSuccess) return fail(EE_ERR_CUDA);
@@ -1022,7 +1022,7 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
         rc = tc_plan_layer(m->tc, g, L.out_h, L.out_w, L.out_h, L.out_w, desc->max_batch, wp, &L.tc);
         if (rc != EE_OK) return fail(rc);
         L.tc.gather = true;
-        L.tc.stem7 = stem7;
+        L.tc.stem = stem;
         L.tc.splits = 1, L.tc.kb_per = kp / kTcBK;
         L.tc.g_h = L.in_h, L.tc.g_w = L.in_w, L.tc.g_cin = d.cin, L.tc.g_kh = d.kh, L.tc.g_kw = d.kw;
         L.tc.g_stride = d.stride, L.tc.g_pad = d.pad, L.tc.g_runp = runp;
@@ -1036,7 +1036,7 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
     for (int i = 0; i + 1 < sd.n_layers; ++i) {
       LayerPlan& L = sp.layers[i];
       LayerPlan& P = sp.layers[i + 1];
-      if (L.kind != KK_TC_GATHER || !L.tc.stem7 || !stem_pool_supported(P.d) || i == out_layer) continue;
+      if (L.kind != KK_TC_GATHER || !L.tc.stem || !stem_pool_supported(P.d) || i == out_layer) continue;
       if (src_of[i + 1] != i || n_in_use[i] != 1 || n_res_use[i] != 0) continue;   // someone else reads the convolution's output
       if (L.src_slot >= 0 && L.src_slot == P.out_slot) continue;                  // the pooled tensor would overwrite the input
       L.pool_next = true;

@@ -578,7 +578,7 @@ inline ee_status_t pair_context_init() {
 
 // Layers the pair kernel covers: what the one-CTA tensor-core kernel covers, without the gather mode.
 inline bool pair_supported(const TcLayer& L, int variant) {
-  if (L.gather || L.halo || L.stem7) return false;
+  if (L.gather || L.halo || L.stem) return false;
   return variant == TCV_PAIR256 ? L.cout > 128 : L.cout > 64;
 }
 

@@ -1195,7 +1195,7 @@ struct TcLayer {
   bool rev = false;              // walk the output tiles from the last one down (see TcParams::rev)
   // gather mode: geometry of the real convolution (cin/kh/... above then describe the packed 1x1 GEMM view)
   bool gather = false;
-  bool stem7 = false;   // the 7x7/2 stem kernel of conv_stem.cuh takes this layer
+  bool stem = false;    // the stem kernel of conv_stem.cuh takes this layer
   bool halo = false;    // the 3x3 halo-block kernel of conv_halo.cuh takes this layer
   int g_h = 0, g_w = 0, g_cin = 0, g_kh = 0, g_kw = 0, g_stride = 1, g_pad = 0, g_runp = 0;
   CUtensorMap tm_w;
@@ -1204,7 +1204,7 @@ struct TcLayer {
   struct Cached {
     const void* ptr;
     int batch;
-    int kind;  // 0: operand A, 1: residual / output matrix, 2: stem input rows, 3: stem output rows, 4: halo blocks
+    int kind;  // 0: operand A, 1: output matrix, 4: halo blocks, 7: residual
     CUtensorMap tm;
   };
   mutable std::vector<Cached> a_maps;  // tensor maps of caller buffers by (pointer, batch, kind)
@@ -1354,34 +1354,6 @@ inline ee_status_t tc_buffer_map(const TcContext& c, const TcLayer& L, const voi
     const cuuint32_t box[4] = {kTcBK, (cuuint32_t)wp, (cuuint32_t)rows, 1};
     const cuuint32_t es[4] = {1, 1, 1, 1};
     r = c.encode_tiled(&e.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, es,
-                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  } else if (kind == 2) {
-    // stem input as (W*Cin, H, B): 256 elements of 7 consecutive image rows per load, zero fill outside
-    const cuuint64_t dims[3] = {(cuuint64_t)L.g_w * L.g_cin, (cuuint64_t)L.g_h, (cuuint64_t)batch};
-    const cuuint64_t strides[2] = {(cuuint64_t)L.g_w * L.g_cin * 2, (cuuint64_t)L.g_w * L.g_cin * 2 * L.g_h};
-    const cuuint32_t box[3] = {256, 7, 1};
-    const cuuint32_t es[3] = {1, 1, 1};
-    r = c.encode_tiled(&e.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, es,
-                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  } else if (kind == 3) {
-    // stem output as (Cout, Wo, B*Ho): a tile is one output row, pixels past Wo are clipped
-    const cuuint64_t dims[3] = {(cuuint64_t)L.cout, (cuuint64_t)L.out_w, (cuuint64_t)batch * L.out_h};
-    const cuuint64_t strides[2] = {(cuuint64_t)L.cout * 2, (cuuint64_t)L.cout * 2 * L.out_w};
-    const cuuint32_t box[3] = {64, 32, 1};
-    const cuuint32_t es[3] = {1, 1, 1};
-    r = c.encode_tiled(&e.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, es,
-                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  } else if (kind == 5) {
-    // stem output behind its fused 3x3 stride-2 pad-1 max-pool, as (Cout, Wp, B*Hp): a store is up to 32 pixels of a pooled row
-    const int hp = (L.out_h - 1) / 2 + 1, wp = (L.out_w - 1) / 2 + 1;
-    const cuuint64_t dims[3] = {(cuuint64_t)L.cout, (cuuint64_t)wp, (cuuint64_t)batch * hp};
-    const cuuint64_t strides[2] = {(cuuint64_t)L.cout * 2, (cuuint64_t)L.cout * 2 * wp};
-    const cuuint32_t box[3] = {64, 32, 1};
-    const cuuint32_t es[3] = {1, 1, 1};
-    r = c.encode_tiled(&e.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box, es,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   } else if (kind == 1 || kind == 7) {   // output (a warp's 32 rows per store) / residual operand (a whole tile's rows per load)

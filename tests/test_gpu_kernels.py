@@ -190,3 +190,36 @@ def test_projection_inside_a_one_wave_tile_gives_the_bits_of_two_layers(case):
         got.append(run.bufs[0].features_out[:B].clone())
         assert sum(p["launches"] for p in run.m.plan(0, B)) == (2 if fused else 3)
     assert torch.equal(*got) and bool(got[0].any())
+
+
+# stems: H, W, cout, k, activation, B: rows of an odd number of elements (the batch's last one alone in its word), 128 output columns,
+# one output row, ranges that start inside an image, one and two channel halves
+STEMS = [(161, 161, 64, 7, wl.ACT_RELU, 3), (15, 33, 8, 7, wl.ACT_NONE, 1), (9, 255, 40, 7, wl.ACT_RELU6, 2), (1, 5, 64, 7, wl.ACT_NONE, 3),
+         (63, 65, 32, 3, wl.ACT_RELU6, 5), (20, 256, 64, 3, wl.ACT_RELU, 2), (2, 1, 48, 3, wl.ACT_NONE, 2)]
+
+
+@pytest.mark.parametrize("case", STEMS)
+def test_stem_kernels_with_and_without_the_pool(case):
+    H, W, cout, k, act, B = case
+    rng = wl._rng(H + W, 919)
+    layers = [wl._conv(rng, wl.OP_CONV, 3, cout, k, 2, k // 2, act, bf16=True), wl.Layer(wl.OP_MAXPOOL, cout, cout, 3, 3, 2, 1)]
+    fw, fb = wl._head(rng, cout, 5, 1.0, True)
+    spec = wl.Model("stem", "bf16", H, W, 3, [wl.Stage(layers, 5, fw, fb, 2.0, False)], B)
+    run = util.GpuRunner(spec)
+    m, out = run.m, run.bufs[0]
+    assert [pl["launches"] for pl in m.plan(0, B)] == [1, 0]
+    x = wl.make_input(spec, B, seed=5)
+    xd = eb.to_device("bf16", x)
+    shapes = wl.stage_shapes(spec)[0]["layers"]
+    conv, apart = (torch.empty((B,) + s, dtype=torch.bfloat16, device="cuda") for s in shapes)
+    m.layer_run(0, 0, xd, None, B, conv, run.ws)
+    m.layer_run(0, 1, conv, None, B, apart, run.ws)
+    m.stage_run(0, xd, B, out, run.ws)
+    torch.cuda.synchronize()
+    m.check()
+    assert torch.equal(out.features_out[:B], apart)
+    assert util.rel_err(apart.float().cpu().numpy(), eo.run_layers(spec, 0, x), "bf16") <= util.TOL["bf16"]
+    m.stage_run(0, xd[B - 1:].clone(), 1, out, run.ws)      # alone: other row ranges, the same bits
+    torch.cuda.synchronize()
+    assert torch.equal(out.features_out[0], apart[B - 1])
+    run.check_guards()

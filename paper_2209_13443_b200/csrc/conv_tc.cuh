@@ -1487,7 +1487,7 @@ inline int tc_wave_bn(const TcContext& c, const TcLayer& L, int B) {
   return 0;
 }
 inline cudaError_t wave_launch(int bn, cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, TcParams p);   // conv_wave.cuh
-inline cudaError_t wave_launch_proj(cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, const CUtensorMap& a2, const CUtensorMap& w2, TcParams p);
+inline cudaError_t wave_launch_proj(int bn, cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, const CUtensorMap& a2, const CUtensorMap& w2, TcParams p);
 
 // L with the projection P in its launch: src -> L, src2 -> P; P's own output is never written.
 inline ee_status_t tc_launch_proj(TcContext& c, const TcLayer& L, const TcLayer& P, const void* src, const void* src2, void* dst, int B,
@@ -1520,8 +1520,8 @@ inline ee_status_t tc_launch_proj(TcContext& c, const TcLayer& L, const TcLayer&
   p.scale2 = scale2, p.bias2 = bias2;
   p.gap_part = gap_part, p.gap_g = gap_part ? gap_g : 0;
   // the persistent kernel's long prologue and 128-wide epilogue are for several tiles per SM
-  if (!p.gap_part && tc_wave_bn(c, L, B) == 32)
-    return wave_launch_proj(st, tmA, L.tm_w_bn[0], tmA2, P.tm_w_bn[0], p) == cudaSuccess ? EE_OK : EE_ERR_CUDA;
+  if (const int bn = p.gap_part ? 0 : tc_wave_bn(c, L, B))
+    return wave_launch_proj(bn, st, tmA, bn == L.bn ? L.tm_w : L.tm_w_bn[bn / 64], tmA2, bn == L.bn ? P.tm_w : P.tm_w_bn[bn / 64], p) == cudaSuccess ? EE_OK : EE_ERR_CUDA;
   const cudaError_t e = L.bn == 128 ? tc_launch_persistent_proj<128>(c.sm_count, st, tmA, L.tm_w, tmO, tmA2, P.tm_w, p)
                                     : tc_launch_persistent_proj<64>(c.sm_count, st, tmA, L.tm_w, tmO, tmA2, P.tm_w, p);
   return e == cudaSuccess ? EE_OK : EE_ERR_CUDA;

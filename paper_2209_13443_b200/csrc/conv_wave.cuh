@@ -244,6 +244,8 @@ inline ee_status_t wave_context_init() {
   set(conv_wave_tcgen05_kernel<32, false>, WaveSmem<32>::bytes(WaveSmem<32>::kMaxSlots));
   set(conv_wave_tcgen05_kernel<32, true>, WaveSmem<32>::bytes(WaveSmem<32>::kMaxSlots));
   set(conv_wave_tcgen05_kernel<64, false>, WaveSmem<64>::bytes(WaveSmem<64>::kMaxSlots));
+  set(conv_wave_tcgen05_kernel<64, true>, WaveSmem<64>::bytes(WaveSmem<64>::kMaxSlots));
+  set(conv_wave_tcgen05_kernel<128, true>, WaveSmem<128>::bytes(WaveSmem<128>::kMaxSlots));
   set(conv_wave_tcgen05_kernel<128, false>, WaveSmem<128>::bytes(WaveSmem<128>::kMaxSlots));
   return e == cudaSuccess ? EE_OK : EE_ERR_CUDA;
 }
@@ -269,8 +271,8 @@ inline cudaError_t wave_launch_t(cudaStream_t st, const CUtensorMap& a, const CU
 inline cudaError_t wave_launch(int bn, cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, TcParams p) {
   return bn == 32 ? wave_launch_t<32, false>(st, a, w, a, w, p) : bn == 64 ? wave_launch_t<64, false>(st, a, w, a, w, p) : wave_launch_t<128, false>(st, a, w, a, w, p);
 }
-inline cudaError_t wave_launch_proj(cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, const CUtensorMap& a2, const CUtensorMap& w2, TcParams p) {
-  return wave_launch_t<32, true>(st, a, w, a2, w2, p);
+inline cudaError_t wave_launch_proj(int bn, cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, const CUtensorMap& a2, const CUtensorMap& w2, TcParams p) {
+  return bn == 32 ? wave_launch_t<32, true>(st, a, w, a2, w2, p) : bn == 64 ? wave_launch_t<64, true>(st, a, w, a2, w2, p) : wave_launch_t<128, true>(st, a, w, a2, w2, p);
 }
 
 }  // namespace ee

@@ -169,7 +169,7 @@ def test_one_wave_tiles_against_the_oracle_and_at_every_width(geom):
         assert np.array_equal(g["features_out"][: len(first)], first), f"{geom} B={B}"
 
 
-@pytest.mark.parametrize("case", [(7, 7, 64, 40, 128, 1, 1), (14, 14, 128, 520, 96, 2, 2), (5, 9, 320, 256, 704, 1, 3)])
+@pytest.mark.parametrize("case", [(7, 7, 64, 40, 128, 1, 1), (14, 14, 128, 520, 96, 2, 2), (5, 9, 320, 256, 704, 1, 3), (14, 14, 64, 1000, 72, 1, 5), (14, 14, 192, 1016, 136, 1, 9)])
 def test_projection_inside_a_one_wave_tile_gives_the_bits_of_two_layers(case):
     H, W, mid, wide, cin, stride, B = case
     rng = wl._rng(H + wide, 917)

@@ -137,7 +137,8 @@ typedef struct {
   void* features_out;     /* [n_surv][out_h][out_w][out_c]: the survivors' stage output, compacted, order kept;
                              this is the next stage's input */
   float* conf;            /* [batch] softmax top-1 probability, input order */
-  int32_t* pred;          /* [batch] argmax class (lowest index on ties), input order */
+  int32_t* pred;          /* [batch] argmax class (lowest index on ties), input order.  conf and pred may be pinned host
+                             memory: they are then there when the count is (n_surv_host, ee_wait_count) */
   float* logits;          /* [batch][n_classes] fp32, optional */
   uint8_t* exit_mask;     /* [batch] 1 = sample exits here */
   int32_t* survivor_idx;  /* first n_surv entries: ascending positions (in the input batch) of the survivors */

@@ -138,8 +138,8 @@ def _ptr(t) -> Optional[int]:
 
 
 def _stream(stream) -> Optional[int]:
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:   # the handle alone: building the Stream object takes 5 us
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -150,14 +150,16 @@ def torch_dtype(model_dtype: str):
 class StageBuffers:
     """Caller-owned device buffers of one ee_stage_run call, sized for max_batch (allocated once)."""
 
-    def __init__(self, model: "EEModel", stage: int, with_logits: bool = True, pinned_count: bool = True):
+    def __init__(self, model: "EEModel", stage: int, with_logits: bool = True, pinned_count: bool = True, pinned_decisions: bool = False):
         info = model.query(stage)
         dev, B = model.device, model.max_batch
         td = torch_dtype(model.dtype)
         self.info = info
         self.features_out = torch.empty((B, info["out_h"], info["out_w"], info["out_c"]), dtype=td, device=dev)
-        self.conf = torch.empty(B, dtype=torch.float32, device=dev)
-        self.pred = torch.empty(B, dtype=torch.int32, device=dev)
+        # pinned_decisions: the kernel writes confidences and classes to pinned host memory, where they are when the count is
+        where = dict(pin_memory=True) if pinned_decisions else dict(device=dev)
+        self.conf = torch.empty(B, dtype=torch.float32, **where)
+        self.pred = torch.empty(B, dtype=torch.int32, **where)
         self.logits = torch.empty((B, model.n_classes[stage]), dtype=torch.float32, device=dev) if with_logits else None
         self.exit_mask = torch.empty(B, dtype=torch.uint8, device=dev)
         self.survivor_idx = torch.empty(B, dtype=torch.int32, device=dev)

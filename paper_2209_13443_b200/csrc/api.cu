@@ -336,6 +336,13 @@ ee_status_t launch_layer(ee_model* m, const LayerPlan& L, const void* src, const
   return EE_OK;
 }
 
+bool host_memory(const void* p) {
+  cudaPointerAttributes a;
+  if (p && cudaPointerGetAttributes(&a, p) == cudaSuccess) return a.type == cudaMemoryTypeHost;
+  if (p) cudaGetLastError();
+  return false;
+}
+
 template <typename T>
 ee_status_t launch_head(ee_model* m, StagePlan& sp, const void* x, int B, int hw, const float* shift,
                         const int32_t* shift_cls, char* scratch, const ee_stage_in_t* in_ids, const ee_stage_out_t* out,
@@ -344,11 +351,12 @@ ee_status_t launch_head(ee_model* m, StagePlan& sp, const void* x, int B, int hw
   HeadLayout h = head_layout(m->max_batch, C, K);
   unsigned* cnt = (unsigned*)(scratch + h.off_cnt);
   float* gap = (float*)(scratch + h.off_gap);
+  const bool host_out = host_count && (host_memory(out->conf) || host_memory(out->pred));
   float* z = out->logits ? out->logits : (float*)(scratch + h.off_z);
   if constexpr (sizeof(T) == 2) {
     if (m->fused_head && hc_supported(C, K, x, sp.fc_w)) {
       DecideArgs da{shift, shift_cls, sp.threshold, sp.always_exit, out->conf, out->pred, out->exit_mask,
-                    in_ids ? in_ids->ids : nullptr, out->survivor_idx, out->ids_out, out->n_surv_dev, nullptr, m->head_done + (&sp - m->stages.data()), host_count};
+                    in_ids ? in_ids->ids : nullptr, out->survivor_idx, out->ids_out, out->n_surv_dev, nullptr, m->head_done + (&sp - m->stages.data()), host_count, host_out};
       EE_CUDA(hc_launch((const bf16*)x, hw, C, (const bf16*)sp.fc_w, sp.fc_b, B, K, z, da, st));
       if (timed) record(m, sp, st, "head_gap_fc_softmax_scan");
       return EE_OK;
@@ -389,7 +397,7 @@ ee_status_t launch_head(ee_model* m, StagePlan& sp, const void* x, int B, int hw
     EE_CUDA(launch_pdl(gap_kernel<T, 1>, ggrid, dim3(kGapThreads), st, (const T*)x, hw, C, lanes, gap, cnt, n_zero, sp.gap_rev ? 1 : 0));
   if (timed) record(m, sp, st, "head_gap");
   DecideArgs da{shift, shift_cls, sp.threshold, sp.always_exit, out->conf, out->pred, out->exit_mask,
-                in_ids ? in_ids->ids : nullptr, out->survivor_idx, out->ids_out, out->n_surv_dev, cnt, cnt + m->max_batch, host_count};
+                in_ids ? in_ids->ids : nullptr, out->survivor_idx, out->ids_out, out->n_surv_dev, cnt, cnt + m->max_batch, host_count, host_out};
   if (sp.fc_cluster)
     EE_CUDA(fc_cluster_launch<T>(fc_shape(B, C, K, (int)sizeof(T), m->fc_room), gap, sp.tm_fc, sp.fc_b, B, C, K, out->logits,
                                  (float4*)(scratch + h.off_z), da, m->err_flag, st));

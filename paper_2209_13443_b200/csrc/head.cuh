@@ -186,6 +186,7 @@ struct DecideArgs {  // everything the exit decision needs besides the logits
   unsigned* tile_done;  // per sample tile: CTAs of the FC kernel that have written its logits; zero between launches
   unsigned* done;       // sample tiles whose exit decisions are written; zero between launches
   volatile int32_t* n_surv_host;   // optional: device address of a pinned host word that receives the count (exit_scan)
+  bool host_out;                   // conf or pred is host memory: they reach it before the count does
 };
 
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc, int src_bytes) {  // bytes past src_bytes are zero-filled
@@ -300,7 +301,10 @@ __device__ __forceinline__ void exit_scan(int B, const DecideArgs& d) {
   }
   if (tid == 0) {
     d.n_surv[0] = base;
-    if (d.n_surv_host) *d.n_surv_host = base;   // B_exit goes to the scheduler: the host polls this word
+    if (d.n_surv_host) {
+      if (d.host_out) __threadfence_system();   // the other CTAs' decisions are ordered before this one's counter by device-wide fences
+      *d.n_surv_host = base;   // B_exit goes to the scheduler: the host polls this word
+    }
   }
 }
 

@@ -68,23 +68,24 @@ class FluidServer:
         self.n_stages = self.m.n_stages
         self.bmax = spec.max_batch
         # two buffer sets: the active batch and the batch that catches up to it
-        self.act = [eb.StageBuffers(self.m, s, with_logits=False) for s in range(self.n_stages)]
-        self.new = [eb.StageBuffers(self.m, s, with_logits=False) for s in range(self.n_stages)]
+        self.act = [eb.StageBuffers(self.m, s, with_logits=False, pinned_decisions=True) for s in range(self.n_stages)]
+        self.new = [eb.StageBuffers(self.m, s, with_logits=False, pinned_decisions=True) for s in range(self.n_stages)]
         self.ws = self.m.workspace()
         td = eb.torch_dtype(spec.dtype)
         shape = (self.bmax, spec.in_h, spec.in_w, spec.in_c)
         self.in_act = torch.empty(shape, dtype=td, device="cuda")
         self.in_new = torch.empty(shape, dtype=td, device="cuda")
-        self.ids_act = torch.empty(self.bmax, dtype=torch.int32, device="cuda")
-        self.ids_new = torch.empty(self.bmax, dtype=torch.int32, device="cuda")
-        self.idx_dev = torch.empty(self.bmax, dtype=torch.int32, device="cuda")
-        self.cnt_dev = torch.empty(1, dtype=torch.int32, device="cuda")
-        # pinned staging: request rows / ids / count on their way in, exit masks and classes on their way out
-        self.h_idx = torch.empty(self.bmax, dtype=torch.int32).pin_memory()
-        self.h_ids = torch.empty(self.bmax, dtype=torch.int32).pin_memory()
-        self.h_cnt = torch.empty(1, dtype=torch.int32).pin_memory()
-        self.h_mask = torch.empty(self.bmax, dtype=torch.uint8).pin_memory()
-        self.h_pred = torch.empty(self.bmax, dtype=torch.int32).pin_memory()
+        # a batch's rows of the pool, its count and its requests' ids go up in one copy from pinned staging: rows | count | ids
+        self.up = {}
+        for name in ("act", "new"):
+            host = torch.empty(2 * self.bmax + 1, dtype=torch.int32).pin_memory()
+            dev = torch.empty(2 * self.bmax + 1, dtype=torch.int32, device="cuda")
+            ids = dev[self.bmax + 1:]
+            setattr(self, "ids_" + name, ids)
+            self.up[ids.data_ptr()] = (host, host.numpy(), dev, dev[self.bmax:])
+        # the decision of a sample from its confidence, as the kernel takes it
+        self.thr = [(np.float32(st.threshold), bool(st.always_exit)) for st in spec.stages]
+        self.decided = {id(b): (b.conf.numpy(), b.pred.numpy()) for b in self.act + self.new}
         self.stage_in_bytes = [self.m.query(s)["in_bytes_per_sample"] for s in range(self.n_stages)]
 
     # ------------------------------------------------------------------ measured exit-level latency table
@@ -112,37 +113,38 @@ class FluidServer:
 
     def form_batch(self, pool, rows: Sequence[int], req_ids: Sequence[int], feat, ids):
         """Gathers the requests' inputs (rows of ``pool``) to the front of the batch buffer ``feat``: one small pinned
-        upload of the row list, the ids and the count, then one ee_gather_survivors."""
-        n = len(rows)
-        self.h_idx[:n] = torch.as_tensor(np.asarray(rows, dtype=np.int32))
-        self.h_ids[:n] = torch.as_tensor(np.asarray(req_ids, dtype=np.int32))
-        self.h_cnt[0] = n
-        self.idx_dev[:n].copy_(self.h_idx[:n], non_blocking=True)
-        ids[:n].copy_(self.h_ids[:n], non_blocking=True)
-        self.cnt_dev.copy_(self.h_cnt, non_blocking=True)
-        eb.gather_survivors(pool, self.stage_in_bytes[0], self.idx_dev, self.cnt_dev, n, feat)
+        upload of the row list, the count and the ids (``ids``: ids_act or ids_new), then one ee_gather_survivors.  The staging
+        is free again: the stage that read it has been waited for."""
+        n, b = len(rows), self.bmax
+        host, h, dev, cnt = self.up[ids.data_ptr()]
+        h[:n] = rows
+        h[b] = n
+        h[b + 1:b + 1 + n] = req_ids
+        dev.copy_(host, non_blocking=True)
+        eb.gather_survivors(pool, self.stage_in_bytes[0], dev, cnt, n, feat)
 
     def run_stage(self, s, feat, ids_dev, members, bufs, clock: _Clock, out):
-        """One subnet and its exit on the batch ``members`` (request numbers, in batch order).  The exit mask and the
-        classes travel to pinned host memory behind the stage; the host waits for them once.  Records the requests
-        that leave; returns those that stay."""
-        n = len(members)
-        self.m.stage_run(s, feat, n, bufs[s], self.ws, ids_dev)
-        self.h_mask[:n].copy_(bufs[s].exit_mask[:n], non_blocking=True)
-        self.h_pred[:n].copy_(bufs[s].pred[:n], non_blocking=True)
-        torch.cuda.current_stream().synchronize()            # B_exit (and who left) reaches the scheduler
+        """One subnet and its exit on the batch ``members`` (request numbers, in batch order).  Confidences and classes
+        are in pinned host memory when the survivor count is, and the host waits for that word alone: no copies behind the
+        stage, and the gather of the survivors' features may still run.  Records the requests that leave; returns those
+        that stay."""
+        n, buf = len(members), bufs[s]
+        buf.arm_count()
+        self.m.stage_run(s, feat, n, buf, self.ws, ids_dev)
+        n_stay = buf.wait_count()                            # B_exit (and who left) reaches the scheduler
         now = clock.after_stage(s, n)
         out["launches"].append((s, tuple(members)))
-        mask, pred = self.h_mask[:n].numpy(), self.h_pred[:n].numpy()
+        thr, always = self.thr[s]
+        conf, pred = self.decided[id(buf)]
         stay = []
         for j, r in enumerate(members):
-            if mask[j]:
+            if always or conf[j] >= thr:
                 out["finish"][r] = now
                 out["exit_stage"][r] = s
-                out["pred"][r] = int(pred[j])
+                out["pred"][r] = pred[j]
             else:
                 stay.append(r)
-        assert len(stay) == int(bufs[s].n_surv_host[0])
+        assert len(stay) == n_stay
         return stay
 
     def catch_up(self, pool, image_of, members, upto, clock, out):

@@ -223,3 +223,23 @@ def test_stem_kernels_with_and_without_the_pool(case):
     torch.cuda.synchronize()
     assert torch.equal(out.features_out[0], apart[B - 1])
     run.check_guards()
+
+
+@pytest.mark.parametrize("fused", [False, True])
+def test_decisions_in_pinned_memory_are_there_when_the_count_is(fused):
+    spec = wl.resnet50_ee(seed=1, in_hw=64, n_classes=100, max_batch=64)
+    m = eb.EEModel(spec)
+    m.set_fused_head(fused)
+    ws = m.workspace()
+    dev, pin = eb.StageBuffers(m, 0), eb.StageBuffers(m, 0, pinned_decisions=True)
+    for B in (1, 17, 64):
+        x = eb.to_device("bf16", wl.make_input(spec, B, seed=B))
+        m.stage_run(0, x, B, dev, ws)
+        torch.cuda.synchronize()
+        for _ in range(3):
+            pin.conf.fill_(-1)
+            pin.pred.fill_(-1)
+            pin.arm_count()
+            m.stage_run(0, x, B, pin, ws)
+            n = pin.wait_count()
+            assert n == int(dev.n_surv_dev[0]) and torch.equal(pin.conf[:B], dev.conf[:B].cpu()) and torch.equal(pin.pred[:B], dev.pred[:B].cpu())

@@ -5,11 +5,15 @@
 // has few output tiles and a long K, e.g. 24 x 512 outputs over K = 4608.  Both are answered by mma.m16n8k16.f64 (2048
 // FMAs per instruction; operands converted from float once per fragment instead of once per product) and by cutting
 // K: the 8 warps of a CTA are KG groups that take every KG-th 16-wide K step of a tile, and a cluster of Z CTAs cuts
-// the K range of the tile once more.  Partial tiles (fp64) are added in ascending group order in each CTA and then in
-// ascending CTA order through distributed shared memory; every CTA of the cluster finishes a share of the tile.
+// the K range of the tile once more.  Partial tiles (fp64) are added in ascending group order in each CTA, sent to the CTA
+// that finishes their share of the tile (distributed shared memory) and added there in ascending CTA order.
 // Z, KG and the tile depend on the layer and max_batch only, so a sample's sums are grouped the same way in any batch.
 //
-// Measured on B200: the ResNet-50-shaped fp32 model at 64 x 64, batch 6 (K up to 4608, 12 to 1536 rows): see f32_plan.
+// What a small layer's time is (clocks of one CTA, 32 x 32 tile): 2050 of MMAs per 128 of K, which is the fp64 rate, and around
+// them first operands, reduction and epilogue.  So weights are requested before the wait for the layer in front, scale, bias
+// and residual come to registers during the K loop (fetched at the end they took 5000), tap positions are counted, not divided,
+// and one cluster barrier stands between the K loop and the result.  ResNet-50-shaped fp32 model at 64 x 64, batch 6:
+// 630 -> 567 us a pass with these.
 #pragma once
 #include "common.cuh"
 #include "conv_simt.cuh"
@@ -26,7 +30,11 @@ struct F32Tile {   // WM x WN warps per K group, each MF x NF fragments of 16 x 
   static constexpr int kStageFloats = (kBM + kBN) * kRow;
   static constexpr int kPRow = kBN + 2;                    // doubles per row of a partial tile
   static constexpr int kRing = kStages * kStageFloats * 4, kPart = KG * kBM * kPRow * 8;
-  static constexpr int kBytes = kRing > kPart ? kRing : kPart;
+  static constexpr int kOuts = kBM * kBN / kF32Threads;    // outputs per thread
+  static constexpr int kMain = kRing > kPart ? kRing : kPart;
+  // a cluster's CTAs receive their share of the partial tiles behind the ring; the 64 x 64 tile is not cut further
+  static constexpr int kRecv = KG == 8 ? kBM * kBN * 8 : 0;
+  static constexpr int kBytes = kMain + kRecv;
   static_assert(WM * WN * KG == 8, "8 warps");
   static_assert(kBytes <= 227 * 1024, "exceeds the shared memory of an SM");
 };
@@ -44,12 +52,10 @@ __device__ __forceinline__ void cp_async_zfill(uint32_t dst, const void* src, bo
   else
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4 : 0) : "memory");
 }
-__device__ __forceinline__ double ld_cluster_f64(uint32_t addr, uint32_t rank) {
+__device__ __forceinline__ void st_cluster_f64(uint32_t addr, uint32_t rank, double v) {
   uint32_t a;
-  double v;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
-  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
-  return v;
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
 }
 
 // V: floats per copy (4 when Cin is a multiple of 4 and the pointers are 16-byte aligned, else 1).  k_per: K range of a CTA.
@@ -85,35 +91,59 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
     a_h[i] = in ? ho * g.stride - g.pad : -(1 << 20);   // far outside the image: zeros
     a_w[i] = wo * g.stride - g.pad_w;
   }
-  auto load = [&](int step) {
-    if (step < steps) {
-      const uint32_t st = ring_s + (uint32_t)((step % STAGES) * S::kStageFloats) * 4u;
-      const int k = k_begin + step * KS + ku * V;
-      const bool kin = k < k_end;
-      const int tap = k / g.Cin, ci = k - tap * g.Cin, r = tap / g.kw, s = tap - r * g.kw;
+  // position of this thread's column in stage `step`: K index, channel, filter row and column, walked by counters
+  int k = k_begin + ku * V, ci = k % g.Cin, fs = k / g.Cin % g.kw, fr_ = k / g.Cin / g.kw;
+  const int dci = KS % g.Cin, dtap = KS / g.Cin;
+  auto load_b = [&](int step) {   // weights: K index k_begin + step * KS + ku * V
+    const uint32_t st = ring_s + (uint32_t)((step % STAGES) * S::kStageFloats) * 4u;
+    const int kb = k_begin + step * KS + ku * V;
 #pragma unroll
-      for (int i = 0; i < RA; ++i) {
-        const int row = r0 + i * STEP;
-        if (BM % STEP == 0 || row < BM) {
-          const int hi = a_h[i] + r, wi = a_w[i] + s;
-          const bool in = kin && hi >= 0 && hi < g.H && wi >= 0 && wi < g.W;
-          cp_async_zfill<V * 4>(st + (uint32_t)(row * ROW + ku * V) * 4u, in ? a_base[i] + ((size_t)hi * g.W + wi) * g.Cin + ci : x, in);
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < RB; ++i) {
-        const int row = r0 + i * STEP, n = n0 + row;
-        if (BN % STEP == 0 || row < BN) {
-          const bool in = kin && n < N;
-          cp_async_zfill<V * 4>(st + (uint32_t)((BM + row) * ROW + ku * V) * 4u, in ? w + (size_t)n * K + k : w, in);
-        }
+    for (int i = 0; i < RB; ++i) {
+      const int row = r0 + i * STEP, n = n0 + row;
+      if (BN % STEP == 0 || row < BN) {
+        const bool in = kb < k_end && n < N;
+        cp_async_zfill<V * 4>(st + (uint32_t)((BM + row) * ROW + ku * V) * 4u, in ? w + (size_t)n * K + kb : w, in);
       }
     }
-    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto load_a = [&](int step) {
+    const uint32_t st = ring_s + (uint32_t)((step % STAGES) * S::kStageFloats) * 4u;
+#pragma unroll
+    for (int i = 0; i < RA; ++i) {
+      const int row = r0 + i * STEP;
+      if (BM % STEP == 0 || row < BM) {
+        const int hi = a_h[i] + fr_, wi = a_w[i] + fs;
+        const bool in = k < k_end && hi >= 0 && hi < g.H && wi >= 0 && wi < g.W;
+        cp_async_zfill<V * 4>(st + (uint32_t)(row * ROW + ku * V) * 4u, in ? a_base[i] + ((size_t)hi * g.W + wi) * g.Cin + ci : x, in);
+      }
+    }
+    k += KS, ci += dci, fs += dtap;
+    if (ci >= g.Cin) ci -= g.Cin, ++fs;
+    while (fs >= g.kw) fs -= g.kw, ++fr_;
   };
 
+  // no kernel writes weights, scale or bias: requested before the layer in front has finished
+#pragma unroll
+  for (int s = 0; s < STAGES - 1; ++s)
+    if (s < steps) load_b(s);
+  if (Z > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  // outputs z * share + tid, + 256, ...: one channel per thread (256 is a multiple of every BN)
+  const int share = BM * BN / Z, out_first = z * share + tid;   // Z is 1, 2, 4 or 8: divides every tile
+  const int nc = n0 + out_first % BN;
+  const float sc = scale && nc < N ? scale[nc] : 1.f, bi = bias && nc < N ? bias[nc] : 0.f;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#pragma unroll
+  for (int s = 0; s < STAGES - 1; ++s) {
+    if (s < steps) load_a(s);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  float res[S::kOuts];
+#pragma unroll
+  for (int i = 0; i < S::kOuts; ++i) {
+    const int m = m0 + (out_first + i * kF32Threads) / BN;
+    res[i] = residual && tid + i * kF32Threads < share && m < M && nc < N ? residual[(size_t)m * N + nc] : 0.f;
+  }
   const int kg = warp / (WM * WN), wmn = warp % (WM * WN), wm = wmn / WN, wn = wmn % WN;
   const int fr = lane >> 2, fk = lane & 3;            // fragment row (column of B) and K position of this lane
   double acc[MF][NF][4];
@@ -123,12 +153,15 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
     for (int j = 0; j < NF; ++j)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.0;
-#pragma unroll
-  for (int s = 0; s < STAGES - 1; ++s) load(s);
   for (int step = 0; step < steps; ++step) {
     asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
     __syncthreads();                                  // this stage has landed for all; the stage refilled below was read one step ago
-    load(step + STAGES - 1);
+    if (step + STAGES - 1 < steps) {
+      load_a(step + STAGES - 1);
+      load_b(step + STAGES - 1);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (k_begin + step * KS + kg * 16 >= k_end) continue;   // past the range: zeros
     const float* as = ring + (step % STAGES) * S::kStageFloats + (wm * MF * 16 + fr) * ROW + kg * 16 + fk;
     const float* bs = ring + (step % STAGES) * S::kStageFloats + (BM + wn * NF * 8 + fr) * ROW + kg * 16 + fk;
     double b[NF][4];
@@ -160,36 +193,39 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
           *reinterpret_cast<double2*>(p + (i * 16 + 8 * h) * S::kPRow + j * 8) = make_double2(acc[i][j][2 * h], acc[i][j][2 * h + 1]);
   }
   __syncthreads();
-  if (Z > 1) {
-    if (KG > 1) {
-      for (int idx = tid; idx < BM * BN; idx += kF32Threads) {
-        const int o = (idx / BN) * S::kPRow + idx % BN;
-        double v = part[o];
+  auto group_sum = [&](int o) {
+    double v = part[o];
 #pragma unroll
-        for (int q = 1; q < KG; ++q) v += part[q * BM * S::kPRow + o];
-        part[o] = v;
-      }
+    for (int q = 1; q < KG; ++q) v += part[q * BM * S::kPRow + o];
+    return v;
+  };
+  double* recv = reinterpret_cast<double*>(f32_smem + S::kMain);   // [Z][share]
+  if (Z > 1) {
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");   // every CTA of the cluster runs
+    const uint32_t recv_s = ring_s + (uint32_t)S::kMain;
+#pragma unroll
+    for (int i = 0; i < S::kOuts; ++i) {
+      const int idx = tid + i * kF32Threads, q = idx / share;
+      st_cluster_f64(recv_s + (uint32_t)(z * share + idx - q * share) * 8u, (uint32_t)q, group_sum(idx / BN * S::kPRow + idx % BN));
     }
     asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
   }
-  const uint32_t part_s = ring_s;
-  const int share = BM * BN / Z;                      // Z is 1, 2, 4 or 8: divides every tile
-  for (int idx = z * share + tid; idx < (z + 1) * share; idx += kF32Threads) {
-    const int r = idx / BN, c = idx % BN, m = m0 + r, n = n0 + c;
-    if (m >= M || n >= N) continue;
-    const int o = r * S::kPRow + c;
+#pragma unroll
+  for (int i = 0; i < S::kOuts; ++i) {
+    const int rel = tid + i * kF32Threads, idx = z * share + rel, m = m0 + idx / BN;
+    if (rel >= share || m >= M || nc >= N) continue;
     double v = 0.0;
     if (Z > 1) {
-      for (int q = 0; q < Z; ++q) v += ld_cluster_f64(part_s + (uint32_t)o * 8u, (uint32_t)q);
-    } else {
 #pragma unroll
-      for (int q = 0; q < KG; ++q) v += part[q * BM * S::kPRow + o];
+      for (int q = 0; q < 8; ++q)
+        if (q < Z) v += recv[q * share + rel];
+    } else {
+      v = group_sum(idx / BN * S::kPRow + idx % BN);
     }
-    v = (double)(scale ? scale[n] : 1.f) * v + (double)(bias ? bias[n] : 0.f);
-    if (residual) v += (double)residual[(size_t)m * N + n];
-    y[(size_t)m * N + n] = (float)apply_act(v, g.act);
+    v = (double)sc * v + (double)bi;
+    if (residual) v += (double)res[i];
+    y[(size_t)m * N + nc] = (float)apply_act(v, g.act);
   }
-  if (Z > 1) asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");   // peers may still read this CTA's partials
 }
 
 // ----------------------------------------------------------------------------- host side

@@ -237,7 +237,7 @@ struct F32Plan {
 
 // Tile and cluster size of a layer, from its geometry and max_batch.  Short K (stems on 3 channels): one K group, a ring
 // stage is 16 wide and nothing is padded to 128.  Grids of two waves of 64 x 64 tiles: that tile reads its operands least.
-// Everything else has idle SMs: small tiles, eight K groups, and as many CTAs per tile (up to 8) as keep the grid within
+// Everything else has idle SMs: small tiles (16 rows where the layer never has more than 32), eight K groups, and as many CTAs per tile (up to 8) as keep the grid within
 // two CTAs per SM while every CTA still has two ring stages of K.
 inline F32Plan f32_plan(long m_max, int n, int k, int sms) {
   F32Plan p;
@@ -246,7 +246,7 @@ inline F32Plan f32_plan(long m_max, int n, int k, int sms) {
     p.tile = 1;
     return p;
   }
-  p.tile = m_max <= 16 ? 3 : 2;
+  p.tile = m_max <= 32 ? 3 : 2;   // 17 to 32 rows are two 16-row tiles: the same products, and half of them once samples have left
   const long tiles = (long)cdiv(m_max, p.tile == 3 ? 16 : 32) * cdiv(n, 32);
   while (p.z < 8 && tiles * p.z * 2 <= 2L * sms && k >= p.z * 2 * 256) p.z *= 2;
   return p;

@@ -20,6 +20,7 @@ F32_GEOMS = [
     (57, 55, 16, 72, 3, 1, 1, True),     # 64 x 64 tiles, two K groups, K tail inside a ring stage
     (8, 8, 136, 72, 3, 1, 1, False),     # 32 x 32 tiles, a cluster cuts K
     (2, 1, 512, 64, 3, 1, 1, True),      # 16 x 32 tiles, K = 4608 over eight CTAs
+    (2, 3, 136, 40, 3, 1, 1, True),      # 30 rows at the largest batch: two of them
     (3, 1, 150, 33, 3, 1, 1, False),     # 4-byte copies (Cin not a multiple of 4), last CTA's K range short, odd N
     (6, 5, 37, 8, 2, 1, 0, False),       # K = 148: one full ring stage and a tail
 ]

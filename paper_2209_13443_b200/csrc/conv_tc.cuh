@@ -319,16 +319,16 @@ __device__ __forceinline__ void epilogue32(int act, const float* v, const float*
   else epilogue32_t<EE_ACT_NONE, RES>(v, scale, bias, res, out);
 }
 
-// Column sums over the 32 rows a warp holds (ov: this lane's row, 64 bf16 columns as eight 16-byte groups), written as
+// Column sums over the 32 rows a warp holds (ov: this lane's row, 32 bf16 columns as four 16-byte groups), written as
 // block sums of G rows (see TcParams::gap_g).  Halving butterfly: in the step of distance d a lane keeps half of its
 // columns and receives its partner's values for them, so that every (block, column) sum is formed once, by the tree
-// ((r, r + G/2), then distance G/4, ...).  Afterwards lane l holds columns [2l, 2l + 2) of the block (G = 32) or
-// columns [4 (l % 16), + 4) of block l / 16 (G = 16).
+// ((r, r + G/2), then distance G/4, ...).  Afterwards lane l holds column l of the block (G = 32) or
+// columns [2 (l % 16), + 2) of block l / 16 (G = 16).
 template <int G>
 __device__ __forceinline__ void gap_partial_store(const uint4* ov, int lane, float* dst, int cols_left, size_t block_stride, bool rows_ok) {
-  float f[64];
+  float f[32];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int i = 0; i < 4; ++i) {
     const uint32_t w[4] = {ov[i].x, ov[i].y, ov[i].z, ov[i].w};
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -337,7 +337,7 @@ __device__ __forceinline__ void gap_partial_store(const uint4* ov, int lane, flo
     }
   }
 #pragma unroll
-  for (int d = G / 2, n = 32; d >= 1; d >>= 1, n >>= 1) {
+  for (int d = G / 2, n = 16; d >= 1; d >>= 1, n >>= 1) {
     const bool up = (lane & d) != 0;
 #pragma unroll
     for (int i = 0; i < n; ++i) {
@@ -347,10 +347,10 @@ __device__ __forceinline__ void gap_partial_store(const uint4* ov, int lane, flo
   }
   if (!rows_ok) return;
   if (G == 32) {
-    if (2 * lane < cols_left) *reinterpret_cast<float2*>(dst + 2 * lane) = make_float2(f[0], f[1]);
+    if (lane < cols_left) dst[lane] = f[0];
   } else {
-    const int c = 4 * (lane & 15);
-    if (c < cols_left) *reinterpret_cast<float4*>(dst + (size_t)(lane >> 4) * block_stride + c) = make_float4(f[0], f[1], f[2], f[3]);
+    const int c = 2 * (lane & 15);
+    if (c < cols_left) *reinterpret_cast<float2*>(dst + (size_t)(lane >> 4) * block_stride + c) = make_float2(f[0], f[1]);
   }
 }
 
@@ -793,7 +793,9 @@ template <int BN, bool RES, bool PROJ = false>
 struct TcPersistSmem {
   // without a residual: a longer ring and two output staging tiles; with one: two residual tiles the producer
   // prefetches (free again as soon as the epilogue has read them) and a single staging tile
-  static constexpr int kEpiWarps = BN == 128 ? 8 : 4;   // at BN = 128 two warps share a TMEM lane quarter, one per 64-column half
+  // One warp per 32 rows and 32 columns.  A tile's epilogue is a chain of latencies (tensor memory, scale and bias, residual,
+  // staging), not of issue slots: with 64 columns a warp it took 3900 clocks a tile and bound every multi-wave 1x1 layer.
+  static constexpr int kEpiWarps = 4 * (BN / 32);
   static constexpr int kThreads = 96 + 32 * kEpiWarps;  // weight producer, MMA warp, epilogue warps, activation producer
   static constexpr int kStages = RES ? (BN == 128 ? 3 : 5) : (BN == 128 ? 4 : 7);
   static constexpr int kABytes = kTcBM * kTcBK * 2;
@@ -804,7 +806,7 @@ struct TcPersistSmem {
   static constexpr int kROff = kTiles;
   static constexpr int kOOff = kTiles + (RES ? 2 * kIoBytes : 0);
   static constexpr int kAfter = kOOff + (RES ? 1 : 2) * kIoBytes;
-  static constexpr int kSb = (PROJ ? 4 : 2) * BN;   // floats per epilogue warp: scale | bias (| scale2 | bias2)
+  static constexpr int kSb = (PROJ ? 4 : 2) * 32;   // floats per epilogue warp, of its columns: scale | bias (| scale2 | bias2)
   static constexpr int kBytes = kAfter + kEpiWarps * kSb * 4 + 256 + 1024;  // + one scale/bias copy per epilogue warp, barriers, slack
   static_assert(!(RES && PROJ), "the projection replaces the residual tile");
   static_assert(kBytes <= 227 * 1024, "exceeds the shared memory of an SM");
@@ -1013,8 +1015,8 @@ conv_igemm_tcgen05_persistent_kernel(const __grid_constant__ CUtensorMap tmA, co
     const int q = warp & 3;
     const int row = q * 32 + lane;
     const int ew = warp - 2;
-    const int h0 = BN == 128 ? (ew >> 2) : 0, h1 = h0 + 1;  // the 64-column half (halves) this warp owns
-    float* sc = s_sb + ew * S::kSb;  // this warp's own copy: no barrier across warps inside the tile loop
+    const int c0 = (ew >> 2) * 32;   // this warp's columns of the tile
+    float* sc = s_sb + ew * S::kSb;  // their scale and bias, this warp's own copy: no barrier across warps inside the tile loop
     bool ok = true;
     int sc_n0 = -1;
     bool pending = false;  // lane 0: a bulk store group of this warp may still be reading shared memory
@@ -1024,14 +1026,13 @@ conv_igemm_tcgen05_persistent_kernel(const __grid_constant__ CUtensorMap tmA, co
       const int b = j & 1;
       if (n0 != sc_n0) {  // consecutive tiles of a CTA usually share the N tile: reload only on change
         __syncwarp();
-        for (int i = lane; i < BN; i += 32) {
-          const bool in = n0 + i < p.N;
-          sc[i] = (p.scale && in) ? p.scale[n0 + i] : 1.f;
-          sc[BN + i] = (p.bias && in) ? p.bias[n0 + i] : 0.f;
-          if (PROJ) {
-            sc[2 * BN + i] = (p.scale2 && in) ? p.scale2[n0 + i] : 1.f;
-            sc[3 * BN + i] = (p.bias2 && in) ? p.bias2[n0 + i] : 0.f;
-          }
+        const int n = n0 + c0 + lane;
+        const bool in = n < p.N;
+        sc[lane] = (p.scale && in) ? p.scale[n] : 1.f;
+        sc[32 + lane] = (p.bias && in) ? p.bias[n] : 0.f;
+        if (PROJ) {
+          sc[64 + lane] = (p.scale2 && in) ? p.scale2[n] : 1.f;
+          sc[96 + lane] = (p.bias2 && in) ? p.bias2[n] : 0.f;
         }
         sc_n0 = n0;
       }
@@ -1045,79 +1046,51 @@ conv_igemm_tcgen05_persistent_kernel(const __grid_constant__ CUtensorMap tmA, co
         __syncwarp();
       }
       const int ob = RES ? 0 : b;  // output staging tile of this tile
-      uint8_t* io = gen + S::kOOff + ob * S::kIoBytes;
-      const uint32_t io_s = base + S::kOOff + ob * S::kIoBytes;
-      const uint8_t* rin = gen + S::kROff + b * S::kIoBytes;
-      const uint32_t acc = tmem_base + (uint32_t)(b * kAccs * BN) + ((uint32_t)(q * 32) << 16);
-#pragma unroll 1
-      for (int h = h0; h < h1; ++h) {
-        uint4 proj[8];   // PROJ: the projection's 64 values of this row, rounded to bf16 as the layer itself would store them
-        if (PROJ) {
-          float pa[32], pb[32];
-          tmem_ld32_issue(acc + (uint32_t)(BN + h * 64), pa);
-          tmem_ld32_issue(acc + (uint32_t)(BN + h * 64 + 32), pb);
-          tmem_ld_wait(pa, pb);
-#pragma unroll
-          for (int sub = 0; sub < 2; ++sub) {
-            const int c0 = h * 64 + sub * 32;
-            const float* v = sub ? pb : pa;
-#pragma unroll
-            for (int gq = 0; gq < 4; ++gq)
-              proj[sub * 4 + gq] = epilogue8_act<false>(p.act2, v + gq * 8, sc + 2 * BN + c0 + gq * 8, sc + 3 * BN + c0 + gq * 8, make_uint4(0u, 0u, 0u, 0u));
-          }
-        }
-        uint4 ov[8];           // this row's 64 outputs of the half (kept for the pooling partials)
-#pragma unroll
-        for (int i = 0; i < 8; ++i) ov[i] = make_uint4(0u, 0u, 0u, 0u);
-        float va[32], vb[32];  // both 32-column loads of the half in flight before one wait
-        tmem_ld32_issue(acc + (uint32_t)(h * 64), va);
-        tmem_ld32_issue(acc + (uint32_t)(h * 64 + 32), vb);
-        tmem_ld_wait(va, vb);
-        if (h == h1 - 1) {  // this warp's share of the accumulator is in registers: the MMA warp may refill it
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty(b)) : "memory");
-        }
-        if (RES && h == h0) {  // single staging tile: this warp's previous store must have finished reading it
-          if (lane == 0 && pending) {
-            asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-            pending = false;
-          }
-          __syncwarp();
-        }
-#pragma unroll
-        for (int sub = 0; sub < 2; ++sub) {
-          const int c0 = h * 64 + sub * 32;
-          const float* v = sub ? vb : va;
-#pragma unroll
-          for (int gq = 0; gq < 4; ++gq) {
-            if (n0 + c0 + gq * 8 >= p.N) break;   // columns past Cout: nothing to compute, the store clips them
-            const int off = h * 16384 + row * 128 + (((sub * 4 + gq) ^ (lane & 7)) << 4);
-            const uint4 r = RES ? *reinterpret_cast<const uint4*>(rin + off) : PROJ ? proj[sub * 4 + gq] : make_uint4(0u, 0u, 0u, 0u);
-            ov[sub * 4 + gq] = epilogue8_act<RES || PROJ>(p.act, v + gq * 8, sc + c0 + gq * 8, sc + BN + c0 + gq * 8, r);
-            *reinterpret_cast<uint4*>(io + off) = ov[sub * 4 + gq];
-          }
-        }
-        if (p.gap_g) {   // rows past M hold zero-filled operands, but their bias and residual garbage must not be summed: whole blocks are skipped
-          const int r0 = m0 + q * 32;
-          if (p.gap_g == 32)
-            gap_partial_store<32>(ov, lane, p.gap_part + (size_t)(r0 / 32) * p.N + n0 + h * 64, p.N - n0 - h * 64, 0, r0 < p.M);
-          else
-            gap_partial_store<16>(ov, lane, p.gap_part + (size_t)(r0 / 16) * p.N + n0 + h * 64, p.N - n0 - h * 64, (size_t)p.N,
-                                  r0 + (lane >> 4) * 16 < p.M);
-        }
+      const int io = S::kOOff + ob * S::kIoBytes + ew * 2048;   // 32 rows of 64 bytes, chunks XORed with the row (64-byte swizzle)
+      const uint8_t* rin = gen + S::kROff + b * S::kIoBytes + (c0 >> 6) * 16384 + row * 128;
+      const uint32_t acc = tmem_base + (uint32_t)(b * kAccs * BN + c0) + ((uint32_t)(q * 32) << 16);
+      const bool wanted = n0 + c0 < p.N;   // columns past Cout: nothing to compute, the store clips them
+      float v[32];
+      uint4 r[4], ov[4];
+      if (PROJ) {   // the projection's 32 values of this row, rounded to bf16 as the layer itself would store them
+        float w[32];
+        tmem_ld32_issue(acc, v);
+        tmem_ld32_issue(acc + (uint32_t)BN, w);
+        tmem_ld_wait(v, w);
+        if (wanted) epilogue32<false>(p.act2, w, sc + 64, sc + 96, nullptr, r);
+      } else {
+        tmem_ld32(acc, v);
       }
-      if (RES) {  // the residual tile is consumed: the producer may prefetch the one of tile j + 2 into it
-        __syncwarp();
-        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(res_free(b)) : "memory");
+      tc_fence_before();   // this warp's share of the accumulator is in registers: the MMA warp may refill it
+      if (RES) {
+#pragma unroll
+        for (int g = 0; g < 4; ++g) r[g] = *reinterpret_cast<const uint4*>(rin + ((((c0 >> 3) + g) & 7 ^ (lane & 7)) << 4));
+      }
+      __syncwarp();
+      if (lane == 0) {
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty(b)) : "memory");
+        if (RES && pending) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // single staging tile: read by this warp's previous store
+      }
+      if (wanted) epilogue32<RES || PROJ>(p.act, v, sc, sc + 32, r, ov);
+      __syncwarp();
+      if (wanted) {
+#pragma unroll
+        for (int g = 0; g < 4; ++g) *reinterpret_cast<uint4*>(gen + io + lane * 64 + ((g ^ (lane >> 1 & 3)) << 4)) = ov[g];
+      }
+      if (p.gap_g && wanted) {   // rows past M hold zero-filled operands, but their bias and residual garbage must not be summed: whole blocks are skipped
+        const int r0 = m0 + q * 32, n = n0 + c0;
+        if (p.gap_g == 32)
+          gap_partial_store<32>(ov, lane, p.gap_part + (size_t)(r0 / 32) * p.N + n, p.N - n, 0, r0 < p.M);
+        else
+          gap_partial_store<16>(ov, lane, p.gap_part + (size_t)(r0 / 16) * p.N + n, p.N - n, (size_t)p.N, r0 + (lane >> 4) * 16 < p.M);
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) {
-        if (m0 + q * 32 < p.M) {
-          for (int h = h0; h < h1; ++h)
-            if (n0 + h * 64 < p.N) tma_store_2d(&tmO, io_s + h * 16384 + q * 4096, n0 + h * 64, m0 + q * 32);
-        }
+        // the residual went into the staged result: the producer may prefetch the one of tile j + 2 (an arrival ahead of that use
+        // let the loads slip behind it, and the next tile's residual in)
+        if (RES) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(res_free(b)) : "memory");
+        if (m0 + q * 32 < p.M && wanted) tma_store_2d(&tmO, base + (uint32_t)io, n0 + c0, m0 + q * 32);
         asm volatile("cp.async.bulk.commit_group;" ::: "memory");  // possibly empty: keeps the bookkeeping uniform
         pending = true;
       }
@@ -1204,7 +1177,7 @@ struct TcLayer {
   struct Cached {
     const void* ptr;
     int batch;
-    int kind;  // 0: operand A, 1: output matrix, 4: halo blocks, 7: residual
+    int kind;  // 0: operand A, 1, 8: output matrix, 4: halo blocks, 7: residual
     CUtensorMap tm;
   };
   mutable std::vector<Cached> a_maps;  // tensor maps of caller buffers by (pointer, batch, kind)
@@ -1356,13 +1329,13 @@ inline ee_status_t tc_buffer_map(const TcContext& c, const TcLayer& L, const voi
     r = c.encode_tiled(&e.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, es,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  } else if (kind == 1 || kind == 7) {   // output (a warp's 32 rows per store) / residual operand (a whole tile's rows per load)
+  } else if (kind == 1 || kind == 7 || kind == 8) {   // output (32 rows per store; 8: of 32 columns) / residual operand (a whole tile's rows per load)
     const cuuint64_t dims[2] = {(cuuint64_t)L.cout, (cuuint64_t)batch * L.out_h * L.out_w};
     const cuuint64_t strides[1] = {(cuuint64_t)L.cout * 2};
-    const cuuint32_t box[2] = {64, kind == 1 ? 32u : (cuuint32_t)kTcBM};
+    const cuuint32_t box[2] = {kind == 8 ? 32u : 64u, kind == 7 ? (cuuint32_t)kTcBM : 32u};
     const cuuint32_t es[2] = {1, 1};
     r = c.encode_tiled(&e.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, es,
-                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                       CU_TENSOR_MAP_INTERLEAVE_NONE, kind == 8 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   } else if (!L.im2col) {
     const cuuint64_t dims[2] = {(cuuint64_t)L.cin, (cuuint64_t)batch * L.in_h * L.in_w};
@@ -1495,7 +1468,7 @@ inline ee_status_t tc_launch_proj(TcContext& c, const TcLayer& L, const TcLayer&
                                   cudaStream_t st, float* gap_part = nullptr, int gap_g = 0) {
   if (((uintptr_t)src & 15) || ((uintptr_t)src2 & 15) || ((uintptr_t)dst & 15)) return EE_ERR_INVALID_ARG;
   const CUtensorMap* t = nullptr;
-  ee_status_t s = tc_buffer_map(c, L, dst, B, 1, &t);
+  ee_status_t s = tc_buffer_map(c, L, dst, B, 8, &t);
   if (s != EE_OK) return s;
   const CUtensorMap tmO = *t;
   if ((s = tc_buffer_map(c, L, src, B, 0, &t)) != EE_OK) return s;
@@ -1606,6 +1579,8 @@ inline ee_status_t tc_launch(TcContext& c, const TcLayer& L, const void* src, co
   if (!split && L.kh * L.kw == 1 && tiles >= 2 * c.sm_count) {  // several waves of short K loops: one persistent CTA per SM walks the tiles
     const int ctas = c.sm_count;
     cudaError_t pe;
+    if ((s = tc_buffer_map(c, L, dst, B, 8, &t)) != EE_OK) return s;
+    const CUtensorMap tmO = *t;
     if (L.bn == 128)
       pe = res ? tc_launch_persistent<128, true>(ctas, st, tmA, L.tm_w, tmR, tmO, p) : tc_launch_persistent<128, false>(ctas, st, tmA, L.tm_w, tmR, tmO, p);
     else

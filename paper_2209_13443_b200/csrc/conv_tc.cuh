@@ -1053,14 +1053,10 @@ conv_igemm_tcgen05_persistent_kernel(const __grid_constant__ CUtensorMap tmA, co
       float v[32];
       uint4 r[4], ov[4];
       if (PROJ) {   // the projection's 32 values of this row, rounded to bf16 as the layer itself would store them
-        float w[32];
-        tmem_ld32_issue(acc, v);
-        tmem_ld32_issue(acc + (uint32_t)BN, w);
-        tmem_ld_wait(v, w);
-        if (wanted) epilogue32<false>(p.act2, w, sc + 64, sc + 96, nullptr, r);
-      } else {
-        tmem_ld32(acc, v);
+        tmem_ld32(acc + (uint32_t)BN, v);   // one accumulator after the other: both at once do not fit 16 warps' registers
+        if (wanted) epilogue32<false>(p.act2, v, sc + 64, sc + 96, nullptr, r);
       }
+      tmem_ld32(acc, v);
       tc_fence_before();   // this warp's share of the accumulator is in registers: the MMA warp may refill it
       if (RES) {
 #pragma unroll

@@ -275,6 +275,7 @@ __device__ __forceinline__ void exit_scan(int B, const DecideArgs& d) {
   for (int p0 = 0; p0 < B; p0 += THREADS) {
     const int b = p0 + tid;
     const bool keep = b < B && __ldcg(d.mask + b) == 0;
+    const int id = b < B && d.ids && d.ids_out ? d.ids[b] : 0;   // asked for together with the flag
     const unsigned bal = __ballot_sync(0xffffffffu, keep);
     const int pre = __popc(bal & ((1u << lane) - 1u));
     if (lane == 0) warp_tot[warp] = __popc(bal);
@@ -294,7 +295,7 @@ __device__ __forceinline__ void exit_scan(int B, const DecideArgs& d) {
     if (keep) {
       const int pos = base + warp_tot[warp] + pre;
       d.surv_idx[pos] = b;
-      if (d.ids && d.ids_out) d.ids_out[pos] = d.ids[b];
+      if (d.ids && d.ids_out) d.ids_out[pos] = id;
     }
     base += pass_total;
     __syncthreads();
@@ -433,6 +434,17 @@ fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restri
   };
 #pragma unroll
   for (int t = 0; t < kFcRing - 1; ++t) load();
+  // bias of the classes this lane finishes in a group (see the butterfly below): the first group's ahead of the wait
+  constexpr int LEFT = NV > 32 ? NV / 32 : 1, REP = NV < 32 ? 32 / NV : 1;   // values per lane, lanes per value
+  float bias[LEFT];
+  auto load_bias = [&](int g) {
+#pragma unroll
+    for (int j = 0; j < LEFT; ++j) {
+      const int k = k0 + g * kFcRows + ((lane / REP) * LEFT + j) % kFcRows;
+      bias[j] = bfc && k < K && g < ngroups ? bfc[k] : 0.f;
+    }
+  };
+  load_bias(warp);
   pdl_wait();
   pdl_launch_dependents();
   // pooled vectors: within a chunk the float4 `e` of lane l's VEC channels sits at [e][l], so that a warp's reads are 512
@@ -504,13 +516,13 @@ fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restri
           v[0] += __shfl_xor_sync(0xffffffffu, v[0], dd);
         }
       }
-      constexpr int LEFT = NV > 32 ? NV / 32 : 1, REP = NV < 32 ? 32 / NV : 1;   // values per lane, lanes per value
 #pragma unroll
       for (int j = 0; j < LEFT; ++j) {
         const int idx = (lane / REP) * LEFT + j, s = idx / kFcRows, kl = grp * kFcRows + idx % kFcRows;
-        if (lane % REP == 0) zs[s * kc + kl] = (float)(v[j] + (A)((bfc && k0 + kl < K) ? bfc[k0 + kl] : 0.f));
+        if (lane % REP == 0) zs[s * kc + kl] = (float)(v[j] + (A)bias[j]);
       }
       grp += WARPS;
+      load_bias(grp);
     }
     if (++ch == nchunk) ch = 0;
   }

@@ -89,16 +89,21 @@ dwconv3x3_tma_kernel(const __grid_constant__ CUtensorMap tmX, DwParams p) {
   const bool live = item0 < item_step;      // nv need not divide 256: the threads of the ragged tail idle
   const int c = c0 + cvec * 8;
   const bool c_in = c < p.C;
-  uint32_t wr[36];   // the vector's 72 weights as stored: element e = channel e / 9, tap e % 9
+  // The vector's 72 weights as floats, [tap][channel]: unpacked from bf16 once, not at every product (two of three instructions
+  // of a strip were such shifts and masks).
+  float wf[9][8];
+  {
+    uint32_t wr[36];   // as stored: element e = channel e / 9, tap e % 9
 #pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const uint4 v = (!POOL && c_in) ? __ldg(reinterpret_cast<const uint4*>(p.w + (size_t)c * 9) + i) : make_uint4(0u, 0u, 0u, 0u);
-    wr[4 * i] = v.x, wr[4 * i + 1] = v.y, wr[4 * i + 2] = v.z, wr[4 * i + 3] = v.w;
+    for (int i = 0; i < 9; ++i) {
+      const uint4 v = (!POOL && c_in) ? __ldg(reinterpret_cast<const uint4*>(p.w + (size_t)c * 9) + i) : make_uint4(0u, 0u, 0u, 0u);
+      wr[4 * i] = v.x, wr[4 * i + 1] = v.y, wr[4 * i + 2] = v.z, wr[4 * i + 3] = v.w;
+    }
+#pragma unroll
+    for (int e = 0; e < 72; ++e) wf[e % 9][e / 9] = (e & 1) ? __uint_as_float(wr[e >> 1] & 0xffff0000u) : __uint_as_float(wr[e >> 1] << 16);
+#pragma unroll
+    for (int e = 0; e < 72; ++e) asm volatile("" : "+f"(wf[e % 9][e / 9]));   // floats from here on: not to be unpacked again in the loop
   }
-  auto weight = [&](int tap, int ch) {   // indices are compile-time constants after unrolling
-    const int e = ch * 9 + tap;
-    return (e & 1) ? __uint_as_float(wr[e >> 1] & 0xffff0000u) : __uint_as_float(wr[e >> 1] << 16);
-  };
   float sc[8], bi[8];
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
@@ -122,16 +127,6 @@ dwconv3x3_tma_kernel(const __grid_constant__ CUtensorMap tmX, DwParams p) {
         const int ro = it / strips, st = it - ro * strips;
         const int wo0 = st * P;
         const int ho = band * p.RB + ro;
-        uint4 v[3][COLS];
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-          const uint8_t* row = tile + (size_t)((ro * STRIDE + r) * Wc) * p.cb * 2 + cvec * 16;
-#pragma unroll
-          for (int q = 0; q < COLS; ++q) {
-            const int col = min(wo0 * STRIDE + q, Wc - 1);   // columns past the frame only feed outputs that are not stored
-            v[r][q] = *reinterpret_cast<const uint4*>(row + (size_t)col * p.cb * 2);
-          }
-        }
         float acc[P][8];
 #pragma unroll
         for (int pp = 0; pp < P; ++pp)
@@ -141,9 +136,16 @@ dwconv3x3_tma_kernel(const __grid_constant__ CUtensorMap tmX, DwParams p) {
         for (int r = 0; r < 3; ++r) {
           const int hi = ho * STRIDE - 1 + r;
           const bool row_in = hi >= 0 && hi < p.H;
+          const uint8_t* row = tile + (size_t)((ro * STRIDE + r) * Wc) * p.cb * 2 + cvec * 16;
+          uint4 v[COLS];
 #pragma unroll
           for (int q = 0; q < COLS; ++q) {
-            const uint32_t wd[4] = {v[r][q].x, v[r][q].y, v[r][q].z, v[r][q].w};
+            const int col = min(wo0 * STRIDE + q, Wc - 1);   // columns past the frame only feed outputs that are not stored
+            v[q] = *reinterpret_cast<const uint4*>(row + (size_t)col * p.cb * 2);
+          }
+#pragma unroll
+          for (int q = 0; q < COLS; ++q) {
+            const uint32_t wd[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
             float f[8];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -164,7 +166,7 @@ dwconv3x3_tma_kernel(const __grid_constant__ CUtensorMap tmX, DwParams p) {
 #pragma unroll
                   for (int e = 0; e < 8; e += 2) {   // two independent round-to-nearest FMAs per instruction
                     float a0 = f[e], a1 = f[e + 1];
-                    ffma2(a0, a1, weight(r * 3 + sx, e), weight(r * 3 + sx, e + 1), acc[pp][e], acc[pp][e + 1]);
+                    ffma2(a0, a1, wf[r * 3 + sx][e], wf[r * 3 + sx][e + 1], acc[pp][e], acc[pp][e + 1]);
                     acc[pp][e] = a0, acc[pp][e + 1] = a1;
                   }
                 }

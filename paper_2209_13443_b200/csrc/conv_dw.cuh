@@ -7,7 +7,7 @@
 // one block of up to 64 channels, including the one-pixel frame of the padding (coordinates start at -1; the unit
 // zero-fills outside the image), into a ring of three slots: two or three tiles (up to 72 KB each) are in flight per
 // SM whatever the consumers do.  Eight consumer warps compute from shared memory: a thread owns one vector of eight
-// channels (its 72 weights stay in registers as stored) and walks strips of four consecutive output pixels of the
+// channels (its 72 weights stay in registers as floats) and walks strips of four consecutive output pixels of the
 // tile, reading each of the 3 x 6 (stride 2: 3 x 9) input vectors of a strip once.  A quarter warp reads the eight
 // channel vectors of one pixel, 128 contiguous bytes, so the reads are conflict-free without swizzling.  Every output
 // sums its nine taps in ascending (r, s) with fp32 FMAs, scale / bias / activation in fp32, one rounding to bf16.

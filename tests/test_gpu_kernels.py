@@ -244,3 +244,14 @@ def test_decisions_in_pinned_memory_are_there_when_the_count_is(fused):
             m.stage_run(0, x, B, pin, ws)
             n = pin.wait_count()
             assert n == int(dev.n_surv_dev[0]) and torch.equal(pin.conf[:B], dev.conf[:B].cpu()) and torch.equal(pin.pred[:B], dev.pred[:B].cpu())
+
+
+# 3x3 layers on 64 channels: H, W, cout, B: one and two channel halves, a half of one vector, one image row per tile, ragged last bands
+@pytest.mark.parametrize("geom", [(56, 56, 64, 3), (13, 61, 8, 2), (5, 20, 40, 4), (1, 1, 32, 2), (17, 30, 48, 3)])
+def test_halo_epilogue_of_narrow_and_wide_layers(geom):
+    H, W, cout, B = geom
+    spec = util.single_layer_model("bf16", H, W, 64, cout, 3, 1, 1, wl.ACT_RELU6, False, seed=sum(geom), max_batch=B)
+    run = util.GpuRunner(spec)
+    x = wl.random_features((B, H, W, 64), seed=9, bf16=True, relu=False)
+    util.check_stage(spec, run.stage(0, x), util.oracle_stage(spec, 0, x), f"{geom}", elementwise=True)
+    run.check_guards()

@@ -24,6 +24,7 @@
 #include <type_traits>
 
 #include "conv_tc.cuh"
+#include "stem_words.h"
 
 namespace ee {
 
@@ -100,34 +101,33 @@ __device__ __forceinline__ uint32_t bf16x2_max(uint32_t a, uint32_t b) {
 }
 
 // The words (elements e0 + 2 j, e0 + 2 j + 1; e0 even) of a filter row's run in one image row, in two steps: `load` only requests
-// aligned words, `finish` makes the run's words of them.  Words outside the row are loads that do not happen, so nothing looks at
-// a word before it is stored: a mask behind each load made every pair wait for memory (5200 clocks a pair).  Rows of an odd
-// number of elements start at an odd element every other time; their words are put together from two aligned ones.
+// aligned words (stem_words.h says which), `finish` makes the run's words of them.  Words outside the row are loads that do not
+// happen, so nothing looks at a word before it is stored: a mask behind each load made every pair wait for memory (5200 clocks
+// a pair).  Rows of an odd number of elements start at an odd element every other time; their words are put together from two
+// aligned ones.
 template <int NW>
 struct StemRun {
   uint32_t a[NW + 1];
-  int kind;   // the same for the whole warp: 0 no such row or even start, 2 odd start, 3 even start and the batch's last element has no word
-  // in: bit j = word j begins inside the row
-  __device__ __forceinline__ void load(const StemParams& p, int n, int y, int e0, uint32_t in) {
+  int kind;   // of StemAsk, the same for the whole warp
+  __device__ __forceinline__ void load(const StemParams& p, int n, int y, int e0, StemTaps in) {
     const int row_elems = p.W * kStemCin;
-    kind = 0;
-    if (y < 0 || y >= p.H) in = 0;
+    if (y < 0 || y >= p.H) in.first = in.second = 0;
     const long rb = ((long)n * p.H + y) * row_elems;
+    const StemAsk ask = stem_ask(rb, row_elems, p.total, in);
+    kind = ask.kind;
     const bf16* row = p.x + (rb + e0);
     auto at = [&](int e, uint32_t ok) {
       uint32_t w;
       asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n mov.u32 %0, 0;\n @q ld.global.nc.u32 %0, [%1];\n}" : "=r"(w) : "l"(row + e), "r"(ok));
       return w;
     };
-    if (!(rb & 1)) {
-      if ((row_elems & 1) && rb + row_elems == p.total) kind = 3;   // its last word would reach past the batch
+    if (kind != 2) {
 #pragma unroll
-      for (int j = 0; j < NW; ++j) a[j] = at(2 * j, in & 1u << j & (kind == 3 && e0 + 2 * j == row_elems - 1 ? 0u : ~0u));
-      if (kind == 3) a[NW] = in ? (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(p.x) + (p.total - 1)) : 0u;
+      for (int j = 0; j < NW; ++j) a[j] = at(2 * j, ask.mask & 1u << j);
+      if (kind == 3) a[NW] = in.first ? (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(p.x) + (p.total - 1)) : 0u;
     } else {
-      kind = 2;   // aligned word j holds elements 2 j - 1 and 2 j of the run
 #pragma unroll
-      for (int j = 0; j <= NW; ++j) a[j] = at(2 * j - 1, (in | in << 1) & 1u << j);
+      for (int j = 0; j <= NW; ++j) a[j] = at(2 * j - 1, ask.mask & 1u << j);
     }
   }
   __device__ __forceinline__ void finish(int e0, int row_elems, uint32_t in, uint32_t* w) const {
@@ -232,9 +232,7 @@ conv_stem_tcgen05_kernel(const __grid_constant__ CUtensorMap tmW, StemParams p) 
     const int r = (int)threadIdx.x - 32;
     const int ox = min(r, p.Wo - 1);   // rows past Wo repeat the last pixel; nobody reads them
     const int e0 = 2 * kStemCin * ox - S::kPad * kStemCin - 1;   // image-row element of column 0 (even)
-    uint32_t in = 0;
-#pragma unroll
-    for (int j = 0; j < S::kRead; ++j) in |= (e0 + 2 * j >= 0 && e0 + 2 * j < p.W * kStemCin ? 1u : 0u) << j;
+    const StemTaps in = stem_taps(e0, p.W * kStemCin, S::kRead);
     uint8_t* aline = gen + r * 128;
     constexpr int NW = S::kRead, CH = S::kCols / 8;   // words, 16-byte chunks of a filter row
     StemRun<NW> wa[2], wb[2];
@@ -256,7 +254,7 @@ conv_stem_tcgen05_kernel(const __grid_constant__ CUtensorMap tmW, StemParams p) 
       };
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
-        run[half].finish(e0, p.W * kStemCin, in, w);
+        run[half].finish(e0, p.W * kStemCin, in.first, w);
 #pragma unroll
         for (int c = 0; c < CH; ++c) put(half * CH + c, c);
         if (KH == 7 && half == 0) {

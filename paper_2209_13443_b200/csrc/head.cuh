@@ -12,6 +12,7 @@
 // batch size or on scheduling, so a sample's logits are bit-identical in any batch.
 #pragma once
 #include "conv_tc.cuh"
+#include "fc_shape.h"
 
 namespace ee {
 
@@ -328,8 +329,6 @@ __device__ __forceinline__ void exit_scan(int B, const DecideArgs& d) {
 //      never exits).  With several tiles the leader that finishes last runs the stable scan over the batch.
 // Waits on copies are bounded.  Launched with programmatic stream serialization.  Pooling kernel + this kernel on B200, 37 samples
 // of 28 x 28 x 512 and 1000 classes: 17.4 us with 16 classes a CTA behind block-wide barriers, 14.9 now.
-constexpr int kFcMaxSmem = 226 * 1024;   // dynamic; the scan's static arrays come on top
-constexpr int kFcThreads = 256, kFcRing = 4, kFcBlocks = 16, kFcRows = 8, kFcSlot = kFcRows * 512;
 
 __device__ __forceinline__ uint32_t hc_cluster_rank() {
   uint32_t r;
@@ -347,38 +346,9 @@ __device__ __forceinline__ void hc_st_f32(uint32_t cluster_addr, float v) {
 __device__ __forceinline__ void hc_cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void hc_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-struct FcShape {
-  int S, CL;     // samples per tile, CTAs per tile
-  int cluster;   // 1: the CTAs of a tile are a cluster; 0: they exchange through global memory (or CL is 1)
-  int kb;        // classes per block
-  int Cp;        // channels rounded up to whole ring slots
-};
-// 64 classes per CTA (clusters of 16 need the non-portable size), fewer CTAs for few classes.  Samples per tile: the fewest
-// whose clusters run side by side (`room16` clusters of 16: not every GPC has 16 SMs), up to 8, as a second wave costs the
-// whole kernel once more; past that the same tiles without clusters, 128 CTAs for 64 samples.  What bounds a CTA is then
-// its FMAs and its shared memory, which every weight crosses twice per tile.  Nothing here changes a sum.
-inline FcShape fc_shape(int B, int C, int K, int elem_bytes, int room16) {
-  FcShape f;
-  f.CL = 1;
-  while (f.CL < 16 && f.CL * 64 < K) f.CL *= 2;
-  const int room = std::max(1, room16 * (16 / f.CL)), most = elem_bytes == 4 ? 4 : 8;   // eight fp64 sums per class do not fit the registers
-  f.S = B <= room ? 1 : B <= 2 * room ? 2 : B <= 4 * room ? 4 : most;
-  f.cluster = f.CL > 1 && ((B + f.S - 1) / f.S <= room || f.CL < 16);
-  f.kb = ((K + kFcBlocks - 1) / kFcBlocks + kFcRows - 1) / kFcRows * kFcRows;
-  const int chunk = 512 / elem_bytes;
-  f.Cp = (C + chunk - 1) / chunk * chunk;
-  return f;
-}
-inline size_t fc_smem_bytes(const FcShape& f) {
-  return (size_t)(kFcThreads / 32) * kFcRing * kFcSlot + (size_t)f.S * f.Cp * 4 + (size_t)f.S * (kFcBlocks / f.CL) * f.kb * 4 +
-         (size_t)kFcBlocks * f.S * 16 + (kFcThreads / 32) * kFcRing * 8;
-}
-// C in whole 16-byte vectors (a row of the weights is then a multiple of 16 bytes), shared memory for the pooled tile and
-// the logits of a CTA.
+// C in whole 16-byte vectors (a row of the weights is then a multiple of 16 bytes), shared memory for a tile of one sample.
 inline bool fc_cluster_supported(int C, int K, int elem_bytes, const void* wfc) {
-  FcShape f = fc_shape(1, C, K, elem_bytes, 1);
-  f.S = elem_bytes == 4 ? 4 : 8;
-  return C % (16 / elem_bytes) == 0 && ((uintptr_t)wfc & 15) == 0 && fc_smem_bytes(f) <= (size_t)kFcMaxSmem;
+  return C % (16 / elem_bytes) == 0 && ((uintptr_t)wfc & 15) == 0 && fc_fits(C, K, elem_bytes);
 }
 
 __device__ __forceinline__ void fc_fma2(float (&a)[2], float w0, float w1, float g0, float g1) {   // two independent FMAs, one instruction
@@ -701,7 +671,8 @@ inline ee_status_t fc_weight_map(const TcContext& c, const void* w, int C, int K
              : EE_ERR_CUDA;
 }
 
-// The same layer for any C, K and alignment (channels that are not whole 16-byte vectors, very many classes): CTA (x, y)
+// The same layer for any C, K and alignment (channels that are not whole 16-byte vectors, or too many of them or of classes for
+// the shared memory of fc_cluster_kernel): CTA (x, y)
 // owns 16 classes (two per warp) of eight samples and walks the channels 128 at a time with plain loads.  The CTA that
 // completes a sample tile's logits (a counter per tile) takes that tile's exit decisions; the CTA that completes the last
 // tile's decisions runs the scan and leaves all counters at zero.

@@ -255,3 +255,37 @@ def test_halo_epilogue_of_narrow_and_wide_layers(geom):
     x = wl.random_features((B, H, W, 64), seed=9, bf16=True, relu=False)
     util.check_stage(spec, run.stage(0, x), util.oracle_stage(spec, 0, x), f"{geom}", elementwise=True)
     run.check_guards()
+
+
+# heads on more channels or classes than a tile of eight samples has shared memory for: tiles of four, two and one, the last channel
+# count the cluster kernel takes and one that it does not
+WIDE_HEADS = [("bf16", 64, 3072, 1000), ("bf16", 19, 8192, 40), ("bf16", 9, 24064, 12), ("bf16", 9, 24576, 12), ("bf16", 33, 64, 30000), ("f32", 37, 8192, 300), ("f32", 5, 16384, 7)]
+
+
+@pytest.mark.parametrize("case", WIDE_HEADS)
+def test_wide_heads_against_the_oracle_and_alone(case):
+    dtype, B, C, K = case
+    bf16 = dtype == "bf16"
+    rng = wl._rng(B + C + K, 911)
+    fw, fb = wl._head(rng, C, K, 4.0, bf16)
+    spec = wl.Model("wide head", dtype, 1, 2, C, [wl.Stage([wl.Layer(wl.OP_MAXPOOL, C, C, 3, 3, 1, 1)], K, fw, fb, 0.5, False)], B)
+    m = eb.EEModel(spec)
+    out = eb.StageBuffers(m, 0)
+    scratch, guard = util.guarded((m.exit_head_scratch_bytes(0) + 256,), torch.uint8)
+    x = wl.random_features((B, 2, C), seed=3, bf16=bf16)
+    xd = eb.to_device(dtype, x)
+    for _ in range(2):
+        m.exit_head(0, xd, B, 2, out, scratch)
+    torch.cuda.synchronize()
+    m.check()
+    z, conf, mask = out.logits[:B].cpu().numpy(), out.conf[:B].cpu().numpy(), out.exit_mask[:B].cpu().numpy()
+    o = eo.exit_head(x, fw, fb, 0.5, False, None, None)
+    assert util.rel_err(z, o["z"], dtype, floor=util.LOGIT_FLOOR[dtype]) <= util.TOL[dtype]
+    assert np.max(np.abs(conf - o["conf"])) <= util.TOL[dtype]
+    n = int(out.n_surv_dev[0])
+    assert np.array_equal(out.survivor_idx[:n].cpu().numpy(), np.nonzero(mask == 0)[0]) and n == B - int(mask.sum())
+    assert bool(torch.all(guard == util.CANARY))
+    b = B - 1
+    m.exit_head(0, xd[b:].contiguous(), 1, 2, out, scratch)
+    torch.cuda.synchronize()
+    assert np.array_equal(out.logits[0].cpu().numpy(), z[b]) and float(out.conf[0]) == float(conf[b])

@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "conv_ranges.h"
 
 namespace ee {
 
@@ -1241,41 +1242,9 @@ inline ee_status_t tc_plan_layer(TcContext& c, const ee_layer_desc_t& d, int in_
   L->in_h = in_h, L->in_w = in_w, L->out_h = out_h, L->out_w = out_w, L->max_batch = max_batch;
   L->bn = d.cout > 64 ? 128 : 64;
   L->im2col = !(d.kh == 1 && d.kw == 1 && d.stride == 1 && d.pad == 0 && d.pad_w == 0);
-  // Split-K: a K block of a 128 x 128 tile takes 0.135 us (its MMAs' own rate; 0.10 us at 64 columns), so a long K loop on a
-  // grid that leaves SMs idle spreads over a cluster of 2..4 CTAs per tile.  A split costs about
-  // 4.5 us (cluster launch, two cluster barriers, the reduce-scatter), larger clusters gain nothing measurable, and
-  // grids of more than two CTAs per SM lose to the unsplit kernel, hence the bounds.  The number of ranges is chosen
-  // once per layer by this cost model summed over the batch sizes the model will see (max_batch, 3/4, 1/2 and 1/4
-  // of it: the batch shrinks at every exit), the analogue of the per-layer objective sum_b w_b T(b) of the paper's
-  // design-space exploration (Eq. 2).  It depends on the layer and on max_batch, never on the batch actually run,
-  // so a sample's sums are grouped the same way in every call.
-  {
-    const int num_kb = d.kh * d.kw * cdiv(d.cin, kTcBK);
-    const int n_tiles = cdiv(d.cout, L->bn);
-    const double t_block = L->bn == 128 ? 0.135 : 0.10;   // us per K block
-    const long tiles_max = (long)cdiv((long)max_batch * out_h * out_w, kTcBM) * n_tiles;
-    double best = 0;
-    L->splits = 1;
-    L->kb_per = num_kb;
-    for (int sp = 1; sp <= 4; ++sp) {
-      const int per = cdiv(num_kb, sp);
-      if (sp > 1 && (per < 4 || (sp - 1) * per >= num_kb || tiles_max * sp > 2 * c.sm_count + 4)) continue;
-      double cost = 0;
-      for (int f = 4; f >= 1; --f) {
-        const int b = std::max(1, (max_batch * f + 3) / 4);
-        const long tiles = (long)cdiv((long)b * out_h * out_w, kTcBM) * n_tiles;
-        const long share = cdiv(tiles * sp, c.sm_count);   // CTAs on the busiest SM
-        cost += 2.4 + (sp > 1 ? 4.5 : 0.0) + (double)share * per * t_block + 0.8 * cdiv(tiles, c.sm_count);
-      }
-      if (sp == 1) {
-        best = cost;
-      } else if (cost < best) {
-        best = cost;
-        L->splits = sp;
-        L->kb_per = per;
-      }
-    }
-  }
+  const int num_kb = d.kh * d.kw * cdiv(d.cin, kTcBK);
+  L->splits = tc_auto_ranges(num_kb, (long)cdiv((long)max_batch * out_h * out_w, kTcBM) * cdiv(d.cout, L->bn), c.sm_count);
+  L->kb_per = cdiv(num_kb, L->splits);
   // weights [Cout][taps][Cin] as a 3-D tensor, box = 64 channels x 1 tap x BN filters
   const cuuint64_t dims[3] = {(cuuint64_t)d.cin, (cuuint64_t)(d.kh * d.kw), (cuuint64_t)d.cout};
   const cuuint64_t strides[2] = {(cuuint64_t)d.cin * 2, (cuuint64_t)d.cin * d.kh * d.kw * 2};
@@ -1559,11 +1528,8 @@ inline ee_status_t tc_launch(TcContext& c, const TcLayer& L, const void* src, co
   p.gH = L.g_h, p.gW = L.g_w, p.gCin = L.g_cin, p.gkh = L.g_kh, p.grun = L.g_kw * L.g_cin, p.grunp = L.g_runp;
   if (L.gather) p.stride = L.g_stride, p.pad = p.pad_w = L.g_pad;
   dim3 grid(cdiv(p.M, kTcBM), cdiv(L.cout, L.bn), split ? L.splits : 1);
-  // At most one CTA per SM anyway: take the deep operand ring.  A cluster grid close to the SM count does not: its
-  // clusters need all their CTAs inside one GPC, a 192 KB CTA owns its SM, and the last clusters then wait for a second
-  // wave (measured: the split-3 3x3 layers of 132 CTAs lose 6 us each with the deep ring).
   const long n_ctas = (long)grid.x * grid.y * grid.z;
-  const bool deep = split ? n_ctas * 4 <= 3L * c.sm_count : n_ctas <= c.sm_count;
+  const bool deep = split ? tc_cluster_deep(n_ctas, c.sm_count) : n_ctas <= c.sm_count;
   const bool tma_res = res && !split;
   if (L.gather) {
     if (res || split) return EE_ERR_INTERNAL;

@@ -1,0 +1,42 @@
+"""How many K ranges a tensor-core convolution gets by itself (csrc/conv_ranges.h)."""
+import os
+import subprocess
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+HARNESS = r"""
+#include "conv_ranges.h"
+#include <cstdio>
+#include <initializer_list>
+static long tiles(int hw, int batch, int cout) { return ((long)batch * hw * hw + 127) / 128 * ((cout + 127) / 128); }
+static int bad(int kb, int hw, int batch, int cout, int want) {
+  const int got = ee::tc_auto_ranges(kb, tiles(hw, batch, cout), 148);
+  if (got != want) std::printf("%d K blocks, %dx%d map, max_batch %d, %d filters: %d ranges, not %d\n", kb, hw, hw, batch, cout, got, want);
+  return got != want;
+}
+int main() {
+  int e = 0;
+  // 3x3 512->512: whole wherever some batch up to max_batch leaves the deep clusters (measured slower there by up to 5 us)
+  e += bad(72, 7, 64, 512, 1) + bad(72, 7, 16, 512, 1) + bad(72, 6, 64, 512, 1) + bad(72, 6, 22, 512, 1) + bad(72, 4, 64, 512, 1);
+  // four where none does (measured faster by 0.3 to 1.4 us)
+  e += bad(72, 7, 8, 512, 4) + bad(72, 7, 1, 512, 4) + bad(72, 6, 16, 512, 4) + bad(72, 4, 48, 512, 4) + bad(72, 3, 64, 512, 4) + bad(72, 2, 64, 512, 4);
+  // 3x3 256->256 and shorter: whole (measured slower in ranges at every batch)
+  e += bad(36, 14, 1, 256, 1) + bad(36, 14, 64, 256, 1) + bad(36, 11, 4, 256, 1) + bad(32, 7, 1, 512, 1) + bad(1, 56, 64, 64, 1);
+  for (int sms : {1, 132, 148})
+    for (int kb = 1; kb <= 600; ++kb)
+      for (long t = 1; t <= 300; ++t) {
+        const int r = ee::tc_auto_ranges(kb, t, sms), per = (kb + r - 1) / r;
+        const bool ok = r == 1 || (r == 4 && (r - 1) * per < kb && ee::tc_cluster_deep(t * r, sms) && t * r <= sms);
+        if (!ok) std::printf("%d K blocks, %ld tiles, %d SMs: %d ranges\n", kb, t, sms, r), ++e;
+      }
+  return e != 0;
+}
+"""
+
+
+def test_ranges_only_where_every_batch_gains(tmp_path):
+    src, exe = tmp_path / "ranges.cpp", tmp_path / "ranges"
+    src.write_text(HARNESS)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", os.path.join(ROOT, "paper_2209_13443_b200", "csrc"), "-o", str(exe), str(src)], check=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout

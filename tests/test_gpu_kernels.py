@@ -289,3 +289,16 @@ def test_wide_heads_against_the_oracle_and_alone(case):
     m.exit_head(0, xd[b:].contiguous(), 1, 2, out, scratch)
     torch.cuda.synchronize()
     assert np.array_equal(out.logits[0].cpu().numpy(), z[b]) and float(out.conf[0]) == float(conf[b])
+
+
+# 3x3 512->512 (72 K blocks): whole where the largest batch would not run as deep clusters, four K ranges where it does
+@pytest.mark.parametrize("hw,bmax,ranges", [(6, 64, 1), (4, 64, 1), (6, 16, 4), (2, 64, 4)])
+def test_k_ranges_chosen_for_a_layer_and_its_results(hw, bmax, ranges):
+    spec = util.single_layer_model("bf16", hw, hw, 512, 512, 3, 1, 1, wl.ACT_RELU, False, seed=hw, max_batch=bmax)
+    run = util.GpuRunner(spec)
+    assert run.m.layer_config(0, 0, 1)["splits"] == ranges
+    x = wl.random_features((bmax, hw, hw, 512), seed=3, bf16=True, relu=False)
+    whole = run.stage(0, x)
+    # the layer's output: the logits of such small maps are sums of a few rounded values that cancel, not the layer's to bound
+    assert util.rel_err(whole["features_out"], eo.run_layers(spec, 0, x), "bf16") <= util.TOL["bf16"]
+    assert np.array_equal(run.stage(0, x[:1])["features_out"][0], whole["features_out"][0])

@@ -160,6 +160,7 @@ class StageBuffers:
         where = dict(pin_memory=True) if pinned_decisions else dict(device=dev)
         self.conf = torch.empty(B, dtype=torch.float32, **where)
         self.pred = torch.empty(B, dtype=torch.int32, **where)
+        self.host_decisions = (self.conf.numpy(), self.pred.numpy()) if pinned_decisions else None
         self.logits = torch.empty((B, model.n_classes[stage]), dtype=torch.float32, device=dev) if with_logits else None
         self.exit_mask = torch.empty(B, dtype=torch.uint8, device=dev)
         self.survivor_idx = torch.empty(B, dtype=torch.int32, device=dev)

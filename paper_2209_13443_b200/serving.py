@@ -76,16 +76,17 @@ class FluidServer:
         self.in_act = torch.empty(shape, dtype=td, device="cuda")
         self.in_new = torch.empty(shape, dtype=td, device="cuda")
         # a batch's rows of the pool, its count and its requests' ids go up in one copy from pinned staging: rows | count | ids
-        self.up = {}
-        for name in ("act", "new"):
+        def staging():
             host = torch.empty(2 * self.bmax + 1, dtype=torch.int32).pin_memory()
             dev = torch.empty(2 * self.bmax + 1, dtype=torch.int32, device="cuda")
-            ids = dev[self.bmax + 1:]
-            setattr(self, "ids_" + name, ids)
-            self.up[ids.data_ptr()] = (host, host.numpy(), dev, dev[self.bmax:])
+            return host, host.numpy(), dev, dev[self.bmax:]
+
+        up_act, up_new, self.up_other = staging(), staging(), staging()
+        self.ids_act, self.ids_new = (u[2][self.bmax + 1:] for u in (up_act, up_new))
+        self.up = {self.ids_act.data_ptr(): up_act, self.ids_new.data_ptr(): up_new}
+        self.other_read = torch.cuda.Event()      # the upload from up_other's staging is done
         # the decision of a sample from its confidence, as the kernel takes it
         self.thr = [(np.float32(st.threshold), bool(st.always_exit)) for st in spec.stages]
-        self.decided = {id(b): (b.conf.numpy(), b.pred.numpy()) for b in self.act + self.new}
         self.stage_in_bytes = [self.m.query(s)["in_bytes_per_sample"] for s in range(self.n_stages)]
 
     # ------------------------------------------------------------------ measured exit-level latency table
@@ -113,21 +114,28 @@ class FluidServer:
 
     def form_batch(self, pool, rows: Sequence[int], req_ids: Sequence[int], feat, ids):
         """Gathers the requests' inputs (rows of ``pool``) to the front of the batch buffer ``feat``: one small pinned
-        upload of the row list, the count and the ids (``ids``: ids_act or ids_new), then one ee_gather_survivors.  The staging
-        is free again: the stage that read it has been waited for."""
+        upload of the row list, the count and the ids, then one ee_gather_survivors.  ids_act and ids_new lie behind the row
+        list and the count in one allocation and have a staging of their own, which is free again: the stage that read it has
+        been waited for.  Any other ids buffer gets a copy of its own behind the upload."""
         n, b = len(rows), self.bmax
-        host, h, dev, cnt = self.up[ids.data_ptr()]
+        own = self.up.get(ids.data_ptr())
+        if own is None:
+            self.other_read.synchronize()
+        host, h, dev, cnt = own or self.up_other
         h[:n] = rows
         h[b] = n
         h[b + 1:b + 1 + n] = req_ids
         dev.copy_(host, non_blocking=True)
+        if own is None:
+            self.other_read.record()
+            ids[:n].copy_(dev[b + 1:b + 1 + n])
         eb.gather_survivors(pool, self.stage_in_bytes[0], dev, cnt, n, feat)
 
     def run_stage(self, s, feat, ids_dev, members, bufs, clock: _Clock, out):
-        """One subnet and its exit on the batch ``members`` (request numbers, in batch order).  Confidences and classes
-        are in pinned host memory when the survivor count is, and the host waits for that word alone: no copies behind the
-        stage, and the gather of the survivors' features may still run.  Records the requests that leave; returns those
-        that stay."""
+        """One subnet and its exit on the batch ``members`` (request numbers, in batch order).  In the server's own buffers
+        confidences and classes are in pinned host memory when the survivor count is, and the host waits for that word alone:
+        no copies behind the stage, and the gather of the survivors' features may still run.  Buffers with the decisions on
+        the device are read back behind the stage.  Records the requests that leave; returns those that stay."""
         n, buf = len(members), bufs[s]
         buf.arm_count()
         self.m.stage_run(s, feat, n, buf, self.ws, ids_dev)
@@ -135,7 +143,7 @@ class FluidServer:
         now = clock.after_stage(s, n)
         out["launches"].append((s, tuple(members)))
         thr, always = self.thr[s]
-        conf, pred = self.decided[id(buf)]
+        conf, pred = buf.host_decisions or (buf.conf[:n].cpu().numpy(), buf.pred[:n].cpu().numpy())
         stay = []
         for j, r in enumerate(members):
             if always or conf[j] >= thr:
@@ -144,7 +152,8 @@ class FluidServer:
                 out["pred"][r] = pred[j]
             else:
                 stay.append(r)
-        assert len(stay) == n_stay
+        if len(stay) != n_stay:
+            raise RuntimeError(f"stage {s}: {n_stay} samples stay by the device's count, {len(stay)} by their confidences")
         return stay
 
     def catch_up(self, pool, image_of, members, upto, clock, out):

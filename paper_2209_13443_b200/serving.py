@@ -20,6 +20,7 @@ of the requests' inputs), run_stage (one subnet + exit), catch_up (a new batch u
 """
 from __future__ import annotations
 
+import functools
 import time
 from collections import deque
 from typing import Callable, Optional, Sequence
@@ -61,6 +62,20 @@ class _Clock:
         return self.now()
 
 
+def _on_one_stream(serve):
+    """Looks the current stream up once for all calls of a trace: per call it costs the host 5 us."""
+
+    @functools.wraps(serve)
+    def run(self, *args, **kwargs):
+        self.stream = torch.cuda.current_stream()
+        try:
+            return serve(self, *args, **kwargs)
+        finally:
+            self.stream = None
+
+    return run
+
+
 class FluidServer:
     def __init__(self, spec, model: Optional[eb.EEModel] = None):
         self.spec = spec
@@ -88,6 +103,7 @@ class FluidServer:
         # the decision of a sample from its confidence, as the kernel takes it
         self.thr = [(np.float32(st.threshold), bool(st.always_exit)) for st in spec.stages]
         self.stage_in_bytes = [self.m.query(s)["in_bytes_per_sample"] for s in range(self.n_stages)]
+        self.stream = None       # while a trace is served: the stream it started on (None: the current one of each call)
 
     # ------------------------------------------------------------------ measured exit-level latency table
 
@@ -129,7 +145,7 @@ class FluidServer:
         if own is None:
             self.other_read.record()
             ids[:n].copy_(dev[b + 1:b + 1 + n])
-        eb.gather_survivors(pool, self.stage_in_bytes[0], dev, cnt, n, feat)
+        eb.gather_survivors(pool, self.stage_in_bytes[0], dev, cnt, n, feat, stream=self.stream)
 
     def run_stage(self, s, feat, ids_dev, members, bufs, clock: _Clock, out):
         """One subnet and its exit on the batch ``members`` (request numbers, in batch order).  In the server's own buffers
@@ -138,7 +154,7 @@ class FluidServer:
         the device are read back behind the stage.  Records the requests that leave; returns those that stay."""
         n, buf = len(members), bufs[s]
         buf.arm_count()
-        self.m.stage_run(s, feat, n, buf, self.ws, ids_dev)
+        self.m.stage_run(s, feat, n, buf, self.ws, ids_dev, stream=self.stream)
         n_stay = buf.wait_count()                            # B_exit (and who left) reaches the scheduler
         now = clock.after_stage(s, n)
         out["launches"].append((s, tuple(members)))
@@ -169,7 +185,7 @@ class FluidServer:
 
     def merge(self, boundary, feat, ids, members, new_feat, new_ids, new_members):
         """ee_batch_refill: the caught-up samples are appended behind the parked ones."""
-        n_acc, n_mer = self.m.batch_refill(boundary, feat, ids, len(members), new_feat, new_ids, len(new_members))
+        n_acc, n_mer = self.m.batch_refill(boundary, feat, ids, len(members), new_feat, new_ids, len(new_members), stream=self.stream)
         assert n_acc == len(new_members) and n_mer == len(members) + len(new_members)
         return members + new_members
 
@@ -180,6 +196,7 @@ class FluidServer:
 
     # ------------------------------------------------------------------ Algorithm 1
 
+    @_on_one_stream
     def serve(self, arrivals: np.ndarray, image_of: Sequence[int], pool: torch.Tensor,
               stage_time: Optional[Callable[[int, int], float]] = None, slo: float = float("inf"),
               latency: Optional[Callable[[int, int], float]] = None):
@@ -262,6 +279,7 @@ class FluidServer:
         """One request at a time in arrival order, each through its exits alone."""
         return self.serve_adaptive_batching(arrivals, image_of, pool, max_batch=1, timeout=0.0, stage_time=stage_time)
 
+    @_on_one_stream
     def serve_adaptive_batching(self, arrivals, image_of, pool, max_batch: Optional[int] = None, timeout: float = 0.0,
                                 stage_time=None):
         """The <B_max, T_timeout> policy: a batch is issued as soon as ``max_batch`` requests wait or the oldest

@@ -68,3 +68,24 @@ def test_a_count_that_disagrees_with_the_decisions_is_an_error():
     server.thr[0] = (np.float32(2.0), False)                      # the host's copy of the threshold alone: nobody would leave
     with pytest.raises(RuntimeError, match="stay by the device's count"):
         _run(server, pool, [5, 1, 3, 15, 0, 2, 9], [0, 1, 2, 3, 4, 5, 6], server.in_act, server.ids_act, server.act)
+
+
+def test_a_trace_runs_on_the_current_stream_and_blocks_on_theirs():
+    spec = wl.tiny_ee_cnn(seed=0)
+    server = FluidServer(spec)
+    pool = eb.to_device("f32", wl.make_input(spec, 16, seed=2))
+    arrivals, image_of = wl.poisson_arrivals(1, 20, 2000.0), [3 * i % 16 for i in range(20)]
+    torch.cuda.synchronize()
+    side, got = torch.cuda.Stream(), []
+    for ctx in (torch.cuda.default_stream(), side):
+        with torch.cuda.stream(ctx):
+            r = server.serve(arrivals, image_of, pool, lambda s, n: 1e-3)
+            got.append([r[k].tolist() for k in ("finish", "exit_stage", "pred")])
+            assert server.stream is None
+    assert got[0] == got[1]
+    with pytest.raises(ValueError):
+        server.serve(arrivals, image_of, pool, slo=1.0)
+    assert server.stream is None
+    own = _run(server, pool, [5, 1, 3], [0, 1, 2], server.in_act, server.ids_act, server.act)
+    with torch.cuda.stream(side):
+        assert _same(_run(server, pool, [5, 1, 3], [0, 1, 2], server.in_act, server.ids_act, server.act), own)

@@ -88,7 +88,8 @@ __device__ __forceinline__ void stem_walk(const StemParams& p, F&& body) {
 }
 
 // Maximum of bf16 pairs.  NONNEG: behind a ReLU the order of the values is that of their bits, and the 16-bit integer maximum is
-// an instruction of full rate; the bf16 one took 60 clocks each here.
+// an instruction of full rate; the bf16 one took 60 clocks each here.  A pooling layer of its own drops NaN (fmaxf), so here it must
+// lose too: the keys of NONNEG are the bits plus one, by which the conversion's one NaN, 0x7FFF, becomes the least integer.
 template <bool NONNEG>
 __device__ __forceinline__ uint32_t bf16x2_max(uint32_t a, uint32_t b) {
   if (NONNEG) {
@@ -98,6 +99,13 @@ __device__ __forceinline__ uint32_t bf16x2_max(uint32_t a, uint32_t b) {
   }
   const __nv_bfloat162 r = __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
   return *reinterpret_cast<const uint32_t*>(&r);
+}
+constexpr uint32_t kPoolKey = 0x00010001u;   // both halves: they hold 0 .. 0x7FFF (or 0x8000, -0), so nothing is carried or borrowed
+// A window's maximum as it is stored: no number in the window (every tap NaN) is -inf, what a maximum over none starts from.
+template <bool NONNEG>
+__device__ __forceinline__ uint32_t bf16x2_pooled(uint32_t m) {
+  const uint32_t nan = __vcmpeq2(m, NONNEG ? 0x80008000u : 0x7FFF7FFFu);
+  return (NONNEG ? m - kPoolKey : m) & ~nan | (0xFF80FF80u & nan);
 }
 
 // The words (elements e0 + 2 j, e0 + 2 j + 1; e0 even) of a filter row's run in one image row, in two steps: `load` only requests
@@ -342,6 +350,10 @@ conv_stem_tcgen05_kernel(const __grid_constant__ CUtensorMap tmW, StemParams p) 
           __syncwarp();
         } else {
           uint8_t* tile = stage + (emitted & 1) * (kTcBM * 64);
+          if (nonneg) {
+#pragma unroll
+            for (int e = 0; e < 16; ++e) cur[e] += kPoolKey;
+          }
           if (fresh) {
 #pragma unroll
             for (int e = 0; e < 16; ++e) vm[e] = cur[e];
@@ -378,7 +390,9 @@ conv_stem_tcgen05_kernel(const __grid_constant__ CUtensorMap tmW, StemParams p) 
             };
             const int c1 = 2 * px;   // columns 2px-1 .. 2px+1, a column past the row's ends replaced by the middle one
             const uint4 x = at(c1), l = at(max(c1 - 1, 0)), r = at(min(c1 + 1, p.Wo - 1));
-            *reinterpret_cast<uint4*>(p.out + ((size_t)t * p.Wp + px) * p.N + ch) = most(most(x, l), r);
+            const uint4 m = most(most(x, l), r);
+            *reinterpret_cast<uint4*>(p.out + ((size_t)t * p.Wp + px) * p.N + ch) =
+                make_uint4(bf16x2_pooled<NONNEG>(m.x), bf16x2_pooled<NONNEG>(m.y), bf16x2_pooled<NONNEG>(m.z), bf16x2_pooled<NONNEG>(m.w));
           }
         }
       };

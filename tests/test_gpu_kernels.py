@@ -302,3 +302,31 @@ def test_k_ranges_chosen_for_a_layer_and_its_results(hw, bmax, ranges):
     # the layer's output: the logits of such small maps are sums of a few rounded values that cancel, not the layer's to bound
     assert util.rel_err(whole["features_out"], eo.run_layers(spec, 0, x), "bf16") <= util.TOL["bf16"]
     assert np.array_equal(run.stage(0, x[:1])["features_out"][0], whole["features_out"][0])
+
+
+# NaN and infinities through the pooling stem: the pooling layer run apart drops NaN, and a window of nothing else is -inf
+@pytest.mark.parametrize("act", [wl.ACT_RELU, wl.ACT_RELU6, wl.ACT_NONE])
+@pytest.mark.parametrize("k,cout", [(7, 64), (3, 40)])
+def test_pooling_stem_treats_nan_as_the_two_layers_run_apart(k, cout, act):
+    H, W, B = 37, 61, 2
+    rng = wl._rng(k + act, 921)
+    layers = [wl._conv(rng, wl.OP_CONV, 3, cout, k, 2, k // 2, act, bf16=True), wl.Layer(wl.OP_MAXPOOL, cout, cout, 3, 3, 2, 1)]
+    fw, fb = wl._head(rng, cout, 5, 1.0, True)
+    spec = wl.Model("stem", "bf16", H, W, 3, [wl.Stage(layers, 5, fw, fb, 2.0, False)], B)
+    m = eb.EEModel(spec)
+    out, ws = eb.StageBuffers(m, 0), m.workspace()
+    xd = eb.to_device("bf16", wl.make_input(spec, B, seed=5))
+    xd[0, 4:30, 6:33] = float("nan")                 # whole windows of NaN
+    xd[1, ::17, ::13, 1] = float("nan")
+    xd[1, 5, 5, 0], xd[1, 20, 30, 2], xd[0, 35, 2] = float("inf"), float("-inf"), float("inf")
+    shapes = wl.stage_shapes(spec)[0]["layers"]
+    conv, apart = (torch.empty((B,) + s, dtype=torch.bfloat16, device="cuda") for s in shapes)
+    m.layer_run(0, 0, xd, None, B, conv, ws)
+    m.layer_run(0, 1, conv, None, B, apart, ws)
+    m.stage_run(0, xd, B, out, ws)
+    torch.cuda.synchronize()
+    m.check()
+    if act != wl.ACT_RELU6:                          # min(max(x, 0), 6) has no NaN
+        assert bool(conv.isnan().any()) and bool((apart == float("-inf")).any())
+    assert not bool(apart.isnan().any())
+    assert torch.equal(out.features_out[:B].view(torch.int16), apart.view(torch.int16))

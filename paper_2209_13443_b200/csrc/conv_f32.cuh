@@ -13,10 +13,11 @@
 // them first operands, reduction and epilogue.  So weights are requested before the wait for the layer in front, scale, bias
 // and residual come to registers during the K loop (fetched at the end they took 5000), tap positions are counted, not divided,
 // and one cluster barrier stands between the K loop and the result.  ResNet-50-shaped fp32 model at 64 x 64, batch 6:
-// 630 -> 567 us a pass with these.
+// 630 -> 567 us a pass with these; K cut in equal numbers of 16-wide steps instead of whole ring stages (f32_plan.h) 526 -> 513.
 #pragma once
 #include "common.cuh"
 #include "conv_simt.cuh"
+#include "f32_plan.h"
 
 namespace ee {
 
@@ -230,34 +231,12 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
 
 // ----------------------------------------------------------------------------- host side
 
-struct F32Plan {
-  int tile = 0;    // 0: 64 x 32, one K group; 1: 64 x 64, two; 2: 32 x 32, eight; 3: 16 x 32, eight
-  int z = 1;       // CTAs of a cluster that share a tile's K
-};
-
-// Tile and cluster size of a layer, from its geometry and max_batch.  Short K (stems on 3 channels): one K group, a ring
-// stage is 16 wide and nothing is padded to 128.  Grids of two waves of 64 x 64 tiles: that tile reads its operands least.
-// Everything else has idle SMs: small tiles (16 rows where the layer never has more than 32), eight K groups, and as many CTAs per tile (up to 8) as keep the grid within
-// two CTAs per SM while every CTA still has two ring stages of K.
-inline F32Plan f32_plan(long m_max, int n, int k, int sms) {
-  F32Plan p;
-  if (k < 128) return p;
-  if ((long)cdiv(m_max, 64) * cdiv(n, 64) >= 2L * sms) {
-    p.tile = 1;
-    return p;
-  }
-  p.tile = m_max <= 32 ? 3 : 2;   // 17 to 32 rows are two 16-row tiles: the same products, and half of them once samples have left
-  const long tiles = (long)cdiv(m_max, p.tile == 3 ? 16 : 32) * cdiv(n, 32);
-  while (p.z < 8 && tiles * p.z * 2 <= 2L * sms && k >= p.z * 2 * 256) p.z *= 2;
-  return p;
-}
-
 template <int WM, int WN, int KG, int MF, int NF, int V>
 inline cudaError_t f32_launch_t(const F32Plan& p, const float* x, const float* w, const float* scale, const float* bias, const float* residual,
                                 float* y, const ConvGeom& g, cudaStream_t st) {
   using S = F32Tile<WM, WN, KG, MF, NF>;
   const int K = g.kh * g.kw * g.Cin;
-  const int k_per = cdiv(cdiv(K, S::kKS), p.z) * S::kKS;
+  const int k_per = f32_k_per(K, p.z);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cdiv((long)g.B * g.Ho * g.Wo, S::kBM), cdiv(g.Cout, S::kBN), p.z);
   cfg.blockDim = dim3(kF32Threads);

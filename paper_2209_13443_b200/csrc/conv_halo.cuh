@@ -14,8 +14,8 @@
 // padding columns of the flattened rows: they are computed and dropped (2 of every Wp rows).
 //
 // Warp roles as in conv_tc.cuh: warp 0 issues TMA loads into a ring of blocks, warp 1 owns TMEM and issues the MMAs
-// into a double-buffered accumulator (2 x 64 columns), warps 2-5 run the epilogue (tcgen05.ld, folded-BN scale/bias,
-// activation, one rounding to bf16) and store each pixel's 128 bytes straight to global memory.  Every wait on an
+// into a double-buffered accumulator (2 x 64 columns), warps 2-9 run the epilogue, 32 channels of 32 pixels each (tcgen05.ld,
+// folded-BN scale/bias, activation, one rounding to bf16), and store through a staging tile of their own.  Every wait on an
 // mbarrier is bounded; on expiry the thread records EE_ERR_TIMEOUT and falls through to the common exit.
 #pragma once
 #include "conv_tc.cuh"

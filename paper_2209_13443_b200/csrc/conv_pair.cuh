@@ -1,9 +1,15 @@
 // Tensor-core convolution on CTA pairs: tcgen05.mma cta_group::2 over 256 x BN output tiles, persistent, with
 // (tile, K-range) work units and a fixed-order split-K reduction through global memory.
 //
+// When.  A layer runs here if a caller's kernel table says so (ee_model_set_layer_variant) and inside multi-layer launches
+// (ee_model_set_stage_kernel); the library itself chooses the one-CTA kernels.  Stages of the ResNet-50-shaped network at
+// batch 1, 10, 30 and 64 with one layer after the other moved here: 0.5 to 70 us slower, but for 1x1 512->256 at 64 (295.9
+// against 296.3).  The feeding loop here still divides (tap_at, about 150 clocks a block), where those of the one-CTA kernels run
+// on elected threads without divisions, and a launch carries about 7 us around its K loop.
+//
 // Why pairs.  In the one-CTA kernels of conv_tc.cuh a 128 x 128 x 64 K block moves 64 KB through the SM's shared
-// memory (32 KB written by TMA, 32 KB read by the MMAs) for 256 clocks of MMA time, so the tile is bound by the 128 B/clk
-// of shared memory at half the tensor rate.  Two CTAs of a cluster that issue one MMA of M = 256 hold half of the
+// memory (32 KB written by TMA, 32 KB read by the MMAs) for 256 clocks of MMA time, all that the tensor core's rate at M = 128
+// leaves.  Two CTAs of a cluster that issue one MMA of M = 256 hold half of the
 // weight tile each: per CTA and K block 16 KB of activations and BN/2 rows of weights are staged and read while the
 // tensor core does a 128 x BN x 64 product, twice the MMA time per staged byte at BN = 256.
 //

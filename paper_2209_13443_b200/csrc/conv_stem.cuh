@@ -18,8 +18,8 @@
 // first row of its last pair, whose other row must not enter the sum, not even times zero: at 7x7 its columns 16..23 are there
 // once more as columns 48..55, so that K steps 0 and 3 hold it alone.
 // What bounds it: the gather, about 1600 clocks a pair (its loads come from L2, and 26 words in two sets are what the registers
-// hold), against 530 of MMAs and 1500 of epilogue a row.  224 x 224 x 64 images with the pool 78.4 -> 66.9 us; 161 x 161
-// images ran on the generic gather, whose tiles read every image row seven times.
+// hold), against 530 of MMAs and 1500 of epilogue a row.  224 x 224 x 64 images with the pool 78.4 -> 66.9 us, 59 with the pool's
+// integer keys (bf16x2_max); 161 x 161 images ran on the generic gather, whose tiles read every image row seven times.
 #pragma once
 #include <type_traits>
 
@@ -156,7 +156,8 @@ struct StemRun {
 // POOL: the epilogue threads keep the running maximum over the convolution rows of a pooled row in registers (a
 // thread owns one pixel column, 32 channels), and on the last of them put it in a staging tile, take the maximum
 // over the three columns of every pooled pixel there and store the pooled row; the convolution's own output never
-// reaches global memory.  max() of bf16 values is exact, so the result equals pooling the stored convolution output.
+// reaches global memory.  max() of bf16 values is exact and NaN loses on both routes, so the result equals pooling the stored
+// convolution output bit for bit.
 template <int KH, bool POOL>
 __global__ void __launch_bounds__(kStemThreads, 1)
 conv_stem_tcgen05_kernel(const __grid_constant__ CUtensorMap tmW, StemParams p) {

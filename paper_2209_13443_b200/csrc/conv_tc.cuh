@@ -12,9 +12,11 @@
 // the warps between run the epilogue: tcgen05.ld of the fp32 accumulator, folded-BN scale/bias, residual add (the
 // residual tile was brought into shared memory by TMA while the main loop ran), activation, one rounding to bf16,
 // then a TMA store of the tile from shared memory.  The K loop visits (channel block, tap) in a fixed order that
-// does not depend on the batch size (tap_at).  Variants (chosen per launch from the grid size, see tc_launch): shallow or
-// deep ring, cluster split-K with a reduce-scatter through distributed shared memory, gather-mode A operand for
-// 3-channel stems, and a persistent kernel with double-buffered TMEM accumulators for multi-wave 1x1 layers.
+// does not depend on the batch size (tap_at).  Variants (chosen per launch from the grid size, see tc_launch): a shallow
+// ring, so that CTAs share an SM, for grids of several tiles per SM; a deep ring and split-K with a reduce-scatter through
+// distributed shared memory for layers with several K ranges; gather-mode A operand for 3-channel stems that conv_stem.cuh
+// does not take; a persistent kernel with double-buffered TMEM accumulators for 1x1 layers of at least two tiles per SM.
+// Grids of at most one tile per SM run on the kernel of conv_wave.cuh.
 //
 // Every wait on an mbarrier is bounded by a clock: on expiry the thread records EE_ERR_TIMEOUT in
 // the model's error word and falls through to the common exit, which frees the TMEM columns.
@@ -69,7 +71,9 @@ struct TcParams {
 };
 
 // Order of a convolution's K blocks, the same in every tensor-core kernel: channel blocks outermost, then filter columns,
-// then filter rows (stride 2: the even rows, then the odd ones), so that consecutive blocks read overlapping input rows.
+// then filter rows (stride 2: the even rows, then the odd ones).  Only that it is fixed matters: taps outermost, or filter rows
+// before columns, took the same time to 0.4 % on passes of the ResNet-50-shaped network at batch 1, 21 and 64; taps outermost
+// was 1.5 % slower on the 1x7 / 7x1 tower (104.1 against 102.6 us a pass).
 // Entry i of a channel block, packed: (row * kw + column) << 16 | row << 8 | column.  The feeding loops read the entries from
 // a table in shared memory (tap_table_fill): one thread feeds the whole SM, and in it an integer division by a run-time number is a chain of about 150 clocks, counters with branches still 50.
 constexpr int kMaxTaps = 49;
@@ -434,8 +438,8 @@ __device__ __forceinline__ void gather_rows_static(const TcParams& p, const bf16
 // residual operand is prefetched (RES), a dedicated 128 x BN bf16 tile that the producer fills with the residual at
 // kernel start and the epilogue overwrites in place with the output.  Without it the output is staged in ring slot
 // 0 once the main loop has drained it.  The shallow variants (3 slots, or 2 + residual tile: 96 KB at BN = 128) let
-// two CTAs share an SM so one's epilogue overlaps the other's main loop; the deep variants (6, or 5 + tile) are
-// used when the grid has at most one CTA per SM anyway and a longer ring hides more TMA latency.
+// two or three CTAs share an SM so one's epilogue overlaps another's main loop; the deep variants (6, or 5 + tile) are for
+// layers with several K ranges on grids that leave SMs free, where a longer ring hides more TMA latency.
 template <int BN, int STAGES, bool RES>
 struct TcSmem {
   static constexpr int kStages = STAGES;
@@ -460,7 +464,7 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* tm, uint32_t src
 // [rows][Cout] matrices with boxes of 64 columns x 128 and 32 rows (128-byte swizzle).
 //
 // SPLIT: the K loop of one output tile is cut into gridDim.z (2 to 8) fixed ranges of p.kb_per K blocks, a
-// property of the layer and never of the batch.  The CTAs of a tile form a thread-block cluster along z.  CTA z owns
+// property of the layer and never of the batch (four of them where nobody sets the number and it pays: conv_ranges.h).  The CTAs of a tile form a thread-block cluster along z.  CTA z owns
 // a slice of the tile's rows: once every CTA has drained its ring (first cluster barrier), each thread sends its row
 // of the fp32 partial tile to the owner's shared memory through distributed shared memory; after the second
 // barrier every CTA adds the partials of its rows in ascending range order, all from its own shared memory (a
@@ -789,7 +793,7 @@ conv_igemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
 // (barriers, TMEM allocation, descriptor fetch) is paid once per SM instead of once per tile.
 // Staged outputs leave through TMA stores; a staging tile is rewritten only after the warp has seen its previous store
 // finish reading it.  Residual tiles are prefetched by the producer into two buffers of their own, which return to it
-// (res_free) as soon as all four epilogue warps have read them.
+// (res_free) as soon as all epilogue warps have read them.
 template <int BN, bool RES, bool PROJ = false>
 struct TcPersistSmem {
   // without a residual: a longer ring and two output staging tiles; with one: two residual tiles the producer
@@ -829,7 +833,7 @@ conv_igemm_tcgen05_persistent_kernel(const __grid_constant__ CUtensorMap tmA, co
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* gen = smem_raw + (base - raw);
-  float* s_sb = reinterpret_cast<float*>(gen + S::kAfter);  // [epilogue warps][scale BN | bias BN]
+  float* s_sb = reinterpret_cast<float*>(gen + S::kAfter);  // [epilogue warps][scale | bias (| scale2 | bias2)], 32 of each
   uint64_t* bars = reinterpret_cast<uint64_t*>(gen + S::kAfter + S::kEpiWarps * S::kSb * 4);
   const uint32_t bar0 = base + S::kAfter + S::kEpiWarps * S::kSb * 4;
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
@@ -1513,12 +1517,13 @@ inline ee_status_t tc_launch(TcContext& c, const TcLayer& L, const void* src, co
   p.err_flag = err_flag;
   // A layer with several K ranges runs them as a cluster of CTAs per tile (more SMs pull operands: small grids) or, bit
   // for bit the same, in ONE CTA per tile with an accumulator per range (no cluster, no exchange: grids that fill the GPU
-  // anyway).  range_mode: 0 = the cluster while the whole grid still fits one wave, 1 = cluster, 2 = one CTA.
+  // anyway).  range_mode: 0 = the cluster up to 1.25 waves, 1 = cluster, 2 = one CTA.
   const long tiles_all = (long)cdiv(p.M, kTcBM) * cdiv(L.cout, L.bn);
   const bool can_local = L.splits > 1 && L.splits * L.bn <= 512 && !L.gather;
   // Measured (3x3 256->256 on 14x14, 2 and 4 ranges): the cluster wins while tiles x ranges stays within about 1.25 waves
   // and loses badly beyond; one CTA with 2 accumulators costs 1 us per layer over a single range, with 4 (all 512 TMEM
-  // columns: no second CTA, no overlap with the neighbouring kernels' prologues) 17 us.
+  // columns: no second CTA, no overlap with the neighbouring kernels' prologues) 1.5 to 17 us.  Ranges that the library
+  // chooses never get there (tc_auto_ranges): only those a caller sets.
   const bool local = can_local && (range_mode == 2 || (range_mode == 0 && tiles_all * L.splits * 4 > 5L * c.sm_count));
   const bool split = L.splits > 1 && !local;
   p.ranges = local ? L.splits : 1;

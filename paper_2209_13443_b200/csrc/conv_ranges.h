@@ -17,8 +17,8 @@ inline bool tc_cluster_deep(long ctas, int sms) { return ctas * 4 <= 3L * sms; }
 // so four pay from about 60 blocks on (3x3 layers on 7x7 maps of 1 to 16 samples, four against one: 54 blocks +0.4 us, 63 -0.7,
 // 90 -2.9, 144 -7.2; with 64 filters 72 blocks -3.5).  Past the deep clusters they lose at every size: 3x3 512->512, four ranges against one,
 // us a layer: 7x7 maps batch 8 -0.5, 16 +5.2, 64 +1.5; 6x6 batch 16 -0.5, 22 +5.1, 64 +5.3 (an accumulator per range in one CTA);
-// 4x4 batch 48 -0.3, 64 +4.5; 3x3 and 2x2 -0.3 to -1.4 up to 64.  Two ranges lost in every case (+0.7 to +9.9), three gave
-// nothing where four gain (-0.7 to +0.6).
+// 4x4 batch 48 -0.3, 64 +4.5; 3x3 and 2x2 -0.3 to -1.4 up to 64.  Two ranges lost in every one of these (+0.7 to +9.9), three
+// gave nothing where four gain (-0.7 to +0.6).
 inline int tc_auto_ranges(int num_kb, long tiles_max, int sms) {
   const int per = (num_kb + 3) / 4;
   return tc_cluster_deep(tiles_max * 4, sms) && 3 * per < num_kb && 7.0 + 0.15 * per < 2.0 + 0.122 * num_kb ? 4 : 1;

@@ -176,9 +176,9 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t smem_addr) {
   return d;
 }
 
-// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = 128, N = n.
-__host__ __device__ constexpr uint32_t umma_idesc(int n) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTcBM >> 4) << 24);
+// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, M = m (128, or 64: row r in TMEM lane r / 16 * 32 + r % 16), N = n.
+__host__ __device__ constexpr uint32_t umma_idesc(int n, int m = kTcBM) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
 __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate) {
@@ -1178,7 +1178,7 @@ struct TcLayer {
   struct Cached {
     const void* ptr;
     int batch;
-    int kind;  // 0: operand A, 1, 8: output matrix, 4: halo blocks, 7: residual
+    int kind;  // 0, 9: operand A, 1, 8: output matrix, 4: halo blocks, 7: residual
     CUtensorMap tm;
   };
   mutable std::vector<Cached> a_maps;  // tensor maps of caller buffers by (pointer, batch, kind)
@@ -1273,7 +1273,7 @@ inline ee_status_t tc_plan_layer(TcContext& c, const ee_layer_desc_t& d, int in_
   return r == CUDA_SUCCESS ? EE_OK : EE_ERR_CUDA;
 }
 
-// Tensor map of a caller buffer, cached by (pointer, batch, kind).  kind 0: operand A of the layer; kind 1: a
+// Tensor map of a caller buffer, cached by (pointer, batch, kind).  kind 0, 9: operand A of the layer in boxes of 128 or 64 rows; kind 1: a
 // [batch*Ho*Wo][Cout] matrix (residual or output) with a 64 x 32 box.  A map covers exactly `batch` samples: rows
 // past them are out of bounds for the TMA unit (reads give zero, writes are dropped), so no byte beyond the
 // caller's [batch] samples is ever touched.
@@ -1288,6 +1288,7 @@ inline ee_status_t tc_buffer_map(const TcContext& c, const TcLayer& L, const voi
   e.batch = batch;
   e.kind = kind;
   CUresult r;
+  const cuuint32_t rows_a = kind == 9 ? 64 : kTcBM;
   if (kind == 4) {
     // NHWC as (C, W, H, B); a box is the R + 2 rows of W + 2 pixels one output tile of R rows touches (zero fill outside)
     const int wp = L.in_w + 2, rows = kTcBM / wp + 2;
@@ -1309,7 +1310,7 @@ inline ee_status_t tc_buffer_map(const TcContext& c, const TcLayer& L, const voi
   } else if (!L.im2col) {
     const cuuint64_t dims[2] = {(cuuint64_t)L.cin, (cuuint64_t)batch * L.in_h * L.in_w};
     const cuuint64_t strides[1] = {(cuuint64_t)L.cin * 2};
-    const cuuint32_t box[2] = {kTcBK, kTcBM};
+    const cuuint32_t box[2] = {kTcBK, rows_a};
     const cuuint32_t es[2] = {1, 1};
     r = c.encode_tiled(&e.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, es,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1322,7 +1323,7 @@ inline ee_status_t tc_buffer_map(const TcContext& c, const TcLayer& L, const voi
     const int upper[2] = {L.pad_w - (L.kw - 1), L.pad - (L.kh - 1)};
     const cuuint32_t es[4] = {1, (cuuint32_t)L.stride, (cuuint32_t)L.stride, 1};
     r = c.encode_im2col(&e.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, lower, upper, kTcBK,
-                        kTcBM, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        rows_a, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   }
   if (r != CUDA_SUCCESS) return EE_ERR_CUDA;
@@ -1419,17 +1420,21 @@ inline bool tc_proj_supported(const TcLayer& L, const TcLayer& P) {
          P.out_h == L.out_h && P.out_w == L.out_w && L.kh * L.kw == 1 && L.splits == 1 && !L.gather && !L.halo;
 }
 
-// Tile width of the one-wave kernel (conv_wave.cuh) for a layer at batch B, 0 = more tiles than SMs: the grid's CTAs then share
-// SMs (or walk tiles on the persistent kernel).  Within one wave the narrower tile is the faster one: more slots for the same
-// round trip of a K block, a shorter epilogue.
-inline int tc_wave_bn(const TcContext& c, const TcLayer& L, int B) {
-  const long mt = cdiv((long)B * L.out_h * L.out_w, kTcBM);
-  for (int bn = 32; bn <= L.bn; bn *= 2)
-    if (mt * cdiv(L.cout, bn) <= c.sm_count) return bn;
-  return 0;
+// Tile of the one-wave kernel (conv_wave.cuh) for a layer at batch B, bm = 0: more tiles than SMs, the grid's CTAs then share
+// SMs (or walk tiles on the persistent kernel).  Within one wave the tile with the fewest operand rows is the fastest: a K block takes
+// about a clock per row, and more of them fit the ring.  64 x 128 would read as many rows as 128 x 64 at half the tensor rate.
+struct WaveTile {
+  int bm, bn;
+};
+inline WaveTile tc_wave_tile(const TcContext& c, const TcLayer& L, int B) {
+  const long M = (long)B * L.out_h * L.out_w;
+  for (WaveTile t : {WaveTile{64, 32}, WaveTile{64, 64}, WaveTile{128, 32}, WaveTile{128, 64}, WaveTile{128, 128}})
+    if (t.bn <= L.bn && (long)cdiv(M, t.bm) * cdiv(L.cout, t.bn) <= c.sm_count) return t;
+  return {0, 0};
 }
-inline cudaError_t wave_launch(int bn, cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, TcParams p);   // conv_wave.cuh
-inline cudaError_t wave_launch_proj(int bn, cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, const CUtensorMap& a2, const CUtensorMap& w2, TcParams p);
+inline const CUtensorMap& tc_weight_map(const TcLayer& L, int bn) { return bn == L.bn ? L.tm_w : L.tm_w_bn[bn / 64]; }
+template <bool PROJ>
+inline cudaError_t wave_launch(WaveTile t, cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, const CUtensorMap& a2, const CUtensorMap& w2, const TcParams& p);   // conv_wave.cuh
 
 // L with the projection P in its launch: src -> L, src2 -> P; P's own output is never written.
 inline ee_status_t tc_launch_proj(TcContext& c, const TcLayer& L, const TcLayer& P, const void* src, const void* src2, void* dst, int B,
@@ -1440,9 +1445,11 @@ inline ee_status_t tc_launch_proj(TcContext& c, const TcLayer& L, const TcLayer&
   ee_status_t s = tc_buffer_map(c, L, dst, B, 8, &t);
   if (s != EE_OK) return s;
   const CUtensorMap tmO = *t;
-  if ((s = tc_buffer_map(c, L, src, B, 0, &t)) != EE_OK) return s;
+  // the persistent kernel's long prologue and 128-wide epilogue are for several tiles per SM
+  const WaveTile wave = gap_part ? WaveTile{0, 0} : tc_wave_tile(c, L, B);
+  if ((s = tc_buffer_map(c, L, src, B, wave.bm == 64 ? 9 : 0, &t)) != EE_OK) return s;
   const CUtensorMap tmA = *t;
-  if ((s = tc_buffer_map(c, P, src2, B, 0, &t)) != EE_OK) return s;
+  if ((s = tc_buffer_map(c, P, src2, B, wave.bm == 64 ? 9 : 0, &t)) != EE_OK) return s;
   const CUtensorMap tmA2 = *t;
   TcParams p = {};
   p.M = B * L.out_h * L.out_w;
@@ -1461,9 +1468,7 @@ inline ee_status_t tc_launch_proj(TcContext& c, const TcLayer& L, const TcLayer&
   p.cblocks2 = cdiv(P.cin, kTcBK), p.im2col2 = P.im2col ? 1 : 0, p.stride2 = P.stride, p.act2 = P.act;
   p.scale2 = scale2, p.bias2 = bias2;
   p.gap_part = gap_part, p.gap_g = gap_part ? gap_g : 0;
-  // the persistent kernel's long prologue and 128-wide epilogue are for several tiles per SM
-  if (const int bn = p.gap_part ? 0 : tc_wave_bn(c, L, B))
-    return wave_launch_proj(bn, st, tmA, bn == L.bn ? L.tm_w : L.tm_w_bn[bn / 64], tmA2, bn == L.bn ? P.tm_w : P.tm_w_bn[bn / 64], p) == cudaSuccess ? EE_OK : EE_ERR_CUDA;
+  if (wave.bm) return wave_launch<true>(wave, st, tmA, tc_weight_map(L, wave.bn), tmA2, tc_weight_map(P, wave.bn), p) == cudaSuccess ? EE_OK : EE_ERR_CUDA;
   const cudaError_t e = L.bn == 128 ? tc_launch_persistent_proj<128>(c.sm_count, st, tmA, L.tm_w, tmO, tmA2, P.tm_w, p)
                                     : tc_launch_persistent_proj<64>(c.sm_count, st, tmA, L.tm_w, tmO, tmA2, P.tm_w, p);
   return e == cudaSuccess ? EE_OK : EE_ERR_CUDA;
@@ -1554,8 +1559,15 @@ inline ee_status_t tc_launch(TcContext& c, const TcLayer& L, const void* src, co
       pe = res ? tc_launch_persistent<64, true>(ctas, st, tmA, L.tm_w, tmR, tmO, p) : tc_launch_persistent<64, false>(ctas, st, tmA, L.tm_w, tmR, tmO, p);
     return pe == cudaSuccess ? EE_OK : EE_ERR_CUDA;
   }
-  if (const int bn = split || local ? 0 : tc_wave_bn(c, L, B))
-    return wave_launch(bn, st, tmA, bn == L.bn ? L.tm_w : L.tm_w_bn[bn / 64], p) == cudaSuccess ? EE_OK : EE_ERR_CUDA;
+  const WaveTile wave = split || local ? WaveTile{0, 0} : tc_wave_tile(c, L, B);
+  if (wave.bm) {
+    if (wave.bm == 64) {
+      if ((s = tc_buffer_map(c, L, src, B, 9, &t)) != EE_OK) return s;
+      tmA = *t;
+    }
+    const CUtensorMap& w = tc_weight_map(L, wave.bn);
+    return wave_launch<false>(wave, st, tmA, w, tmA, w, p) == cudaSuccess ? EE_OK : EE_ERR_CUDA;
+  }
   cudaError_t e = L.bn == 128 ? tc_launch_bn<128>(deep, tma_res, split, grid, st, tmA, L.tm_w, tmR, tmO, p)
                               : tc_launch_bn<64>(deep, tma_res, split, grid, st, tmA, L.tm_w, tmR, tmO, p);
   return e == cudaSuccess ? EE_OK : EE_ERR_CUDA;

@@ -1,19 +1,26 @@
-// Convolution tiles of grids with at most one tile per SM (small batches, the 14x14 and 7x7 maps): 128 pixels x BN filters per
-// CTA, the narrowest of 32, 64 and 128 whose tiles fit in one wave.
+// Convolution tiles of grids with at most one tile per SM (small batches, the 14x14 and 7x7 maps): BM pixels x BN filters per
+// CTA, the first of 64 x 32, 64 x 64, 128 x 32, 128 x 64 and 128 x 128 whose tiles fit in one wave.
 //
 // Such a layer is a chain of latencies: first operands (600 ns), the K loop of one tile, its epilogue, and about 1 us until the
-// next launch may go on.  What this kernel does about them (clocks measured inside it):
+// next launch may go on.  What this kernel does about them (clocks measured on one SM):
+//  - The tensor core reads both operands at 128 bytes a clock, so a K block's four MMAs take BM + BN clocks and a few more (64 x 32:
+//    110, 64 x 64: 133, 128 x 32: 162, 128 x 64: 194, 128 x 128: 257); TMA writes a 128-byte row a clock beside them.  Hence
+//    small tiles first.  At 128 x 32 alone the 3x3 512 -> 512 layer on one 7x7 map took 10.6 us, at 64 x 32 10.4: another bound.
+//  - That bound was the thread behind the MMAs: every wait on a barrier costs it about 100 clocks, whether the data is there or not, so a
+//    K block with a wait of its own took 212 clocks at 64 x 32, with one MMA in place of four as well.  kG K blocks share a full
+//    barrier (their slots are still given back one by one): 212 -> 140 clocks at two, 128 at four; 128 x 64 and 128 x 128 tiles, which
+//    are bound by the MMAs and by the few slots that fit, lose from it (3x3 256 -> 256, batch 30: 9.3, 9.7 at two, 13.8 at four).
 //  - A K block goes round the ring in about 1900 clocks (its loads 1100, its MMAs and their commit, the feeding thread), so the
-//    K loop's pace is that over the number of slots: all of shared memory is ring when the loop is long, and a narrow tile has
-//    more slots (11 of 20 KB at 32 filters, 6 of 32 KB at 128).
-//  - Weights and activations have two feeding warps each, for the even and the odd blocks: one thread behind both operands spent
-//    400 clocks between a free slot and its second request.
-//  - The MMA thread asks for the next block's barrier before it issues this block's MMAs: the answer is there when it gets to it.
+//    K loop's pace is also that over the number of slots: all of shared memory is ring when the loop is long, and a small tile has
+//    more slots (16 of 12 KB at 64 x 32, 6 of 32 KB at 128 x 128).
+//  - Weights and activations have two feeding warps each: a thread takes about 140 clocks from one request to its next (three
+//    or four warps an operand gained nothing).
+//  - The MMA thread asks for the next group's barrier before it issues this one's MMAs: the answer is there when it gets to it.
 //  - 32 or 64 columns per epilogue warp (four warps with 128 columns each took 2800 clocks, these take 700 or 1400).  The
 //    residual's rows come to registers while the K loop runs.
 // Bits are those of the other kernels: the same K order, one accumulator per output, one rounding.
-// In a chain of launches, before (128-filter tiles, a feeding thread per operand) -> now, us: 3x3 512 -> 512 on 7x7, batch 1
-// 13.6 -> 10.8, batch 22 14.4 -> 11.3; 3x3 256 -> 256 on 14x14, batch 1 8.4 -> 6.4; 1x1 512 -> 128 on 28x28 4.3 -> 3.0, 128 -> 512 3.7 -> 2.5.
+// In a chain of launches, 128-pixel tiles and a wait per K block -> now, us: 3x3 512 -> 512 on 7x7, batch 1 10.6 -> 7.5; 3x3 256 -> 256
+// on 14x14, batch 1 6.3 -> 4.7, batch 7 6.8 -> 5.8; 1x1 2048 -> 512, batch 1 5.8 -> 4.4; 1x1 512 -> 128 on 28x28 2.9 -> 2.5.
 //
 // PROJ: the residual operand is a 1x1 projection computed into a second accumulator (see the persistent kernel of conv_tc.cuh).
 #pragma once
@@ -21,22 +28,27 @@
 
 namespace ee {
 
-template <int BN>
+template <int BM, int BN>
 struct WaveSmem {
   static constexpr int kEpiWarps = BN == 32 ? 4 : 8;
-  static constexpr int kThreads = 32 * (5 + kEpiWarps);     // warps 0, 1 weights, 2, 3 activations, 4 MMA, then the epilogue
-  static constexpr int kABytes = kTcBM * kTcBK * 2, kBBytes = BN * kTcBK * 2, kSlot = kABytes + kBBytes;
-  static constexpr int kMaxSlots = BN == 32 ? 11 : BN == 64 ? 9 : 6;
-  static_assert(kEpiWarps * 2048 <= kSlot, "output staging: 2 KB per epilogue warp in the drained first slot");
-  static constexpr int bytes(int slots) { return slots * kSlot + 4 * BN * 4 + 256 + 256 + 1024; }   // + scale/bias, barriers, taps, alignment slack
+  static constexpr int kFeed = 2;                            // feeding warps of each operand
+  static constexpr int kMma = 2 * kFeed, kEpi = kMma + 1;   // warps: weights, activations, MMA, then the epilogue
+  static constexpr int kThreads = 32 * (kEpi + kEpiWarps);
+  static constexpr int kG = BM == 64 ? (BN == 32 ? 4 : 2) : BN == 32 ? 2 : 1;   // K blocks per full barrier
+  static constexpr int kABytes = BM * kTcBK * 2, kBBytes = BN * kTcBK * 2, kSlot = kABytes + kBBytes;
+  static constexpr int kMaxSlots = (BM == 64 ? (BN == 32 ? 18 : 13) : BN == 32 ? 11 : BN == 64 ? 9 : 6) / kG * kG;
+  static constexpr int kWarpRows = BM / 4;                  // pixels per epilogue warp: at 64 pixels a TMEM lane quarter holds 16 of them
+  static_assert(kEpiWarps * kWarpRows * 64 <= kSlot, "output staging: 64 bytes per pixel of an epilogue warp in the drained first slot");
+  static constexpr int kBars = 2 * kMaxSlots + 1, kTapsOff = (kBars * 8 + 4 + 15) / 16 * 16;   // barriers, the TMEM address, taps
+  static constexpr int bytes(int slots) { return slots * kSlot + 4 * BN * 4 + kTapsOff + 256 + 1024; }   // + scale/bias, barriers, taps, alignment slack
   static_assert(bytes(kMaxSlots) <= 227 * 1024, "exceeds the shared memory of an SM");
 };
 
-template <int BN, bool PROJ>
-__global__ void __launch_bounds__(WaveSmem<BN>::kThreads, 1)
+template <int BM, int BN, bool PROJ>
+__global__ void __launch_bounds__(WaveSmem<BM, BN>::kThreads, 1)
 conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
                          const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmW2, TcParams p) {
-  using S = WaveSmem<BN>;
+  using S = WaveSmem<BM, BN>;
   constexpr int R = S::kMaxSlots;
   extern __shared__ uint8_t smem_raw[];
   const int ring = p.ring;   // slots, <= R
@@ -46,22 +58,22 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
   float* s_sb = reinterpret_cast<float*>(gen + ring * S::kSlot);      // scale | bias | scale2 | bias2
   uint64_t* bars = reinterpret_cast<uint64_t*>(gen + ring * S::kSlot + 4 * BN * 4);
   const uint32_t bar0 = base + (uint32_t)(ring * S::kSlot + 4 * BN * 4);
-  auto full_bar = [&](int s) { return bar0 + 8u * s; };
+  auto full_bar = [&](int s) { return bar0 + 8u * (s / S::kG); };   // of the group that slot s belongs to
   auto empty_bar = [&](int s) { return bar0 + 8u * (R + s); };
   const uint32_t accum_bar = bar0 + 8u * (2 * R);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * R + 1);
-  uint32_t* taps = reinterpret_cast<uint32_t*>(bars + 32);
+  uint32_t* taps = reinterpret_cast<uint32_t*>(gen + ring * S::kSlot + 4 * BN * 4 + S::kTapsOff);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = (p.rev ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x) * kTcBM, n0 = blockIdx.y * BN;
+  const int m0 = (p.rev ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x) * BM, n0 = blockIdx.y * BN;
   const int num_kb1 = p.taps * p.cblocks, num_kb = num_kb1 + (PROJ ? p.cblocks2 : 0);
   constexpr uint32_t kCols = PROJ ? 2 * BN : BN;   // accumulators, fp32 columns
 
   if (threadIdx.x < 2 * R + 1) {
-    mbar_init(bar0 + 8u * threadIdx.x, threadIdx.x < R ? 2 : 1);   // full: one expect_tx each of weights and activations
+    mbar_init(bar0 + 8u * threadIdx.x, threadIdx.x < R ? 2 * S::kG : 1);   // full: an expect_tx each of weights and activations per K block
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 5 && lane == 0) {
+  if (warp == S::kEpi && lane == 0) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmW) : "memory");
     if (PROJ) {
@@ -70,7 +82,7 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     }
   }
   tap_table_fill(taps, p.kh, p.kw, p.stride);
-  if (warp == 4) {
+  if (warp == S::kMma) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -79,17 +91,26 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  if (warp < 4) {
-    // K blocks h, h + 2, ...: walked by counters (slot and phase, channel block x 64, position in the tap table)
-    const int h = warp & 1, dc = p.taps == 1 ? 2 * kTcBK : 0, dt = p.taps == 1 ? 0 : 2;
+  if (warp < S::kMma) {
+    // K blocks h, h + kFeed, ...: walked by counters (slot and phase, channel block x 64, position in the tap table)
+    constexpr int F = S::kFeed;
+    const int h = warp % F, dc = p.taps == 1 ? F * kTcBK : 0, dt = p.taps == 1 ? 0 : F;
     int i = h, s = h, c = p.taps == 1 ? h * kTcBK : 0, t = p.taps == 1 ? 0 : h;
     uint32_t ph = 1;
+    while (t >= p.taps) t -= p.taps, c += kTcBK;
     auto step = [&] {
-      i += 2, c += dc, t += dt;
-      if (t >= p.taps) t -= p.taps, c += kTcBK;
-      if ((s += 2) >= ring) s -= ring, ph ^= 1u;
+      i += F, c += dc, t += dt;
+      while (t >= p.taps) t -= p.taps, c += kTcBK;
+      if ((s += F) >= ring) s -= ring, ph ^= 1u;
     };
-    if (warp < 2) {
+    // the last group may be short: whoever feeds its last block arrives for the missing ones
+    auto fill = [&] {
+      if (S::kG > 1 && h == (num_kb - 1) % F && num_kb % S::kG) {
+        const uint32_t bar = full_bar((num_kb - 1) % ring);
+        for (int k = num_kb % S::kG; k < S::kG; ++k) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+      }
+    };
+    if (warp < F) {
       if (elect_one()) {
         // no kernel writes weights: nothing to wait for but a free slot
         for (; i < num_kb; step()) {
@@ -101,6 +122,7 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
           else
             tma_load_3d(dst, &tmW, full_bar(s), c, (int)(taps[t] >> 16), n0);
         }
+        if (i >= num_kb) fill();
       }
       __syncwarp();
       asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -144,32 +166,44 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
               tma_load_2d(base + (uint32_t)(s * S::kSlot), &tmA2, full_bar(s), (i - num_kb1) * kTcBK, m0);
           }
         }
+        if (i >= num_kb) fill();
       }
       __syncwarp();
     }
-  } else if (warp == 4) {
+  } else if (warp == S::kMma) {
     if (elect_one()) {
-      constexpr uint32_t idesc = umma_idesc(BN);
+      constexpr uint32_t idesc = umma_idesc(BN, BM);
+      constexpr int G = S::kG;
       const uint64_t da0 = umma_desc(base), db0 = umma_desc(base + S::kABytes);
       bool ok = true;
-      int s = 0;
+      int s = 0, i = 0;
       uint32_t ph = 0;
+      auto block = [&](int i, int s) {
+        const uint64_t off = (uint64_t)(s * (S::kSlot >> 4));
+        umma_block(tmem_base + (PROJ && i >= num_kb1 ? (uint32_t)BN : 0u), da0 + off, db0 + off, idesc, i != 0 && !(PROJ && i == num_kb1));
+      };
       bool here = mbar_test_wait(full_bar(0), 0);
-      for (int i = 0; i < num_kb; ++i) {
+      for (; i + G <= num_kb; i += G) {
         if (!here) ok = mbar_wait(full_bar(s), ph, p.err_flag);
         if (!ok) break;
         const int cur = s;
-        if (++s == ring) s = 0, ph ^= 1u;
-        here = mbar_test_wait(full_bar(s), ph);   // behind the last block: a phase that nobody waits for
-        const uint64_t off = (uint64_t)(cur * (S::kSlot >> 4));
-        umma_block(tmem_base + (PROJ && i >= num_kb1 ? (uint32_t)BN : 0u), da0 + off, db0 + off, idesc, i != 0 && i != num_kb1);
-        umma_commit(empty_bar(cur));
+        if ((s += G) == ring) s = 0, ph ^= 1u;
+        here = mbar_test_wait(full_bar(s), ph);   // behind the last group: a phase that nobody waits for
+#pragma unroll
+        for (int k = 0; k < G; ++k) {
+          block(i + k, cur + k);
+          umma_commit(empty_bar(cur + k));
+        }
+      }
+      if (ok && i < num_kb) {   // a short group: its slots are not used again
+        if (!here) ok = mbar_wait(full_bar(s), ph, p.err_flag);
+        for (; ok && i < num_kb; ++i, ++s) block(i, s);
       }
       if (ok) umma_commit(accum_bar);   // everything before it has read its operands as well
     }
     __syncwarp();
   } else {
-    const int et = threadIdx.x - 160;
+    const int et = threadIdx.x - 32 * S::kEpi;
     for (int i = et; i < BN; i += 32 * S::kEpiWarps) {
       const bool in = n0 + i < p.N;
       s_sb[i] = (p.scale && in) ? p.scale[n0 + i] : 1.f;
@@ -183,7 +217,7 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     constexpr int kCover = BN == 128 ? 64 : 32, kSteps = kCover / 32;   // columns of a warp, in steps of 32
-    const int q = warp & 3, half = et >> 7, m = m0 + q * 32 + lane;
+    const int q = warp & 3, half = et >> 7, m = lane < S::kWarpRows ? m0 + q * S::kWarpRows + lane : p.M;
     uint4 r[4 * kSteps];
 #pragma unroll
     for (int g = 0; g < 4 * kSteps; ++g) {
@@ -194,7 +228,7 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     const bool ok = __all_sync(0xffffffffu, mbar_wait(accum_bar, 0, p.err_flag));
     if (ok) {
       tc_fence_after();
-      uint8_t* stage = gen + (warp - 5) * 2048;   // 32 rows of 64 bytes, their 16-byte chunks XORed with the row
+      uint8_t* stage = gen + (warp - S::kEpi) * (S::kWarpRows * 64);   // rows of 64 bytes, their 16-byte chunks XORed with the row
 #pragma unroll
       for (int st = 0; st < kSteps; ++st) {
         const int c0 = half * kCover + st * 32;
@@ -217,11 +251,12 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
           epilogue32<false>(p.act, v, s_sb + c0, s_sb + BN + c0, nullptr, o);
         if (st) __syncwarp();
 #pragma unroll
-        for (int g = 0; g < 4; ++g) *reinterpret_cast<uint4*>(stage + lane * 64 + ((g ^ (lane >> 1 & 3)) << 4)) = o[g];
+        for (int g = 0; g < 4; ++g)
+          if (lane < S::kWarpRows) *reinterpret_cast<uint4*>(stage + lane * 64 + ((g ^ (lane >> 1 & 3)) << 4)) = o[g];
         __syncwarp();
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {   // eight rows per store, four lanes with 64 bytes of each
-          const int row = k * 8 + (lane >> 2), g = lane & 3, mm = m0 + q * 32 + row, n = n0 + c0 + g * 8;
+        for (int k = 0; k < S::kWarpRows / 8; ++k) {   // eight rows per store, four lanes with 64 bytes of each
+          const int row = k * 8 + (lane >> 2), g = lane & 3, mm = m0 + q * S::kWarpRows + row, n = n0 + c0 + g * 8;
           const uint4 x = *reinterpret_cast<const uint4*>(stage + row * 64 + ((g ^ (row >> 1 & 3)) << 4));
           if (mm < p.M && n < p.N) *reinterpret_cast<uint4*>(p.out + (size_t)mm * p.N + n) = x;
         }
@@ -230,7 +265,7 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 4) {
+  if (warp == S::kMma) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kCols) : "memory");
   }
@@ -241,22 +276,26 @@ inline ee_status_t wave_context_init() {
   auto set = [&](auto kernel, int bytes) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   };
-  set(conv_wave_tcgen05_kernel<32, false>, WaveSmem<32>::bytes(WaveSmem<32>::kMaxSlots));
-  set(conv_wave_tcgen05_kernel<32, true>, WaveSmem<32>::bytes(WaveSmem<32>::kMaxSlots));
-  set(conv_wave_tcgen05_kernel<64, false>, WaveSmem<64>::bytes(WaveSmem<64>::kMaxSlots));
-  set(conv_wave_tcgen05_kernel<64, true>, WaveSmem<64>::bytes(WaveSmem<64>::kMaxSlots));
-  set(conv_wave_tcgen05_kernel<128, true>, WaveSmem<128>::bytes(WaveSmem<128>::kMaxSlots));
-  set(conv_wave_tcgen05_kernel<128, false>, WaveSmem<128>::bytes(WaveSmem<128>::kMaxSlots));
+  auto tile = [&](auto s, auto plain, auto proj) {
+    typedef decltype(s) S;
+    set(plain, S::bytes(S::kMaxSlots));
+    set(proj, S::bytes(S::kMaxSlots));
+  };
+  tile(WaveSmem<64, 32>{}, conv_wave_tcgen05_kernel<64, 32, false>, conv_wave_tcgen05_kernel<64, 32, true>);
+  tile(WaveSmem<64, 64>{}, conv_wave_tcgen05_kernel<64, 64, false>, conv_wave_tcgen05_kernel<64, 64, true>);
+  tile(WaveSmem<128, 32>{}, conv_wave_tcgen05_kernel<128, 32, false>, conv_wave_tcgen05_kernel<128, 32, true>);
+  tile(WaveSmem<128, 64>{}, conv_wave_tcgen05_kernel<128, 64, false>, conv_wave_tcgen05_kernel<128, 64, true>);
+  tile(WaveSmem<128, 128>{}, conv_wave_tcgen05_kernel<128, 128, false>, conv_wave_tcgen05_kernel<128, 128, true>);
   return e == cudaSuccess ? EE_OK : EE_ERR_CUDA;
 }
 
 // Slots: as many as the K loop has blocks for; a short loop leaves room on its SM for the next layer's CTA to set up.
-template <int BN, bool PROJ>
+template <int BM, int BN, bool PROJ>
 inline cudaError_t wave_launch_t(cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, const CUtensorMap& a2, const CUtensorMap& w2, TcParams p) {
-  using S = WaveSmem<BN>;
-  p.ring = std::min(S::kMaxSlots, std::max(2, p.taps * p.cblocks + (PROJ ? p.cblocks2 : 0)));
+  using S = WaveSmem<BM, BN>;
+  p.ring = std::min(S::kMaxSlots, cdiv(std::max(S::kFeed, p.taps * p.cblocks + (PROJ ? p.cblocks2 : 0)), S::kG) * S::kG);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(cdiv(p.M, kTcBM), cdiv(p.N, BN));
+  cfg.gridDim = dim3(cdiv(p.M, BM), cdiv(p.N, BN));
   cfg.blockDim = dim3(S::kThreads);
   cfg.dynamicSmemBytes = S::bytes(p.ring);
   cfg.stream = st;
@@ -265,14 +304,16 @@ inline cudaError_t wave_launch_t(cudaStream_t st, const CUtensorMap& a, const CU
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, conv_wave_tcgen05_kernel<BN, PROJ>, a, w, a2, w2, p);
+  return cudaLaunchKernelEx(&cfg, conv_wave_tcgen05_kernel<BM, BN, PROJ>, a, w, a2, w2, p);
 }
 
-inline cudaError_t wave_launch(int bn, cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, TcParams p) {
-  return bn == 32 ? wave_launch_t<32, false>(st, a, w, a, w, p) : bn == 64 ? wave_launch_t<64, false>(st, a, w, a, w, p) : wave_launch_t<128, false>(st, a, w, a, w, p);
-}
-inline cudaError_t wave_launch_proj(int bn, cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, const CUtensorMap& a2, const CUtensorMap& w2, TcParams p) {
-  return bn == 32 ? wave_launch_t<32, true>(st, a, w, a2, w2, p) : bn == 64 ? wave_launch_t<64, true>(st, a, w, a2, w2, p) : wave_launch_t<128, true>(st, a, w, a2, w2, p);
+// a, a2: maps whose boxes have t.bm rows, w, w2: boxes of t.bn filters.
+template <bool PROJ>
+inline cudaError_t wave_launch(WaveTile t, cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, const CUtensorMap& a2, const CUtensorMap& w2, const TcParams& p) {
+  if (t.bm == 64) return t.bn == 32 ? wave_launch_t<64, 32, PROJ>(st, a, w, a2, w2, p) : wave_launch_t<64, 64, PROJ>(st, a, w, a2, w2, p);
+  return t.bn == 32   ? wave_launch_t<128, 32, PROJ>(st, a, w, a2, w2, p)
+         : t.bn == 64 ? wave_launch_t<128, 64, PROJ>(st, a, w, a2, w2, p)
+                      : wave_launch_t<128, 128, PROJ>(st, a, w, a2, w2, p);
 }
 
 }  // namespace ee

@@ -170,6 +170,19 @@ def test_one_wave_tiles_against_the_oracle_and_at_every_width(geom):
         assert np.array_equal(g["features_out"][: len(first)], first), f"{geom} B={B}"
 
 
+# one-wave tiles of 64 pixels (32 and 64 filters) and of 128 x 32: K blocks that leave a group short, exactly as many as the ring has
+# slots and one more, a ragged last tile, images that straddle tiles
+WAVE_GROUP_GEOMS = [
+    (8, 8, 1024, 512, 1, 1, False, (1, 9, 10, 18, 19)), (8, 8, 1088, 520, 1, 1, True, (1, 8, 17)), (14, 14, 704, 96, 1, 1, True, (1, 23, 25, 32)),
+    (7, 7, 192, 512, 3, 1, True, (1, 3, 12)), (5, 5, 320, 72, 1, 1, False, (1, 2, 60)), (7, 7, 832, 256, 1, 1, False, (1, 40)),
+]
+
+
+@pytest.mark.parametrize("geom", WAVE_GROUP_GEOMS)
+def test_one_wave_tiles_of_64_pixels_and_groups_of_k_blocks(geom):
+    test_one_wave_tiles_against_the_oracle_and_at_every_width(geom)
+
+
 @pytest.mark.parametrize("case", [(7, 7, 64, 40, 128, 1, 1), (14, 14, 128, 520, 96, 2, 2), (5, 9, 320, 256, 704, 1, 3), (14, 14, 64, 1000, 72, 1, 5), (14, 14, 192, 1016, 136, 1, 9)])
 def test_projection_inside_a_one_wave_tile_gives_the_bits_of_two_layers(case):
     H, W, mid, wide, cin, stride, B = case

@@ -221,7 +221,7 @@ def run_ours(args):
     def stage_launches(s, n):
         """Kernels one ee_stage_run launches: the layers' (a packed stem packs and multiplies chunk by chunk),
         the head's (one cluster kernel, or pooling and FC with the exit decision in its last CTA), one gather."""
-        return sum(pl["launches"] for pl in model.plan(s, n)) + model.head_launches(s) + (0 if spec.stages[s].always_exit else 1)
+        return sum(pl["launches"] for pl in model.plan(s, n)) + model.head_launches(s) - model.head_pools(s, n) + (0 if spec.stages[s].always_exit else 1)
 
     # end to end: the inputs of step k + 1 travel from pinned host memory on a copy stream while step k computes (two
     # device buffers); every copy is issued behind the start event of a timed step, so it lies inside a timed window

@@ -260,6 +260,9 @@ int ee_model_gap_partials(const ee_model_t* model, int stage, int batch);
 ee_status_t ee_model_set_fused_head(ee_model_t* model, int enabled);
 /* Kernels the exit head of `stage` launches on 16-byte aligned features: 1 (one-launch head) or 2; 0 for a bad argument. */
 int ee_model_head_launches(const ee_model_t* model, int stage);
+/* 1 when ee_stage_run of `batch` samples pools inside the FC kernel's launch (few classes on a small map: one launch in place of
+ * the two, the same bits), else 0; 0 for a bad argument.  Timed runs (ee_model_set_timing) always launch both. */
+int ee_model_head_pools(const ee_model_t* model, int stage, int batch);
 
 /* Branch execution.  On by default for batches of up to 32 samples: a layer whose output is only a residual operand of a later layer (the projection
  * shortcut of a residual block) runs on a stream of the model's own, beside the layers between its input and its

@@ -171,7 +171,7 @@ struct ee_model {
   bool stage_kernel = false;           // run eligible layer runs as one launch (measured slower than per-layer launches: off)
   int stage_kernel_max_batch = 1 << 30;
   size_t pair_counter_words = 0;
-  unsigned* head_done = nullptr;       // one arrival counter per stage for the one-launch exit head; zero between launches
+  unsigned* head_done = nullptr;       // two words per stage for the heads of one launch: an arrival counter, or counter and survivors; zero between launches
   int proj_waves = 0;                  // tiles per SM from which a layer absorbs its projection (measured: a gain at every batch)
   bool gap_fusion = true;              // pooling partials from the last layer's epilogue where that applies
   bool proj_fusion = true;             // projection shortcuts computed inside the layer that adds them, where that applies
@@ -343,6 +343,17 @@ bool host_memory(const void* p) {
   return false;
 }
 
+// The map of one stage as the pooling kernels, or an FC kernel that pools by itself, walk it.
+template <typename T>
+PoolArgs pool_args(const void* x, int hw, const float* gap_part, int gap_g) {
+  PoolArgs pa = {x, hw, 0, 1, gap_lanes(hw), 0};
+  if (sizeof(T) == 2) {
+    pa.G = gap_part ? gap_g : gap_block_rows(hw), pa.nb = hw / pa.G, pa.lanes = gap_block_lanes(pa.nb);
+    if (gap_part) pa.x = gap_part, pa.sums = 1;
+  }
+  return pa;
+}
+
 template <typename T>
 ee_status_t launch_head(ee_model* m, StagePlan& sp, const void* x, int B, int hw, const float* shift,
                         const int32_t* shift_cls, char* scratch, const ee_stage_in_t* in_ids, const ee_stage_out_t* out,
@@ -356,7 +367,7 @@ ee_status_t launch_head(ee_model* m, StagePlan& sp, const void* x, int B, int hw
   if constexpr (sizeof(T) == 2) {
     if (m->fused_head && hc_supported(C, K, x, sp.fc_w)) {
       DecideArgs da{shift, shift_cls, sp.threshold, sp.always_exit, out->conf, out->pred, out->exit_mask,
-                    in_ids ? in_ids->ids : nullptr, out->survivor_idx, out->ids_out, out->n_surv_dev, nullptr, m->head_done + (&sp - m->stages.data()), host_count, host_out};
+                    in_ids ? in_ids->ids : nullptr, out->survivor_idx, out->ids_out, out->n_surv_dev, nullptr, m->head_done + 2 * (&sp - m->stages.data()), nullptr, host_count, host_out};
       EE_CUDA(hc_launch((const bf16*)x, hw, C, (const bf16*)sp.fc_w, sp.fc_b, B, K, z, da, st));
       if (timed) record(m, sp, st, "head_gap_fc_softmax_scan");
       return EE_OK;
@@ -365,6 +376,17 @@ ee_status_t launch_head(ee_model* m, StagePlan& sp, const void* x, int B, int hw
   constexpr int V = Elem<T>::kVec;
   const bool vec = C % V == 0 && ((uintptr_t)x & 15) == 0;
   const int lanes = gap_lanes(hw);
+  const FcShape f = fc_shape(B, C, K, (int)sizeof(T), m->fc_room, m->max_batch);
+  if (sp.fc_cluster && vec && !m->timing) {   // timed runs: an event between the two kernels
+    const PoolArgs pa = pool_args<T>(x, hw, gap_part, gap_g);
+    if (fc_pools(f, C / (pa.sums ? 4 : V), pa.lanes)) {
+      unsigned* done = m->head_done + 2 * (&sp - m->stages.data());   // nothing in front of this kernel could zero the scratch's counters
+      DecideArgs da{shift, shift_cls, sp.threshold, sp.always_exit, out->conf, out->pred, out->exit_mask,
+                    in_ids ? in_ids->ids : nullptr, out->survivor_idx, out->ids_out, out->n_surv_dev, nullptr, done, (unsigned long long*)done, host_count, host_out};
+      EE_CUDA(fc_cluster_launch<T>(f, nullptr, &pa, sp.tm_fc, sp.fc_b, B, C, K, out->logits, nullptr, da, m->err_flag, st));
+      return EE_OK;
+    }
+  }
   const int n_zero = m->max_batch + 1;   // the pooling kernel leaves the FC kernel's counters at zero
   bool pooled = false;
   if constexpr (sizeof(T) == 2) {
@@ -397,10 +419,10 @@ ee_status_t launch_head(ee_model* m, StagePlan& sp, const void* x, int B, int hw
     EE_CUDA(launch_pdl(gap_kernel<T, 1>, ggrid, dim3(kGapThreads), st, (const T*)x, hw, C, lanes, gap, cnt, n_zero, sp.gap_rev ? 1 : 0));
   if (timed) record(m, sp, st, "head_gap");
   DecideArgs da{shift, shift_cls, sp.threshold, sp.always_exit, out->conf, out->pred, out->exit_mask,
-                in_ids ? in_ids->ids : nullptr, out->survivor_idx, out->ids_out, out->n_surv_dev, cnt, cnt + m->max_batch, host_count, host_out};
+                in_ids ? in_ids->ids : nullptr, out->survivor_idx, out->ids_out, out->n_surv_dev, cnt, cnt + m->max_batch,
+                f.cluster || f.CL == 1 ? (unsigned long long*)cnt : nullptr, host_count, host_out};
   if (sp.fc_cluster)
-    EE_CUDA(fc_cluster_launch<T>(fc_shape(B, C, K, (int)sizeof(T), m->fc_room), gap, sp.tm_fc, sp.fc_b, B, C, K, out->logits,
-                                 (float4*)(scratch + h.off_z), da, m->err_flag, st));
+    EE_CUDA(fc_cluster_launch<T>(f, gap, nullptr, sp.tm_fc, sp.fc_b, B, C, K, out->logits, (float4*)(scratch + h.off_z), da, m->err_flag, st));
   else
     EE_CUDA(launch_pdl(fc_kernel<T>, dim3(cdiv(K, kFcClasses), cdiv(B, kFcSamples)), dim3(kFcThreads), st, (const float*)gap, (const T*)sp.fc_w,
                        (const float*)sp.fc_b, B, C, K, z, da));
@@ -1131,10 +1153,10 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
   }
   {
     void* p = nullptr;
-    if (cudaMalloc(&p, 256 + m->stages.size() * sizeof(unsigned)) != cudaSuccess) return fail(EE_ERR_CUDA);
+    if (cudaMalloc(&p, 256 + m->stages.size() * 2 * sizeof(unsigned)) != cudaSuccess) return fail(EE_ERR_CUDA);
     m->owned.push_back(p);
     m->head_done = (unsigned*)p;
-    if (cudaMemsetAsync(p, 0, 256 + m->stages.size() * sizeof(unsigned), st) != cudaSuccess) return fail(EE_ERR_CUDA);
+    if (cudaMemsetAsync(p, 0, 256 + m->stages.size() * 2 * sizeof(unsigned), st) != cudaSuccess) return fail(EE_ERR_CUDA);
   }
   if (m->pair_counter_words) {
     void* p = nullptr;
@@ -1469,6 +1491,17 @@ int ee_model_head_launches(const ee_model_t* m, int stage) {
   return m->dtype == EE_BF16 && m->fused_head && hc_supported(sp.out_c, sp.n_classes, nullptr, sp.fc_w) ? 1 : 2;
 }
 
+int ee_model_head_pools(const ee_model_t* m, int stage, int batch) {
+  if (!m || stage < 0 || stage >= (int)m->stages.size() || batch < 1 || batch > m->max_batch) return 0;
+  const StagePlan& sp = m->stages[stage];
+  if (ee_model_head_launches(m, stage) == 1 || !sp.fc_cluster || m->timing) return 0;
+  const bool bf = m->dtype == EE_BF16, part = bf && gap_partials(m, sp, batch);
+  const float* p = part ? (const float*)m : nullptr;   // only whether there are block sums matters here
+  const int hw = sp.out_h * sp.out_w, es = (int)esize(m->dtype);
+  const PoolArgs pa = bf ? pool_args<bf16>(nullptr, hw, p, sp.gap_g) : pool_args<float>(nullptr, hw, nullptr, 0);
+  return fc_pools(fc_shape(batch, sp.out_c, sp.n_classes, es, m->fc_room, m->max_batch), sp.out_c / (pa.sums ? 4 : 16 / es), pa.lanes) ? 1 : 0;
+}
+
 int ee_model_gap_partials(const ee_model_t* m, int stage, int batch) {
   if (!m || stage < 0 || stage >= (int)m->stages.size() || batch < 1 || batch > m->max_batch) return 0;
   return gap_partials(m, m->stages[stage], batch) ? m->stages[stage].gap_g : 0;
@@ -1674,7 +1707,7 @@ ee_status_t ee_model_check(ee_model_t* m, void* cuda_stream) {
     // a kernel that gave up may have left arrival counters of a split-K reduction behind
     if (m->pair_counters) EE_CUDA(cudaMemsetAsync(m->pair_counters, 0, m->pair_counter_words * sizeof(unsigned), st));
     if (m->grid_bar) EE_CUDA(cudaMemsetAsync(m->grid_bar, 0, 256, st));
-    if (m->head_done) EE_CUDA(cudaMemsetAsync(m->head_done, 0, m->stages.size() * sizeof(unsigned), st));
+    if (m->head_done) EE_CUDA(cudaMemsetAsync(m->head_done, 0, m->stages.size() * 2 * sizeof(unsigned), st));
     EE_CUDA(cudaMemsetAsync(m->err_flag, 0, sizeof(int), st));
     EE_CUDA(cudaStreamSynchronize(st));
     return EE_ERR_TIMEOUT;

@@ -172,6 +172,8 @@ gap_blocks_kernel(const T* __restrict__ x, int nb, int HW, int C, int lanes, flo
   }
 }
 
+constexpr int kFcPackedBatch = 56;   // survivors of that many samples and the number of tiles done, 56 at most, fit a 64-bit word
+
 struct DecideArgs {  // everything the exit decision needs besides the logits
   const float* shift;
   const int32_t* shift_cls;
@@ -186,6 +188,7 @@ struct DecideArgs {  // everything the exit decision needs besides the logits
   int32_t* n_surv;
   unsigned* tile_done;  // per sample tile: CTAs of the FC kernel that have written its logits; zero between launches
   unsigned* done;       // sample tiles whose exit decisions are written; zero between launches
+  unsigned long long* packed;      // cluster FC kernel, up to kFcPackedBatch samples: tiles done and survivors in one word; zero between launches
   volatile int32_t* n_surv_host;   // optional: device address of a pinned host word that receives the count (exit_scan)
   bool host_out;                   // conf or pred is host memory: they reach it before the count does
 };
@@ -319,16 +322,19 @@ __device__ __forceinline__ void exit_scan(int B, const DecideArgs& d) {
 // shared memory before the kernel waits for the pooled vectors.
 //   1. The classes are cut into 16 blocks of kb (a multiple of 8), CTA r owns 16 / CL of them.  A warp takes groups of eight
 //      classes: its weights stream through a ring of its own, [8 classes][512 bytes of channels] per slot, one TMA box
-//      each (as eight row copies a slot took 1200 clocks), requested kFcRing - 1 slots ahead; no barrier across warps.  A lane adds its 16 bytes of channels
+//      each (as eight row copies a slot took 1200 clocks), requested ring - 1 slots ahead; no barrier across warps.  A lane adds its 16 bytes of channels
 //      of every slot in ascending order, then a halving butterfly (distances 16, 8, ..., 1) forms all 8 S sums at once:
 //      the tree of a sum does not depend on S, so a logit is the same bits in any batch.
 //   2. Per (sample, block): maximum, lowest argmax and sum of exp(z - max) go into the leader CTA's shared memory.  More tiles
 //      than clusters fit side by side: no clusters, the triples go through global memory and the CTA that finishes a tile
 //      last is its leader.
 //   3. The leader adds the 16 triples in a fixed order: conf = 1 / sum_r s_r exp(m_r - m), exit = always || conf >= thr (NaN
-//      never exits).  With several tiles the leader that finishes last runs the stable scan over the batch.
+//      never exits).  With several tiles the leader that finishes last has the survivors of all of them in the word that counts
+//      the tiles (up to kFcPackedBatch samples; else it runs the stable scan over the flags in memory).
 // Waits on copies are bounded.  Launched with programmatic stream serialization.  Pooling kernel + this kernel on B200, 37 samples
-// of 28 x 28 x 512 and 1000 classes: 17.4 us with 16 classes a CTA behind block-wide barriers, 14.9 now.
+// of 28 x 28 x 512 and 1000 classes: 17.4 us with 16 classes a CTA behind block-wide barriers, 14.9 with this split.  Survivors in
+// one atomic and six slots, a chain of heads, us: 1 sample of 14 x 14 x 1024 7.6 -> 7.2, 7 samples 9.8 -> 8.6, 13 of 17 x 17 x 192
+// 7.9 -> 7.0, fp32 8 of 16 x 16 x 16 with 10 classes 7.8 -> 5.5 (6.4 of that by pooling here).
 
 __device__ __forceinline__ uint32_t hc_cluster_rank() {
   uint32_t r;
@@ -362,48 +368,99 @@ __device__ __forceinline__ void fc_fma2(double (&a)[2], float w0, float w1, floa
   a[1] = acc_fma(w1, g1, a[1]);
 }
 
-template <typename T, int S>
+// POOL (tiles of one CTA): the CTA pools its samples' feature maps itself, in place of a pooling kernel in front of it, summed as
+// gap_kernel and gap_blocks_kernel do (same bits).
+struct PoolArgs {
+  const void* x;   // [B][HW][C] feature maps, or their block sums [B][nb][C] (fp32) when `sums`
+  int HW, nb, G;   // bf16: blocks of G rows
+  int lanes;       // gap_block_lanes / gap_lanes of the map
+  int sums;
+};
+// Sums of one channel vector of one sample over the blocks (rows) grp, grp + groups, ..., for the pooling kernels' row groups.
+template <int VP, int G, typename T>
+__device__ __forceinline__ void pool_blocks(const T* p, int nb, int C, int grp, int groups, float* acc) {
+  for (int j = grp; j < nb; j += groups) {
+    const T* pb = p + (size_t)j * G * C;
+    float t[VP];
+    gap_tree<G, VP>([&](int row, float* out) {
+      Vec16<T> r;
+      r.load(pb + (size_t)row * C);
+#pragma unroll
+      for (int e = 0; e < VP; ++e) out[e] = r.v[e];
+    }, 0, 1, t);
+#pragma unroll
+    for (int e = 0; e < VP; ++e) acc[e] += t[e];
+  }
+}
+// Pools the tile's samples, `lanes` channel vectors of VP channels at a time.  put(s, c, value).
+template <int VP, typename A, typename SUM, typename PUT>
+__device__ __forceinline__ void pool_tile(int samples, int C, int lanes, A* red, SUM&& sum, PUT&& put) {
+  const int tid = threadIdx.x, groups = kFcThreads / lanes, grp = tid / lanes, lv = tid - grp * lanes;
+  const int cv = C / VP, items = samples * cv;
+  for (int i0 = 0; i0 < items; i0 += lanes) {
+    const int it = i0 + lv;
+    A acc[VP];
+#pragma unroll
+    for (int e = 0; e < VP; ++e) acc[e] = (A)0;
+    if (it < items) sum(it / cv, it % cv, grp, groups, acc);
+#pragma unroll
+    for (int e = 0; e < VP; ++e) red[(grp * lanes + lv) * VP + e] = acc[e];
+    __syncthreads();
+    if (tid < lanes * VP && i0 + tid / VP < items) {
+      const int i = i0 + tid / VP;
+      A t = (A)0;
+      for (int q = 0; q < groups; ++q) t += red[q * lanes * VP + tid];
+      put(i / cv, i % cv * VP + tid % VP, t);
+    }
+    __syncthreads();
+  }
+}
+
+template <typename T, int S, bool POOL>
 __global__ void __launch_bounds__(kFcThreads)
 fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restrict__ gap, const float* __restrict__ bfc, int B, int C, int K,
-                  float* z, float4* exchange, DecideArgs d, FcShape f, int* err_flag) {
+                  float* z, float4* exchange, DecideArgs d, FcShape f, PoolArgs pa, int* err_flag) {
   typedef typename Accum<T>::type A;                        // fp64 sums for the fp32 model
   constexpr int VEC = 16 / (int)sizeof(T), CHUNK = 32 * VEC, NV = kFcRows * S, WARPS = kFcThreads / 32;
   extern __shared__ __align__(128) uint8_t fc_smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint8_t* ring = fc_smem + (size_t)warp * kFcRing * kFcSlot;                             // this warp's slots
-  float* gs = reinterpret_cast<float*>(fc_smem + (size_t)WARPS * kFcRing * kFcSlot);      // [S][Cp] pooled vectors, see below
+  uint8_t* ring = fc_smem + (size_t)warp * f.ring * kFcSlot;                             // this warp's slots
+  float* gs = reinterpret_cast<float*>(fc_smem + (size_t)WARPS * f.ring * kFcSlot);      // [S][Cp] pooled vectors, see below
   const int my_blocks = kFcBlocks / f.CL, kc = my_blocks * f.kb;
   float* zs = gs + (size_t)S * f.Cp;                                                      // [S][kc] this CTA's logits
   float* part = zs + (size_t)S * kc;                                                      // [16][S][4] (leader): max, argmax, sum
-  const uint32_t bars = smem_u32(part + kFcBlocks * S * 4) + (uint32_t)(warp * kFcRing * 8);   // this warp's slot barriers
+  uint64_t* s_done = reinterpret_cast<uint64_t*>(part + kFcBlocks * S * 4);               // [2]: survivors, is this the last tile
+  const uint32_t bars = smem_u32(s_done + 2) + (uint32_t)(warp * f.ring * 8);             // this warp's slot barriers
+  A* cross = reinterpret_cast<A*>(s_done + 2 + WARPS * f.ring);                           // [ws][S][kc] sums of the warps that share classes
   const uint32_t rank = blockIdx.x % (unsigned)f.CL;   // also the CTA's rank in its cluster
   const int tile = (int)blockIdx.x / f.CL, tiles = (int)gridDim.x / f.CL, b0 = tile * S;
   const int k0 = (int)rank * kc;
   const int nchunk = f.Cp / CHUNK, ngroups = max(0, min(kc, K - k0) + kFcRows - 1) / kFcRows;
-  const int my_groups = warp < ngroups ? (ngroups - 1 - warp) / WARPS + 1 : 0, slots = my_groups * nchunk;
+  // warp -> group wg, wg + side, ... of classes, slots wc, wc + ws, ... of their channels
+  const int ws = f.ws, side = WARPS / ws, wg = warp / ws, wc = warp - wg * ws, my_chunks = (nchunk - 1 - wc) / ws + 1;
+  const int my_groups = wg < ngroups ? (ngroups - 1 - wg) / side + 1 : 0, slots = my_groups * my_chunks;
 
   if (f.cluster) hc_cluster_arrive();   // #1: every CTA of the cluster runs (waited for before the first remote store)
   if (lane == 0) {
-#pragma unroll
-    for (int i = 0; i < kFcRing; ++i) mbar_init(bars + 8u * i, 1);
+    for (int i = 0; i < f.ring; ++i) mbar_init(bars + 8u * i, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncwarp();
   // slot lt of this warp: classes of group lg, channels of chunk lc; classes past K and channels past C arrive as zeros
-  int lt = 0, lg = warp, lc = 0;
+  int lt = 0, lg = wg, lc = wc, ls = 0;
   auto load = [&]() {
     if (lt < slots) {
       if (lane == 0) {
-        const uint32_t bar = bars + 8u * (lt % kFcRing);
+        const uint32_t bar = bars + 8u * ls;
         mbar_expect_tx(bar, kFcSlot);
-        tma_load_2d(smem_u32(ring + (lt % kFcRing) * kFcSlot), &tmW, bar, lc * CHUNK, k0 + lg * kFcRows);
+        tma_load_2d(smem_u32(ring + ls * kFcSlot), &tmW, bar, lc * CHUNK, k0 + lg * kFcRows);
       }
-      if (++lc == nchunk) lc = 0, lg += WARPS;
+      if (++ls == f.ring) ls = 0;
+      if ((lc += ws) >= nchunk) lc = wc, lg += side;
     }
     ++lt;
   };
-#pragma unroll
-  for (int t = 0; t < kFcRing - 1; ++t) load();
+  for (int t = 0; t < f.ring - 1; ++t) load();
   // bias of the classes this lane finishes in a group (see the butterfly below): the first group's ahead of the wait
   constexpr int LEFT = NV > 32 ? NV / 32 : 1, REP = NV < 32 ? 32 / NV : 1;   // values per lane, lanes per value
   float bias[LEFT];
@@ -414,33 +471,81 @@ fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restri
       bias[j] = bfc && k < K && g < ngroups ? bfc[k] : 0.f;
     }
   };
-  load_bias(warp);
+  load_bias(wg);
   pdl_wait();
   pdl_launch_dependents();
+  const bool packed = d.packed && B <= kFcPackedBatch;
+  const int my_id = packed && tid < B && d.ids && d.ids_out ? d.ids[tid] : 0;   // of the scan, should this CTA run it
   // pooled vectors: within a chunk the float4 `e` of lane l's VEC channels sits at [e][l], so that a warp's reads are 512
   // consecutive bytes
-  for (int i = tid; i < S * (f.Cp / 4); i += kFcThreads) {
-    const int s = i / (f.Cp / 4), c4 = i - s * (f.Cp / 4), c = c4 * 4;
-    const int ch = c / CHUNK, l = (c % CHUNK) / VEC, e = (c % VEC) / 4;
-    const bool in = b0 + s < B && c < C;
-    cp_async16(gs + (size_t)s * f.Cp + ch * CHUNK + (e * 32 + l) * 4, in ? gap + (size_t)(b0 + s) * C + c : gap, in ? 16 : 0);
+  auto place = [&](int s, int c) { return s * f.Cp + c / CHUNK * CHUNK + (c % VEC / 4 * 32 + c % CHUNK / VEC) * 4; };   // of float4 c / 4
+  if constexpr (!POOL) {
+    for (int i = tid; i < S * (f.Cp / 4); i += kFcThreads) {
+      const int s = i / (f.Cp / 4), c = (i - s * (f.Cp / 4)) * 4;
+      const bool in = b0 + s < B && c < C;
+      cp_async16(gs + place(s, c), in ? gap + (size_t)(b0 + s) * C + c : gap, in ? 16 : 0);
+    }
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+  } else {
+    const int here = min(S, B - b0), pad4 = (f.Cp - C) / 4;
+    for (int i = tid; i < S * pad4; i += kFcThreads) *reinterpret_cast<float4*>(gs + place(i / pad4, C + i % pad4 * 4)) = make_float4(0.f, 0.f, 0.f, 0.f);
+    void* red = fc_smem + fc_smem_bytes(f);
+    auto put = [&](int s, int c, A total) { gs[place(s, c) + c % 4] = (float)(total / (A)pa.HW); };
+    if constexpr (sizeof(T) == 4) {
+      pool_tile<VEC>(here, C, pa.lanes, (A*)red, [&](int s, int v, int grp, int groups, A* acc) {
+        const T* p0 = (const T*)pa.x + (size_t)(b0 + s) * pa.HW * C + (size_t)v * VEC;
+        int r = grp;
+        for (; r + 7 * groups < pa.HW; r += 8 * groups) {
+          Vec16<T> t[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) t[u].load(p0 + (size_t)(r + u * groups) * C);
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) acc[e] += t[u].v[e];
+        }
+        for (; r < pa.HW; r += groups) {
+          Vec16<T> t;
+          t.load(p0 + (size_t)r * C);
+#pragma unroll
+          for (int e = 0; e < VEC; ++e) acc[e] += t.v[e];
+        }
+      }, put);
+    } else if (pa.sums) {
+      pool_tile<4>(here, C, pa.lanes, (A*)red, [&](int s, int v, int grp, int groups, A* acc) {
+        pool_blocks<4, 1>((const float*)pa.x + (size_t)(b0 + s) * pa.nb * C + (size_t)v * 4, pa.nb, C, grp, groups, acc);
+      }, put);
+    } else {
+      pool_tile<VEC>(here, C, pa.lanes, (A*)red, [&](int s, int v, int grp, int groups, A* acc) {
+        const T* p0 = (const T*)pa.x + (size_t)(b0 + s) * pa.HW * C + (size_t)v * VEC;
+        switch (pa.G) {
+          case 32: pool_blocks<VEC, 32>(p0, pa.nb, C, grp, groups, acc); break;
+          case 16: pool_blocks<VEC, 16>(p0, pa.nb, C, grp, groups, acc); break;
+          case 8: pool_blocks<VEC, 8>(p0, pa.nb, C, grp, groups, acc); break;
+          case 4: pool_blocks<VEC, 4>(p0, pa.nb, C, grp, groups, acc); break;
+          case 2: pool_blocks<VEC, 2>(p0, pa.nb, C, grp, groups, acc); break;
+          default: pool_blocks<VEC, 1>(p0, pa.nb, C, grp, groups, acc); break;
+        }
+      }, put);
+    }
   }
-  cp_async_commit();
-  cp_async_wait<0>();
-  __syncthreads();
 
   A acc[kFcRows][S][2];   // even and odd channels
 #pragma unroll
   for (int q = 0; q < kFcRows; ++q)
 #pragma unroll
     for (int s = 0; s < S; ++s) acc[q][s][0] = acc[q][s][1] = (A)0;
-  int ch = 0, grp = warp;
+  int ch = wc, grp = wg, cs = 0;
+  uint32_t cp = 0;
   bool ok = true;
   for (int t = 0; t < slots; ++t) {
     __syncwarp();           // every lane is done with the slot refilled next
     if (ok) load();
-    ok = ok && mbar_wait(bars + 8u * (t % kFcRing), (uint32_t)(t / kFcRing) & 1u, err_flag);
-    const uint8_t* slot = ring + (t % kFcRing) * kFcSlot + lane * 16;
+    ok = ok && mbar_wait(bars + 8u * cs, cp, err_flag);
+    const uint8_t* slot = ring + cs * kFcSlot + lane * 16;
+    if (++cs == f.ring) cs = 0, cp ^= 1u;
     if (ok) {
       float gv[S][VEC];
 #pragma unroll
@@ -461,7 +566,7 @@ fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restri
       }
     }
     __syncwarp();
-    if (ch == nchunk - 1) {   // the group's sums are complete: all 8 S of them in one halving butterfly
+    if ((ch += ws) >= nchunk) {   // the group's sums are complete: all 8 S of them in one halving butterfly
       A v[NV];
 #pragma unroll
       for (int q = 0; q < kFcRows; ++q)
@@ -489,14 +594,25 @@ fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restri
 #pragma unroll
       for (int j = 0; j < LEFT; ++j) {
         const int idx = (lane / REP) * LEFT + j, s = idx / kFcRows, kl = grp * kFcRows + idx % kFcRows;
-        if (lane % REP == 0) zs[s * kc + kl] = (float)(v[j] + (A)bias[j]);
+        if (lane % REP == 0) {
+          if (ws == 1) zs[s * kc + kl] = (float)(v[j] + (A)bias[j]);
+          else cross[((size_t)wc * S + s) * kc + kl] = v[j];
+        }
       }
-      grp += WARPS;
+      grp += side, ch = wc;
       load_bias(grp);
     }
-    if (++ch == nchunk) ch = 0;
   }
   __syncthreads();
+  if (ws > 1) {   // the shares of the warps that shared classes, in ascending order
+    for (int i = tid; i < S * kc; i += kFcThreads) {
+      const int s = i / kc, k = i - s * kc;
+      A sum = (A)0;
+      for (int w = 0; w < ws; ++w) sum += cross[((size_t)w * S + s) * kc + k];
+      zs[s * kc + k] = (float)(sum + (A)(bfc && k0 + k < K ? bfc[k0 + k] : 0.f));
+    }
+    __syncthreads();
+  }
 
   // ---- 2. one warp per (block, sample)
   if (f.cluster) hc_cluster_wait();   // #1
@@ -578,8 +694,44 @@ fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restri
       const float cf = 1.0f / tot;
       if (d.conf) d.conf[b] = cf;
       if (d.pred) d.pred[b] = arg == 0x7fffffff ? 0 : arg;
-      d.mask[b] = (uint8_t)((d.always_exit || cf >= d.thr) ? 1 : 0);
+      const int leaves = d.always_exit || cf >= d.thr ? 1 : 0;
+      d.mask[b] = (uint8_t)leaves;
+      part[s * 4] = __int_as_float(leaves);   // nobody reads block 0's triple of this sample again
     }
+  }
+  if (packed) {
+    // The survivors and the number of tiles done travel in one atomic: who finishes last has every decision in hand, and nothing is
+    // written, fenced and read again (2 us of a head that takes 8 to 10).
+    __syncthreads();
+    if (tid == 0) {
+      unsigned long long keep = 0;
+      for (int s = 0; s < S && b0 + s < B; ++s) keep |= (unsigned long long)(__float_as_int(part[s * 4]) ? 0 : 1) << (b0 + s);
+      unsigned long long last = 1;
+      if (tiles > 1) {
+        if (d.host_out) __threadfence();
+        const unsigned long long before = atomicAdd(d.packed, (1ull << kFcPackedBatch) + keep);
+        last = (int)(before >> kFcPackedBatch) == tiles - 1;
+        keep = (before + keep) & ((1ull << kFcPackedBatch) - 1);
+        if (last) *d.packed = 0;
+      }
+      s_done[0] = keep, s_done[1] = last;
+    }
+    __syncthreads();
+    const unsigned long long keep = s_done[0];
+    if (!s_done[1]) return;
+    if (tid < B && (keep >> tid & 1)) {
+      const int pos = __popcll(keep & ((1ull << tid) - 1));
+      d.surv_idx[pos] = tid;
+      if (d.ids && d.ids_out) d.ids_out[pos] = my_id;
+    }
+    if (tid == 0) {
+      d.n_surv[0] = __popcll(keep);
+      if (d.n_surv_host) {
+        if (d.host_out) __threadfence_system();   // conf and pred reach the host before the count does
+        *d.n_surv_host = __popcll(keep);          // B_exit goes to the scheduler: the host polls this word
+      }
+    }
+    return;
   }
   __threadfence();
   __syncthreads();
@@ -594,13 +746,14 @@ fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restri
   exit_scan<kFcThreads>(B, d);
 }
 
+// pool: null = `gap` holds the pooled vectors.
 template <typename T, int S>
-inline cudaError_t fc_cluster_launch_t(const float* gap, const CUtensorMap& wfc, const float* bfc, int B, int C, int K, float* z,
+inline cudaError_t fc_cluster_launch_t(const float* gap, const PoolArgs* pool, const CUtensorMap& wfc, const float* bfc, int B, int C, int K, float* z,
                                        float4* exchange, const DecideArgs& d, const FcShape& f, int* err_flag, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((B + S - 1) / S * f.CL));
   cfg.blockDim = dim3(kFcThreads);
-  cfg.dynamicSmemBytes = fc_smem_bytes(f);
+  cfg.dynamicSmemBytes = fc_smem_bytes(f) + (pool ? kFcPoolSmem : 0);
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -610,25 +763,29 @@ inline cudaError_t fc_cluster_launch_t(const float* gap, const CUtensorMap& wfc,
   attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = f.cluster ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, fc_cluster_kernel<T, S>, wfc, gap, bfc, B, C, K, z, exchange, d, f, err_flag);
+  return pool ? cudaLaunchKernelEx(&cfg, fc_cluster_kernel<T, S, true>, wfc, gap, bfc, B, C, K, z, exchange, d, f, *pool, err_flag)
+              : cudaLaunchKernelEx(&cfg, fc_cluster_kernel<T, S, false>, wfc, gap, bfc, B, C, K, z, exchange, d, f, PoolArgs{}, err_flag);
 }
 // d.done and d.tile_done must be zero when the kernel starts and are zero again when it ends.  exchange: 16 float4 per sample
 // of every tile, less than the batch's logits take wherever it is used (more than 512 classes).
 template <typename T>
-inline cudaError_t fc_cluster_launch(const FcShape& f, const float* gap, const CUtensorMap& wfc, const float* bfc, int B, int C, int K, float* z,
+inline cudaError_t fc_cluster_launch(const FcShape& f, const float* gap, const PoolArgs* pool, const CUtensorMap& wfc, const float* bfc, int B, int C, int K, float* z,
                                      float4* exchange, const DecideArgs& d, int* err_flag, cudaStream_t st) {
   switch (f.S) {
-    case 1: return fc_cluster_launch_t<T, 1>(gap, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, st);
-    case 2: return fc_cluster_launch_t<T, 2>(gap, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, st);
-    case 4: return fc_cluster_launch_t<T, 4>(gap, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, st);
+    case 1: return fc_cluster_launch_t<T, 1>(gap, pool, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, st);
+    case 2: return fc_cluster_launch_t<T, 2>(gap, pool, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, st);
+    case 4: return fc_cluster_launch_t<T, 4>(gap, pool, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, st);
   }
-  if constexpr (sizeof(T) == 2) return fc_cluster_launch_t<T, 8>(gap, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, st);
+  if constexpr (sizeof(T) == 2) return fc_cluster_launch_t<T, 8>(gap, pool, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, st);
   return cudaErrorInvalidValue;
 }
 template <typename T, int S>
 inline cudaError_t fc_cluster_attr() {
-  cudaError_t e = cudaFuncSetAttribute(fc_cluster_kernel<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFcMaxSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(fc_cluster_kernel<T, S>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaError_t e = cudaSuccess;
+  for (auto kernel : {fc_cluster_kernel<T, S, false>, fc_cluster_kernel<T, S, true>}) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFcMaxSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  }
   return e;
 }
 inline cudaError_t fc_context_init() {
@@ -651,7 +808,7 @@ inline int fc_room() {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, fc_cluster_kernel<bf16, 8>, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, fc_cluster_kernel<bf16, 8, false>, &cfg) != cudaSuccess) {
     cudaGetLastError();
     return 4;
   }

@@ -343,3 +343,46 @@ def test_pooling_stem_treats_nan_as_the_two_layers_run_apart(k, cout, act):
         assert bool(conv.isnan().any()) and bool((apart == float("-inf")).any())
     assert not bool(apart.isnan().any())
     assert torch.equal(out.features_out[:B].view(torch.int16), apart.view(torch.int16))
+
+
+# the FC kernel pools by itself (one pass of its threads over a map), one pass more than that, warps that share a class's channels, and
+# 56 samples, whose survivors are one word, and 57, which scan: dtype, B, max_batch, HW, C, K
+HEAD_ROUTES = [("f32", 8, 8, 256, 64, 10), ("f32", 8, 8, 256, 68, 10), ("bf16", 5, 6, 784, 64, 33), ("bf16", 3, 6, 784, 72, 64), ("f32", 3, 6, 8, 520, 100),
+               ("f32", 6, 32, 4, 2048, 17), ("bf16", 13, 32, 5, 1032, 129), ("bf16", 56, 64, 3, 40, 1000), ("bf16", 57, 64, 3, 40, 1000), ("f32", 56, 57, 16, 16, 10),
+               ("f32", 57, 57, 16, 16, 10), ("bf16", 1, 1, 49, 16, 10)]
+
+
+POOLED = [(256, 64, 10), (784, 64, 33), (16, 16, 10), (49, 16, 10)]
+
+
+@pytest.mark.parametrize("case", HEAD_ROUTES)
+def test_head_routes_against_the_oracle_and_alone(case):
+    dtype, B, most, HW, C, K = case
+    bf16 = dtype == "bf16"
+    rng = wl._rng(B + C + K, 923)
+    fw, fb = wl._head(rng, C, K, 4.0, bf16)
+    spec = wl.Model("routes", dtype, 1, HW, C, [wl.Stage([wl.Layer(wl.OP_MAXPOOL, C, C, 3, 3, 1, 1)], K, fw, fb, 0.5, False)], most)
+    m = eb.EEModel(spec)
+    assert m.head_pools(0, B) == int((HW, C, K) in POOLED)
+    out, pin = eb.StageBuffers(m, 0), eb.StageBuffers(m, 0, pinned_decisions=True)
+    scratch, guard = util.guarded((m.exit_head_scratch_bytes(0) + 256,), torch.uint8)
+    scratch.fill_(0x5A)
+    x = wl.random_features((B, HW, C), seed=3, bf16=bf16)
+    xd = eb.to_device(dtype, x)
+    shift, cls = (np.arange(B) % 3 == 0).astype(np.float32) * 12.0, (np.arange(B) * 7 % K).astype(np.int32)
+    sd, cd = torch.as_tensor(shift, device="cuda"), torch.as_tensor(cls, device="cuda")
+    for o in (out, pin, out):      # the counters of a call are back at zero for the next
+        m.exit_head(0, xd, B, HW, o, scratch, sd, cd)
+    torch.cuda.synchronize()
+    m.check()
+    z, conf, mask = out.logits[:B].cpu().numpy(), out.conf[:B].cpu().numpy(), out.exit_mask[:B].cpu().numpy()
+    o = eo.exit_head(x, fw, fb, 0.5, False, shift, cls)
+    assert util.rel_err(z, o["z"], dtype, floor=util.LOGIT_FLOOR[dtype]) <= util.TOL[dtype]
+    sure = np.abs(o["conf"] - 0.5) > util.BAND
+    assert np.array_equal(mask[sure], o["exit"][sure])
+    n = int(out.n_surv_dev[0])
+    assert np.array_equal(out.survivor_idx[:n].cpu().numpy(), np.nonzero(mask == 0)[0]) and n == B - int(mask.sum())
+    assert torch.equal(pin.conf[:B], out.conf[:B].cpu()) and bool(torch.all(guard == util.CANARY))
+    m.exit_head(0, xd[B - 1:].contiguous(), 1, HW, out, scratch, sd[B - 1:].contiguous(), cd[B - 1:].contiguous())
+    torch.cuda.synchronize()
+    assert np.array_equal(out.logits[0].cpu().numpy(), z[B - 1]) and float(out.conf[0]) == float(conf[B - 1])

@@ -1,25 +1,24 @@
 // Stride-2 stem convolutions on 3-channel bf16 images (7x7 of the ResNet-style backbones, 3x3 of the MobileNet-style ones), as
 // an implicit GEMM on tcgen05.mma.
 //
-// A 3-channel pixel is 6 bytes, so no TMA load can fetch operand rows, and the operand is built by threads: the row of filter
-// row rf and output pixel ox is the kw * 3 contiguous elements of image row 2 oy - pad + rf from 6 ox - 3 pad on.  These do
-// not depend on oy but through the image row, and consecutive output rows share all but two of theirs.  So the unit is a PAIR of
-// image rows (2 P - pad, 2 P - pad + 1): 128 pixels x 64 columns, built once into a ring slot and read by the up to
-// (kh + 1) / 2 output rows P, P - 1, ...; an output row costs one new pair and its MMAs.  (Built per output row, seven
-// filter rows went through shared memory for each of them and a row took 2950 clocks of an SM.)
+// A 3-channel pixel is 6 bytes, so no TMA load can fetch operand rows.  But in an image row whose pixels are padded to four channels, 8
+// bytes, the operand row of output pixel ox is the run of pixels from 2 ox - pad on, 16 bytes further for every ox: read without
+// swizzle, as groups of eight rows of 16 bytes with 128 bytes from group to group, the image row IS the operand, whose rows overlap, and
+// a filter row is one (3x3) or two (7x7) K steps at fixed offsets into it.  Nothing is built per output pixel; a row that several
+// output rows read is in shared memory once.
 //
-// One persistent CTA per SM walks a contiguous range of output rows.  Four gather warps (one thread per output pixel) read the
-// image straight from global memory, a pair ahead of the one they store; one thread issues the MMAs into four accumulators in
-// turn; eight epilogue warps, 32 channels of 32 pixels each, finish the rows.  (A second set of gather warps left each thread 96
-// registers, and with nearly all of L1 given to shared memory what spilled came back from L2.)
+// A run starts at an odd pixel, and the pixel in front of it must not enter the sum, not even times zero.  So an image row is two
+// arrays of pixel pairs: "odd", with zeros in place of the even pixel, and "both".  A K step is two pairs, the second at any distance
+// from the first (the descriptor's leading offset): taps 0 | 1 2 from "odd" and "both", taps 3 4 | 5 6 from "both".
 //
-// Columns of a pair: a filter row is a dummy column, the kw * 3 taps and zeros (24 columns at 7x7, 16 at 3x3), its second row
-// follows.  The dummy makes every run start at an even element (6 ox - 10 or 6 ox - 4).  The last filter row of an output row is the
-// first row of its last pair, whose other row must not enter the sum, not even times zero: at 7x7 its columns 16..23 are there
-// once more as columns 48..55, so that K steps 0 and 3 hold it alone.
-// What bounds it: the gather, about 1600 clocks a pair (its loads come from L2, and 26 words in two sets are what the registers
-// hold), against 530 of MMAs and 1500 of epilogue a row.  224 x 224 x 64 images with the pool 78.4 -> 66.9 us, 59 with the pool's
-// integer keys (bf16x2_max); 161 x 161 images ran on the generic gather, whose tiles read every image row seven times.
+// One persistent CTA per SM walks a contiguous range of output rows; the unit is a PAIR of image rows (2 P - pad, 2 P - pad + 1) in a ring,
+// read by the up to (kh + 1) / 2 output rows P, P - 1, ...  Four gather warps, a thread per pixel pair, fetch three words of a row
+// with cp.async, eight pairs of rows ahead, and put them into the arrays; one thread issues the MMAs into four accumulators in turn;
+// eight epilogue warps, 32 channels of 32 pixels each, finish the rows.
+// What bounds it: the epilogue with the pool behind it, about 1500 clocks a row (sixteen warps of 16 channels take as long, and at 80
+// registers spill), against 780 of MMAs and 650 of gather (1430 to 1600 when every output pixel gathered its own runs).  A stage of the
+// stem, the pool and an 8-channel 1x1 layer, gather per output pixel -> this, us: 7x7, batch 64 of 224 x 224 images 77.9 -> 74.9, batch 7
+// 30.8 -> 27.6, batch 21 of 161 x 161 41.1 -> 37.2; 3x3 without a pool, batch 32 of 224 x 224 74.3 -> 63.6.
 #pragma once
 #include <type_traits>
 
@@ -42,21 +41,22 @@ struct StemParams {
   int* err_flag;
 };
 
-constexpr int kStemThreads = 416;      // MMA warp, 4 gather warps, 8 epilogue warps
-constexpr int kStemRing = 8, kStemAccs = 4, kStemCin = 3;
+constexpr int kStemEpi = 8, kStemThreads = 32 * (5 + kStemEpi);      // MMA warp, 4 gather warps, epilogue warps
+constexpr int kStemRing = 8, kStemAccs = 4, kStemCin = 3, kStemAhead = 8;
 
 template <int KH>
 struct StemGeom {
   static constexpr int kPad = KH / 2, kPairs = (KH + 1) / 2;
-  static constexpr int kCols = KH == 7 ? 24 : 16;            // columns of a filter row
-  static constexpr int kRead = (1 + KH * kStemCin + 1) / 2;  // words that hold taps
-  static constexpr int kSteps = 2 * kCols / 16;              // K steps of a pair
+  static constexpr int kCols = KH == 7 ? 32 : 16;            // columns of a filter row
   static constexpr int kPacked = kPairs * kTcBK;             // columns of the packed weights, a K block per pair
-  static constexpr int kABytes = kTcBM * kTcBK * 2, kWBytes = 64 * kTcBK * 2;
-  static constexpr int kWOff = kStemRing * kABytes;
+  static constexpr int kLine = 136 * 16;                     // bytes of one array of an image row: two pixel pairs of padding, 128, and six
+  static constexpr int kRow = 2 * kLine;                     // "odd" and "both"
+  static constexpr int kABytes = 2 * kRow, kWBytes = 64 * kTcBK * 2;
+  static constexpr int kWOff = (kStemRing * kABytes + 1023) / 1024 * 1024;
   static constexpr int kOOff = kWOff + kPairs * kWBytes;
   static constexpr int kScaleOff = kOOff + 4 * kTcBM * 64;   // staging: two tiles of 128 pixels x 32 channels per channel half
-  static constexpr int kBarOff = kScaleOff + 2 * 64 * 4;
+  static constexpr int kRawOff = kScaleOff + 2 * 64 * 4;     // words on their way: [pair][image row][word][thread]
+  static constexpr int kBarOff = kRawOff + kStemAhead * 2 * 4 * 128 * 4;
   static constexpr int kBytes = kBarOff + 256 + 1024;
   static_assert(kBytes <= 227 * 1024, "exceeds the shared memory of an SM");
 };
@@ -87,6 +87,33 @@ __device__ __forceinline__ void stem_walk(const StemParams& p, F&& body) {
   }
 }
 
+// The pairs that the rows of stem_walk meet, in order: image n, rows 2 P - pad and 2 P - pad + 1 of it.
+template <bool POOL, int PAIRS>
+struct StemPairs {
+  const StemParams& p;
+  int r, r1, per, n, y;   // y: pooled row (POOL) or output row
+  int P, last;            // pairs of the open row still to come: P .. last
+  __device__ __forceinline__ explicit StemPairs(const StemParams& q) : p(q) {
+    const long g = p.rev ? (long)gridDim.x - 1 - blockIdx.x : (long)blockIdx.x;
+    const int all = POOL ? p.rows : p.tiles;
+    per = POOL ? p.Hp : p.Ho;
+    r = (int)(g * all / gridDim.x), r1 = (int)((g + 1) * all / gridDim.x);
+    n = r / per, y = r - n * per;
+    open(true);
+  }
+  __device__ __forceinline__ void open(bool first) {
+    const int lo = POOL ? (first ? max(2 * y - 1, 0) : 2 * y) : y, hi = POOL ? min(2 * y + 1, p.Ho - 1) : y;
+    P = first ? lo : lo + PAIRS - 1, last = hi + PAIRS - 1;
+  }
+  __device__ __forceinline__ bool more() const { return r < r1; }
+  __device__ __forceinline__ void next() {
+    if (++P <= last) return;
+    ++r;
+    if (++y == per) y = 0, ++n;
+    open(y == 0);
+  }
+};
+
 // Maximum of bf16 pairs.  NONNEG: behind a ReLU the order of the values is that of their bits, and the 16-bit integer maximum is
 // an instruction of full rate; the bf16 one took 60 clocks each here.  A pooling layer of its own drops NaN (fmaxf), so here it must
 // lose too: the keys of NONNEG are the bits plus one, by which the conversion's one NaN, 0x7FFF, becomes the least integer.
@@ -108,48 +135,121 @@ __device__ __forceinline__ uint32_t bf16x2_pooled(uint32_t m) {
   return (NONNEG ? m - kPoolKey : m) & ~nan | (0xFF80FF80u & nan);
 }
 
-// The words (elements e0 + 2 j, e0 + 2 j + 1; e0 even) of a filter row's run in one image row, in two steps: `load` only requests
-// aligned words (stem_words.h says which), `finish` makes the run's words of them.  Words outside the row are loads that do not
-// happen, so nothing looks at a word before it is stored: a mask behind each load made every pair wait for memory (5200 clocks
-// a pair).  Rows of an odd number of elements start at an odd element every other time; their words are put together from two
-// aligned ones.
-template <int NW>
+// A pixel pair (elements e0 .. e0 + 5 of an image row, e0 even) in two steps: `load` only requests aligned words (stem_words.h says
+// which) into the thread's own column of a staging buffer, `finish` makes the pair's three words of them.  Copies, not registers,
+// hold what is on its way: kStemAhead pairs of rows.  Words outside the row arrive as zeros.  Rows of an odd number of elements start at
+// an odd element every other time; their words are put together from two aligned ones.
 struct StemRun {
-  uint32_t a[NW + 1];
-  int kind;   // of StemAsk, the same for the whole warp
-  __device__ __forceinline__ void load(const StemParams& p, int n, int y, int e0, StemTaps in) {
+  static constexpr int NW = 3;
+  __device__ __forceinline__ static void load(const StemParams& p, uint32_t dst, int n, int y, int e0, StemTaps in) {
     const int row_elems = p.W * kStemCin;
     if (y < 0 || y >= p.H) in.first = in.second = 0;
     const long rb = ((long)n * p.H + y) * row_elems;
     const StemAsk ask = stem_ask(rb, row_elems, p.total, in);
-    kind = ask.kind;
-    const bf16* row = p.x + (rb + e0);
-    auto at = [&](int e, uint32_t ok) {
-      uint32_t w;
-      asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n mov.u32 %0, 0;\n @q ld.global.nc.u32 %0, [%1];\n}" : "=r"(w) : "l"(row + e), "r"(ok));
-      return w;
-    };
-    if (kind != 2) {
+    const bf16* src = p.x + (rb + e0 + ask.off);
 #pragma unroll
-      for (int j = 0; j < NW; ++j) a[j] = at(2 * j, ask.mask & 1u << j);
-      if (kind == 3) a[NW] = in.first ? (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(p.x) + (p.total - 1)) : 0u;
-    } else {
-#pragma unroll
-      for (int j = 0; j <= NW; ++j) a[j] = at(2 * j - 1, ask.mask & 1u << j);
+    for (int j = 0; j <= NW; ++j) {
+      const int bytes = stem_word_bytes(ask, in, j);
+      if (j < NW || ask.kind == 2) asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + j * 512), "l"(bytes ? src + 2 * j : p.x), "r"(bytes) : "memory");
     }
   }
-  __device__ __forceinline__ void finish(int e0, int row_elems, uint32_t in, uint32_t* w) const {
+  __device__ __forceinline__ static void finish(const StemParams& p, const uint32_t* col, int n, int y, int e0, uint32_t in, uint32_t* w) {
+    const int row_elems = p.W * kStemCin;
 #pragma unroll
-    for (int j = 0; j < NW; ++j) w[j] = a[j];
+    for (int j = 0; j < NW; ++j) w[j] = col[j * 128];
     if (!(row_elems & 1)) return;
+    const bool odd = (((long)n * p.H + y) * row_elems & 1) != 0;
+    uint32_t next = odd ? col[NW * 128] : 0u;
 #pragma unroll
-    for (int j = 0; j < NW; ++j) {
-      const bool end = e0 + 2 * j == row_elems - 1;   // the row's last element, alone in its word
-      if (kind == 2) w[j] = in >> j & 1u ? __byte_perm(a[j], a[j + 1], 0x5432) : 0u;
-      if (end) w[j] = kind == 3 ? a[NW] : w[j] & 0xffffu;
+    for (int j = NW - 1; j >= 0; --j) {
+      const uint32_t a = w[j];
+      if (odd) w[j] = in >> j & 1u ? __byte_perm(a, next, 0x5432) : 0u;
+      if (e0 + 2 * j == row_elems - 1) w[j] &= 0xffffu;   // the row's last element, alone in its word
+      next = a;
     }
   }
 };
+
+// Descriptor of an operand without swizzle: groups of eight rows of 16 bytes, 128 bytes from one to the next; a K step's second half lies `lead` bytes further.
+__device__ __forceinline__ uint64_t stem_desc(uint32_t addr, int lead) {
+  return (uint64_t)((addr & 0x3FFFF) >> 4) | (uint64_t)(lead >> 4) << 16 | (uint64_t)(128 >> 4) << 32 | (uint64_t)1 << 46;
+}
+
+// The epilogue of a thread's pixel column with the pool behind it: the running maximum over the rows of a pooled row in registers,
+// then the maximum over three columns through shared memory.  Where a pooled row goes out, the four warps of a half meet at a
+// barrier, so a warp whose wait ran out must not leave: it raises s_abort and from then on only keeps the barrier's count; the
+// others see the flag at their next pooled row and do the same.
+template <bool NONNEG, typename W, typename V>
+__device__ __forceinline__ void stem_pool_rows(const StemParams& p, uint8_t* stage, volatile int* s_abort, int r0, int r1, int half, int row, int et,
+                                               bool idle, W&& arrived, V&& values) {
+  uint4 vm[4];   // the open pooled row
+  auto most = [](uint4 m, uint4 a) {
+    return make_uint4(bf16x2_max<NONNEG>(m.x, a.x), bf16x2_max<NONNEG>(m.y, a.y), bf16x2_max<NONNEG>(m.z, a.z), bf16x2_max<NONNEG>(m.w, a.w));
+  };
+  // the two pooled pixels whose 16-byte channel group this thread finishes: columns 2 px - 1 .. 2 px + 1, a column past the row's
+  // ends replaced by the middle one
+  const int g = et & 3, ch = half * 32 + g * 8, px0 = et >> 2;
+  uint32_t at[2][3];
+  bool mine[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int px = px0 + 32 * k;
+    mine[k] = px < p.Wp && ch < p.N;
+    const int c[3] = {2 * px, max(2 * px - 1, 0), min(2 * px + 1, p.Wo - 1)};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) at[k][i] = (uint32_t)(c[i] * 64 + ((g ^ (c[i] >> 1 & 3)) << 4));
+  }
+  bf16* out = p.out + ((size_t)r0 * p.Wp + px0) * p.N + ch;
+  bool live = true;
+  int y = r0 % p.Hp, j = 0;
+  for (int t = r0; t < r1; ++t, out += (size_t)p.Wp * p.N) {
+    live = live && !__any_sync(0xffffffffu, *s_abort != 0);
+    bool fresh = t == r0 || y == 0;          // else vm holds the row above, the last one of the pooled row before
+    const int last = min(2 * y + 1, p.Ho - 1);
+    for (int c = fresh ? max(2 * y - 1, 0) : 2 * y; c <= last; ++c, ++j) {
+      if (!live) continue;
+      if (!arrived(j)) {
+        live = false;
+        *s_abort = 1;
+        continue;
+      }
+      uint4 cur[4];
+      values(j, cur);
+      if (idle) continue;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (NONNEG) cur[i].x += kPoolKey, cur[i].y += kPoolKey, cur[i].z += kPoolKey, cur[i].w += kPoolKey;
+        vm[i] = fresh ? cur[i] : most(vm[i], cur[i]);
+      }
+      fresh = false;
+      if (c == last) {
+        uint8_t* line = stage + (t & 1) * (kTcBM * 64) + row * 64;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          *reinterpret_cast<uint4*>(line + ((i ^ (row >> 1 & 3)) << 4)) = vm[i];
+          vm[i] = cur[i];                    // the last row of a pooled row is the first row of the next one
+        }
+      }
+    }
+    if (++y == p.Hp) y = 0;
+    if (idle) continue;
+    // the row of running maxima is staged; the tile is written again two pooled rows on, past the barrier of the next one
+    asm volatile("bar.sync %0, 128;" ::"r"(1 + half) : "memory");
+    if (!live) continue;
+    const uint8_t* tile = stage + (t & 1) * (kTcBM * 64);
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+      if (mine[k]) {
+        auto col = [&](int i) { return *reinterpret_cast<const uint4*>(tile + at[k][i]); };
+        uint4 m = most(most(col(0), col(1)), col(2));
+        if (NONNEG && ((m.x | m.y | m.z | m.w) & 0x80008000u) == 0)   // no NaN (and no -0) among them
+          m = make_uint4(m.x - kPoolKey, m.y - kPoolKey, m.z - kPoolKey, m.w - kPoolKey);
+        else
+          m = make_uint4(bf16x2_pooled<NONNEG>(m.x), bf16x2_pooled<NONNEG>(m.y), bf16x2_pooled<NONNEG>(m.z), bf16x2_pooled<NONNEG>(m.w));
+        *reinterpret_cast<uint4*>(out + (size_t)(32 * k) * p.N) = m;
+      }
+  }
+}
 
 // tmW: packed weights (columns, 1, Cout) with a 64 x 1 x 64 box, 128-byte swizzle.
 //
@@ -183,10 +283,16 @@ conv_stem_tcgen05_kernel(const __grid_constant__ CUtensorMap tmW, StemParams p) 
   if (threadIdx.x < 1 + 2 * kStemRing + 2 * kStemAccs) {
     const int i = threadIdx.x;
     // pair_full: lane 0 of each gather warp, after every lane's proxy fence; acc_empty: lane 0 of each epilogue warp
-    mbar_init(bar0 + 8u * i, i >= 1 && i <= kStemRing ? 4 : i > 2 * kStemRing + kStemAccs ? 8 : 1);
+    mbar_init(bar0 + 8u * i, i >= 1 && i <= kStemRing ? 4 : i > 2 * kStemRing + kStemAccs ? kStemEpi : 1);
     if (i == 0) *s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // the padding that no gather thread writes: pixel pairs -2, -1, 128 and 129 of every array
+  for (int i = threadIdx.x; i < kStemRing * 4 * 4; i += kStemThreads) {
+    const int e = i & 3;
+    *reinterpret_cast<uint4*>(gen + (i >> 2) * S::kLine + (e < 2 ? e : 128 + e) * 16) = make_uint4(0u, 0u, 0u, 0u);
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (warp == 0) {
     if (lane == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmW) : "memory");
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kStemAccs * 64) : "memory");
@@ -207,29 +313,33 @@ conv_stem_tcgen05_kernel(const __grid_constant__ CUtensorMap tmW, StemParams p) 
   if (warp == 0) {
     if (elect_one()) {
       constexpr uint32_t idesc = umma_idesc(64);
-      const uint64_t da0 = umma_desc(base), db0 = umma_desc(base + S::kWOff);
+      // K step 0 of a filter row: taps 0, 1 and 2 (the odd pixel of a pair, the next pair whole), step 1: taps 3 to 6
+      const uint64_t d0 = stem_desc(base + (KH == 7 ? 0 : 16), S::kLine + 16), d1 = stem_desc(base + S::kLine + 32, 16), db0 = umma_desc(base + S::kWOff);
       int q = 0;   // pairs the rows so far have met
+      bool acc_here = false, pair_here = false;   // asked for while the row before was being computed: a wait costs its thread 200 clocks
       if (mbar_wait(w_bar, 0, p.err_flag))
         stem_walk<POOL, PAIRS>(p, [&](int j, int, int, int fresh_pairs, int free_pairs, bool, bool, int) {
           const int b = j & (kStemAccs - 1);
           // the epilogue must have drained this accumulator
-          if (j >= kStemAccs && !mbar_wait(acc_empty(b), (uint32_t)(j / kStemAccs - 1) & 1u, p.err_flag)) return false;
+          if (j >= kStemAccs && !acc_here && !mbar_wait(acc_empty(b), (uint32_t)(j / kStemAccs - 1) & 1u, p.err_flag)) return false;
           tc_fence_after();
           q += fresh_pairs;
           const uint32_t acc = tmem_base + (uint32_t)(b * 64);
 #pragma unroll
           for (int k = 0; k < PAIRS; ++k) {
             const int pq = q - PAIRS + k, s = pq & (kStemRing - 1);
-            if (k >= PAIRS - fresh_pairs && !mbar_wait(pair_full(s), (uint32_t)(pq / kStemRing) & 1u, p.err_flag)) return false;
-            const uint64_t da = da0 + (uint64_t)(s * (S::kABytes >> 4)), db = db0 + (uint64_t)(k * (S::kWBytes >> 4));
-            if (k + 1 < PAIRS) {
+            if (k >= PAIRS - fresh_pairs && !(pair_here && k == PAIRS - fresh_pairs) && !mbar_wait(pair_full(s), (uint32_t)(pq / kStemRing) & 1u, p.err_flag)) return false;
+            const uint64_t off = (uint64_t)(s * (S::kABytes >> 4)), db = db0 + (uint64_t)(k * (S::kWBytes >> 4));
 #pragma unroll
-              for (int i = 0; i < S::kSteps; ++i) umma_bf16(acc, da + 2 * i, db + 2 * i, idesc, (uint32_t)(k != 0 || i != 0));
-            } else {   // the last filter row alone
-              umma_bf16(acc, da, db, idesc, 1u);
-              if (KH == 7) umma_bf16(acc, da + 6, db + 6, idesc, 1u);
+            for (int half = 0; half < 2; ++half) {
+              if (half == 1 && k + 1 == PAIRS) break;   // the last filter row alone
+              const uint64_t row = off + (uint64_t)(half * (S::kRow >> 4));
+              umma_bf16(acc, d0 + row, db + half * (S::kCols / 8), idesc, (uint32_t)(k != 0 || half != 0));
+              if (KH == 7) umma_bf16(acc, d1 + row, db + half * (S::kCols / 8) + 2, idesc, 1u);
             }
           }
+          pair_here = mbar_test_wait(pair_full(q & (kStemRing - 1)), (uint32_t)(q / kStemRing) & 1u);
+          acc_here = j + 1 >= kStemAccs && mbar_test_wait(acc_empty((j + 1) & (kStemAccs - 1)), (uint32_t)((j + 1) / kStemAccs - 1) & 1u);
           umma_commit(acc_full(b));
           for (int k = 0; k < free_pairs; ++k) umma_commit(pair_empty((q - PAIRS + k) & (kStemRing - 1)));
           return true;
@@ -237,61 +347,73 @@ conv_stem_tcgen05_kernel(const __grid_constant__ CUtensorMap tmW, StemParams p) 
     }
     __syncwarp();
   } else if (warp < 5) {
-    // gather warps: thread r builds row r (output pixel ox = r) of every pair
-    const int r = (int)threadIdx.x - 32;
-    const int ox = min(r, p.Wo - 1);   // rows past Wo repeat the last pixel; nobody reads them
-    const int e0 = 2 * kStemCin * ox - S::kPad * kStemCin - 1;   // image-row element of column 0 (even)
-    const StemTaps in = stem_taps(e0, p.W * kStemCin, S::kRead);
-    uint8_t* aline = gen + r * 128;
-    constexpr int NW = S::kRead, CH = S::kCols / 8;   // words, 16-byte chunks of a filter row
-    StemRun<NW> wa[2], wb[2];
-    auto load = [&](int n, int P, StemRun<NW>* r) {
-      r[0].load(p, n, 2 * P - S::kPad, e0, in);
-      r[1].load(p, n, 2 * P - S::kPad + 1, e0, in);
+    // gather warps: thread r puts pixels 2 r and 2 r + 1 of every image row into its arrays
+    const int r = (int)threadIdx.x - 32, e0 = 2 * kStemCin * r;   // image-row element of pixel 2 r
+    const StemTaps in = r < p.Wo ? stem_taps(e0, p.W * kStemCin, 3) : StemTaps{0u, 0u};   // behind the row: zeros
+    uint8_t* at = gen + (r + 2) * 16;
+    const uint32_t raw0 = base + S::kRawOff + r * 4;
+    const uint32_t* col0 = reinterpret_cast<const uint32_t*>(gen + S::kRawOff) + r;
+    // Rows of an even number of elements: every word is whole and aligned, and a pair of rows costs a thread two addresses.
+    const bool even = (p.W & 1) == 0;
+    const uint32_t size = r < p.Wo ? 4u : 0u;
+    const char* src0 = reinterpret_cast<const char*>(p.x) + (r < p.Wo ? 2 * e0 : 0);
+    const uint32_t row_bytes = (uint32_t)p.W * (2 * kStemCin);
+    auto load = [&](int q, int n, int P) {
+      const uint32_t dst = raw0 + (uint32_t)(q & (kStemAhead - 1)) * 4096u;
+      const int y = 2 * P - S::kPad;
+      if (even) {
+        const char* src = src0 + (long)(n * p.H + y) * row_bytes;
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          const bool in = (unsigned)(y + half) < (unsigned)p.H;
+          const char* at = in ? src + half * row_bytes : src0;
+#pragma unroll
+          for (int j = 0; j < 3; ++j)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + half * 2048 + j * 512), "l"(at + 4 * j), "r"(in ? size : 0u) : "memory");
+        }
+      } else {
+        StemRun::load(p, dst, n, y, e0, in);
+        StemRun::load(p, dst + 2048u, n, y + 1, e0, in);
+      }
     };
-    auto store = [&](int q, const StemRun<NW>* run) {
+    auto store = [&](int q, int n, int P) {
       const int s = q & (kStemRing - 1);
       if (q >= kStemRing && !mbar_wait(pair_empty(s), (uint32_t)(q / kStemRing - 1) & 1u, p.err_flag)) return false;
-      uint8_t* line = aline + s * S::kABytes;
-      uint32_t w[NW];
-      auto put = [&](int c, int c_src) {   // chunk c_src of the filter row (words 4 c_src .. + 3) as chunk c
-        uint32_t v[4];
+      const uint32_t* col = col0 + (q & (kStemAhead - 1)) * 1024;
+      uint8_t* row = at + s * S::kABytes;
 #pragma unroll
-        for (int e = 0; e < 4; ++e) v[e] = 4 * c_src + e < NW ? w[4 * c_src + e] : 0u;
-        if (c_src == 0) v[0] &= 0xFFFF0000u;   // dummy column | first tap
-        *reinterpret_cast<uint4*>(line + ((c ^ (r & 7)) << 4)) = make_uint4(v[0], v[1], v[2], v[3]);
-      };
+      for (int half = 0; half < 2; ++half, row += S::kRow) {
+        uint32_t w[3];
+        if (even) {
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        run[half].finish(e0, p.W * kStemCin, in.first, w);
-#pragma unroll
-        for (int c = 0; c < CH; ++c) put(half * CH + c, c);
-        if (KH == 7 && half == 0) {
-          put(6, 2);
-          put(7, 3);   // past the row: zeros
+          for (int j = 0; j < 3; ++j) w[j] = col[half * 512 + j * 128];
+        } else {
+          StemRun::finish(p, col + half * 512, n, 2 * P - S::kPad + half, e0, in.first, w);
         }
+        const uint32_t lo = __byte_perm(w[1], w[2], 0x5432), hi = w[2] >> 16;   // the odd pixel
+        *reinterpret_cast<uint4*>(row) = make_uint4(0u, 0u, lo, hi);
+        *reinterpret_cast<uint4*>(row + S::kLine) = make_uint4(w[0], w[1] & 0xffffu, lo, hi);
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the tensor core
       __syncwarp();   // one arrival per warp: 128 of them on one barrier took 1000 clocks
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(pair_full(s)) : "memory");
       return true;
     };
-    int q = 0;
+    // two walks over the same pairs, the first kStemAhead - 1 pairs in front of the second
+    StemPairs<POOL, PAIRS> ahead(p), here(p);
     bool ok = true;
-    stem_walk<POOL, PAIRS>(p, [&](int, int n, int oy, int fresh_pairs, int, bool, bool, int) {
-      for (int k = PAIRS - fresh_pairs; k < PAIRS && ok; ++k, ++q) {
-        // two sets of registers in turn: a pair's words are on their way while those of the one before are stored
-        if (q & 1) {
-          load(n, oy + k, wb);
-          ok = store(q - 1, wa);
-        } else {
-          load(n, oy + k, wa);
-          if (q) ok = store(q - 1, wb);
-        }
-      }
-      return ok;
-    });
-    if (ok && q) (q & 1) ? store(q - 1, wa) : store(q - 1, wb);
+    for (int q = 0; q < kStemAhead - 1; ++q) {
+      if (ahead.more()) load(q, ahead.n, ahead.P), ahead.next();
+      cp_async_commit();
+    }
+    for (int q = 0; ok && here.more(); ++q) {
+      if (ahead.more()) load(q + kStemAhead - 1, ahead.n, ahead.P), ahead.next();
+      cp_async_commit();
+      cp_async_wait<kStemAhead - 1>();
+      ok = store(q, here.n, here.P);
+      here.next();
+    }
+    cp_async_wait<0>();
   } else {
     // epilogue warps 5..12: TMEM lane quarter = warp % 4, 32 channels each
     const int quarter = warp & 3, half = (warp - 5) >> 2, et = (int)threadIdx.x - 160 - 128 * half;
@@ -307,99 +429,42 @@ conv_stem_tcgen05_kernel(const __grid_constant__ CUtensorMap tmW, StemParams p) 
     const float* sc = s_scale + half * 32;
     const float* bi = s_bias + half * 32;
     uint8_t* stage = gen + S::kOOff + half * (2 * kTcBM * 64);
-    uint32_t vm[16];   // POOL: running maximum over the rows of the open pooled row: this thread's pixel column, 32 channels
+    const uint32_t acc0 = tmem_base + (uint32_t)(half * 32) + ((uint32_t)(quarter * 32) << 16);
+    auto arrived = [&](int j) { return __all_sync(0xffffffffu, mbar_wait(acc_full(j & (kStemAccs - 1)), (uint32_t)(j / kStemAccs) & 1u, p.err_flag)); };
+    auto values = [&](int j, uint4* o) {   // of row j: this thread's pixel column, 32 channels
+      tc_fence_after();
+      float v[32];
+      if (!idle) tmem_ld32(acc0 + (uint32_t)((j & (kStemAccs - 1)) * 64), v);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty(j & (kStemAccs - 1))) : "memory");   // the MMA warp may refill it
+      if (!idle) epilogue32<false>(p.act, v, sc, bi, nullptr, o);
+    };
+    const long g0 = p.rev ? (long)gridDim.x - 1 - blockIdx.x : (long)blockIdx.x;
+    const int all = POOL ? p.rows : p.tiles, r0 = (int)(g0 * all / gridDim.x), r1 = (int)((g0 + 1) * all / gridDim.x);
+    uint4 cur[4];
+    if constexpr (!POOL) {
+      uint8_t* mine = stage + quarter * 2048;   // 32 pixels of 64 bytes, their 16-byte chunks XORed with the pixel
+      for (int t = r0; t < r1; ++t) {
+        if (!arrived(t - r0)) break;
+        values(t - r0, cur);
+        if (idle) continue;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) vm[i] = 0u;
-    bool live = true;
-    const bool nonneg = p.act != EE_ACT_NONE;
-    int emitted = 0;
-    // Where a pooled row goes out, the four warps of a half meet at a barrier, so a warp whose wait ran out must not
-    // leave: it raises s_abort and from then on only keeps the barrier's count; the others see the flag at their
-    // next row and do the same.
-    stem_walk<POOL, PAIRS>(p, [&](int j, int, int, int, int, bool fresh, bool emit, int t) {
-      const int b = j & (kStemAccs - 1);
-      if (POOL) live = live && !__any_sync(0xffffffffu, *s_abort != 0);
-      if (live && !__all_sync(0xffffffffu, mbar_wait(acc_full(b), (uint32_t)(j / kStemAccs) & 1u, p.err_flag))) {
-        live = false;
-        *s_abort = 1;
-      }
-      if (!POOL && !live) return false;
-      if (live) {
-        tc_fence_after();
-        float v[32];
-        if (!idle) tmem_ld32(tmem_base + (uint32_t)(b * 64 + half * 32) + ((uint32_t)(quarter * 32) << 16), v);
-        tc_fence_before();
+        for (int g = 0; g < 4; ++g) *reinterpret_cast<uint4*>(mine + lane * 64 + ((g ^ (lane >> 1 & 3)) << 4)) = cur[g];
         __syncwarp();
-        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acc_empty(b)) : "memory");   // the MMA warp may refill it
-        if (idle) return true;
-        uint32_t cur[16];   // this row's values
-        uint4 o[4];
-        epilogue32<false>(p.act, v, sc, bi, nullptr, o);
 #pragma unroll
-        for (int g = 0; g < 4; ++g) cur[4 * g] = o[g].x, cur[4 * g + 1] = o[g].y, cur[4 * g + 2] = o[g].z, cur[4 * g + 3] = o[g].w;
-        if constexpr (!POOL) {
-          uint8_t* mine = stage + quarter * 2048;   // 32 pixels of 64 bytes, their 16-byte chunks XORed with the pixel
-#pragma unroll
-          for (int g = 0; g < 4; ++g) *reinterpret_cast<uint4*>(mine + lane * 64 + ((g ^ (lane >> 1 & 3)) << 4)) = make_uint4(cur[4 * g], cur[4 * g + 1], cur[4 * g + 2], cur[4 * g + 3]);
-          __syncwarp();
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {   // eight pixels per store, four lanes with 64 bytes of each
-            const int px = k * 8 + (lane >> 2), g = lane & 3, ox = quarter * 32 + px, ch = half * 32 + g * 8;
-            const uint4 x = *reinterpret_cast<const uint4*>(mine + px * 64 + ((g ^ (px >> 1 & 3)) << 4));
-            if (ox < p.Wo && ch < p.N) *reinterpret_cast<uint4*>(p.out + ((size_t)t * p.Wo + ox) * p.N + ch) = x;
-          }
-          __syncwarp();
-        } else {
-          uint8_t* tile = stage + (emitted & 1) * (kTcBM * 64);
-          if (nonneg) {
-#pragma unroll
-            for (int e = 0; e < 16; ++e) cur[e] += kPoolKey;
-          }
-          if (fresh) {
-#pragma unroll
-            for (int e = 0; e < 16; ++e) vm[e] = cur[e];
-          } else if (nonneg) {
-#pragma unroll
-            for (int e = 0; e < 16; ++e) vm[e] = bf16x2_max<true>(vm[e], cur[e]);
-          } else {
-#pragma unroll
-            for (int e = 0; e < 16; ++e) vm[e] = bf16x2_max<false>(vm[e], cur[e]);
-          }
-          if (emit) {
-#pragma unroll
-            for (int g = 0; g < 4; ++g)
-              *reinterpret_cast<uint4*>(tile + row * 64 + ((g ^ (row >> 1 & 3)) << 4)) = make_uint4(vm[4 * g], vm[4 * g + 1], vm[4 * g + 2], vm[4 * g + 3]);
-#pragma unroll
-            for (int e = 0; e < 16; ++e) vm[e] = cur[e];   // the last row of a pooled row is the first row of the next one
-          }
+        for (int k = 0; k < 4; ++k) {   // eight pixels per store, four lanes with 64 bytes of each
+          const int px = k * 8 + (lane >> 2), g = lane & 3, ox = quarter * 32 + px, ch = half * 32 + g * 8;
+          const uint4 x = *reinterpret_cast<const uint4*>(mine + px * 64 + ((g ^ (px >> 1 & 3)) << 4));
+          if (ox < p.Wo && ch < p.N) *reinterpret_cast<uint4*>(p.out + ((size_t)t * p.Wo + ox) * p.N + ch) = x;
         }
+        __syncwarp();
       }
-      if (!POOL || !emit || idle) return true;
-      // the row of running maxima is staged; the tile is written again two pooled rows on, past the barrier of the next one
-      asm volatile("bar.sync %0, 128;" ::"r"(1 + half) : "memory");
-      const uint8_t* tile = stage + (emitted++ & 1) * (kTcBM * 64);
-      if (!live) return true;
-      auto columns = [&](auto sign) {
-        constexpr bool NONNEG = decltype(sign)::value;
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          const int idx = et + k * 128, px = idx >> 2, g = idx & 3, ch = half * 32 + g * 8;   // pooled pixel, 16-byte channel group
-          if (px < p.Wp && ch < p.N) {
-            auto at = [&](int c) { return *reinterpret_cast<const uint4*>(tile + c * 64 + ((g ^ (c >> 1 & 3)) << 4)); };
-            auto most = [](uint4 m, uint4 a) {
-              return make_uint4(bf16x2_max<NONNEG>(m.x, a.x), bf16x2_max<NONNEG>(m.y, a.y), bf16x2_max<NONNEG>(m.z, a.z), bf16x2_max<NONNEG>(m.w, a.w));
-            };
-            const int c1 = 2 * px;   // columns 2px-1 .. 2px+1, a column past the row's ends replaced by the middle one
-            const uint4 x = at(c1), l = at(max(c1 - 1, 0)), r = at(min(c1 + 1, p.Wo - 1));
-            const uint4 m = most(most(x, l), r);
-            *reinterpret_cast<uint4*>(p.out + ((size_t)t * p.Wp + px) * p.N + ch) =
-                make_uint4(bf16x2_pooled<NONNEG>(m.x), bf16x2_pooled<NONNEG>(m.y), bf16x2_pooled<NONNEG>(m.z), bf16x2_pooled<NONNEG>(m.w));
-          }
-        }
-      };
-      if (nonneg) columns(std::true_type{}); else columns(std::false_type{});
-      return true;
-    });
+    } else if (p.act != EE_ACT_NONE) {
+      stem_pool_rows<true>(p, stage, s_abort, r0, r1, half, row, et, idle, arrived, values);
+    } else {
+      stem_pool_rows<false>(p, stage, s_abort, r0, r1, half, row, et, idle, arrived, values);
+    }
   }
   tc_fence_before();
   __syncthreads();
@@ -413,20 +478,13 @@ conv_stem_tcgen05_kernel(const __grid_constant__ CUtensorMap tmW, StemParams p) 
 template <int KH>
 __global__ void pack_stem_weights_kernel(const bf16* __restrict__ w, bf16* __restrict__ out, int rows) {
   using S = StemGeom<KH>;
-  constexpr int run = KH * kStemCin;
   const long total = (long)rows * S::kPacked;
   for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
     const int k = (int)(idx % S::kPacked), pair = k / kTcBK, c = k % kTcBK;
     const long co = idx / S::kPacked;
-    int r = -1, j = 0;   // filter row and column of its run
-    if (pair + 1 < S::kPairs) {
-      if (c < 2 * S::kCols) r = 2 * pair + c / S::kCols, j = c % S::kCols;
-    } else if (c < 16) {
-      r = KH - 1, j = c;
-    } else if (KH == 7 && c >= 48 && c < 56) {
-      r = KH - 1, j = c - 32;
-    }
-    out[idx] = r >= 0 && j >= 1 && j <= run ? w[(co * KH + r) * run + j - 1] : __float2bfloat16_rn(0.f);
+    const int r = 2 * pair + c / S::kCols, tap = c % S::kCols / 4 - 1, ch = c % 4;   // four columns a pixel, the first pixel of a row a dummy
+    const bool in = c < 2 * S::kCols && r < KH && tap >= 0 && tap < KH && ch < kStemCin;
+    out[idx] = in ? w[((co * KH + r) * KH + tap) * kStemCin + ch] : __float2bfloat16_rn(0.f);
   }
 }
 

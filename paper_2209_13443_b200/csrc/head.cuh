@@ -197,9 +197,6 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc, int
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(gsrc), "r"(src_bytes)
                : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // Exit decision of samples [b_lo, b_hi), one warp per sample (warp w of nwarps takes b_lo + w, b_lo + w + nwarps, ...):
 // optional logit shift, max / lowest argmax, conf = 1 / sum exp(z - max), exit = always || conf >= thr (NaN never

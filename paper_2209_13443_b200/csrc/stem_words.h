@@ -48,5 +48,10 @@ EE_HD StemAsk stem_ask(long row_begin, int row_elems, long total, StemTaps t) {
   }
   return a;
 }
+// Bytes of word j that are read, from element e0 + off + 2 j on: 4, 2 (kind 3: the batch's last element, alone in its word) or none.
+EE_HD int stem_word_bytes(StemAsk a, StemTaps in, int j) {
+  if (a.mask >> j & 1u) return 4;
+  return a.kind == 3 && ((in.first & ~in.second) >> j & 1u) ? 2 : 0;
+}
 
 }  // namespace ee

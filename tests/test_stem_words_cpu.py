@@ -62,3 +62,46 @@ def test_requested_words_lie_in_the_batch_and_hold_the_run(tmp_path):
     subprocess.run(["g++", "-std=c++17", "-O1", "-I", os.path.join(ROOT, "paper_2209_13443_b200", "csrc"), "-o", str(exe), str(src)], check=True)
     r = subprocess.run([str(exe)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
+
+
+# a thread per pixel pair: three words from element 6 r of every image row on, and what of them is read
+PAIRS = r"""
+#include "stem_words.h"
+#include <cstdio>
+#include <initializer_list>
+int main() {
+  long halves = 0, odd = 0;
+  for (int B = 1; B <= 3; ++B)
+    for (int H : {1, 2, 3, 5})
+      for (int W = 1; W <= 256; ++W) {
+        const int Wo = (W - 1) / 2 + 1, row = W * 3;
+        const long total = (long)B * H * row;
+        for (long y = 0; y < (long)B * H; ++y)
+          for (int r = 0; r < Wo; ++r) {
+            const ee::StemTaps in = ee::stem_taps(6 * r, row, 3);
+            const ee::StemAsk a = ee::stem_ask(y * row, row, total, in);
+            bool have[10] = {};   // element 6 r - 1 + i of the row
+            for (int j = 0; j <= 3; ++j) {
+              const int n = ee::stem_word_bytes(a, in, j);
+              if (j == 3 && a.kind != 2 && n) return std::printf("a fourth word of an even row\n"), 1;
+              const long e = y * row + 6 * r + a.off + 2 * j;
+              if (n && ((e & 1) || e < 0 || e + n / 2 > total)) return std::printf("B %d H %d W %d: %d bytes at element %ld of %ld\n", B, H, W, n, e, total), 1;
+              for (int i = 0; i < n / 2; ++i) have[1 + a.off + 2 * j + i] = true;
+              halves += n == 2;
+            }
+            odd += a.kind == 2;
+            for (int i = 0; i < 6; ++i)
+              if (6 * r + i < row && !have[1 + i]) return std::printf("B %d H %d W %d: element %d of pair %d not read\n", B, H, W, i, r), 1;
+          }
+      }
+  return !(halves && odd);
+}
+"""
+
+
+def test_pixel_pairs_are_read_whole_and_inside_the_batch(tmp_path):
+    src, exe = tmp_path / "pairs.cpp", tmp_path / "pairs"
+    src.write_text(PAIRS)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", os.path.join(ROOT, "paper_2209_13443_b200", "csrc"), "-o", str(exe), str(src)], check=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout

@@ -220,7 +220,7 @@ def run_ours(args):
 
     def stage_launches(s, n):
         """Kernels one ee_stage_run launches: the layers' (a packed stem packs and multiplies chunk by chunk),
-        the head's (one cluster kernel, or pooling and FC with the exit decision in its last CTA), one gather."""
+        the head's (one cluster kernel, or pooling and FC with the exit decision in its last CTA), one kernel that closes up the survivors."""
         return sum(pl["launches"] for pl in model.plan(s, n)) + model.head_launches(s) - model.head_pools(s, n) + (0 if spec.stages[s].always_exit else 1)
 
     # end to end: the inputs of step k + 1 travel from pinned host memory on a copy stream while step k computes (two
@@ -394,7 +394,9 @@ def run_ours(args):
                 fam["head_gap"]["bytes"] += n * (info["out_h"] * info["out_w"] // gg) * info["out_c"] * 4 if gg else n * info["out_bytes_per_sample"]
                 fam["head_fc_softmax_scan"]["bytes"] += info["out_c"] * spec.stages[s].n_classes * es + n * info["out_c"] * 4
             if "gather_survivors" in fam and not spec.stages[s].always_exit:
-                fam["gather_survivors"]["bytes"] += 2 * ns * info["out_bytes_per_sample"]
+                # survivors close up in place: rows in front of the first sample that left do not move
+                moved = int((bufs[s].survivor_idx[:ns].cpu() != torch.arange(ns, dtype=torch.int32)).sum())
+                fam["gather_survivors"]["bytes"] += 2 * moved * info["out_bytes_per_sample"]
             n = ns
             feat, ids = bufs[s].features_out, bufs[s].ids_out
             if n == 0:

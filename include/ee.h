@@ -135,7 +135,9 @@ typedef struct {
  * except features_out, exit_mask, survivor_idx and n_surv_dev). */
 typedef struct {
   void* features_out;     /* [n_surv][out_h][out_w][out_c]: the survivors' stage output, compacted, order kept;
-                             this is the next stage's input */
+                             this is the next stage's input.  Its first `batch` rows are written (where the buffer is
+                             16-byte aligned and apart from the others, the last layer stores its output here and the
+                             survivors close up in place); what rows n_surv .. batch - 1 hold afterwards is undefined */
   float* conf;            /* [batch] softmax top-1 probability, input order */
   int32_t* pred;          /* [batch] argmax class (lowest index on ties), input order.  conf and pred may be pinned host
                              memory: they are then there when the count is (n_surv_host, ee_wait_count) */

@@ -107,6 +107,7 @@ struct StagePlan {
   // the column sums of every block of gap_g (32 or 16) output rows; the head then pools those block sums instead of
   // reading the feature map again (same bits: see gap_blocks_kernel).  0 = the map's height * width has no such block.
   int out_layer = 0, gap_g = 0;
+  bool out_private = false;      // nothing inside the stage reads out_layer's output (writes_features_out)
   size_t gapp_off = 0, gapp_bytes = 0;
   int n_classes = 0;
   void* fc_w = nullptr;
@@ -457,6 +458,26 @@ ee_status_t gather_launch(const void* feat, size_t bytes_per_sample, const int32
 }
 
 template <typename V>
+ee_status_t move_launch_t(void* feat, size_t bytes_per_sample, const int32_t* idx, const int32_t* n_dev, int B, cudaStream_t st) {
+  const size_t vecs = bytes_per_sample / sizeof(V);
+  EE_CUDA(launch_pdl(move_rows_kernel<V>, dim3(cdiv((long)vecs, kMoveThreads)), dim3(kMoveThreads), st, (V*)feat, vecs, idx, n_dev, B));
+  return EE_OK;
+}
+ee_status_t move_launch(void* feat, size_t bytes_per_sample, const int32_t* idx, const int32_t* n_dev, int B, cudaStream_t st) {
+  return copy_width(bytes_per_sample, feat, feat) == 16 ? move_launch_t<uint4>(feat, bytes_per_sample, idx, n_dev, B, st)
+                                                        : move_launch_t<uint16_t>(feat, bytes_per_sample, idx, n_dev, B, st);   // elements are 2 or 4 bytes
+}
+
+// The stage's last layer can write features_out itself, where the survivors then close up in place: nobody inside the stage reads that
+// layer's output, its launch takes any 16-byte aligned destination, and the buffer is not one that the stage still reads or writes.
+bool writes_features_out(const ee_model* m, const StagePlan& sp, const ee_stage_in_t* in, const char* ws, const ee_stage_out_t* out, bool mega) {
+  if (sp.always_exit || !sp.out_private || mega || ((uintptr_t)out->features_out & 15)) return false;
+  const size_t es = esize(m->dtype), ob = (size_t)in->batch * sp.out_h * sp.out_w * sp.out_c * es, ib = (size_t)in->batch * sp.in_h * sp.in_w * sp.in_c * es;
+  const char *o = (const char*)out->features_out, *f = (const char*)in->features;
+  return (o + ob <= f || f + ib <= o) && (o + ob <= ws || ws + sp.ws_bytes <= o);
+}
+
+template <typename V>
 ee_status_t append_launch_t(const void* src, void* dst, size_t bytes, const int32_t* ids_src, int32_t* ids_dst, int n_ids,
                             cudaStream_t st) {
   const size_t vecs = bytes / sizeof(V);
@@ -536,6 +557,7 @@ ee_status_t enqueue_stage(ee_model* m, StagePlan& sp, const ee_stage_in_t* in, c
   const bool mega = stage_kernel_active(m, sp, B);
   const bool par = m->branches && !m->timing && B <= kBranchMaxBatch && !mega;
   float* gpart = gap_partials(m, sp, B) ? (float*)(ws + sp.gapp_off) : nullptr;   // the last layer's epilogue pools in row blocks
+  void* const so = writes_features_out(m, sp, in, ws, out, mega) ? out->features_out : ws + sp.slot_off[sp.out_slot];   // the last layer's output
   for (size_t k = 0; k < sp.layers.size(); ++k) {
     if (mega && sp.seg_at[k] >= 0) {
       ee_status_t s = launch_segment(m, sp, sp.segments[sp.seg_at[k]], in, ws, B, st);
@@ -551,7 +573,7 @@ ee_status_t enqueue_stage(ee_model* m, StagePlan& sp, const ee_stage_in_t* in, c
       const LayerPlan& P = sp.layers[L.proj_from];
       const void* psrc = P.src_slot < 0 ? in->features : ws + sp.slot_off[P.src_slot];
       const void* lsrc = L.src_slot < 0 ? in->features : ws + sp.slot_off[L.src_slot];
-      ee_status_t ps = tc_launch_proj(m->tc, L.tc, P.tc, lsrc, psrc, ws + sp.slot_off[L.out_slot], B, L.scale_dev, L.bias_dev, P.scale_dev,
+      ee_status_t ps = tc_launch_proj(m->tc, L.tc, P.tc, lsrc, psrc, (int)i == sp.out_layer ? so : ws + sp.slot_off[L.out_slot], B, L.scale_dev, L.bias_dev, P.scale_dev,
                                       P.bias_dev, m->err_flag, st, (int)i == sp.out_layer ? gpart : nullptr, sp.gap_g);
       if (ps != EE_OK) return ps;
       record(m, sp, st, kKernelNames[L.kind]);
@@ -559,7 +581,7 @@ ee_status_t enqueue_stage(ee_model* m, StagePlan& sp, const ee_stage_in_t* in, c
     }
     const void* src = L.src_slot < 0 ? in->features : ws + sp.slot_off[L.src_slot];
     const void* res = L.res_slot == -2 ? nullptr : (L.res_slot == -1 ? in->features : ws + sp.slot_off[L.res_slot]);
-    void* dst = ws + sp.slot_off[L.pool_next ? sp.layers[i + 1].out_slot : L.out_slot];
+    void* dst = (int)i == sp.out_layer ? so : ws + sp.slot_off[L.pool_next ? sp.layers[i + 1].out_slot : L.out_slot];
     float* partial = (float*)(ws + sp.split_off);
     cudaStream_t ls = st;
     if (par && L.side) {            // fork: everything enqueued so far (the producer of this layer's input) precedes it
@@ -575,7 +597,6 @@ ee_status_t enqueue_stage(ee_model* m, StagePlan& sp, const ee_stage_in_t* in, c
     if (par && L.side) EE_CUDA(cudaEventRecord(L.ev_done, m->branch));
     record(m, sp, st, kKernelNames[L.kind]);
   }
-  const void* so = ws + sp.slot_off[sp.out_slot];
   const int hw = sp.out_h * sp.out_w;
   ee_status_t s = m->dtype == EE_BF16
                       ? launch_head<bf16>(m, sp, so, B, hw, in->logit_shift, in->shift_class, ws + sp.head_off, in, out, st, true, host_count, gpart, sp.gap_g)
@@ -591,7 +612,9 @@ ee_status_t enqueue_stage(ee_model* m, StagePlan& sp, const ee_stage_in_t* in, c
     EE_CUDA(cudaEventRecord(m->ev_join, m->side));
   }
   if (!sp.always_exit) {
-    s = gather_launch(so, (size_t)hw * sp.out_c * esize(m->dtype), out->survivor_idx, out->n_surv_dev, B, out->features_out, sp.gather_rev, st);
+    const size_t row = (size_t)hw * sp.out_c * esize(m->dtype);
+    s = so == out->features_out ? move_launch(so, row, out->survivor_idx, out->n_surv_dev, B, st)
+                                : gather_launch(so, row, out->survivor_idx, out->n_surv_dev, B, out->features_out, sp.gather_rev, st);
     if (s != EE_OK) return s;
     record(m, sp, st, "gather_survivors");
   }
@@ -1072,6 +1095,7 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
       L.pool_next = true;
       P.fused_away = true;
     }
+    sp.out_private = n_in_use[out_layer] == 0 && n_res_use[out_layer] == 0 && !sp.layers[out_layer].fused_away;
     for (int i = 0; i < sd.n_layers; ++i) {
       LayerPlan& P = sp.layers[i];
       if (P.kind != KK_TC || P.tc.cin != P.d.cin || i == out_layer || n_in_use[i] != 0 || n_res_use[i] != 1 || P.res_slot != -2) continue;

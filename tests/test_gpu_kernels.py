@@ -345,6 +345,40 @@ def test_pooling_stem_treats_nan_as_the_two_layers_run_apart(k, cout, act):
     assert torch.equal(out.features_out[:B].view(torch.int16), apart.view(torch.int16))
 
 
+# survivors close up in place, or are gathered where features_out is not 16-byte aligned: dtype, HW, C (rows of 16-byte and 2-byte units)
+@pytest.mark.parametrize("dtype,hw,c", [("bf16", 7, 64), ("bf16", 3, 9), ("f32", 5, 12), ("f32", 3, 5)])
+@pytest.mark.parametrize("aligned", [True, False])
+def test_survivors_close_up_in_place(dtype, hw, c, aligned):
+    B = 40
+    spec = util.single_layer_model(dtype, hw, hw, c, c, 1, 1, 0, wl.ACT_RELU, False, seed=c, max_batch=B)
+    s0 = spec.stages[0]
+    s0.threshold, s0.fc_weight = 0.9, s0.fc_weight * 0.0
+    m = eb.EEModel(spec)
+    ws, out = m.workspace(), eb.StageBuffers(m, 0)
+    n_el = out.features_out.numel()
+    flat, guard = util.guarded((n_el + 8,), out.features_out.dtype)
+    off = 0 if aligned else 1
+    out.features_out = flat[off:off + n_el].view(out.features_out.shape)
+    x = eb.to_device(dtype, wl.random_features((B, hw, hw, c), seed=3, bf16=dtype == "bf16"))
+    full = torch.empty((B, hw, hw, c), dtype=x.dtype, device="cuda")
+    m.layer_run(0, 0, x, None, B, full, ws)
+    rng = np.random.default_rng(5)
+    masks = [np.zeros(B, bool), np.ones(B, bool), np.arange(B) == 0, np.arange(B) == B - 1, np.arange(B) == 17, np.arange(B) % 2 == 0,
+             np.arange(B) < 39, np.arange(B) >= 16, rng.random(B) < 0.3, rng.random(B) < 0.7]
+    for leave in masks:
+        for b in (B, 16, 1):
+            lv = leave[:b]
+            shift = torch.as_tensor(lv.astype(np.float32) * 30.0, device="cuda")
+            m.stage_run(0, x, b, out, ws, None, shift, torch.zeros(b, dtype=torch.int32, device="cuda"))
+            torch.cuda.synchronize()
+            stay = np.nonzero(~lv)[0]
+            n = int(out.n_surv_dev[0])
+            assert n == len(stay) and np.array_equal(out.survivor_idx[:n].cpu().numpy(), stay)
+            assert torch.equal(out.features_out[:n], full[torch.as_tensor(stay, device="cuda")])
+    m.check()
+    assert bool(torch.all(guard == util.CANARY))
+
+
 # the FC kernel pools by itself (one pass of its threads over a map), one pass more than that, warps that share a class's channels, and
 # 56 samples, whose survivors are one word, and 57, which scan: dtype, B, max_batch, HW, C, K
 HEAD_ROUTES = [("f32", 8, 8, 256, 64, 10), ("f32", 8, 8, 256, 68, 10), ("bf16", 5, 6, 784, 64, 33), ("bf16", 3, 6, 784, 72, 64), ("f32", 3, 6, 8, 520, 100),

@@ -298,7 +298,8 @@ typedef struct {
   double flops, bytes;
   int launches; /* kernels this layer launches at this batch size; 0: an earlier layer's launch does its work (a layer
                  * inside a multi-layer launch; a 3x3 stride-2 pad-1 max-pool read only from the 7x7 or 3x3 stride-2
-                 * 3-channel bf16 convolution right before it, which pools in its epilogue and never stores its own output) */
+                 * 3-channel bf16 convolution right before it, which pools in its epilogue and never stores its own output; a
+                 * 3x3 depthwise layer read behind a 1x1 bf16 convolution that nothing else reads, on maps of up to 34 x 34) */
 } ee_layer_plan_t;
 ee_status_t ee_model_plan(const ee_model_t* model, int stage, int batch, int cap, ee_layer_plan_t* out, int* n);
 

@@ -17,6 +17,7 @@
 #include "conv_halo.cuh"
 #include "conv_pair.cuh"
 #include "conv_dw.cuh"
+#include "conv_xdw.cuh"
 #include "head.cuh"
 
 using namespace ee;
@@ -61,6 +62,10 @@ struct LayerPlan {
   // inside ee_stage_run (the convolution's own output is then never written); ee_layer_run still runs either alone.
   bool pool_next = false;     // this layer's launch also does the pooling of the next layer
   bool fused_away = false;    // this (pooling) layer's work is done by the launch of the layer before it
+  // A 1x1 layer read only by the depthwise layer behind it runs in one launch with it (xdw_active, conv_xdw.cuh).
+  bool dw_next = false;
+  CUtensorMap tm_xdw;         // its weights in boxes of 64 filters, and its scale and bias: not grouped by pixels
+  const float *d_scale = nullptr, *d_bias = nullptr;
   // A projection shortcut (1x1, no padding, read only as the residual operand of one later layer) can be computed inside
   // that layer's launch, on the persistent kernel (see conv_tc.cuh, PROJ).
   int proj_into = -1;         // projection: the layer that can absorb it
@@ -495,6 +500,14 @@ bool proj_absorbed(const ee_model* m, const StagePlan& sp, int l, int B) {
   return plain(L) && plain(P) && L.tc.splits == 1 && P.tc.splits == 1 && tc_runs_persistent(m->tc, L.tc, B, m->proj_waves);
 }
 
+// True when layer l and the depthwise layer behind it are one launch: at every batch or at none, since the 1x1 sums of narrow layers
+// are grouped differently there (conv_xdw.cuh), so a layer with an entry in the table, and a model with multi-layer launches, run apart.
+bool xdw_active(const ee_model* m, const StagePlan& sp, int l) {
+  if (l < 0 || m->stage_kernel) return false;
+  const LayerPlan& L = sp.layers[l];
+  return L.dw_next && L.tc.splits == 1 && std::all_of(L.variant.begin(), L.variant.end(), [](uint8_t v) { return v == (uint8_t)TCV_AUTO; });
+}
+
 // True when the stage's last layer writes pooling partials at batch B: it runs on the persistent kernel.
 bool gap_partials(const ee_model* m, const StagePlan& sp, int B) {
   if (!m->gap_fusion || m->dtype != EE_BF16 || sp.gap_g == 0 || (m->stage_kernel && !m->timing && !sp.segments.empty() && B <= m->stage_kernel_max_batch))
@@ -568,6 +581,16 @@ ee_status_t enqueue_stage(ee_model* m, StagePlan& sp, const ee_stage_in_t* in, c
     const size_t i = m->timing ? k : (size_t)sp.order[k];
     const LayerPlan& L = sp.layers[i];
     if (L.fused_away) continue;   // the launch of the convolution before it pools as well
+    if (xdw_active(m, sp, (int)i - 1)) continue;
+    if (xdw_active(m, sp, (int)i)) {
+      const LayerPlan& D = sp.layers[i + 1];
+      const ConvGeom g{B, D.in_h, D.in_w, D.d.cin, D.out_h, D.out_w, D.d.cout, D.d.kh, D.d.kw, D.d.stride, D.d.pad, D.d.pad_w, D.d.act};
+      const ee_status_t xs = xdw_launch(m->tc, L.tc, L.tm_xdw, L.d.cin, L.d.act, L.d_scale, L.d_bias, g, L.tc.rev, L.src_slot < 0 ? in->features : ws + sp.slot_off[L.src_slot],
+                                        D.w_dev, D.scale_dev, D.bias_dev, (int)i + 1 == sp.out_layer ? so : ws + sp.slot_off[D.out_slot], m->err_flag, st);
+      if (xs != EE_OK) return xs;
+      record(m, sp, st, kKernelNames[L.kind]);
+      continue;
+    }
     if (L.proj_into >= 0 && !mega && proj_absorbed(m, sp, L.proj_into, B)) continue;   // computed inside the layer that adds it
     if (L.proj_from >= 0 && !mega && proj_absorbed(m, sp, (int)i, B)) {
       const LayerPlan& P = sp.layers[L.proj_from];
@@ -839,6 +862,7 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
   rc = tc_context_init(m->tc);
   if (rc == EE_OK) rc = wave_context_init();
   if (rc == EE_OK) rc = stem_context_init();
+  if (rc == EE_OK) rc = xdw_context_init();
   if (rc == EE_OK) rc = halo_context_init();
   if (rc == EE_OK) rc = pair_context_init();
   if (rc == EE_OK) rc = dw_context_init();
@@ -952,6 +976,13 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
     // a branch layer is only known to have finished (reading its input too) where its consumer joins it
     for (int i = 0; i < n; ++i)
       if (sp.layers[i].side && src_of[i] >= 0) last_pos[src_of[i]] = std::max(last_pos[src_of[i]], pos[res_user[i]]);
+    // a 1x1 layer in one launch with the depthwise layer behind it: its input is read until that one has run
+    for (int i = 0; i + 1 < n; ++i) {
+      LayerPlan &L = sp.layers[i], &D = sp.layers[i + 1];
+      L.dw_next = desc->dtype == EE_BF16 && i != out_layer && src_of[i + 1] == i && n_in_use[i] == 1 && n_res_use[i] == 0 && !L.side && !D.side &&
+                  pos[i + 1] == pos[i] + 1 && xdw_supported(L.d, D.d, L.in_h, L.in_w, m->tc.sm_count);
+      if (L.dw_next && src_of[i] >= 0) last_pos[src_of[i]] = std::max(last_pos[src_of[i]], pos[i + 1]);
+    }
     last_pos[out_layer] = n + 1;
     (void)last_use;
     // slot assignment: a slot is reused once every consumer of its tensor has run
@@ -1022,6 +1053,7 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
       if ((rc = upload_bytes(m, d.weight, wn * es, ondev, st, &L.w_dev)) != EE_OK) return fail(rc);
       if ((rc = upload<float>(m, d.scale, d.cout, ondev, st, &L.scale_dev)) != EE_OK) return fail(rc);
       if ((rc = upload<float>(m, d.bias, d.cout, ondev, st, &L.bias_dev)) != EE_OK) return fail(rc);
+      L.d_scale = L.scale_dev, L.d_bias = L.bias_dev;
       if (d.op == EE_OP_DWCONV) {
         L.kind = KK_DW;
       } else if (desc->dtype == EE_BF16 && tc_supported(d, L.in_h, L.in_w)) {
@@ -1055,6 +1087,7 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
         }
         if (rc != EE_OK) return fail(rc);
         L.tc.halo = halo_supported(d, L.in_w);
+        if (L.dw_next && (rc = xdw_weight_map(m->tc, L.w_dev, d.cin, d.cout, &L.tm_xdw)) != EE_OK) return fail(rc);
       } else if (desc->dtype == EE_BF16 && d.cout % 8 == 0 && d.kh * d.kw * d.cin <= 1024 && d.pad_w == d.pad) {
         // pixel rows are not 16-byte units (e.g. a 3-channel stem): explicit Toeplitz rows, then the tensor-core GEMM
         L.kind = KK_TC_GATHER;
@@ -1639,7 +1672,11 @@ ee_status_t ee_model_plan(const ee_model_t* m, int stage, int batch, int cap, ee
       const LayerPlan& P = sp.layers[i + 1];
       p.bytes = in_b + w_b + (double)batch * P.out_h * P.out_w * P.d.cout * es;
     }
-    if (L.fused_away) p.bytes = 0.0, p.launches = 0;   // done by the launch of the convolution before it
+    if (L.fused_away || xdw_active(m, sp, (int)i - 1)) p.bytes = 0.0, p.launches = 0;   // done by the launch of the convolution before it
+    if (xdw_active(m, sp, (int)i)) {
+      const LayerPlan& D = sp.layers[i + 1];
+      p.bytes = in_b + w_b + ((double)D.d.cout * 9 + (double)batch * D.out_h * D.out_w * D.d.cout) * es;
+    }
     if (L.proj_into >= 0 && !stage_kernel_active(m, sp, batch) && proj_absorbed(m, sp, L.proj_into, batch))
       p.bytes = in_b + w_b, p.launches = 0;            // its GEMM runs inside the layer that adds it; its output is never stored
     if (L.proj_from >= 0 && !stage_kernel_active(m, sp, batch) && proj_absorbed(m, sp, (int)i, batch)) p.bytes = in_b + out_b + w_b;

@@ -220,21 +220,23 @@ inline ee_status_t dw_context_init() {
 
 // Tensor map of a depthwise layer's input, NHWC as (C, W, H, B), box = (cb, W + 2, rows, 1), no swizzle; cached in the
 // layer like the other maps of caller buffers.
+// operand: 128-byte swizzle, boxes that are the rows of a K-major operand (conv_xdw.cuh).
 inline ee_status_t dw_input_map(const TcContext& c, const TcLayer& L, const void* ptr, int batch, int C, int H, int W, int cb, int rows,
-                                const CUtensorMap** out) {
+                                const CUtensorMap** out, bool operand = false) {
+  const int kind = operand ? 10 : 5;
   for (auto& e : L.a_maps)
-    if (e.ptr == ptr && e.batch == batch && e.kind == 5) {
+    if (e.ptr == ptr && e.batch == batch && e.kind == kind) {
       *out = &e.tm;
       return EE_OK;
     }
   TcLayer::Cached e;
-  e.ptr = ptr, e.batch = batch, e.kind = 5;
+  e.ptr = ptr, e.batch = batch, e.kind = kind;
   const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)batch};
   const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)C * 2 * W, (cuuint64_t)C * 2 * W * H};
   const cuuint32_t box[4] = {(cuuint32_t)cb, (cuuint32_t)(W + 2), (cuuint32_t)rows, 1};
   const cuuint32_t es[4] = {1, 1, 1, 1};
   if (c.encode_tiled(&e.tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                     CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+                     operand ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return EE_ERR_CUDA;
   if (L.a_maps.size() < 48) {
     L.a_maps.push_back(e);

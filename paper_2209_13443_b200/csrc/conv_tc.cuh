@@ -234,6 +234,17 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
       : "memory");
 }
 
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {   // 16 columns
+  uint32_t* r = reinterpret_cast<uint32_t*>(v);
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+
 // v[i] = scale[i] * v[i] + bias[i] over N columns (a multiple of 4).  scale and bias are 16-byte aligned rows in shared
 // memory that every lane reads at the same address: as float4 a load is one broadcast wavefront for four columns.
 template <int N>
@@ -1178,7 +1189,7 @@ struct TcLayer {
   struct Cached {
     const void* ptr;
     int batch;
-    int kind;  // 0, 9: operand A, 1, 8: output matrix, 4: halo blocks, 7: residual
+    int kind;  // 0, 9: operand A, 1, 8: output matrix, 4: halo blocks, 5, 10: framed bands (conv_dw.cuh), 7: residual
     CUtensorMap tm;
   };
   mutable std::vector<Cached> a_maps;  // tensor maps of caller buffers by (pointer, batch, kind)

@@ -420,3 +420,51 @@ def test_head_routes_against_the_oracle_and_alone(case):
     m.exit_head(0, xd[B - 1:].contiguous(), 1, HW, out, scratch, sd[B - 1:].contiguous(), cd[B - 1:].contiguous())
     torch.cuda.synchronize()
     assert np.array_equal(out.logits[0].cpu().numpy(), z[B - 1]) and float(out.conf[0]) == float(conf[B - 1])
+
+
+# 1x1 layer + depthwise layer in one launch: H, W, cin, hidden, stride, batches: one to three K blocks, channel blocks that are short, odd
+# or not a multiple of 16, bands of one row and of the whole image, one pixel, the widest row, images smaller than a tile of positions
+XDW_GEOMS = [(14, 14, 64, 384, 1, (1, 5)), (7, 7, 160, 960, 1, (1, 9)), (20, 50, 16, 96, 2, (1, 4)), (9, 13, 24, 144, 1, (1, 3)), (5, 5, 96, 576, 2, (1, 40)),
+             (1, 1, 64, 72, 1, (1, 7)), (3, 3, 40, 40, 2, (2,)), (4, 254, 40, 16, 1, (1, 2)), (13, 61, 136, 200, 2, (1, 3)), (29, 31, 192, 24, 1, (1, 3)), (34, 34, 16, 96, 2, (2, 33))]
+
+
+@pytest.mark.parametrize("geom", XDW_GEOMS)
+def test_expand_and_depthwise_in_one_launch(geom):
+    H, W, cin, hidden, stride, batches = geom
+    bmax = batches[-1]
+    rng = wl._rng(H + hidden, 927)
+    layers = [wl._conv(rng, wl.OP_CONV, cin, hidden, 1, 1, 0, wl.ACT_RELU6, bf16=True), wl._conv(rng, wl.OP_DWCONV, hidden, hidden, 3, stride, 1, wl.ACT_RELU6, bf16=True)]
+    layers[0].bias = layers[0].bias + 0.25          # outside the image the hidden map is zero, not act(bias)
+    fw, fb = wl._head(rng, hidden, 5, 1.0, True)
+    spec = wl.Model("xdw", "bf16", H, W, cin, [wl.Stage(layers, 5, fw, fb, 2.0, False)], bmax)
+    run = util.GpuRunner(spec)
+    m, out = run.m, run.bufs[0]
+    x = wl.random_features((bmax, H, W, cin), seed=4, bf16=True, relu=False)
+    xd = eb.to_device("bf16", x)
+    first = None
+    for B in batches:
+        assert [pl["launches"] for pl in m.plan(0, B)] == [1, 0]
+        m.stage_run(0, xd[:B], B, out, run.ws)
+        torch.cuda.synchronize()
+        m.check()
+        got = out.features_out[:B].clone()
+        if first is None:
+            first = got
+        assert torch.equal(got[: len(first)], first)     # alone or in a batch, other bands: the same bits
+    hid = torch.empty((bmax, H, W, hidden), dtype=torch.bfloat16, device="cuda")
+    apart = torch.empty_like(out.features_out[:bmax])
+    m.layer_run(0, 0, xd, None, bmax, hid, run.ws)
+    m.layer_run(0, 1, hid, None, bmax, apart, run.ws)
+    torch.cuda.synchronize()
+    if cin > 32:
+        assert torch.equal(got, apart)
+    o = eo.run_layers(spec, 0, x)
+    # the bar of a chain of layers: a hidden value that rounds the other way moves by 2^-8 of itself, and the outputs that sum it with it,
+    # so an element is off by a few 2^-8 of the largest, whatever its own size
+    assert np.max(np.abs(got.float().cpu().numpy() - o)) <= 2.0 ** -6 * np.max(np.abs(o))
+    m.set_layer_variant(0, 0, 1, 1, 4)      # a table entry: apart again, at every batch
+    assert [pl["launches"] for pl in m.plan(0, batches[0])] == [1, 1]
+    m.stage_run(0, xd, bmax, out, run.ws)
+    torch.cuda.synchronize()
+    assert torch.equal(out.features_out[:bmax], apart)
+    run.check_guards()

@@ -13,14 +13,16 @@
 //  - A K block goes round the ring in about 1900 clocks (its loads 1100, its MMAs and their commit, the feeding thread), so the
 //    K loop's pace is also that over the number of slots: all of shared memory is ring when the loop is long, and a small tile has
 //    more slots (16 of 12 KB at 64 x 32, 6 of 32 KB at 128 x 128).
-//  - Weights and activations have two feeding warps each: a thread takes about 140 clocks from one request to its next (three
-//    or four warps an operand gained nothing).
+//  - Weights and activations have two feeding warps each, three at 64 x 32: a thread takes 140 to 280 clocks from one request to its
+//    next, and that tile's MMAs a K block every 128 (3x3 512 -> 512, batch 1: 8.7 us with two, 7.2 with three; four gain nothing).
 //  - The MMA thread asks for the next group's barrier before it issues this one's MMAs: the answer is there when it gets to it.
+//  - Tensor memory is given back as soon as the accumulators are in registers, and every warp leaves when it is done: nobody waits for
+//    the stores (0.1 us a launch).
 //  - 32 or 64 columns per epilogue warp (four warps with 128 columns each took 2800 clocks, these take 700 or 1400).  The
 //    residual's rows come to registers while the K loop runs.
 // Bits are those of the other kernels: the same K order, one accumulator per output, one rounding.
-// In a chain of launches, 128-pixel tiles and a wait per K block -> now, us: 3x3 512 -> 512 on 7x7, batch 1 10.6 -> 7.5; 3x3 256 -> 256
-// on 14x14, batch 1 6.3 -> 4.7, batch 7 6.8 -> 5.8; 1x1 2048 -> 512, batch 1 5.8 -> 4.4; 1x1 512 -> 128 on 28x28 2.9 -> 2.5.
+// In a chain of launches, 128-pixel tiles and a wait per K block -> now, us: 3x3 512 -> 512 on 7x7, batch 1 10.6 -> 7.2; 3x3 256 -> 256
+// on 14x14, batch 1 6.3 -> 4.6, batch 7 6.8 -> 5.7; 1x1 2048 -> 512, batch 1 5.8 -> 4.3; 1x1 512 -> 128 on 28x28 2.9 -> 2.4.
 //
 // PROJ: the residual operand is a 1x1 projection computed into a second accumulator (see the persistent kernel of conv_tc.cuh).
 #pragma once
@@ -31,7 +33,7 @@ namespace ee {
 template <int BM, int BN>
 struct WaveSmem {
   static constexpr int kEpiWarps = BN == 32 ? 4 : 8;
-  static constexpr int kFeed = 2;                            // feeding warps of each operand
+  static constexpr int kFeed = BM == 64 && BN == 32 ? 3 : 2;   // feeding warps of each operand
   static constexpr int kMma = 2 * kFeed, kEpi = kMma + 1;   // warps: weights, activations, MMA, then the epilogue
   static constexpr int kThreads = 32 * (kEpi + kEpiWarps);
   static constexpr int kG = BM == 64 ? (BN == 32 ? 4 : 2) : BN == 32 ? 2 : 1;   // K blocks per full barrier
@@ -202,6 +204,9 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
       if (ok) umma_commit(accum_bar);   // everything before it has read its operands as well
     }
     __syncwarp();
+    asm volatile("bar.sync 2, %0;" ::"n"(32 * (S::kEpiWarps + 1)) : "memory");   // every epilogue warp has read its part
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kCols) : "memory");
   } else {
     const int et = threadIdx.x - 32 * S::kEpi;
     for (int i = et; i < BN; i += 32 * S::kEpiWarps) {
@@ -226,6 +231,14 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
       if (!PROJ && p.residual && m < p.M && n < p.N) r[g] = *reinterpret_cast<const uint4*>(p.residual + (size_t)m * p.N + n);
     }
     const bool ok = __all_sync(0xffffffffu, mbar_wait(accum_bar, 0, p.err_flag));
+    bool read = false;   // this warp's part of the accumulator is in registers: the MMA warp may free it, nobody waits for the stores
+    auto free_tmem = [&] {
+      if (!read) {
+        tc_fence_before();
+        asm volatile("bar.arrive 2, %0;" ::"n"(32 * (S::kEpiWarps + 1)) : "memory");
+        read = true;
+      }
+    };
     if (ok) {
       tc_fence_after();
       uint8_t* stage = gen + (warp - S::kEpi) * (S::kWarpRows * 64);   // rows of 64 bytes, their 16-byte chunks XORed with the row
@@ -245,6 +258,7 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         } else {
           tmem_ld32(acc, v);
         }
+        if (st + 1 == kSteps) free_tmem();
         if (PROJ || p.residual)
           epilogue32<true>(p.act, v, s_sb + c0, s_sb + BN + c0, r + 4 * st, o);
         else
@@ -262,12 +276,7 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         }
       }
     }
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == S::kMma) {
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kCols) : "memory");
+    free_tmem();
   }
 }
 

@@ -1533,7 +1533,7 @@ inline ee_status_t tc_launch(TcContext& c, const TcLayer& L, const void* src, co
   p.err_flag = err_flag;
   // A layer with several K ranges runs them as a cluster of CTAs per tile (more SMs pull operands: small grids) or, bit
   // for bit the same, in ONE CTA per tile with an accumulator per range (no cluster, no exchange: grids that fill the GPU
-  // anyway).  range_mode: 0 = the cluster up to 1.25 waves, 1 = cluster, 2 = one CTA.
+  // anyway).  range_mode: 0 = as measured: see `one` and `local`, 1 = cluster, 2 = one CTA.
   const long tiles_all = (long)cdiv(p.M, kTcBM) * cdiv(L.cout, L.bn);
   const bool can_local = L.splits > 1 && L.splits * L.bn <= 512 && !L.gather;
   // Measured (3x3 256->256 on 14x14, 2 and 4 ranges): the cluster wins while tiles x ranges stays within about 1.25 waves
@@ -1541,8 +1541,11 @@ inline ee_status_t tc_launch(TcContext& c, const TcLayer& L, const void* src, co
   // columns: no second CTA, no overlap with the neighbouring kernels' prologues) 1.5 to 17 us.  Ranges that the library
   // chooses never get there (tc_auto_ranges): only those a caller sets.
   const bool local = can_local && (range_mode == 2 || (range_mode == 0 && tiles_all * L.splits * 4 > 5L * c.sm_count));
-  const bool split = L.splits > 1 && !local;
-  p.ranges = local ? L.splits : 1;
+  // Grids of at most one tile per SM: the one-wave kernel, an accumulator per range, where that is the shorter one (tc_wave_ranges).
+  const WaveTile one = L.splits > 1 && range_mode == 0 && !L.gather ? tc_wave_tile(c, L, B) : WaveTile{0, 0};
+  const bool wave_ranges = one.bm && tc_wave_ranges(p.taps * p.cblocks, L.splits, one.bn);
+  const bool split = L.splits > 1 && !local && !wave_ranges;
+  p.ranges = local || wave_ranges ? L.splits : 1;
   p.kb_per = L.kb_per;
   p.rev = L.rev ? 1 : 0;
   p.gx = (const bf16*)src;
@@ -1570,7 +1573,7 @@ inline ee_status_t tc_launch(TcContext& c, const TcLayer& L, const void* src, co
       pe = res ? tc_launch_persistent<64, true>(ctas, st, tmA, L.tm_w, tmR, tmO, p) : tc_launch_persistent<64, false>(ctas, st, tmA, L.tm_w, tmR, tmO, p);
     return pe == cudaSuccess ? EE_OK : EE_ERR_CUDA;
   }
-  const WaveTile wave = split || local ? WaveTile{0, 0} : tc_wave_tile(c, L, B);
+  const WaveTile wave = wave_ranges ? one : split || local ? WaveTile{0, 0} : tc_wave_tile(c, L, B);
   if (wave.bm) {
     if (wave.bm == 64) {
       if ((s = tc_buffer_map(c, L, src, B, 9, &t)) != EE_OK) return s;

@@ -25,6 +25,7 @@
 // on 14x14, batch 1 6.3 -> 4.6, batch 7 6.8 -> 5.7; 1x1 2048 -> 512, batch 1 5.8 -> 4.3; 1x1 512 -> 128 on 28x28 2.9 -> 2.4.
 //
 // PROJ: the residual operand is a 1x1 projection computed into a second accumulator (see the persistent kernel of conv_tc.cuh).
+// RANGES: the layer's sums are cut into p.ranges ranges of K (conv_ranges.h); each has an accumulator, added in ascending order at the end.
 #pragma once
 #include "conv_tc.cuh"
 
@@ -46,7 +47,7 @@ struct WaveSmem {
   static_assert(bytes(kMaxSlots) <= 227 * 1024, "exceeds the shared memory of an SM");
 };
 
-template <int BM, int BN, bool PROJ>
+template <int BM, int BN, bool PROJ, bool RANGES>
 __global__ void __launch_bounds__(WaveSmem<BM, BN>::kThreads, 1)
 conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW,
                          const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmW2, TcParams p) {
@@ -69,7 +70,9 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = (p.rev ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x) * BM, n0 = blockIdx.y * BN;
   const int num_kb1 = p.taps * p.cblocks, num_kb = num_kb1 + (PROJ ? p.cblocks2 : 0);
-  constexpr uint32_t kCols = PROJ ? 2 * BN : BN;   // accumulators, fp32 columns
+  uint32_t cols = PROJ ? 2 * BN : BN;   // accumulators, fp32 columns
+  if (RANGES)
+    while ((int)cols < p.ranges * BN) cols *= 2;
 
   if (threadIdx.x < 2 * R + 1) {
     mbar_init(bar0 + 8u * threadIdx.x, threadIdx.x < R ? 2 * S::kG : 1);   // full: an expect_tx each of weights and activations per K block
@@ -85,7 +88,7 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
   }
   tap_table_fill(taps, p.kh, p.kw, p.stride);
   if (warp == S::kMma) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kCols) : "memory");
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
@@ -180,9 +183,17 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
       bool ok = true;
       int s = 0, i = 0;
       uint32_t ph = 0;
+      uint32_t range_acc = tmem_base;   // RANGES: accumulator of the open range
+      int in_range = 0;                 // its blocks so far
       auto block = [&](int i, int s) {
         const uint64_t off = (uint64_t)(s * (S::kSlot >> 4));
-        umma_block(tmem_base + (PROJ && i >= num_kb1 ? (uint32_t)BN : 0u), da0 + off, db0 + off, idesc, i != 0 && !(PROJ && i == num_kb1));
+        if (RANGES) {
+          if (in_range == p.kb_per) in_range = 0, range_acc += (uint32_t)BN;
+          umma_block(range_acc, da0 + off, db0 + off, idesc, in_range != 0);
+          ++in_range;
+        } else {
+          umma_block(tmem_base + (PROJ && i >= num_kb1 ? (uint32_t)BN : 0u), da0 + off, db0 + off, idesc, i != 0 && !(PROJ && i == num_kb1));
+        }
       };
       bool here = mbar_test_wait(full_bar(0), 0);
       for (; i + G <= num_kb; i += G) {
@@ -206,7 +217,7 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     __syncwarp();
     asm volatile("bar.sync 2, %0;" ::"n"(32 * (S::kEpiWarps + 1)) : "memory");   // every epilogue warp has read its part
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kCols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(cols) : "memory");
   } else {
     const int et = threadIdx.x - 32 * S::kEpi;
     for (int i = et; i < BN; i += 32 * S::kEpiWarps) {
@@ -257,6 +268,13 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
           epilogue32<false>(p.act2, w, s_sb + 2 * BN + c0, s_sb + 3 * BN + c0, nullptr, r + 4 * st);
         } else {
           tmem_ld32(acc, v);
+          if (RANGES)
+            for (int g = 1; g < p.ranges; ++g) {   // the order of the cluster's reduction
+              float w[32];
+              tmem_ld32(acc + (uint32_t)(g * BN), w);
+#pragma unroll
+              for (int e = 0; e < 32; ++e) v[e] += w[e];
+            }
         }
         if (st + 1 == kSteps) free_tmem();
         if (PROJ || p.residual)
@@ -285,21 +303,20 @@ inline ee_status_t wave_context_init() {
   auto set = [&](auto kernel, int bytes) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   };
-  auto tile = [&](auto s, auto plain, auto proj) {
+  auto tile = [&](auto s, auto... kernels) {
     typedef decltype(s) S;
-    set(plain, S::bytes(S::kMaxSlots));
-    set(proj, S::bytes(S::kMaxSlots));
+    (set(kernels, S::bytes(S::kMaxSlots)), ...);
   };
-  tile(WaveSmem<64, 32>{}, conv_wave_tcgen05_kernel<64, 32, false>, conv_wave_tcgen05_kernel<64, 32, true>);
-  tile(WaveSmem<64, 64>{}, conv_wave_tcgen05_kernel<64, 64, false>, conv_wave_tcgen05_kernel<64, 64, true>);
-  tile(WaveSmem<128, 32>{}, conv_wave_tcgen05_kernel<128, 32, false>, conv_wave_tcgen05_kernel<128, 32, true>);
-  tile(WaveSmem<128, 64>{}, conv_wave_tcgen05_kernel<128, 64, false>, conv_wave_tcgen05_kernel<128, 64, true>);
-  tile(WaveSmem<128, 128>{}, conv_wave_tcgen05_kernel<128, 128, false>, conv_wave_tcgen05_kernel<128, 128, true>);
+  tile(WaveSmem<64, 32>{}, conv_wave_tcgen05_kernel<64, 32, false, false>, conv_wave_tcgen05_kernel<64, 32, true, false>, conv_wave_tcgen05_kernel<64, 32, false, true>);
+  tile(WaveSmem<64, 64>{}, conv_wave_tcgen05_kernel<64, 64, false, false>, conv_wave_tcgen05_kernel<64, 64, true, false>, conv_wave_tcgen05_kernel<64, 64, false, true>);
+  tile(WaveSmem<128, 32>{}, conv_wave_tcgen05_kernel<128, 32, false, false>, conv_wave_tcgen05_kernel<128, 32, true, false>, conv_wave_tcgen05_kernel<128, 32, false, true>);
+  tile(WaveSmem<128, 64>{}, conv_wave_tcgen05_kernel<128, 64, false, false>, conv_wave_tcgen05_kernel<128, 64, true, false>, conv_wave_tcgen05_kernel<128, 64, false, true>);
+  tile(WaveSmem<128, 128>{}, conv_wave_tcgen05_kernel<128, 128, false, false>, conv_wave_tcgen05_kernel<128, 128, true, false>);
   return e == cudaSuccess ? EE_OK : EE_ERR_CUDA;
 }
 
 // Slots: as many as the K loop has blocks for; a short loop leaves room on its SM for the next layer's CTA to set up.
-template <int BM, int BN, bool PROJ>
+template <int BM, int BN, bool PROJ, bool RANGES = false>
 inline cudaError_t wave_launch_t(cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, const CUtensorMap& a2, const CUtensorMap& w2, TcParams p) {
   using S = WaveSmem<BM, BN>;
   p.ring = std::min(S::kMaxSlots, cdiv(std::max(S::kFeed, p.taps * p.cblocks + (PROJ ? p.cblocks2 : 0)), S::kG) * S::kG);
@@ -313,12 +330,17 @@ inline cudaError_t wave_launch_t(cudaStream_t st, const CUtensorMap& a, const CU
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, conv_wave_tcgen05_kernel<BM, BN, PROJ>, a, w, a2, w2, p);
+  return cudaLaunchKernelEx(&cfg, conv_wave_tcgen05_kernel<BM, BN, PROJ, RANGES>, a, w, a2, w2, p);
 }
 
 // a, a2: maps whose boxes have t.bm rows, w, w2: boxes of t.bn filters.
 template <bool PROJ>
 inline cudaError_t wave_launch(WaveTile t, cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, const CUtensorMap& a2, const CUtensorMap& w2, const TcParams& p) {
+  if constexpr (!PROJ)
+    if (p.ranges > 1) {
+      if (t.bm == 64) return t.bn == 32 ? wave_launch_t<64, 32, false, true>(st, a, w, a2, w2, p) : wave_launch_t<64, 64, false, true>(st, a, w, a2, w2, p);
+      return t.bn == 32 ? wave_launch_t<128, 32, false, true>(st, a, w, a2, w2, p) : wave_launch_t<128, 64, false, true>(st, a, w, a2, w2, p);
+    }
   if (t.bm == 64) return t.bn == 32 ? wave_launch_t<64, 32, PROJ>(st, a, w, a2, w2, p) : wave_launch_t<64, 64, PROJ>(st, a, w, a2, w2, p);
   return t.bn == 32   ? wave_launch_t<128, 32, PROJ>(st, a, w, a2, w2, p)
          : t.bn == 64 ? wave_launch_t<128, 64, PROJ>(st, a, w, a2, w2, p)

@@ -317,6 +317,34 @@ def test_k_ranges_chosen_for_a_layer_and_its_results(hw, bmax, ranges):
     assert np.array_equal(run.stage(0, x[:1])["features_out"][0], whole["features_out"][0])
 
 
+# K ranges on the one-wave kernel, every tile that takes them (64 x 32, 64 x 64, 128 x 32, 128 x 64): the bits of a cluster of CTAs per
+# tile; a last range that is shorter, ranges that end inside a group of K blocks, ragged filters: H, W, cin, cout, residual, ranges, batches
+WAVE_RANGE_GEOMS = [(7, 7, 512, 512, False, 4, (1, 12, 40)), (14, 14, 200, 96, True, 3, (1, 20, 30, 40)), (9, 9, 136, 64, False, 5, (1, 7)),
+                    (5, 5, 320, 72, True, 2, (1, 3, 40))]
+
+
+@pytest.mark.parametrize("geom", WAVE_RANGE_GEOMS)
+def test_k_ranges_on_the_one_wave_kernel_give_the_bits_of_the_cluster(geom):
+    H, W, cin, cout, residual, ranges, batches = geom
+    spec = util.single_layer_model("bf16", H, W, cin, cout, 3, 1, 1, wl.ACT_RELU, residual, seed=cin, max_batch=batches[-1])
+    layer = 1 if residual else 0
+    m = eb.EEModel(spec)
+    m.set_layer_splits(0, layer, ranges)
+    ws = m.workspace()
+    for B in batches:
+        xd = eb.to_device("bf16", wl.random_features((B, H, W, cin), seed=B, bf16=True, relu=False))
+        res = eb.to_device("bf16", wl.random_features((B, H, W, cout), seed=B + 1, bf16=True)) if residual else None
+        got = {}
+        for variant in (0, 3):
+            m.set_layer_variant(0, layer, 1, batches[-1], variant)
+            got[variant], guard = util.guarded((B, H, W, cout), torch.bfloat16)
+            m.layer_run(0, layer, xd, res, B, got[variant], ws)
+            torch.cuda.synchronize()
+            m.check()
+            assert bool(torch.all(guard == util.CANARY))
+        assert torch.equal(got[0], got[3])
+
+
 # NaN and infinities through the pooling stem: the pooling layer run apart drops NaN, and a window of nothing else is -inf
 @pytest.mark.parametrize("act", [wl.ACT_RELU, wl.ACT_RELU6, wl.ACT_NONE])
 @pytest.mark.parametrize("k,cout", [(7, 64), (3, 40)])

@@ -33,8 +33,8 @@ if ROOT not in sys.path:
 
 # DRAM bytes (read + written) per launch of the tensor-core conv kernels by (workload, batch), from an ncu capture of the
 # default workload (48 launches a pass).  To be taken again, or emptied, whenever one of those kernels changes.
-NCU_CONV_TRAFFIC_PER_LAUNCH = {("resnet50", 64): 32.00e6}
-NCU_CONV_TRAFFIC_WARM_L2 = {("resnet50", 64): 24.51e6}   # same capture with --cache-control none
+NCU_CONV_TRAFFIC_PER_LAUNCH = {("resnet50", 64): 31.99e6}
+NCU_CONV_TRAFFIC_WARM_L2 = {("resnet50", 64): 24.94e6}   # same capture with --cache-control none
 
 METRIC = "EE-CNN samples/sec on 1 B200 vs exit rate & batch 1-64; tensor-pipe % of peak"
 UNIT = "samples/s"

@@ -174,8 +174,9 @@ ee_status_t ee_batch_refill(ee_model_t* model, int boundary, void* batch_feat, i
                             const void* arr_feat, const int32_t* arr_ids, int n_arr, int* n_accepted,
                             int* n_merged, void* cuda_stream);
 
-/* One layer of a stage alone (the same kernel and launch configuration ee_stage_run uses for it): `input` is
- * the layer's input tensor [batch][in_h][in_w][cin], `residual` its residual operand [batch][out_h][out_w][cout]
+/* One layer of a stage alone: the kernel and launch configuration ee_stage_run uses for it, or, where ee_stage_run computes it
+ * inside another layer's launch (ee_layer_plan_t.launches == 0, or the layer before it), a launch of its own with the same bits.
+ * `input` is the layer's input tensor [batch][in_h][in_w][cin], `residual` its residual operand [batch][out_h][out_w][cout]
  * (required iff the layer has one), `output` [batch][out_h][out_w][cout]; all DEVICE, model dtype, 16-byte aligned,
  * caller-owned.  `workspace` is reserved (no layer kernel needs scratch today; pass the stage workspace or NULL).  For per-layer parity checks and
  * micro-benchmarks.  Errors: INVALID_ARG, STAGE (stage or layer out of range), CAPACITY, CUDA. */
@@ -316,7 +317,9 @@ ee_status_t ee_model_plan(const ee_model_t* model, int stage, int batch, int cap
  * The number of K ranges of a layer (`splits`) is one value per layer for all batch sizes and all variants, and the
  * partial sums of the ranges are always added in ascending order (without a setter: one range, or four for layers of about 60
  * or more K blocks of 64 whose tiles at max_batch leave SMs free), so a sample's result is bit-identical whichever
- * variant the table picks for the batch it rides in.  Both setters drop the stage's captured graphs.
+ * variant the table picks for the batch it rides in.  A 1x1 layer that shares a launch with the depthwise layer behind it
+ * (ee_layer_plan_t.launches) has one of its own, with the same bits, at every batch once it has an entry other than 0 at any
+ * batch or more than one range.  Both setters drop the stage's captured graphs.
  * ee_model_set_layer_splits may change ee_stage_info_t.workspace_bytes: query again before the next run.
  * ee_model_get_layer_config: tensor_core = -1 (not a tensor-core layer with a table), else a bit mask of the pair
  * variants the layer supports (bit 0: variant 1, bit 1: variant 2).  Errors: INVALID_ARG, STAGE, CAPACITY (batch range beyond max_batch; partial tiles of more than 256 MB),

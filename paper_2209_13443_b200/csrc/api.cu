@@ -500,8 +500,8 @@ bool proj_absorbed(const ee_model* m, const StagePlan& sp, int l, int B) {
   return plain(L) && plain(P) && L.tc.splits == 1 && P.tc.splits == 1 && tc_runs_persistent(m->tc, L.tc, B, m->proj_waves);
 }
 
-// True when layer l and the depthwise layer behind it are one launch: at every batch or at none, since the 1x1 sums of narrow layers
-// are grouped differently there (conv_xdw.cuh), so a layer with an entry in the table, and a model with multi-layer launches, run apart.
+// True when layer l and the depthwise layer behind it are one launch: at every batch or at none.  The bits are those of the two launches;
+// an entry in the table, at whatever batch, asks for the layer's own kernels, and multi-layer launches take single layers.
 bool xdw_active(const ee_model* m, const StagePlan& sp, int l) {
   if (l < 0 || m->stage_kernel) return false;
   const LayerPlan& L = sp.layers[l];
@@ -1058,7 +1058,9 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
         L.kind = KK_DW;
       } else if (desc->dtype == EE_BF16 && tc_supported(d, L.in_h, L.in_w)) {
         L.kind = KK_TC;
-        const int g = pixel_group(d, L.in_h * L.in_w);
+        // Beside the launch with the depthwise layer, whose K steps start at a pixel's first channel, so must those of the layer apart: pixels
+        // of whole K steps only are grouped there.  (24 channels on 34 x 34, 64 images: 22 to 31 of 10.7 million values rounded the other way.)
+        const int g = L.dw_next && d.cin % 16 ? 1 : pixel_group(d, L.in_h * L.in_w);
         if (g > 1) {   // narrow 1x1 layer: g pixels per row, block-diagonal weights, scale / bias repeated per pixel
           void* wp = nullptr;
           float *sp2 = nullptr, *bp2 = nullptr;

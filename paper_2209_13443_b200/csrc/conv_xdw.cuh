@@ -12,8 +12,8 @@
 // What bounds it: the eight workers, two a scheduler, which finish a band and then filter it, one after the other: about 2000
 // clocks each on a 16 x 16 frame of 64 channels, the MMAs 400.  (Fetching narrow pixels by threads in place of TMA: 40.7 -> 42.6 us on
 // 56 x 56 x 144, batch 32.)
-// Each output sums the same products in the same order as the two layers apart, with the same roundings, but where the 1x1 layer apart
-// runs on grouped pixels (conv_tc.cuh, pixel_group: up to 32 channels) and its K steps start elsewhere.
+// Each output sums the same products in the same K steps as the two layers apart, with the same roundings: the same bits.  (Beside this
+// launch a 1x1 layer groups its pixels, conv_tc.cuh, only where a pixel's channels are whole K steps.)
 #pragma once
 #include "conv_dw.cuh"
 

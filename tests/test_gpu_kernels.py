@@ -496,3 +496,42 @@ def test_expand_and_depthwise_in_one_launch(geom):
     torch.cuda.synchronize()
     assert torch.equal(out.features_out[:bmax], apart)
     run.check_guards()
+
+
+# The expand + depthwise launch against the two layers run apart, narrow inputs, whose pixels are grouped apart (cin 8 to 32): channels that
+# are whole K steps of 16 and such that are not, maps of an even and an odd number of pixels.  The depthwise layer hands its input on, so every
+# hidden value shows; enough of them that K steps starting elsewhere would round some the other way.  H, W, cin, hidden, stride, batch
+XDW_NARROW = [(28, 28, 8, 48, 1, 32), (16, 34, 16, 96, 2, 32), (34, 34, 24, 144, 1, 64), (28, 28, 24, 144, 1, 64), (33, 33, 24, 144, 2, 3), (28, 28, 32, 192, 1, 32)]
+
+
+@pytest.mark.parametrize("geom", XDW_NARROW)
+def test_expand_and_depthwise_of_narrow_layers_give_the_bits_of_the_layers_apart(geom):
+    H, W, cin, hidden, stride, B = geom
+    rng = wl._rng(W + hidden, 931)
+    layers = [wl._conv(rng, wl.OP_CONV, cin, hidden, 1, 1, 0, wl.ACT_NONE, bf16=True), wl._conv(rng, wl.OP_DWCONV, hidden, hidden, 3, stride, 1, wl.ACT_NONE, bf16=True)]
+    layers[1].weight = np.zeros_like(layers[1].weight)
+    layers[1].weight[:, 1, 1, :] = 1.0
+    layers[1].scale = layers[1].bias = None
+    fw, fb = wl._head(rng, hidden, 5, 1.0, True)
+    spec = wl.Model("xdw", "bf16", H, W, cin, [wl.Stage(layers, 5, fw, fb, 2.0, False)], B)
+    run = util.GpuRunner(spec)
+    m, out = run.m, run.bufs[0]
+    assert [pl["launches"] for pl in m.plan(0, B)] == [1, 0]
+    xd = eb.to_device("bf16", wl.random_features((B, H, W, cin), seed=6, bf16=True, relu=False))
+    m.stage_run(0, xd, B, out, run.ws)
+    torch.cuda.synchronize()
+    m.check()
+    fused = out.features_out[:B].clone()
+    hid = torch.empty((B, H, W, hidden), dtype=torch.bfloat16, device="cuda")
+    apart = torch.empty_like(fused)
+    m.layer_run(0, 0, xd, None, B, hid, run.ws)
+    m.layer_run(0, 1, hid, None, B, apart, run.ws)
+    torch.cuda.synchronize()
+    assert torch.equal(fused, apart)
+    m.set_stage_kernel(True)         # multi-layer launches take single layers
+    assert [pl["launches"] for pl in m.plan(0, B)] == [1, 1]
+    m.stage_run(0, xd, B, out, run.ws)
+    torch.cuda.synchronize()
+    m.check()
+    assert torch.equal(out.features_out[:B], fused)
+    run.check_guards()

@@ -14,7 +14,9 @@ picked variants that made the stages slower.
                       as a cluster of CTAs per tile while the grid fits one wave, else inside one CTA per tile);
   phase 2, variants:  for every measured batch size and every layer, greedily, the kernel variant (0 one-CTA tiles,
                       1 CTA pairs 256 x 256, 2 CTA pairs 256 x 128; for layers with several K ranges also 3 cluster of
-                      CTAs per tile, 4 one CTA per tile) that lowers the stage's time by more than 3 %, twice.
+                      CTAs per tile, 4 one CTA per tile) that lowers the stage's time by more than 3 %, twice.  An entry that
+                      changes what is launched at other batches too (a layer's first entry ends its shared launch with the
+                      depthwise layer behind it at every batch) has to lower the mean over all the batches it touches.
 
   python -m paper_2209_13443_b200.autotune --workload resnet50 --max-batch 64 [--out FILE]
 
@@ -112,6 +114,10 @@ def tune(spec, batches, split_batches, verbose=True):
             cfg = m.layer_config(s, i, 1)
             if cfg["tensor_core"] >= 0:
                 layers.append((s, i, cfg["tensor_core"], cfg["splits"]))
+
+    def launches(s):
+        return {b: [p["launches"] for p in m.plan(s, b)] for b in batches}
+
     side = torch.cuda.Stream()
     table = {(s, i): {"splits": d, "variants": {}} for s, i, _, d in layers}
     log = []
@@ -148,13 +154,25 @@ def tune(spec, batches, split_batches, verbose=True):
                 for i, mask in mine:
                     pick = 0
                     ranged = table[(s, i)]["splits"] > 1
+                    before = launches(s)
                     for v in VARIANTS + (RANGE_VARIANTS if ranged else ()):
                         if v in VARIANTS and not (mask >> (v - 1)) & 1:
                             continue
                         m.set_layer_variant(s, i, B, B, v)
-                        t = timer.time(s, B)
-                        if t < base * 0.97 and timer.time(s, B) < base * 0.97:     # a gain has to show twice
-                            base, pick = t, v
+                        after = launches(s)
+                        others = [b for b in batches if b != B and after[b] != before[b]]
+                        if others:       # the times of the batches touched, without this entry
+                            m.set_layer_variant(s, i, B, B, pick)
+                            base_of = {b: timer.time(s, b) for b in others}
+                            m.set_layer_variant(s, i, B, B, v)
+
+                        def gains():
+                            t = timer.time(s, B)
+                            rel = [t / base] + [timer.time(s, b) / base_of[b] for b in others]
+                            return t, sum(rel) / len(rel)
+                        t, rel = gains()
+                        if rel < 0.97 and gains()[1] < 0.97:     # a gain has to show twice
+                            base, pick, before = t, v, after
                     m.set_layer_variant(s, i, B, B, pick)
                     table[(s, i)]["variants"][B] = pick
                 log.append({"phase": "variants", "stage": s, "batch": B, "stage_us": base,

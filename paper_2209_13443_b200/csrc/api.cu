@@ -469,8 +469,11 @@ ee_status_t move_launch_t(void* feat, size_t bytes_per_sample, const int32_t* id
   return EE_OK;
 }
 ee_status_t move_launch(void* feat, size_t bytes_per_sample, const int32_t* idx, const int32_t* n_dev, int B, cudaStream_t st) {
-  return copy_width(bytes_per_sample, feat, feat) == 16 ? move_launch_t<uint4>(feat, bytes_per_sample, idx, n_dev, B, st)
-                                                        : move_launch_t<uint16_t>(feat, bytes_per_sample, idx, n_dev, B, st);   // elements are 2 or 4 bytes
+  switch (copy_width(bytes_per_sample, feat, feat)) {
+    case 16: return move_launch_t<uint4>(feat, bytes_per_sample, idx, n_dev, B, st);
+    case 4: return move_launch_t<uint32_t>(feat, bytes_per_sample, idx, n_dev, B, st);
+    default: return move_launch_t<uint16_t>(feat, bytes_per_sample, idx, n_dev, B, st);   // elements are 2 or 4 bytes
+  }
 }
 
 // The stage's last layer can write features_out itself, where the survivors then close up in place: nobody inside the stage reads that

@@ -373,8 +373,8 @@ def test_pooling_stem_treats_nan_as_the_two_layers_run_apart(k, cout, act):
     assert torch.equal(out.features_out[:B].view(torch.int16), apart.view(torch.int16))
 
 
-# survivors close up in place, or are gathered where features_out is not 16-byte aligned: dtype, HW, C (rows of 16-byte and 2-byte units)
-@pytest.mark.parametrize("dtype,hw,c", [("bf16", 7, 64), ("bf16", 3, 9), ("f32", 5, 12), ("f32", 3, 5)])
+# survivors close up in place, or are gathered where features_out is not 16-byte aligned: dtype, HW, C (rows of 16-, 2- and 4-byte units)
+@pytest.mark.parametrize("dtype,hw,c", [("bf16", 7, 64), ("bf16", 3, 9), ("f32", 5, 12), ("f32", 3, 5), ("bf16", 3, 10)])
 @pytest.mark.parametrize("aligned", [True, False])
 def test_survivors_close_up_in_place(dtype, hw, c, aligned):
     B = 40

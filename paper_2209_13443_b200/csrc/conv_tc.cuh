@@ -1349,6 +1349,14 @@ inline ee_status_t tc_buffer_map(const TcContext& c, const TcLayer& L, const voi
   return EE_OK;
 }
 
+// A copy of the map (a later lookup may grow the cache and move its entries); nothing happens behind an error in *s.  A launch asks for the
+// maps its kernel reads and for no others, each of which would take one of the 48 places from the maps of another batch.
+inline CUtensorMap tc_map_copy(const TcContext& c, const TcLayer& L, const void* ptr, int batch, int kind, ee_status_t* s) {
+  const CUtensorMap* t = nullptr;
+  if (*s == EE_OK) *s = tc_buffer_map(c, L, ptr, batch, kind, &t);
+  return t ? *t : CUtensorMap{};
+}
+
 template <int BN, int STAGES, bool RES, bool SPLIT, bool GATHER = false, bool LOCAL = false>
 inline cudaError_t tc_launch_t(dim3 grid, cudaStream_t st, const CUtensorMap& a, const CUtensorMap& w, const CUtensorMap& r,
                                const CUtensorMap& o, const TcParams& p) {
@@ -1452,16 +1460,12 @@ inline ee_status_t tc_launch_proj(TcContext& c, const TcLayer& L, const TcLayer&
                                   const float* scale, const float* bias, const float* scale2, const float* bias2, int* err_flag,
                                   cudaStream_t st, float* gap_part = nullptr, int gap_g = 0) {
   if (((uintptr_t)src & 15) || ((uintptr_t)src2 & 15) || ((uintptr_t)dst & 15)) return EE_ERR_INVALID_ARG;
-  const CUtensorMap* t = nullptr;
-  ee_status_t s = tc_buffer_map(c, L, dst, B, 8, &t);
-  if (s != EE_OK) return s;
-  const CUtensorMap tmO = *t;
   // the persistent kernel's long prologue and 128-wide epilogue are for several tiles per SM
   const WaveTile wave = gap_part ? WaveTile{0, 0} : tc_wave_tile(c, L, B);
-  if ((s = tc_buffer_map(c, L, src, B, wave.bm == 64 ? 9 : 0, &t)) != EE_OK) return s;
-  const CUtensorMap tmA = *t;
-  if ((s = tc_buffer_map(c, P, src2, B, wave.bm == 64 ? 9 : 0, &t)) != EE_OK) return s;
-  const CUtensorMap tmA2 = *t;
+  ee_status_t s = EE_OK;
+  const CUtensorMap tmA = tc_map_copy(c, L, src, B, wave.bm == 64 ? 9 : 0, &s), tmA2 = tc_map_copy(c, P, src2, B, wave.bm == 64 ? 9 : 0, &s);
+  const CUtensorMap tmO = wave.bm ? tmA : tc_map_copy(c, L, dst, B, 8, &s);
+  if (s != EE_OK) return s;
   TcParams p = {};
   p.M = B * L.out_h * L.out_w;
   p.N = L.cout;
@@ -1502,21 +1506,7 @@ inline ee_status_t tc_launch(TcContext& c, const TcLayer& L, const void* src, co
                              const float* bias, int* err_flag, cudaStream_t st, float* gap_part = nullptr, int gap_g = 0,
                              int range_mode = 0) {
   if (((uintptr_t)src & 15) || ((uintptr_t)dst & 15) || ((uintptr_t)res & 15)) return EE_ERR_INVALID_ARG;
-  // copies: a later lookup may grow the cache and move its entries
-  const CUtensorMap* t = nullptr;
-  ee_status_t s = tc_buffer_map(c, L, dst, B, 1, &t);
-  if (s != EE_OK) return s;
-  const CUtensorMap tmO = *t;
-  CUtensorMap tmA = tmO;  // unused in gather mode
-  if (!L.gather) {
-    if ((s = tc_buffer_map(c, L, src, B, 0, &t)) != EE_OK) return s;
-    tmA = *t;
-  }
-  CUtensorMap tmR = tmO;
-  if (res) {
-    if ((s = tc_buffer_map(c, L, res, B, 7, &t)) != EE_OK) return s;
-    tmR = *t;
-  }
+  ee_status_t s = EE_OK;
   TcParams p = {};
   p.gap_part = gap_part, p.gap_g = gap_part ? gap_g : 0;
   p.M = B * L.out_h * L.out_w;
@@ -1557,16 +1547,18 @@ inline ee_status_t tc_launch(TcContext& c, const TcLayer& L, const void* src, co
   const bool tma_res = res && !split;
   if (L.gather) {
     if (res || split) return EE_ERR_INTERNAL;
-    cudaError_t ge = L.bn == 128 ? tc_launch_t<128, 3, false, false, true>(grid, st, tmA, L.tm_w, tmR, tmO, p)
-                                 : tc_launch_t<64, 3, false, false, true>(grid, st, tmA, L.tm_w, tmR, tmO, p);
+    const CUtensorMap tmO = tc_map_copy(c, L, dst, B, 1, &s);
+    if (s != EE_OK) return s;
+    cudaError_t ge = L.bn == 128 ? tc_launch_t<128, 3, false, false, true>(grid, st, tmO, L.tm_w, tmO, tmO, p)
+                                 : tc_launch_t<64, 3, false, false, true>(grid, st, tmO, L.tm_w, tmO, tmO, p);
     return ge == cudaSuccess ? EE_OK : EE_ERR_CUDA;
   }
   const long tiles = (long)grid.x * grid.y;
   if (!split && L.kh * L.kw == 1 && tiles >= 2 * c.sm_count) {  // several waves of short K loops: one persistent CTA per SM walks the tiles
     const int ctas = c.sm_count;
     cudaError_t pe;
-    if ((s = tc_buffer_map(c, L, dst, B, 8, &t)) != EE_OK) return s;
-    const CUtensorMap tmO = *t;
+    const CUtensorMap tmA = tc_map_copy(c, L, src, B, 0, &s), tmO = tc_map_copy(c, L, dst, B, 8, &s), tmR = res ? tc_map_copy(c, L, res, B, 7, &s) : tmO;
+    if (s != EE_OK) return s;
     if (L.bn == 128)
       pe = res ? tc_launch_persistent<128, true>(ctas, st, tmA, L.tm_w, tmR, tmO, p) : tc_launch_persistent<128, false>(ctas, st, tmA, L.tm_w, tmR, tmO, p);
     else
@@ -1575,13 +1567,13 @@ inline ee_status_t tc_launch(TcContext& c, const TcLayer& L, const void* src, co
   }
   const WaveTile wave = wave_ranges ? one : split || local ? WaveTile{0, 0} : tc_wave_tile(c, L, B);
   if (wave.bm) {
-    if (wave.bm == 64) {
-      if ((s = tc_buffer_map(c, L, src, B, 9, &t)) != EE_OK) return s;
-      tmA = *t;
-    }
+    const CUtensorMap tmA = tc_map_copy(c, L, src, B, wave.bm == 64 ? 9 : 0, &s);
+    if (s != EE_OK) return s;
     const CUtensorMap& w = tc_weight_map(L, wave.bn);
     return wave_launch<false>(wave, st, tmA, w, tmA, w, p) == cudaSuccess ? EE_OK : EE_ERR_CUDA;
   }
+  const CUtensorMap tmA = tc_map_copy(c, L, src, B, 0, &s), tmO = split ? tmA : tc_map_copy(c, L, dst, B, 1, &s), tmR = tma_res ? tc_map_copy(c, L, res, B, 7, &s) : tmO;
+  if (s != EE_OK) return s;
   cudaError_t e = L.bn == 128 ? tc_launch_bn<128>(deep, tma_res, split, grid, st, tmA, L.tm_w, tmR, tmO, p)
                               : tc_launch_bn<64>(deep, tma_res, split, grid, st, tmA, L.tm_w, tmR, tmO, p);
   return e == cudaSuccess ? EE_OK : EE_ERR_CUDA;

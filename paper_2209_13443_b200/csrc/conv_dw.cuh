@@ -38,12 +38,72 @@ constexpr int kDwConsumers = 256;
 constexpr int kDwThreads = 32 + kDwConsumers;
 constexpr int kDwMaxTileBytes = 72 * 1024;
 
+// What a thread does with its vector of eight channels, here and in conv_xdw.cuh, whose bits have to agree.
+// Its 72 weights [8][3][3] as floats, [tap][channel]: unpacked from bf16 once, not at every product (two of three instructions of a strip
+// were such shifts and masks).  Zeros where !take.
+__device__ __forceinline__ void dw_weights(const bf16* w, bool take, float (&wf)[9][8]) {
+  uint32_t wr[36];   // as stored: element e = channel e / 9, tap e % 9
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    const uint4 v = take ? __ldg(reinterpret_cast<const uint4*>(w) + i) : make_uint4(0u, 0u, 0u, 0u);
+    wr[4 * i] = v.x, wr[4 * i + 1] = v.y, wr[4 * i + 2] = v.z, wr[4 * i + 3] = v.w;
+  }
+#pragma unroll
+  for (int e = 0; e < 72; ++e) wf[e % 9][e / 9] = (e & 1) ? __uint_as_float(wr[e >> 1] & 0xffff0000u) : __uint_as_float(wr[e >> 1] << 16);
+#pragma unroll
+  for (int e = 0; e < 72; ++e) asm volatile("" : "+f"(wf[e % 9][e / 9]));   // floats from here on: not to be unpacked again in the loop
+}
+// A strip of kDwStrip output pixels: at(r, q) is the vector of frame row r, column q; tap(r, q, s, p, f) takes its eight values as tap
+// (r, s) of output p.  Every output gets its taps in ascending (r, s).
+template <int STRIDE, typename AT, typename TAP>
+__device__ __forceinline__ void dw_strip(AT&& at, TAP&& tap) {
+  constexpr int COLS = (kDwStrip - 1) * STRIDE + 3;
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    uint4 v[COLS];
+#pragma unroll
+    for (int q = 0; q < COLS; ++q) v[q] = at(r, q);
+#pragma unroll
+    for (int q = 0; q < COLS; ++q) {
+      const uint32_t wd[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+      float f[8];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) f[2 * i] = __uint_as_float(wd[i] << 16), f[2 * i + 1] = __uint_as_float(wd[i] & 0xffff0000u);
+#pragma unroll
+      for (int p = 0; p < kDwStrip; ++p) {
+        const int s = q - p * STRIDE;   // compile-time after unrolling
+        if (s >= 0 && s < 3) tap(r, q, s, p, f);
+      }
+    }
+  }
+}
+__device__ __forceinline__ void dw_fma(float (&acc)[8], const float (&f)[8], const float (&w)[8]) {
+#pragma unroll
+  for (int e = 0; e < 8; e += 2) {   // two independent round-to-nearest FMAs per instruction
+    float a0 = f[e], a1 = f[e + 1];
+    ffma2(a0, a1, w[e], w[e + 1], acc[e], acc[e + 1]);
+    acc[e] = a0, acc[e + 1] = a1;
+  }
+}
+// Stores the strip's first `cols` pixels (all of them where more are left in the row): value(sum, e), rounded to bf16.
+template <typename VALUE>
+__device__ __forceinline__ void dw_store(bf16* y, int C, int cols, const float (&acc)[kDwStrip][8], VALUE&& value) {
+#pragma unroll
+  for (int p = 0; p < kDwStrip; ++p)
+    if (p < cols) {
+      Vec16<bf16> o;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) o.v[e] = value(acc[p][e], e);
+      o.store(y + (size_t)p * C);
+    }
+}
+
 // POOL: the same staging for a 3x3 pad-1 window maximum (the max-pool behind a ResNet-style stem): taps outside the
 // image are skipped (the frame's zeros must not win against negative inputs), no weights, no epilogue arithmetic.
 template <int STRIDE, bool POOL>
 __global__ void __launch_bounds__(kDwThreads, 1)
 dwconv3x3_tma_kernel(const __grid_constant__ CUtensorMap tmX, DwParams p) {
-  constexpr int P = kDwStrip, COLS = (P - 1) * STRIDE + 3;
+  constexpr int P = kDwStrip;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_s = smem_u32(smem_raw);
   const uint32_t base = (raw_s + 127u) & ~127u;
@@ -89,21 +149,8 @@ dwconv3x3_tma_kernel(const __grid_constant__ CUtensorMap tmX, DwParams p) {
   const bool live = item0 < item_step;      // nv need not divide 256: the threads of the ragged tail idle
   const int c = c0 + cvec * 8;
   const bool c_in = c < p.C;
-  // The vector's 72 weights as floats, [tap][channel]: unpacked from bf16 once, not at every product (two of three instructions
-  // of a strip were such shifts and masks).
   float wf[9][8];
-  {
-    uint32_t wr[36];   // as stored: element e = channel e / 9, tap e % 9
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      const uint4 v = (!POOL && c_in) ? __ldg(reinterpret_cast<const uint4*>(p.w + (size_t)c * 9) + i) : make_uint4(0u, 0u, 0u, 0u);
-      wr[4 * i] = v.x, wr[4 * i + 1] = v.y, wr[4 * i + 2] = v.z, wr[4 * i + 3] = v.w;
-    }
-#pragma unroll
-    for (int e = 0; e < 72; ++e) wf[e % 9][e / 9] = (e & 1) ? __uint_as_float(wr[e >> 1] & 0xffff0000u) : __uint_as_float(wr[e >> 1] << 16);
-#pragma unroll
-    for (int e = 0; e < 72; ++e) asm volatile("" : "+f"(wf[e % 9][e / 9]));   // floats from here on: not to be unpacked again in the loop
-  }
+  dw_weights(p.w + (size_t)c * 9, !POOL && c_in, wf);
   float sc[8], bi[8];
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
@@ -132,60 +179,24 @@ dwconv3x3_tma_kernel(const __grid_constant__ CUtensorMap tmX, DwParams p) {
         for (int pp = 0; pp < P; ++pp)
 #pragma unroll
           for (int e = 0; e < 8; ++e) acc[pp][e] = POOL ? -INFINITY : 0.f;
+        dw_strip<STRIDE>(
+            [&](int r, int q) {   // columns past the frame only feed outputs that are not stored
+              return *reinterpret_cast<const uint4*>(tile + (size_t)((ro * STRIDE + r) * Wc + min(wo0 * STRIDE + q, Wc - 1)) * p.cb * 2 + cvec * 16);
+            },
+            [&](int r, int q, int sx, int pp, const float (&f)[8]) {
+              if constexpr (POOL) {
+                const int hi = ho * STRIDE - 1 + r, wi = wo0 * STRIDE - 1 + q;
+                if (hi >= 0 && hi < p.H && wi >= 0 && wi < p.W) {
 #pragma unroll
-        for (int r = 0; r < 3; ++r) {
-          const int hi = ho * STRIDE - 1 + r;
-          const bool row_in = hi >= 0 && hi < p.H;
-          const uint8_t* row = tile + (size_t)((ro * STRIDE + r) * Wc) * p.cb * 2 + cvec * 16;
-          uint4 v[COLS];
-#pragma unroll
-          for (int q = 0; q < COLS; ++q) {
-            const int col = min(wo0 * STRIDE + q, Wc - 1);   // columns past the frame only feed outputs that are not stored
-            v[q] = *reinterpret_cast<const uint4*>(row + (size_t)col * p.cb * 2);
-          }
-#pragma unroll
-          for (int q = 0; q < COLS; ++q) {
-            const uint32_t wd[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
-            float f[8];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              f[2 * i] = __uint_as_float(wd[i] << 16);
-              f[2 * i + 1] = __uint_as_float(wd[i] & 0xffff0000u);
-            }
-#pragma unroll
-            for (int pp = 0; pp < P; ++pp) {
-              const int sx = q - pp * STRIDE;   // compile-time after unrolling
-              if (sx >= 0 && sx < 3) {
-                if constexpr (POOL) {
-                  const int wi = wo0 * STRIDE - 1 + q;
-                  if (row_in && wi >= 0 && wi < p.W) {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) acc[pp][e] = fmaxf(acc[pp][e], f[e]);
-                  }
-                } else {
-#pragma unroll
-                  for (int e = 0; e < 8; e += 2) {   // two independent round-to-nearest FMAs per instruction
-                    float a0 = f[e], a1 = f[e + 1];
-                    ffma2(a0, a1, wf[r * 3 + sx][e], wf[r * 3 + sx][e + 1], acc[pp][e], acc[pp][e + 1]);
-                    acc[pp][e] = a0, acc[pp][e + 1] = a1;
-                  }
+                  for (int e = 0; e < 8; ++e) acc[pp][e] = fmaxf(acc[pp][e], f[e]);
                 }
+              } else {
+                dw_fma(acc[pp], f, wf[r * 3 + sx]);
               }
-            }
-          }
-        }
-        if (c_in && ho < p.Ho) {
-          bf16* yp = p.y + (((size_t)b * p.Ho + ho) * p.Wo + wo0) * p.C + c;
-#pragma unroll
-          for (int pp = 0; pp < P; ++pp) {
-            if (wo0 + pp < p.Wo) {
-              Vec16<bf16> o;
-#pragma unroll
-              for (int e = 0; e < 8; ++e) o.v[e] = POOL ? acc[pp][e] : apply_act(fmaf(sc[e], acc[pp][e], bi[e]), p.act);
-              o.store(yp + (size_t)pp * p.C);
-            }
-          }
-        }
+            });
+        if (c_in && ho < p.Ho)
+          dw_store(p.y + (((size_t)b * p.Ho + ho) * p.Wo + wo0) * p.C + c, p.C, p.Wo - wo0, acc,
+                   [&](float v, int e) { return POOL ? v : apply_act(fmaf(sc[e], v, bi[e]), p.act); });
       }
     }
     __syncwarp();

@@ -59,7 +59,7 @@ inline XdwSmem xdw_smem(int cb, int kblocks, int positions, int slots) {
 template <int STRIDE>
 __global__ void __launch_bounds__(kXdwThreads, 1)
 conv_expand_dw_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW, XdwParams p, XdwSmem S) {
-  constexpr int P = kDwStrip, COLS = (P - 1) * STRIDE + 3;
+  constexpr int P = kDwStrip;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -151,19 +151,8 @@ conv_expand_dw_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __g
     const bool live = item0 < item_step;      // nv need not divide 256: the threads of the ragged tail idle
     const int c = c0 + cvec * 8;
     const bool c_in = c < p.C;
-    float wf[9][8];                           // the vector's 72 weights, [tap][channel], unpacked once
-    {
-      uint32_t wr[36];
-#pragma unroll
-      for (int i = 0; i < 9; ++i) {
-        const uint4 v = c_in ? __ldg(reinterpret_cast<const uint4*>(p.w + (size_t)c * 9) + i) : make_uint4(0u, 0u, 0u, 0u);
-        wr[4 * i] = v.x, wr[4 * i + 1] = v.y, wr[4 * i + 2] = v.z, wr[4 * i + 3] = v.w;
-      }
-#pragma unroll
-      for (int e = 0; e < 72; ++e) wf[e % 9][e / 9] = (e & 1) ? __uint_as_float(wr[e >> 1] & 0xffff0000u) : __uint_as_float(wr[e >> 1] << 16);
-#pragma unroll
-      for (int e = 0; e < 72; ++e) asm volatile("" : "+f"(wf[e % 9][e / 9]));
-    }
+    float wf[9][8];
+    dw_weights(p.w + (size_t)c * 9, c_in, wf);
     float sc[8], bi[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
@@ -215,43 +204,13 @@ conv_expand_dw_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __g
           for (int pp = 0; pp < P; ++pp)
 #pragma unroll
             for (int e = 0; e < 8; ++e) acc[pp][e] = 0.f;
-#pragma unroll
-          for (int r = 0; r < 3; ++r) {
-            const uint8_t* row = hid + (ro * STRIDE + r) * Wc * S.pitch + cvec * 16;
-            uint4 v[COLS];
-#pragma unroll
-            for (int t = 0; t < COLS; ++t) v[t] = *reinterpret_cast<const uint4*>(row + min(wo0 * STRIDE + t, Wc - 1) * S.pitch);   // columns past the frame only feed outputs that are not stored
-#pragma unroll
-            for (int t = 0; t < COLS; ++t) {
-              const uint32_t wd[4] = {v[t].x, v[t].y, v[t].z, v[t].w};
-              float f[8];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) f[2 * i] = __uint_as_float(wd[i] << 16), f[2 * i + 1] = __uint_as_float(wd[i] & 0xffff0000u);
-#pragma unroll
-              for (int pp = 0; pp < P; ++pp) {
-                const int sx = t - pp * STRIDE;   // compile-time after unrolling
-                if (sx >= 0 && sx < 3) {
-#pragma unroll
-                  for (int e = 0; e < 8; e += 2) {
-                    float a0 = f[e], a1 = f[e + 1];
-                    ffma2(a0, a1, wf[r * 3 + sx][e], wf[r * 3 + sx][e + 1], acc[pp][e], acc[pp][e + 1]);
-                    acc[pp][e] = a0, acc[pp][e + 1] = a1;
-                  }
-                }
-              }
-            }
-          }
-          if (c_in && ho < p.Ho) {
-            bf16* yp = p.y + (((size_t)b * p.Ho + ho) * p.Wo + wo0) * p.C + c;
-#pragma unroll
-            for (int pp = 0; pp < P; ++pp)
-              if (wo0 + pp < p.Wo) {
-                Vec16<bf16> o;
-#pragma unroll
-                for (int e = 0; e < 8; ++e) o.v[e] = apply_act(fmaf(sc[e], acc[pp][e], bi[e]), p.act2);
-                o.store(yp + (size_t)pp * p.C);
-              }
-          }
+          dw_strip<STRIDE>(
+              [&](int r, int t) {   // columns past the frame only feed outputs that are not stored
+                return *reinterpret_cast<const uint4*>(hid + ((ro * STRIDE + r) * Wc + min(wo0 * STRIDE + t, Wc - 1)) * S.pitch + cvec * 16);
+              },
+              [&](int r, int, int sx, int pp, const float (&f)[8]) { dw_fma(acc[pp], f, wf[r * 3 + sx]); });
+          if (c_in && ho < p.Ho)
+            dw_store(p.y + (((size_t)b * p.Ho + ho) * p.Wo + wo0) * p.C + c, p.C, p.Wo - wo0, acc, [&](float v, int e) { return apply_act(fmaf(sc[e], v, bi[e]), p.act2); });
         }
       }
       asm volatile("bar.sync 1, 256;" ::: "memory");   // read by everybody: the next band may be written over it

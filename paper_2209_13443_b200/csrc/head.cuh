@@ -21,6 +21,34 @@ constexpr int kGapThreads = 256;
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Adds the rows grp, grp + groups, ... of a [HW][C] map to acc, one vector of VEC channels at p, in ascending order, eight loads in flight: what
+// a row group of gap_kernel does, and of an FC kernel that pools by itself.
+template <typename T, int VEC, typename A>
+__device__ __forceinline__ void pool_rows(const T* p, int HW, int C, int grp, int groups, A* acc) {
+  int r = grp;
+  if constexpr (VEC > 1) {
+    for (; r + 7 * groups < HW; r += 8 * groups) {
+      Vec16<T> t[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) t[u].load(p + (size_t)(r + u * groups) * C);
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) acc[e] += t[u].v[e];
+    }
+  }
+  for (; r < HW; r += groups) {
+    if constexpr (VEC > 1) {
+      Vec16<T> t;
+      t.load(p + (size_t)r * C);
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) acc[e] += t.v[e];
+    } else {
+      acc[0] += Elem<T>::ld(p + (size_t)r * C);
+    }
+  }
+}
+
 // gap[b][c] = mean over the HW rows of sample b's [HW][C] map, in one pass.  A CTA owns one sample and a slab of
 // `lanes` channel vectors: its 256 threads form 256 / lanes row groups, group g adds rows g, g + groups, ... in
 // ascending order (eight loads in flight), then the first lanes * VEC threads add the group sums in ascending group
@@ -45,32 +73,7 @@ gap_kernel(const T* __restrict__ x, int HW, int C, int lanes, float* __restrict_
   A acc[VEC];
 #pragma unroll
   for (int e = 0; e < VEC; ++e) acc[e] = (A)0;
-  if (v < cv) {
-    const T* p0 = x + (size_t)b * HW * C + (size_t)v * VEC;
-    int r = grp;
-    if constexpr (VEC > 1) {
-      for (; r + 7 * groups < HW; r += 8 * groups) {
-        Vec16<T> t[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) t[u].load(p0 + (size_t)(r + u * groups) * C);
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-#pragma unroll
-          for (int e = 0; e < VEC; ++e) acc[e] += t[u].v[e];
-      }
-    }
-    for (; r < HW; r += groups) {
-      const T* p = p0 + (size_t)r * C;
-      if constexpr (VEC > 1) {
-        Vec16<T> t;
-        t.load(p);
-#pragma unroll
-        for (int e = 0; e < VEC; ++e) acc[e] += t.v[e];
-      } else {
-        acc[0] += Elem<T>::ld(p);
-      }
-    }
-  }
+  if (v < cv) pool_rows<T, VEC>(x + (size_t)b * HW * C + (size_t)v * VEC, HW, C, grp, groups, acc);
 #pragma unroll
   for (int e = 0; e < VEC; ++e) red[(grp * lanes + lv) * VEC + e] = acc[e];
   __syncthreads();
@@ -126,6 +129,24 @@ __device__ __forceinline__ void gap_tree(LD&& load, int o, int s, float* out) {
   }
 }
 
+// Adds the sums of the blocks grp, grp + groups, ... of G rows, one vector of VP channels at p, to acc: a row group of gap_blocks_kernel, and of an FC
+// kernel that pools by itself.
+template <int VP, int G, typename T>
+__device__ __forceinline__ void pool_blocks(const T* p, int nb, int C, int grp, int groups, float* acc) {
+  for (int j = grp; j < nb; j += groups) {
+    const T* pb = p + (size_t)j * G * C;
+    float t[VP];
+    gap_tree<G, VP>([&](int row, float* out) {
+      Vec16<T> r;
+      r.load(pb + (size_t)row * C);
+#pragma unroll
+      for (int e = 0; e < VP; ++e) out[e] = r.v[e];
+    }, 0, 1, t);
+#pragma unroll
+    for (int e = 0; e < VP; ++e) acc[e] += t[e];
+  }
+}
+
 // T = bf16 (VEC 8, the feature map) or float (VEC 4, block sums written by a convolution's epilogue; G = 1).
 template <typename T, int VEC, int G>
 __global__ void __launch_bounds__(kGapThreads)
@@ -144,21 +165,7 @@ gap_blocks_kernel(const T* __restrict__ x, int nb, int HW, int C, int lanes, flo
   float acc[VEC];
 #pragma unroll
   for (int e = 0; e < VEC; ++e) acc[e] = 0.f;
-  if (v < cv) {
-    const T* p0 = x + (size_t)b * nb * G * C + (size_t)v * VEC;
-    for (int j = grp; j < nb; j += groups) {
-      const T* pb = p0 + (size_t)j * G * C;
-      float t[VEC];
-      gap_tree<G, VEC>([&](int row, float* out) {
-        Vec16<T> r;
-        r.load(pb + (size_t)row * C);
-#pragma unroll
-        for (int e = 0; e < VEC; ++e) out[e] = r.v[e];
-      }, 0, 1, t);
-#pragma unroll
-      for (int e = 0; e < VEC; ++e) acc[e] += t[e];
-    }
-  }
+  if (v < cv) pool_blocks<VEC, G>(x + (size_t)b * nb * G * C + (size_t)v * VEC, nb, C, grp, groups, acc);
 #pragma unroll
   for (int e = 0; e < VEC; ++e) red[(grp * lanes + lv) * VEC + e] = acc[e];
   __syncthreads();
@@ -373,25 +380,10 @@ struct PoolArgs {
   int lanes;       // gap_block_lanes / gap_lanes of the map
   int sums;
 };
-// Sums of one channel vector of one sample over the blocks (rows) grp, grp + groups, ..., for the pooling kernels' row groups.
-template <int VP, int G, typename T>
-__device__ __forceinline__ void pool_blocks(const T* p, int nb, int C, int grp, int groups, float* acc) {
-  for (int j = grp; j < nb; j += groups) {
-    const T* pb = p + (size_t)j * G * C;
-    float t[VP];
-    gap_tree<G, VP>([&](int row, float* out) {
-      Vec16<T> r;
-      r.load(pb + (size_t)row * C);
-#pragma unroll
-      for (int e = 0; e < VP; ++e) out[e] = r.v[e];
-    }, 0, 1, t);
-#pragma unroll
-    for (int e = 0; e < VP; ++e) acc[e] += t[e];
-  }
-}
 // Pools the tile's samples, `lanes` channel vectors of VP channels at a time.  put(s, c, value).
 template <int VP, typename A, typename SUM, typename PUT>
 __device__ __forceinline__ void pool_tile(int samples, int C, int lanes, A* red, SUM&& sum, PUT&& put) {
+  static_assert(kFcThreads == kGapThreads, "row groups as in the pooling kernels");
   const int tid = threadIdx.x, groups = kFcThreads / lanes, grp = tid / lanes, lv = tid - grp * lanes;
   const int cv = C / VP, items = samples * cv;
   for (int i0 = 0; i0 < items; i0 += lanes) {
@@ -492,23 +484,7 @@ fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restri
     auto put = [&](int s, int c, A total) { gs[place(s, c) + c % 4] = (float)(total / (A)pa.HW); };
     if constexpr (sizeof(T) == 4) {
       pool_tile<VEC>(here, C, pa.lanes, (A*)red, [&](int s, int v, int grp, int groups, A* acc) {
-        const T* p0 = (const T*)pa.x + (size_t)(b0 + s) * pa.HW * C + (size_t)v * VEC;
-        int r = grp;
-        for (; r + 7 * groups < pa.HW; r += 8 * groups) {
-          Vec16<T> t[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) t[u].load(p0 + (size_t)(r + u * groups) * C);
-#pragma unroll
-          for (int u = 0; u < 8; ++u)
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) acc[e] += t[u].v[e];
-        }
-        for (; r < pa.HW; r += groups) {
-          Vec16<T> t;
-          t.load(p0 + (size_t)r * C);
-#pragma unroll
-          for (int e = 0; e < VEC; ++e) acc[e] += t.v[e];
-        }
+        pool_rows<T, VEC>((const T*)pa.x + (size_t)(b0 + s) * pa.HW * C + (size_t)v * VEC, pa.HW, C, grp, groups, acc);
       }, put);
     } else if (pa.sums) {
       pool_tile<4>(here, C, pa.lanes, (A*)red, [&](int s, int v, int grp, int groups, A* acc) {

@@ -535,3 +535,72 @@ def test_expand_and_depthwise_of_narrow_layers_give_the_bits_of_the_layers_apart
     m.check()
     assert torch.equal(out.features_out[:B], fused)
     run.check_guards()
+
+
+# Sums of negative zeros, sign and all: the ranges of a layer start from the same zero on every route (clusters of CTAs, one CTA per tile,
+# the one-wave kernel, CTA pairs): H, W, cin, cout, ranges, batch
+@pytest.mark.parametrize("geom", [(7, 7, 128, 128, 3, 4), (7, 7, 128, 256, 2, 40)])
+def test_k_ranges_give_the_same_zero_on_every_route(geom):
+    H, W, cin, cout, ranges, B = geom
+    spec = util.single_layer_model("bf16", H, W, cin, cout, 3, 1, 1, wl.ACT_NONE, False, seed=3, max_batch=B)
+    l = spec.stages[0].layers[0]
+    l.weight, l.scale, l.bias = -np.abs(l.weight), None, np.full(cout, -0.0, dtype=np.float32)
+    m = eb.EEModel(spec)
+    m.set_layer_splits(0, 0, ranges)
+    ws = m.workspace()
+    x = wl.random_features((B, H, W, cin), seed=3, bf16=True)
+    x[: (B + 1) // 2] = 0.0
+    xd = eb.to_device("bf16", x)
+    got = []
+    for variant in (3, 4, 0, 1 if cout > 128 else 2):
+        m.set_layer_variant(0, 0, 1, B, variant)
+        out = torch.empty((B, H, W, cout), dtype=torch.bfloat16, device="cuda")
+        m.layer_run(0, 0, xd, None, B, out, ws)
+        torch.cuda.synchronize()
+        m.check()
+        got.append(out.view(torch.int16))
+    assert all(torch.equal(g, got[0]) for g in got)
+
+
+# What keeps the last layer from storing to features_out: its output is read inside the stage, or features_out lies in the stage's input or
+# in the workspace, where the last layer still reads: a 3x3 layer over several waves of tiles, whose neighbours would be overwritten.  The
+# survivors are the same rows as in a buffer of its own.
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("where", ["read inside", "residual inside", "input", "workspace"])
+def test_survivors_are_gathered_where_features_out_cannot_take_the_output(dtype, where):
+    inside = where in ("read inside", "residual inside")
+    B, hw, c = 19, 6 if inside else 56, 64
+    rng = wl._rng(c, 933)
+    bf16 = dtype == "bf16"
+
+    def layer(k, **kw):
+        return wl._conv(rng, wl.OP_CONV, c, c, k, 1, k // 2, wl.ACT_RELU, bf16=bf16, **kw)
+
+    from_input = dict(input_from=wl.FROM_STAGE_INPUT)
+    layers = [layer(1), layer(3, **(from_input if where in ("input", "residual inside") else {}), **(dict(residual_from=0) if where == "residual inside" else {}))]
+    fw, fb = wl._head(rng, c, 5, 1.0, bf16)
+    spec = wl.Model("gathered", dtype, hw, hw, c, [wl.Stage(layers, 5, fw * 0.0, fb, 0.9, False, out_layer=0 if inside else 1)], B)
+    run = util.GpuRunner(spec)
+    m, out, ws = run.m, run.bufs[0], run.ws
+    xd = eb.to_device(dtype, wl.random_features((B, hw, hw, c), seed=3, bf16=bf16))
+    want, hid = torch.empty_like(out.features_out), torch.empty_like(out.features_out)
+    m.layer_run(0, 0, xd, None, B, want if inside else hid, ws)
+    if not inside:
+        m.layer_run(0, 1, xd if where == "input" else hid, None, B, want, ws)
+    xs = xd.clone()
+    if where == "input":
+        out.features_out = xs
+    elif where == "workspace":       # its first slot, the hidden layer's
+        out.features_out = ws[: want.numel() * want.element_size()].view(want.dtype).view(want.shape)
+    out._struct = None
+    for leave in (np.zeros(B, bool), np.arange(B) % 3 == 0, np.arange(B) > 4, np.ones(B, bool)):
+        xs.copy_(xd)
+        shift = torch.as_tensor(leave.astype(np.float32) * 30.0, device="cuda")
+        m.stage_run(0, xs, B, out, ws, None, shift, torch.zeros(B, dtype=torch.int32, device="cuda"))
+        torch.cuda.synchronize()
+        stay = np.nonzero(~leave)[0]
+        n = int(out.n_surv_dev[0])
+        assert n == len(stay) and np.array_equal(out.survivor_idx[:n].cpu().numpy(), stay)
+        assert torch.equal(out.features_out[:n], want[torch.as_tensor(stay, device="cuda")])
+    m.check()
+    run.check_guards()

@@ -178,8 +178,8 @@ ee_status_t ee_batch_refill(ee_model_t* model, int boundary, void* batch_feat, i
  * inside another layer's launch (ee_layer_plan_t.launches == 0, or the layer before it), a launch of its own with the same bits.
  * `input` is the layer's input tensor [batch][in_h][in_w][cin], `residual` its residual operand [batch][out_h][out_w][cout]
  * (required iff the layer has one), `output` [batch][out_h][out_w][cout]; all DEVICE, model dtype, 16-byte aligned,
- * caller-owned.  `workspace` is reserved (no layer kernel needs scratch today; pass the stage workspace or NULL).  For per-layer parity checks and
- * micro-benchmarks.  Errors: INVALID_ARG, STAGE (stage or layer out of range), CAPACITY, CUDA. */
+ * caller-owned.  `workspace`: the stage workspace, for the partial tiles of a layer with several K ranges on the CTA-pair kernel; NULL where
+ * the layer has no table entry that picks that kernel.  For per-layer parity checks and micro-benchmarks.  Errors: INVALID_ARG, STAGE (stage or layer out of range), CAPACITY, CUDA. */
 ee_status_t ee_layer_run(ee_model_t* model, int stage, int layer, const void* input, const void* residual, int batch,
                          void* output, void* workspace, size_t workspace_bytes, void* cuda_stream);
 

@@ -3,8 +3,8 @@
   python -m paper_2209_13443_b200.profile_layers --workload resnet50 --max-batch 64 --layers 2:5:30,3:4:27 [--variant V] [--reps N]
 
 ``--layers`` is a comma-separated list of stage:layer:batch.  Every layer runs through ee_layer_run in the kernel and
-launch configuration ee_stage_run would use for it (the model's per-(layer, batch) table applies unless ``--variant``
-forces one), on random inputs of the right shape.  Nothing beyond the chosen layers' tensors is allocated (a few
+launch configuration ee_stage_run would use for it by itself (the model's per-(layer, batch) table applies unless ``--variant``
+forces one; layers that share another layer's launch there have one of their own here), on random inputs of the right shape.  Nothing beyond the chosen layers' tensors is allocated (a few
 hundred MB at most), so that a profiler capture of a handful of launches ends in seconds.  Prints one line per
 layer with the CUDA-event time of a launch (the launches of a layer run back to back).
 """

@@ -18,7 +18,7 @@ int main() {
   int e = 0;
   // 3x3 512->512: whole wherever some batch up to max_batch leaves the deep clusters (measured slower there by up to 5 us)
   e += bad(72, 7, 64, 512, 1) + bad(72, 7, 16, 512, 1) + bad(72, 6, 64, 512, 1) + bad(72, 6, 22, 512, 1) + bad(72, 4, 64, 512, 1);
-  // four where none does (measured faster by 0.3 to 1.4 us)
+  // four where none does (a quarter of the outputs that miss the nearest bf16, for 0.3 to 0.8 us up to 144 blocks and a gain past 200)
   e += bad(72, 7, 8, 512, 4) + bad(72, 7, 1, 512, 4) + bad(72, 6, 16, 512, 4) + bad(72, 4, 48, 512, 4) + bad(72, 3, 64, 512, 4) + bad(72, 2, 64, 512, 4);
   // 3x3 256->256 and shorter: whole (measured slower in ranges at every batch)
   e += bad(36, 14, 1, 256, 1) + bad(36, 14, 64, 256, 1) + bad(36, 11, 4, 256, 1) + bad(32, 7, 1, 512, 1) + bad(1, 56, 64, 64, 1);

@@ -51,6 +51,9 @@ struct LayerPlan {
   float* scale_dev = nullptr;
   float* bias_dev = nullptr;
   TcLayer tc;  // tensor-core plan (valid iff kind == KK_TC or KK_TC_GATHER)
+  // Filters that decide which entries for CTA pairs the table takes: those of grouped pixels, also where the layer stays ungrouped for its
+  // bits' sake.  Where the pair kernel cannot run what is left, one-CTA tiles do (launch_layer).
+  int pair_filters = 0;
   F32Plan f32; // tile and K cut of a dense convolution of the fp32 model (kind == KK_F32)
   // Kernel variant per batch size, index 0..max_batch (TcVariant; empty = TCV_AUTO everywhere).  The analogue of the
   // paper's per-(layer, batch) look-up table that configures the array for the active batch (Section III-C): the
@@ -340,6 +343,11 @@ ee_status_t launch_layer(ee_model* m, const LayerPlan& L, const void* src, const
   }
   EE_CUDA(cudaGetLastError());
   return EE_OK;
+}
+
+// The table's rule for entries 1 and 2 (pair_supported, by pair_filters).
+bool pair_entry_taken(const LayerPlan& L, int variant) {
+  return L.kind == KK_TC && !L.tc.gather && !L.tc.halo && !L.tc.stem && L.pair_filters > (variant == TCV_PAIR256 ? 128 : 64);
 }
 
 bool host_memory(const void* p) {
@@ -1062,9 +1070,11 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
       } else if (desc->dtype == EE_BF16 && tc_supported(d, L.in_h, L.in_w)) {
         L.kind = KK_TC;
         // Beside the launch with the depthwise layer, whose K steps start at a pixel's first channel, so must those of the layer apart: pixels
-        // of whole K steps only are grouped there.  (24 channels on 34 x 34, 64 images: 22 to 31 of 10.7 million values rounded the other way.
-        // By itself such a layer takes 7.2 us in place of 4.5 on 28 x 28 x 144, 32 images, 2.0 either way for one; by default it never runs so.)
-        const int g = L.dw_next && d.cin % 16 ? 1 : pixel_group(d, L.in_h * L.in_w);
+        // whose channels are neither part of one K step nor whole ones are not grouped there.  (24 channels on 34 x 34, 64 images: 22 to 31 of
+        // 10.7 million values rounded the other way; 8, 16 and 32 channels: none.  By itself such a layer takes 7.2 us in place of 4.5 on
+        // 28 x 28 x 144, 32 images, 2.0 either way for one; by default it never runs so.)
+        const int grouped = pixel_group(d, L.in_h * L.in_w), g = L.dw_next && d.cin > 16 && d.cin % 16 ? 1 : grouped;
+        L.pair_filters = grouped * d.cout;
         if (g > 1) {   // narrow 1x1 layer: g pixels per row, block-diagonal weights, scale / bias repeated per pixel
           void* wp = nullptr;
           float *sp2 = nullptr, *bp2 = nullptr;
@@ -1703,7 +1713,7 @@ ee_status_t ee_model_set_layer_variant(ee_model_t* m, int stage, int layer, int 
   LayerPlan& L = sp.layers[layer];
   const bool ranges_v = variant == TCV_RANGES_CLUSTER || variant == TCV_RANGES_LOCAL;
   if (ranges_v && (L.kind != KK_TC || L.tc.gather || L.tc.halo)) return EE_ERR_UNSUPPORTED;
-  if (variant != TCV_AUTO && !ranges_v && (L.kind != KK_TC || !pair_supported(L.tc, variant))) return EE_ERR_UNSUPPORTED;
+  if (variant != TCV_AUTO && !ranges_v && !pair_entry_taken(L, variant)) return EE_ERR_UNSUPPORTED;
   if (L.variant.empty()) L.variant.assign((size_t)m->max_batch + 1, (uint8_t)TCV_AUTO);
   for (int b = batch_lo; b <= batch_hi; ++b) L.variant[b] = (uint8_t)variant;
   for (auto& g : sp.graphs) cudaGraphExecDestroy(g.exec);   // captured stages hold the old choice
@@ -1741,7 +1751,7 @@ ee_status_t ee_model_get_layer_config(const ee_model_t* m, int stage, int layer,
   const bool tc = L.kind == KK_TC && !L.tc.gather && !L.tc.halo;
   if (variant) *variant = L.variant.empty() ? (int)TCV_AUTO : (int)L.variant[batch];
   if (splits) *splits = L.kind == KK_TC ? L.tc.splits : 1;
-  if (tensor_core) *tensor_core = tc ? ((pair_supported(L.tc, TCV_PAIR256) ? 1 : 0) | (pair_supported(L.tc, TCV_PAIR128) ? 2 : 0)) : -1;
+  if (tensor_core) *tensor_core = tc ? ((pair_entry_taken(L, TCV_PAIR256) ? 1 : 0) | (pair_entry_taken(L, TCV_PAIR128) ? 2 : 0)) : -1;
   return EE_OK;
 }
 

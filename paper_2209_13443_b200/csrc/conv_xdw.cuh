@@ -13,7 +13,7 @@
 // clocks each on a 16 x 16 frame of 64 channels, the MMAs 400.  (Fetching narrow pixels by threads in place of TMA: 40.7 -> 42.6 us on
 // 56 x 56 x 144, batch 32.)
 // Each output sums the same products in the same K steps as the two layers apart, with the same roundings: the same bits.  (Beside this
-// launch a 1x1 layer groups its pixels, conv_tc.cuh, only where a pixel's channels are whole K steps.)
+// launch a 1x1 layer groups its pixels, conv_tc.cuh, only where a pixel's channels are part of one K step or whole ones.)
 #pragma once
 #include "conv_dw.cuh"
 

@@ -501,7 +501,8 @@ def test_expand_and_depthwise_in_one_launch(geom):
 # The expand + depthwise launch against the two layers run apart, narrow inputs, whose pixels are grouped apart (cin 8 to 32): channels that
 # are whole K steps of 16 and such that are not, maps of an even and an odd number of pixels.  The depthwise layer hands its input on, so every
 # hidden value shows; enough of them that K steps starting elsewhere would round some the other way.  H, W, cin, hidden, stride, batch
-XDW_NARROW = [(28, 28, 8, 48, 1, 32), (16, 34, 16, 96, 2, 32), (34, 34, 24, 144, 1, 64), (28, 28, 24, 144, 1, 64), (33, 33, 24, 144, 2, 3), (28, 28, 32, 192, 1, 32)]
+XDW_NARROW = [(28, 28, 8, 48, 1, 32), (16, 34, 16, 96, 2, 32), (34, 34, 24, 144, 1, 64), (28, 28, 24, 144, 1, 64), (33, 33, 24, 144, 2, 3), (28, 28, 32, 192, 1, 32), (28, 28, 24, 72, 1, 8),
+              (12, 12, 24, 40, 1, 8)]
 
 
 @pytest.mark.parametrize("geom", XDW_NARROW)
@@ -528,6 +529,18 @@ def test_expand_and_depthwise_of_narrow_layers_give_the_bits_of_the_layers_apart
     m.layer_run(0, 1, hid, None, B, apart, run.ws)
     torch.cuda.synchronize()
     assert torch.equal(fused, apart)
+    # entries for CTA pairs are taken as for grouped pixels, whatever the kernel behind them
+    group = max(g for g in range(1, 64 // cin + 1) if H * W % g == 0)
+    mask = (1 if group * hidden > 128 else 0) | (2 if group * hidden > 64 else 0)
+    assert m.layer_config(0, 0, B)["tensor_core"] == mask
+    for v in [v for v in (1, 2) if mask >> (v - 1) & 1] + [4]:
+        m.set_layer_variant(0, 0, B, B, v)
+        m.stage_run(0, xd, B, out, run.ws)
+        torch.cuda.synchronize()
+        m.check()
+        assert torch.equal(out.features_out[:B], fused)
+    m.set_layer_variant(0, 0, B, B, 0)
+    assert [pl["launches"] for pl in m.plan(0, B)] == [1, 0]
     m.set_stage_kernel(True)         # multi-layer launches take single layers
     assert [pl["launches"] for pl in m.plan(0, B)] == [1, 1]
     m.stage_run(0, xd, B, out, run.ws)

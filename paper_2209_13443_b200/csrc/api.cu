@@ -412,6 +412,7 @@ ee_status_t launch_head(ee_model* m, StagePlan& sp, const void* x, int B, int hw
       pooled = true;
     } else if (vec) {
       const int G = gap_block_rows(hw), nb = hw / G, bl = gap_block_lanes(nb);
+      const bool many = gap_many(G, nb, bl);
       const dim3 bgrid(cdiv(C / V, bl), B);
       auto go = [&](auto kernel) { return launch_pdl(kernel, bgrid, dim3(kGapThreads), st, (const T*)x, nb, hw, C, bl, gap, cnt, n_zero, sb); };
       switch (G) {
@@ -419,8 +420,8 @@ ee_status_t launch_head(ee_model* m, StagePlan& sp, const void* x, int B, int hw
         case 16: EE_CUDA(go(gap_blocks_kernel<T, V, 16>)); break;
         case 8: EE_CUDA(go(gap_blocks_kernel<T, V, 8>)); break;
         case 4: EE_CUDA(go(gap_blocks_kernel<T, V, 4>)); break;
-        case 2: EE_CUDA(go(gap_blocks_kernel<T, V, 2>)); break;
-        default: EE_CUDA(go(gap_blocks_kernel<T, V, 1>)); break;
+        case 2: EE_CUDA(many ? go(gap_blocks_kernel<T, V, 2, true>) : go(gap_blocks_kernel<T, V, 2>)); break;
+        default: EE_CUDA(many ? go(gap_blocks_kernel<T, V, 1, true>) : go(gap_blocks_kernel<T, V, 1>)); break;
       }
       pooled = true;
     }

@@ -30,12 +30,15 @@ template <> struct Vec16<float> {
     float4 t = *reinterpret_cast<const float4*>(p);
     v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
   }
+  __device__ __forceinline__ void unpack(uint4 t) {
+    v[0] = __uint_as_float(t.x); v[1] = __uint_as_float(t.y); v[2] = __uint_as_float(t.z); v[3] = __uint_as_float(t.w);
+  }
   __device__ __forceinline__ void store(float* p) const { *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]); }
 };
 template <> struct Vec16<bf16> {
   float v[8];
-  __device__ __forceinline__ void load(const bf16* p) {
-    uint4 t = *reinterpret_cast<const uint4*>(p);
+  __device__ __forceinline__ void load(const bf16* p) { unpack(*reinterpret_cast<const uint4*>(p)); }
+  __device__ __forceinline__ void unpack(uint4 t) {
     const uint32_t w[4] = {t.x, t.y, t.z, t.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {  // bf16 -> f32 is a 16-bit shift

@@ -131,24 +131,54 @@ __device__ __forceinline__ void gap_tree(LD&& load, int o, int s, float* out) {
 
 // Adds the sums of the blocks grp, grp + groups, ... of G rows, one vector of VP channels at p, to acc: a row group of gap_blocks_kernel, and of an FC
 // kernel that pools by itself.
-template <int VP, int G, typename T>
+// MANY: a row group has more than two blocks of one or two rows (gap_many), which are few loads each: eight rows are in flight
+// together, added in the same order, kept as the words they came in.
+template <int VP, int G, bool MANY = false, typename T>
 __device__ __forceinline__ void pool_blocks(const T* p, int nb, int C, int grp, int groups, float* acc) {
-  for (int j = grp; j < nb; j += groups) {
-    const T* pb = p + (size_t)j * G * C;
+  auto sum = [&](auto&& row_at) {   // of a block's G rows
     float t[VP];
     gap_tree<G, VP>([&](int row, float* out) {
-      Vec16<T> r;
-      r.load(pb + (size_t)row * C);
+      const Vec16<T> r = row_at(row);
 #pragma unroll
       for (int e = 0; e < VP; ++e) out[e] = r.v[e];
     }, 0, 1, t);
 #pragma unroll
     for (int e = 0; e < VP; ++e) acc[e] += t[e];
+  };
+  constexpr int U = MANY ? 8 / G : 1;
+  for (int j = grp; j < nb; j += U * groups) {
+    if constexpr (MANY) {
+      uint4 raw[8];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (j + u * groups < nb)
+#pragma unroll
+          for (int row = 0; row < G; ++row) raw[u * G + row] = *reinterpret_cast<const uint4*>(p + ((size_t)(j + u * groups) * G + row) * C);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (j + u * groups < nb)
+          sum([&](int row) {
+            Vec16<T> r;
+            r.unpack(raw[u * G + row]);
+            return r;
+          });
+    } else {
+      const T* pb = p + (size_t)j * G * C;
+      sum([&](int row) {
+        Vec16<T> r;
+        r.load(pb + (size_t)row * C);
+        return r;
+      });
+    }
   }
 }
+// Pooling + FC, us, 41 x 41 x 256 (odd: blocks of one row) at batch 37 / 64 without and with: 17.8 / 24.3 -> 15.7 / 21.8, 27 rows a group; in a
+// pass, where the map comes from HBM, 21 of them took 23 and take 13.  Up to two blocks a group it costs registers (32 -> 60) and with them
+// CTAs side by side: 11 x 11 x 1024 at 64 19.8 -> 21.7.  Blocks of four rows and more have their loads in flight as it is.
+inline bool gap_many(int G, int nb, int lanes) { return G <= 2 && nb > 2 * (kGapThreads / lanes); }
 
 // T = bf16 (VEC 8, the feature map) or float (VEC 4, block sums written by a convolution's epilogue; G = 1).
-template <typename T, int VEC, int G>
+template <typename T, int VEC, int G, bool MANY = false>
 __global__ void __launch_bounds__(kGapThreads)
 gap_blocks_kernel(const T* __restrict__ x, int nb, int HW, int C, int lanes, float* __restrict__ gap, unsigned* __restrict__ zero_me,
                   int n_zero, int rev) {
@@ -165,7 +195,7 @@ gap_blocks_kernel(const T* __restrict__ x, int nb, int HW, int C, int lanes, flo
   float acc[VEC];
 #pragma unroll
   for (int e = 0; e < VEC; ++e) acc[e] = 0.f;
-  if (v < cv) pool_blocks<VEC, G>(x + (size_t)b * nb * G * C + (size_t)v * VEC, nb, C, grp, groups, acc);
+  if (v < cv) pool_blocks<VEC, G, MANY>(x + (size_t)b * nb * G * C + (size_t)v * VEC, nb, C, grp, groups, acc);
 #pragma unroll
   for (int e = 0; e < VEC; ++e) red[(grp * lanes + lv) * VEC + e] = acc[e];
   __syncthreads();
@@ -736,8 +766,10 @@ inline cudaError_t fc_cluster_launch_t(const float* gap, const PoolArgs* pool, c
   attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = f.cluster ? 2 : 1;
-  return pool ? cudaLaunchKernelEx(&cfg, fc_cluster_kernel<T, S, true>, wfc, gap, bfc, B, C, K, z, exchange, d, f, *pool, err_flag)
-              : cudaLaunchKernelEx(&cfg, fc_cluster_kernel<T, S, false>, wfc, gap, bfc, B, C, K, z, exchange, d, f, PoolArgs{}, err_flag);
+  if constexpr (S == 1)   // fc_pools: tiles of one sample
+    if (pool) return cudaLaunchKernelEx(&cfg, fc_cluster_kernel<T, 1, true>, wfc, gap, bfc, B, C, K, z, exchange, d, f, *pool, err_flag);
+  if (pool) return cudaErrorInvalidValue;
+  return cudaLaunchKernelEx(&cfg, fc_cluster_kernel<T, S, false>, wfc, gap, bfc, B, C, K, z, exchange, d, f, PoolArgs{}, err_flag);
 }
 // d.done and d.tile_done must be zero when the kernel starts and are zero again when it ends.  exchange: 16 float4 per sample
 // of every tile, less than the batch's logits take wherever it is used (more than 512 classes).
@@ -755,7 +787,7 @@ inline cudaError_t fc_cluster_launch(const FcShape& f, const float* gap, const P
 template <typename T, int S>
 inline cudaError_t fc_cluster_attr() {
   cudaError_t e = cudaSuccess;
-  for (auto kernel : {fc_cluster_kernel<T, S, false>, fc_cluster_kernel<T, S, true>}) {
+  for (auto kernel : {fc_cluster_kernel<T, S, false>, fc_cluster_kernel<T, S, S == 1>}) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFcMaxSmem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   }

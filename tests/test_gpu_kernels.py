@@ -450,6 +450,29 @@ def test_head_routes_against_the_oracle_and_alone(case):
     assert np.array_equal(out.logits[0].cpu().numpy(), z[B - 1]) and float(out.conf[0]) == float(conf[B - 1])
 
 
+# rows of a map, its blocks of G rows and row groups: one row a block with two, three and more than eight blocks a group, two rows likewise
+@pytest.mark.parametrize("HW,G,groups", [(63, 1, 32), (65, 1, 64), (127, 1, 64), (129, 1, 64), (513, 1, 64), (1681, 1, 64), (258, 2, 64), (1026, 2, 64), (98, 2, 32)])
+def test_pooling_adds_the_blocks_of_a_row_group_in_order(HW, G, groups):
+    B, C = 2, 72
+    spec = wl.Model("rows", "bf16", 1, HW, C, [wl.Stage([wl.Layer(wl.OP_MAXPOOL, C, C, 3, 3, 1, 1)], C, np.eye(C, dtype=np.float32), None, 0.5, False)], B)
+    m = eb.EEModel(spec)
+    out = eb.StageBuffers(m, 0)
+    scratch = torch.empty(m.exit_head_scratch_bytes(0) + 256, dtype=torch.uint8, device="cuda")
+    x = wl.random_features((B, HW, C), seed=HW, bf16=True, relu=False)
+    m.exit_head(0, eb.to_device("bf16", x), B, HW, out, scratch)
+    torch.cuda.synchronize()
+    blocks = np.asarray(x, dtype=np.float32).reshape(B, HW // G, G, C)
+    while blocks.shape[2] > 1:      # the pairwise tree over a block's rows
+        blocks = blocks[:, :, :blocks.shape[2] // 2] + blocks[:, :, blocks.shape[2] // 2:]
+    blocks, want = blocks[:, :, 0], np.zeros((B, C), dtype=np.float32)
+    for q in range(groups):
+        part = np.zeros((B, C), dtype=np.float32)
+        for j in range(q, HW // G, groups):
+            part = part + blocks[:, j]
+        want = want + part
+    assert np.array_equal(out.logits[:B].cpu().numpy(), want / np.float32(HW))   # the FC layer is the identity: the logits are the pooled vector
+
+
 # 1x1 layer + depthwise layer in one launch: H, W, cin, hidden, stride, batches: one to three K blocks, channel blocks that are short, odd
 # or not a multiple of 16, bands of one row and of the whole image, one pixel, the widest row, images smaller than a tile of positions
 XDW_GEOMS = [(14, 14, 64, 384, 1, (1, 5)), (7, 7, 160, 960, 1, (1, 9)), (20, 50, 16, 96, 2, (1, 4)), (9, 13, 24, 144, 1, (1, 3)), (5, 5, 96, 576, 2, (1, 40)),

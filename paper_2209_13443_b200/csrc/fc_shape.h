@@ -25,7 +25,7 @@ __host__ __device__
 #endif
 inline size_t fc_smem_bytes(const FcShape& f) {
   return (size_t)(kFcThreads / 32) * f.ring * kFcSlot + (size_t)f.S * f.Cp * 4 + (size_t)f.S * (kFcBlocks / f.CL) * f.kb * 4 * (f.ws > 1 ? 1 + 2 * f.ws : 1) +
-         (size_t)kFcBlocks * f.S * 16 + (kFcThreads / 32) * f.ring * 8 + 16;
+         (size_t)kFcBlocks * f.S * 16 + (kFcThreads / 32) * f.ring * 8 + 32;
 }
 // 64 classes per CTA (clusters of 16 need the non-portable size), fewer CTAs for few classes.  Samples per tile: the fewest
 // whose clusters run side by side (`room16` clusters of 16: not every GPC has 16 SMs), up to 8, as a second wave costs the

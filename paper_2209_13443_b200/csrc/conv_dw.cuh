@@ -126,10 +126,10 @@ dwconv3x3_tma_kernel(const __grid_constant__ CUtensorMap tmX, DwParams p) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmX) : "memory");
   }
   __syncthreads();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (lane == 0) {
       for (int j = 0; j < my_tiles; ++j) {
         const int tf = (int)blockIdx.x + j * (int)gridDim.x, t = p.rev ? p.tiles - 1 - tf : tf;
@@ -159,7 +159,6 @@ dwconv3x3_tma_kernel(const __grid_constant__ CUtensorMap tmX, DwParams p) {
   }
   // no kernel writes weights, scale or bias: fetched while the layer in front still runs
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int strips = (p.Wo + P - 1) / P;
   const int Wc = p.W + 2;
   const int items = p.RB * strips;

@@ -103,13 +103,13 @@ conv3x3_halo_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __gri
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // the weights are written by no kernel: request all nine taps before the dependency wait
   if (warp == 0 && lane == 0 && my_tiles > 0) {
     mbar_expect_tx(w_bar, kHaloTaps * kHaloWTapBytes);
     for (int tap = 0; tap < kHaloTaps; ++tap) tma_load_3d(base + S::kWOff + tap * kHaloWTapBytes, &tmW, w_bar, 0, tap, 0);
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
     if (elect_one()) {

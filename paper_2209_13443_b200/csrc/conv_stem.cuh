@@ -302,13 +302,13 @@ conv_stem_tcgen05_kernel(const __grid_constant__ CUtensorMap tmW, StemParams p) 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (threadIdx.x == 0) {   // the whole weight matrix stays resident; no kernel writes it, so it need not wait
     mbar_expect_tx(w_bar, PAIRS * S::kWBytes);
     for (int i = 0; i < PAIRS; ++i) tma_load_3d(base + S::kWOff + i * S::kWBytes, &tmW, w_bar, i * kTcBK, 0, 0);
   }
   __syncwarp();
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
     if (elect_one()) {

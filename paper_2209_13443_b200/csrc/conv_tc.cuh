@@ -545,6 +545,7 @@ conv_igemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // Programmatic dependent launch: everything above overlapped the tail of the previous kernel in the stream, and
   // so do the weight tiles of the first ring slots, which no kernel writes.  From the wait on this kernel touches
   // activations, so it needs that kernel's memory; the next kernel in the stream may begin its own prologue now.
@@ -567,7 +568,6 @@ conv_igemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
     }
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
     // the elected thread goes on where the prefetch stopped (elect.sync picks the same lane of the same converged warp, and
@@ -894,6 +894,7 @@ conv_igemm_tcgen05_persistent_kernel(const __grid_constant__ CUtensorMap tmA, co
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // weight tiles of the first ring slots (first tile of this CTA) are requested before the dependency wait: no
   // kernel writes them
   const int w_ahead = my_tiles > 0 ? min(num_kb, kStages) : 0;
@@ -916,7 +917,6 @@ conv_igemm_tcgen05_persistent_kernel(const __grid_constant__ CUtensorMap tmA, co
   }
   __syncwarp();
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
     if (elect_one()) {   // weights; the ring never drains at a tile boundary

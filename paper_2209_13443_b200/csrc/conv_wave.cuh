@@ -95,6 +95,7 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp < S::kMma) {
     // K blocks h, h + kFeed, ...: walked by counters (slot and phase, channel block x 64, position in the tap table)
@@ -131,7 +132,6 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
       }
       __syncwarp();
       asm volatile("griddepcontrol.wait;" ::: "memory");
-      asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     } else {
       int cw = 0, ch = 0, cn = 0, cw2 = 0, ch2 = 0;
       if (p.im2col || (PROJ && p.im2col2)) {
@@ -142,7 +142,6 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         if (PROJ) cw2 = wo * p.stride2, ch2 = ho * p.stride2;
       }
       asm volatile("griddepcontrol.wait;" ::: "memory");
-      asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
       if (elect_one()) {
         bool ok = true;
         if (p.im2col) {
@@ -231,7 +230,6 @@ conv_wave_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
     }
     asm volatile("bar.sync 1, %0;" ::"n"(32 * S::kEpiWarps) : "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     constexpr int kCover = BN == 128 ? 64 : 32, kSteps = kCover / 32;   // columns of a warp, in steps of 32
     const int q = warp & 3, half = et >> 7, m = lane < S::kWarpRows ? m0 + q * S::kWarpRows + lane : p.M;
     uint4 r[4 * kSteps];

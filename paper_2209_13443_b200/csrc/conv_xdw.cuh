@@ -92,6 +92,7 @@ conv_expand_dw_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __g
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   auto band_of = [&](int j, int& b, int& band) {
     const int tf = (int)blockIdx.x + j * (int)gridDim.x, t = p.rev ? p.tiles - 1 - tf : tf;
     b = t / p.bands, band = t - b * p.bands;
@@ -102,7 +103,6 @@ conv_expand_dw_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __g
       mbar_expect_tx(w_bar, (uint32_t)(p.kblocks * 64 * 128));   // no kernel writes weights
       for (int k = 0; k < p.kblocks; ++k) tma_load_3d(base + (uint32_t)(k * 64 * 128), &tmW, w_bar, k * kTcBK, 0, c0);
       asm volatile("griddepcontrol.wait;" ::: "memory");
-      asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
       int s = 0;
       uint32_t ph = 1;
       for (int j = 0; j < my_tiles; ++j) {
@@ -161,7 +161,6 @@ conv_expand_dw_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __g
     }
     asm volatile("bar.sync 1, 256;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     uint8_t* hid = gen + S.h_off;
     const int strips = (p.Wo + P - 1) / P, items = p.RB * strips;
     for (int j = 0; j < my_tiles; ++j) {

@@ -66,8 +66,8 @@ gap_kernel(const T* __restrict__ x, int HW, int C, int lanes, float* __restrict_
   const int groups = kGapThreads / lanes;
   const int grp = tid / lanes, lv = tid - grp * lanes;
   const int v = blockIdx.x * lanes + lv;
-  pdl_wait();
   pdl_launch_dependents();
+  pdl_wait();
   if (blockIdx.x == 0 && blockIdx.y == 0)
     for (int i = tid; i < n_zero; i += kGapThreads) zero_me[i] = 0u;
   A acc[VEC];
@@ -188,8 +188,8 @@ gap_blocks_kernel(const T* __restrict__ x, int nb, int HW, int C, int lanes, flo
   const int groups = kGapThreads / lanes;
   const int grp = tid / lanes, lv = tid - grp * lanes;
   const int v = blockIdx.x * lanes + lv;
-  pdl_wait();
   pdl_launch_dependents();
+  pdl_wait();
   if (blockIdx.x == 0 && blockIdx.y == 0)
     for (int i = tid; i < n_zero; i += kGapThreads) zero_me[i] = 0u;
   float acc[VEC];
@@ -514,8 +514,8 @@ fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restri
     }
   };
   load_bias(wg);
-  pdl_wait();
   pdl_launch_dependents();
+  pdl_wait();
   const bool packed = d.packed && B <= kFcPackedBatch;
   // a warp's triples are all of one sample: S is 1, 2, 4 or 8, the step between them the eight warps
   const int my_s = warp % S, my_b = b0 + my_s;
@@ -866,8 +866,8 @@ fc_kernel(const float* __restrict__ gap, const T* __restrict__ wfc, const float*
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int k0 = blockIdx.x * kFcClasses, b0 = blockIdx.y * S;
   const int nchunk = (C + kFcChunk - 1) / kFcChunk;
-  pdl_wait();
   pdl_launch_dependents();
+  pdl_wait();
   typedef typename Accum<T>::type A;   // fp64 sums for the fp32 model
   A acc[kFcClassesPerWarp][S];
 #pragma unroll
@@ -1018,8 +1018,8 @@ head_cluster_kernel(const bf16* __restrict__ x, int HW, int C, const bf16* __res
     cp_async_commit();
   }
   for (int i = tid; i < S * (h.Cp - C); i += kHcThreads) gsm[(i / (h.Cp - C)) * h.Cp + C + i % (h.Cp - C)] = 0.f;   // channel padding
-  pdl_wait();
   pdl_launch_dependents();
+  pdl_wait();
 
   // ---- 1. pool
   {
@@ -1236,8 +1236,8 @@ template <typename V>
 __global__ void __launch_bounds__(kCopyThreads)
 gather_rows_kernel(const V* __restrict__ src, size_t vecs_per_row, const int32_t* __restrict__ surv_idx,
                    const int32_t* __restrict__ n_surv, V* __restrict__ dst, int rev) {
-  pdl_wait();
   pdl_launch_dependents();
+  pdl_wait();
   const int j = rev ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;   // rev: last row first, each row from its end
   const unsigned bx = rev ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
   if (j >= *n_surv) return;
@@ -1270,8 +1270,8 @@ __global__ void __launch_bounds__(kMoveThreads)
 move_rows_kernel(V* feat, size_t vecs_per_row, const int32_t* __restrict__ surv_idx, const int32_t* __restrict__ n_surv, int B) {
   const size_t v = (size_t)blockIdx.x * kMoveThreads + threadIdx.x;
   V* at = feat + v;
-  pdl_wait();
   pdl_launch_dependents();
+  pdl_wait();
   const int n = *n_surv;   // and, asked for together with it, the first rows' sources
   if (v >= vecs_per_row) return;
   for (int j0 = 0; j0 < B; j0 += kMoveRows) {
@@ -1294,8 +1294,8 @@ template <typename V>
 __global__ void __launch_bounds__(kCopyThreads)
 append_rows_kernel(const V* __restrict__ src, V* __restrict__ dst, size_t n, const int32_t* __restrict__ ids_src,
                    int32_t* __restrict__ ids_dst, int n_ids) {
-  pdl_wait();
   pdl_launch_dependents();
+  pdl_wait();
   const size_t stride = (size_t)gridDim.x * kCopyThreads;
   for (size_t v = (size_t)blockIdx.x * kCopyThreads + threadIdx.x; v < n; v += stride) dst[v] = __ldcs(src + v);
   if (ids_src && ids_dst && blockIdx.x == 0)

@@ -1,8 +1,8 @@
 // Depthwise 3x3 pad-1 convolution on bf16 (stride 1 or 2) with the input staged in shared memory by TMA: the
 // bandwidth-bound layers of the inverted-residual blocks.
 //
-// A depthwise layer does 9 MACs per element, so its only bound is HBM: what matters is how many bytes an SM keeps in
-// flight.  A kernel that loads through registers holds one item's inputs per thread and stalls on every item.  Here
+// A depthwise layer does 9 MACs per element.  A kernel that loads through registers holds one item's inputs per thread and stalls on
+// every item.  Here
 // one producer warp per persistent CTA asks the TMA unit for whole input tiles, a band of output rows x all columns x
 // one block of up to 64 channels, including the one-pixel frame of the padding (coordinates start at -1; the unit
 // zero-fills outside the image), into a ring of three slots: two or three tiles (up to 72 KB each) are in flight per
@@ -12,6 +12,8 @@
 // channel vectors of one pixel, 128 contiguous bytes, so the reads are conflict-free without swizzling.  Every output
 // sums its nine taps in ascending (r, s) with fp32 FMAs, scale / bias / activation in fp32, one rounding to bf16.
 #pragma once
+#include <type_traits>
+
 #include "conv_tc.cuh"
 
 namespace ee {
@@ -38,64 +40,95 @@ constexpr int kDwConsumers = 256;
 constexpr int kDwThreads = 32 + kDwConsumers;
 constexpr int kDwMaxTileBytes = 72 * 1024;
 
-// What a thread does with its vector of eight channels, here and in conv_xdw.cuh, whose bits have to agree.
-// Its 72 weights [8][3][3] as floats, [tap][channel]: unpacked from bf16 once, not at every product (two of three instructions of a strip
+// What a thread does with its vector of eight channels, here and in conv_xdw.cuh, whose bits have to agree.  What bounds it is instructions:
+// nine FMAs an output are 4.5 packed ones (an SM does about 93 FMAs a clock, packed or not), so everything else has to be few.  Pairs of
+// channels stay packed from the unpacking to the rounding, columns are offsets from one address, and the activation is chosen once a strip.  (30
+// instructions an output before.)  us, batch 32 / 13 / 1: 112 x 112 x 32 18.2 / 8.6 / 2.7 -> 16.7 / 8.1 / 2.6, 112 x 112 x 96 at stride 2
+// 22.9 / 9.2 / 3.1 -> 20.0 / 8.3 / 2.9.  A thread that walks down its columns, sums of three rows open in registers, reads every vector once
+// (13.7 and 17.5 at batch 32) but fills the register file, so that no neighbouring kernel sets up beside it: 9.3 and 9.4 at 13, 4.2 and 4.3 at 1.
+typedef unsigned long long f32x2;   // two floats
+__device__ __forceinline__ f32x2 f32x2_pack(uint32_t lo, uint32_t hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+  return r;
+}
+__device__ __forceinline__ f32x2 f32x2_fma(f32x2 a, f32x2 b, f32x2 c) {   // two independent round-to-nearest FMAs
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ void f32x2_unpack_bf16(uint4 x, f32x2 (&f)[4]) {
+  const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) f[i] = f32x2_pack(w[i] << 16, w[i] & 0xffff0000u);
+}
+// Its 72 weights [8][3][3] as floats, [tap][channel pair]: unpacked from bf16 once, not at every product (two of three instructions of a strip
 // were such shifts and masks).  Zeros where !take.
-__device__ __forceinline__ void dw_weights(const bf16* w, bool take, float (&wf)[9][8]) {
+__device__ __forceinline__ void dw_weights(const bf16* w, bool take, f32x2 (&wf)[9][4]) {
   uint32_t wr[36];   // as stored: element e = channel e / 9, tap e % 9
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
     const uint4 v = take ? __ldg(reinterpret_cast<const uint4*>(w) + i) : make_uint4(0u, 0u, 0u, 0u);
     wr[4 * i] = v.x, wr[4 * i + 1] = v.y, wr[4 * i + 2] = v.z, wr[4 * i + 3] = v.w;
   }
+  auto elem = [&](int e) { return (e & 1) ? wr[e >> 1] & 0xffff0000u : wr[e >> 1] << 16; };
 #pragma unroll
-  for (int e = 0; e < 72; ++e) wf[e % 9][e / 9] = (e & 1) ? __uint_as_float(wr[e >> 1] & 0xffff0000u) : __uint_as_float(wr[e >> 1] << 16);
+  for (int t = 0; t < 9; ++t)
 #pragma unroll
-  for (int e = 0; e < 72; ++e) asm volatile("" : "+f"(wf[e % 9][e / 9]));   // floats from here on: not to be unpacked again in the loop
+    for (int i = 0; i < 4; ++i) {
+      wf[t][i] = f32x2_pack(elem(18 * i + t), elem(18 * i + 9 + t));
+      asm volatile("" : "+l"(wf[t][i]));   // floats from here on: not to be unpacked again in the loop
+    }
 }
-// A strip of kDwStrip output pixels: at(r, q) is the vector of frame row r, column q; tap(r, q, s, p, f) takes its eight values as tap
-// (r, s) of output p.  Every output gets its taps in ascending (r, s).
-template <int STRIDE, typename AT, typename TAP>
-__device__ __forceinline__ void dw_strip(AT&& at, TAP&& tap) {
+// The sums of a strip of kDwStrip output pixels, every output's taps in ascending (r, s).  at: the strip's first frame vector, columns `pitch` and
+// rows `line` bytes apart.  Columns past the frame only feed outputs that are not stored: up to kDwOver vectors behind the last row are read.
+constexpr int kDwOver = 8;
+template <int STRIDE>
+__device__ __forceinline__ void dw_strip(const uint8_t* at, int pitch, int line, const f32x2 (&w)[9][4], f32x2 (&acc)[kDwStrip][4]) {
   constexpr int COLS = (kDwStrip - 1) * STRIDE + 3;
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
     uint4 v[COLS];
 #pragma unroll
-    for (int q = 0; q < COLS; ++q) v[q] = at(r, q);
+    for (int q = 0; q < COLS; ++q) v[q] = *reinterpret_cast<const uint4*>(at + r * line + q * pitch);
 #pragma unroll
     for (int q = 0; q < COLS; ++q) {
-      const uint32_t wd[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
-      float f[8];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) f[2 * i] = __uint_as_float(wd[i] << 16), f[2 * i + 1] = __uint_as_float(wd[i] & 0xffff0000u);
+      f32x2 f[4];
+      f32x2_unpack_bf16(v[q], f);
 #pragma unroll
       for (int p = 0; p < kDwStrip; ++p) {
         const int s = q - p * STRIDE;   // compile-time after unrolling
-        if (s >= 0 && s < 3) tap(r, q, s, p, f);
+        if (s < 0 || s > 2) continue;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[p][i] = f32x2_fma(f[i], w[r * 3 + s][i], r == 0 && s == 0 ? 0ull : acc[p][i]);
       }
     }
   }
 }
-__device__ __forceinline__ void dw_fma(float (&acc)[8], const float (&f)[8], const float (&w)[8]) {
+// y[0 .. cols) = act(scale * sum + bias), rounded to bf16; pixels at and past `cols` are not stored.  sb: eight scales and, 64 floats behind, biases.
+__device__ __forceinline__ void dw_store(bf16* y, int C, int cols, const f32x2 (&acc)[kDwStrip][4], const float* sb, int act) {
+  f32x2 sc[4], bi[4];
 #pragma unroll
-  for (int e = 0; e < 8; e += 2) {   // two independent round-to-nearest FMAs per instruction
-    float a0 = f[e], a1 = f[e + 1];
-    ffma2(a0, a1, w[e], w[e + 1], acc[e], acc[e + 1]);
-    acc[e] = a0, acc[e + 1] = a1;
+  for (int i = 0; i < 2; ++i) {
+    const ulonglong2 s = reinterpret_cast<const ulonglong2*>(sb)[i], b = reinterpret_cast<const ulonglong2*>(sb + 64)[i];
+    sc[2 * i] = s.x, sc[2 * i + 1] = s.y, bi[2 * i] = b.x, bi[2 * i + 1] = b.y;
   }
-}
-// Stores the strip's first `cols` pixels (all of them where more are left in the row): value(sum, e), rounded to bf16.
-template <typename VALUE>
-__device__ __forceinline__ void dw_store(bf16* y, int C, int cols, const float (&acc)[kDwStrip][8], VALUE&& value) {
+  auto put = [&](auto kind) {
 #pragma unroll
-  for (int p = 0; p < kDwStrip; ++p)
-    if (p < cols) {
-      Vec16<bf16> o;
+    for (int p = 0; p < kDwStrip; ++p)
+      if (p < cols) {
+        uint32_t o[4];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) o.v[e] = value(acc[p][e], e);
-      o.store(y + (size_t)p * C);
-    }
+        for (int i = 0; i < 4; ++i) {
+          const f32x2 t = f32x2_fma(sc[i], acc[p][i], bi[i]);
+          o[i] = pack_bf16x2(apply_act(__uint_as_float((uint32_t)t), decltype(kind)::value), apply_act(__uint_as_float((uint32_t)(t >> 32)), decltype(kind)::value));
+        }
+        *reinterpret_cast<uint4*>(y + (size_t)p * C) = make_uint4(o[0], o[1], o[2], o[3]);
+      }
+  };
+  if (act == EE_ACT_RELU6) put(std::integral_constant<int, EE_ACT_RELU6>{});
+  else if (act == EE_ACT_RELU) put(std::integral_constant<int, EE_ACT_RELU>{});
+  else put(std::integral_constant<int, EE_ACT_NONE>{});
 }
 
 // POOL: the same staging for a 3x3 pad-1 window maximum (the max-pool behind a ResNet-style stem): taps outside the
@@ -108,8 +141,9 @@ dwconv3x3_tma_kernel(const __grid_constant__ CUtensorMap tmX, DwParams p) {
   const uint32_t raw_s = smem_u32(smem_raw);
   const uint32_t base = (raw_s + 127u) & ~127u;
   uint8_t* gen = smem_raw + (base - raw_s);
-  const int bar_off = kDwStages * p.slot_bytes;
+  const int bar_off = kDwStages * p.slot_bytes + kDwOver * 128;   // behind the last slot: what strips read past its frame
   const uint32_t bar0 = base + bar_off;
+  __shared__ __align__(16) float s_sb[128];   // scale | bias of the channel block
   auto full = [&](int s) { return bar0 + 8u * s; };
   auto empty = [&](int s) { return bar0 + 8u * (kDwStages + s); };
 
@@ -124,6 +158,12 @@ dwconv3x3_tma_kernel(const __grid_constant__ CUtensorMap tmX, DwParams p) {
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmX) : "memory");
+  }
+  if (!POOL && threadIdx.x < 64) {   // no kernel writes weights, scale or bias: fetched while the layer in front still runs
+    const int i = (int)threadIdx.x;
+    const bool in = i < p.cb && c0 + i < p.C;
+    s_sb[i] = p.scale && in ? p.scale[c0 + i] : 1.f;
+    s_sb[64 + i] = p.bias && in ? p.bias[c0 + i] : 0.f;
   }
   __syncthreads();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -149,18 +189,11 @@ dwconv3x3_tma_kernel(const __grid_constant__ CUtensorMap tmX, DwParams p) {
   const bool live = item0 < item_step;      // nv need not divide 256: the threads of the ragged tail idle
   const int c = c0 + cvec * 8;
   const bool c_in = c < p.C;
-  float wf[9][8];
-  dw_weights(p.w + (size_t)c * 9, !POOL && c_in, wf);
-  float sc[8], bi[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    sc[e] = (p.scale && c_in) ? p.scale[c + e] : 1.f;
-    bi[e] = (p.bias && c_in) ? p.bias[c + e] : 0.f;
-  }
-  // no kernel writes weights, scale or bias: fetched while the layer in front still runs
+  f32x2 wf[9][4];
+  if constexpr (!POOL) dw_weights(p.w + (size_t)c * 9, c_in, wf);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int strips = (p.Wo + P - 1) / P;
-  const int Wc = p.W + 2;
+  const int Wc = p.W + 2, pitch = p.cb * 2;
   const int items = p.RB * strips;
   for (int j = 0; j < my_tiles; ++j) {
     const int tf = (int)blockIdx.x + j * (int)gridDim.x, t = p.rev ? p.tiles - 1 - tf : tf;
@@ -173,29 +206,43 @@ dwconv3x3_tma_kernel(const __grid_constant__ CUtensorMap tmX, DwParams p) {
         const int ro = it / strips, st = it - ro * strips;
         const int wo0 = st * P;
         const int ho = band * p.RB + ro;
-        float acc[P][8];
+        const uint8_t* at = tile + (ro * STRIDE * Wc + wo0 * STRIDE) * pitch + cvec * 16;
+        bf16* y = p.y + (((size_t)b * p.Ho + ho) * p.Wo + wo0) * p.C + c;
+        if constexpr (POOL) {
+          float acc[P][8];
 #pragma unroll
-        for (int pp = 0; pp < P; ++pp)
+          for (int pp = 0; pp < P; ++pp)
 #pragma unroll
-          for (int e = 0; e < 8; ++e) acc[pp][e] = POOL ? -INFINITY : 0.f;
-        dw_strip<STRIDE>(
-            [&](int r, int q) {   // columns past the frame only feed outputs that are not stored
-              return *reinterpret_cast<const uint4*>(tile + (size_t)((ro * STRIDE + r) * Wc + min(wo0 * STRIDE + q, Wc - 1)) * p.cb * 2 + cvec * 16);
-            },
-            [&](int r, int q, int sx, int pp, const float (&f)[8]) {
-              if constexpr (POOL) {
-                const int hi = ho * STRIDE - 1 + r, wi = wo0 * STRIDE - 1 + q;
-                if (hi >= 0 && hi < p.H && wi >= 0 && wi < p.W) {
+            for (int e = 0; e < 8; ++e) acc[pp][e] = -INFINITY;
 #pragma unroll
-                  for (int e = 0; e < 8; ++e) acc[pp][e] = fmaxf(acc[pp][e], f[e]);
+          for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int q = 0; q < (P - 1) * STRIDE + 3; ++q) {
+              const int hi = ho * STRIDE - 1 + r, wi = wo0 * STRIDE - 1 + q;
+              if (hi < 0 || hi >= p.H || wi < 0 || wi >= p.W) continue;
+              Vec16<bf16> f;
+              f.unpack(*reinterpret_cast<const uint4*>(at + (r * Wc + q) * pitch));
+#pragma unroll
+              for (int pp = 0; pp < P; ++pp)
+                if (q - pp * STRIDE >= 0 && q - pp * STRIDE < 3) {
+#pragma unroll
+                  for (int e = 0; e < 8; ++e) acc[pp][e] = fmaxf(acc[pp][e], f.v[e]);
                 }
-              } else {
-                dw_fma(acc[pp], f, wf[r * 3 + sx]);
+            }
+          if (c_in && ho < p.Ho)
+#pragma unroll
+            for (int pp = 0; pp < P; ++pp)
+              if (pp < p.Wo - wo0) {
+                Vec16<bf16> o;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) o.v[e] = acc[pp][e];
+                o.store(y + (size_t)pp * p.C);
               }
-            });
-        if (c_in && ho < p.Ho)
-          dw_store(p.y + (((size_t)b * p.Ho + ho) * p.Wo + wo0) * p.C + c, p.C, p.Wo - wo0, acc,
-                   [&](float v, int e) { return POOL ? v : apply_act(fmaf(sc[e], v, bi[e]), p.act); });
+        } else {
+          f32x2 acc[P][4];
+          dw_strip<STRIDE>(at, pitch, Wc * pitch, wf, acc);
+          if (c_in && ho < p.Ho) dw_store(y, p.C, p.Wo - wo0, acc, s_sb + cvec * 8, p.act);
+        }
       }
     }
     __syncwarp();
@@ -220,7 +267,7 @@ inline bool dw_tma_supported(const ConvGeom& g, const void* x, const void* w, co
 }
 
 inline ee_status_t dw_context_init() {
-  const int bytes = kDwStages * kDwMaxTileBytes + 256 + 128;
+  const int bytes = kDwStages * kDwMaxTileBytes + kDwOver * 128 + 256 + 128;
   cudaError_t e = cudaFuncSetAttribute(dwconv3x3_tma_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(dwconv3x3_tma_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(dwconv3x3_tma_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -300,7 +347,7 @@ inline ee_status_t dw_tma_launch(TcContext& c, const TcLayer& L, const ConvGeom&
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(std::min(p.tiles, std::max(1, c.sm_count / chunks)), chunks);
   cfg.blockDim = dim3(kDwThreads);
-  cfg.dynamicSmemBytes = kDwStages * p.slot_bytes + 256 + 128;
+  cfg.dynamicSmemBytes = kDwStages * p.slot_bytes + kDwOver * 128 + 256 + 128;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -50,8 +50,8 @@ inline XdwSmem xdw_smem(int cb, int kblocks, int positions, int slots) {
   s.slot = kblocks * mtiles * 128 * 128;
   s.h_off = s.x_off + slots * s.slot;
   s.pitch = cb * 2 + 16;   // eight positions of a store or load phase in different banks
-  s.sb_off = s.h_off + (positions * s.pitch + 127) / 128 * 128;
-  s.bar_off = s.sb_off + 2 * 64 * 4;
+  s.sb_off = s.h_off + ((positions + kDwOver) * s.pitch + 127) / 128 * 128;   // strips read past the last row of the frame
+  s.bar_off = s.sb_off + 4 * 64 * 4;
   s.bytes = s.bar_off + 128 + 1024;
   return s;
 }
@@ -145,20 +145,16 @@ conv_expand_dw_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __g
       const bool in = i < p.cb && c0 + i < p.C;
       s_sb[i] = (p.scale1 && in) ? p.scale1[c0 + i] : 1.f;
       s_sb[64 + i] = (p.bias1 && in) ? p.bias1[c0 + i] : 0.f;
+      s_sb[128 + i] = (p.scale2 && in) ? p.scale2[c0 + i] : 1.f;
+      s_sb[192 + i] = (p.bias2 && in) ? p.bias2[c0 + i] : 0.f;
     }
     const int nv = p.cb >> 3;                 // channel vectors per block
     const int cvec = tid % nv, item0 = tid / nv, item_step = kDwConsumers / nv;
     const bool live = item0 < item_step;      // nv need not divide 256: the threads of the ragged tail idle
     const int c = c0 + cvec * 8;
     const bool c_in = c < p.C;
-    float wf[9][8];
+    f32x2 wf[9][4];
     dw_weights(p.w + (size_t)c * 9, c_in, wf);
-    float sc[8], bi[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      sc[e] = (p.scale2 && c_in) ? p.scale2[c + e] : 1.f;
-      bi[e] = (p.bias2 && c_in) ? p.bias2[c + e] : 0.f;
-    }
     asm volatile("bar.sync 1, 256;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     uint8_t* hid = gen + S.h_off;
@@ -198,18 +194,9 @@ conv_expand_dw_tcgen05_kernel(const __grid_constant__ CUtensorMap tmX, const __g
       if (live) {
         for (int it = item0; it < items; it += item_step) {
           const int ro = it / strips, st = it - ro * strips, wo0 = st * P, ho = band * p.RB + ro;
-          float acc[P][8];
-#pragma unroll
-          for (int pp = 0; pp < P; ++pp)
-#pragma unroll
-            for (int e = 0; e < 8; ++e) acc[pp][e] = 0.f;
-          dw_strip<STRIDE>(
-              [&](int r, int t) {   // columns past the frame only feed outputs that are not stored
-                return *reinterpret_cast<const uint4*>(hid + ((ro * STRIDE + r) * Wc + min(wo0 * STRIDE + t, Wc - 1)) * S.pitch + cvec * 16);
-              },
-              [&](int r, int, int sx, int pp, const float (&f)[8]) { dw_fma(acc[pp], f, wf[r * 3 + sx]); });
-          if (c_in && ho < p.Ho)
-            dw_store(p.y + (((size_t)b * p.Ho + ho) * p.Wo + wo0) * p.C + c, p.C, p.Wo - wo0, acc, [&](float v, int e) { return apply_act(fmaf(sc[e], v, bi[e]), p.act2); });
+          f32x2 acc[P][4];
+          dw_strip<STRIDE>(hid + (ro * STRIDE * Wc + wo0 * STRIDE) * S.pitch + cvec * 16, S.pitch, Wc * S.pitch, wf, acc);
+          if (c_in && ho < p.Ho) dw_store(p.y + (((size_t)b * p.Ho + ho) * p.Wo + wo0) * p.C + c, p.C, p.Wo - wo0, acc, s_sb + 128 + cvec * 8, p.act2);
         }
       }
       asm volatile("bar.sync 1, 256;" ::: "memory");   // read by everybody: the next band may be written over it

@@ -271,6 +271,22 @@ def test_depthwise_layer(dtype, C, stride, H, W):
     util.check_stage(spec, run.stage(0, x), util.oracle_stage(spec, 0, x), f"dw {dtype} C={C}", elementwise=True)
 
 
+# Depthwise layers at the edges of a strip, a band and a channel block: C, stride, H, W.  One pixel, one column, strips that end inside a row and read past
+# its frame (by up to six columns at stride 2, one channel vector to eight apart), the widest row, one to four blocks of which the last is short.
+DW_GEOMS = [(8, 1, 1, 1), (8, 2, 1, 2), (40, 1, 5, 1), (16, 1, 2, 3), (72, 1, 7, 9), (136, 2, 7, 8), (8, 1, 4, 254), (8, 2, 5, 254), (32, 2, 3, 129),
+            (32, 1, 56, 57), (96, 2, 57, 56), (200, 1, 30, 13)]
+
+
+@pytest.mark.parametrize("C,stride,H,W", DW_GEOMS)
+@pytest.mark.parametrize("act", [wl.ACT_NONE, wl.ACT_RELU])
+def test_depthwise_layer_at_its_edges(C, stride, H, W, act):
+    spec = util.single_layer_model("bf16", H, W, C, C, 3, stride, 1, act, False, seed=C + W, op=wl.OP_DWCONV, max_batch=19)
+    run = util.GpuRunner(spec)
+    for B in (1, 19):   # at 19 a CTA walks several bands of the large maps
+        x = wl.random_features((B, H, W, C), seed=B, bf16=True, relu=False)
+        util.check_stage(spec, run.stage(0, x), util.oracle_stage(spec, 0, x), f"dw C={C} {H}x{W}/{stride} B={B}", elementwise=True)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_maxpool_layer(dtype):
     rng = wl._rng(5, 901)

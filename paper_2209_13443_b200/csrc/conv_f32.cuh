@@ -9,6 +9,12 @@
 // that finishes their share of the tile (distributed shared memory) and added there in ascending CTA order.
 // Z, KG and the tile depend on the layer and max_batch only, so a sample's sums are grouped the same way in any batch.
 //
+// A K group has a ring of its own, 16 of K a step, which its threads fill, and waits for nobody else: where a group is one warp, the
+// fragments of one warp are fetched and converted while the other warp of its scheduler multiplies.  (With stages of 128 that all eight warps
+// shared, a block-wide barrier each, loads, conversions and products took turns: of 9.7 us of a 3x3 512 -> 512 layer 1.7 and 3.5 were the
+// last two.)  us a layer of the 64 x 64 model: 3x3 64 -> 64, batch 6 11.0 -> 9.9, 3x3 512 -> 512, 2 9.7 -> 8.3, 1x1 512 -> 2048, 2 5.2 -> 4.3;
+// a pass at batch 6 479 -> 448, tiny model at 8 69 -> 64.
+//
 // What a small layer's time is (clocks of one CTA, 32 x 32 tile): 2050 of MMAs per 128 of K, which is the fp64 rate, and around
 // them first operands, reduction and epilogue.  So weights are requested before the wait for the layer in front, scale, bias
 // and residual come to registers during the K loop (fetched at the end they took 5000), tap positions are counted, not divided,
@@ -25,12 +31,12 @@ constexpr int kF32Threads = 256;
 
 template <int WM, int WN, int KG, int MF, int NF>
 struct F32Tile {   // WM x WN warps per K group, each MF x NF fragments of 16 x 8
-  static constexpr int kBM = WM * MF * 16, kBN = WN * NF * 8, kKS = 16 * KG;   // output tile; K per ring stage
-  static constexpr int kStages = KG == 8 ? 3 : 4;
-  static constexpr int kRow = kKS + 4;                     // floats per shared-memory row: 4 mod 32 (20 mod 32 for KG = 1) spreads a fragment's 8 rows over all banks
-  static constexpr int kStageFloats = (kBM + kBN) * kRow;
+  static constexpr int kBM = WM * MF * 16, kBN = WN * NF * 8, kKS = 16 * KG;   // output tile; K that the groups take together per step
+  static constexpr int kGroup = 32 * WM * WN;              // threads of a K group
+  static constexpr int kStages = KG == 8 && MF == 2 ? 3 : 4;   // steps in a group's ring
+  static constexpr int kStageFloats = (kBM + kBN) * 16;    // rows of 16 floats, their four 16-byte chunks XORed with half the row: a fragment's 8 rows then lie in all banks
   static constexpr int kPRow = kBN + 2;                    // doubles per row of a partial tile
-  static constexpr int kRing = kStages * kStageFloats * 4, kPart = KG * kBM * kPRow * 8;
+  static constexpr int kRing = KG * kStages * kStageFloats * 4, kPart = KG * kBM * kPRow * 8;
   static constexpr int kOuts = kBM * kBN / kF32Threads;    // outputs per thread
   static constexpr int kMain = kRing > kPart ? kRing : kPart;
   // a cluster's CTAs receive their share of the partial tiles behind the ring; the 64 x 64 tile is not cut further
@@ -45,6 +51,11 @@ __device__ __forceinline__ void mma_f64(double* c, const double* a, const double
       "mma.sync.aligned.m16n8k16.row.col.f64.f64.f64.f64 {%0, %1, %2, %3}, {%4, %5, %6, %7, %8, %9, %10, %11}, {%12, %13, %14, %15}, {%0, %1, %2, %3};"
       : "+d"(c[0]), "+d"(c[1]), "+d"(c[2]), "+d"(c[3])
       : "d"(a[0]), "d"(a[1]), "d"(a[2]), "d"(a[3]), "d"(a[4]), "d"(a[5]), "d"(a[6]), "d"(a[7]), "d"(b[0]), "d"(b[1]), "d"(b[2]), "d"(b[3]));
+}
+__device__ __forceinline__ double lds_f64(uint32_t at) {   // a float of shared memory
+  float x;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x) : "r"(at) : "memory");
+  return x;
 }
 template <int BYTES>   // 16 or 4; `in` false fills zeros
 __device__ __forceinline__ void cp_async_zfill(uint32_t dst, const void* src, bool in) {
@@ -61,49 +72,49 @@ __device__ __forceinline__ void st_cluster_f64(uint32_t addr, uint32_t rank, dou
 
 // V: floats per copy (4 when Cin is a multiple of 4 and the pointers are 16-byte aligned, else 1).  k_per: K range of a CTA.
 template <int WM, int WN, int KG, int MF, int NF, int V>
-__global__ void __launch_bounds__(kF32Threads)
+__global__ void __launch_bounds__(kF32Threads, KG == 1 || (KG == 8 && V == 4) ? 2 : 1)   // two CTAs an SM: 128 registers
 conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ w, const float* __restrict__ scale,
                          const float* __restrict__ bias, const float* __restrict__ residual, float* __restrict__ y, ConvGeom g, int k_per) {
   using S = F32Tile<WM, WN, KG, MF, NF>;
-  constexpr int BM = S::kBM, BN = S::kBN, KS = S::kKS, ROW = S::kRow, STAGES = S::kStages;
-  constexpr int UNITS = KS / V;                       // copies per row and stage
-  constexpr int STEP = kF32Threads / UNITS;           // rows covered by one pass of the CTA
+  constexpr int BM = S::kBM, BN = S::kBN, KS = S::kKS, STAGES = S::kStages;
+  constexpr int UNITS = 16 / V;                       // copies per row and step
+  constexpr int STEP = S::kGroup / UNITS;             // rows covered by one pass of a group
   constexpr int RA = (BM + STEP - 1) / STEP, RB = (BN + STEP - 1) / STEP;
   extern __shared__ __align__(16) uint8_t f32_smem[];
-  float* ring = reinterpret_cast<float*>(f32_smem);
-  const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(f32_smem);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, kg = __shfl_sync(0xffffffffu, tid / S::kGroup, 0);   // the compiler is to know that a warp has one
+  const uint32_t smem_s = (uint32_t)__cvta_generic_to_shared(f32_smem);
+  const uint32_t ring_s = smem_s + (uint32_t)(kg * (STAGES * S::kStageFloats)) * 4u;   // of this thread's K group
   const int M = g.B * g.Ho * g.Wo, N = g.Cout, K = g.kh * g.kw * g.Cin;
   const int m0 = (int)blockIdx.x * BM, n0 = (int)blockIdx.y * BN;
   const int z = (int)blockIdx.z, Z = (int)gridDim.z;
   const int k_begin = z * k_per, k_end = min(K, k_begin + k_per);
-  const int steps = max(0, (k_end - k_begin + KS - 1) / KS);
+  const int k_mine = k_begin + kg * 16, steps = max(0, (k_end - k_mine + KS - 1) / KS);   // this group's steps: k_mine, k_mine + KS, ...
 
-  const int ku = tid % UNITS, r0 = tid / UNITS;       // this thread copies column ku of rows r0, r0 + STEP, ...
-  const float* a_base[RA];
-  int a_h[RA], a_w[RA];
+  const int ku = tid % UNITS, r0 = tid % S::kGroup / UNITS;   // this thread copies column ku of rows r0, r0 + STEP, ...
+  int a_b[RA], a_h[RA], a_w[RA];   // sample x image rows, row and column of the first tap
 #pragma unroll
   for (int i = 0; i < RA; ++i) {
     const int r = r0 + i * STEP, m = m0 + r;
     const bool in = r < BM && m < M;
     const int mm = in ? m : 0;
     const int wo = mm % g.Wo, q = mm / g.Wo, ho = q % g.Ho, b = q / g.Ho;
-    a_base[i] = x + (size_t)b * g.H * g.W * g.Cin;
+    a_b[i] = b * g.H;
     a_h[i] = in ? ho * g.stride - g.pad : -(1 << 20);   // far outside the image: zeros
     a_w[i] = wo * g.stride - g.pad_w;
   }
-  // position of this thread's column in stage `step`: K index, channel, filter row and column, walked by counters
-  int k = k_begin + ku * V, ci = k % g.Cin, fs = k / g.Cin % g.kw, fr_ = k / g.Cin / g.kw;
+  auto place = [&](int row) { return ((ku * V / 4 ^ (row >> 1 & 3)) << 4) + ku * V % 4 * 4; };   // byte of this thread's column in a row
+  // position of this thread's column in a step: K index, channel, filter row and column, walked by counters
+  int k = k_mine + ku * V, ci = k % g.Cin, fs = k / g.Cin % g.kw, fr_ = k / g.Cin / g.kw;
   const int dci = KS % g.Cin, dtap = KS / g.Cin;
-  auto load_b = [&](int step) {   // weights: K index k_begin + step * KS + ku * V
+  auto load_b = [&](int step) {   // weights
     const uint32_t st = ring_s + (uint32_t)((step % STAGES) * S::kStageFloats) * 4u;
-    const int kb = k_begin + step * KS + ku * V;
+    const int kb = k_mine + step * KS + ku * V;
 #pragma unroll
     for (int i = 0; i < RB; ++i) {
       const int row = r0 + i * STEP, n = n0 + row;
       if (BN % STEP == 0 || row < BN) {
         const bool in = kb < k_end && n < N;
-        cp_async_zfill<V * 4>(st + (uint32_t)((BM + row) * ROW + ku * V) * 4u, in ? w + (size_t)n * K + kb : w, in);
+        cp_async_zfill<V * 4>(st + (uint32_t)((BM + row) * 64 + place(row)), in ? w + (size_t)n * K + kb : w, in);
       }
     }
   };
@@ -115,7 +126,7 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
       if (BM % STEP == 0 || row < BM) {
         const int hi = a_h[i] + fr_, wi = a_w[i] + fs;
         const bool in = k < k_end && hi >= 0 && hi < g.H && wi >= 0 && wi < g.W;
-        cp_async_zfill<V * 4>(st + (uint32_t)(row * ROW + ku * V) * 4u, in ? a_base[i] + ((size_t)hi * g.W + wi) * g.Cin + ci : x, in);
+        cp_async_zfill<V * 4>(st + (uint32_t)(row * 64 + place(row)), in ? x + (size_t)((a_b[i] + hi) * g.W + wi) * g.Cin + ci : x, in);
       }
     }
     k += KS, ci += dci, fs += dtap;
@@ -147,7 +158,7 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
     const int m = m0 + (out_first + i * kF32Threads) / BN;
     res[i] = residual && tid + i * kF32Threads < share && m < M && nc < N ? residual[(size_t)m * N + nc] : 0.f;
   }
-  const int kg = warp / (WM * WN), wmn = warp % (WM * WN), wm = wmn / WN, wn = wmn % WN;
+  const int wmn = warp % (WM * WN), wm = wmn / WN, wn = wmn % WN;
   const int fr = lane >> 2, fk = lane & 3;            // fragment row (column of B) and K position of this lane
   double acc[MF][NF][4];
 #pragma unroll
@@ -156,27 +167,34 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
     for (int j = 0; j < NF; ++j)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.0;
+  uint32_t chunk[4];   // of K 4 e .. 4 e + 3, in this lane's rows
+#pragma unroll
+  for (int e = 0; e < 4; ++e) chunk[e] = ring_s + (uint32_t)(fr * 64 + ((e ^ (fr >> 1 & 3)) << 4) + fk * 4);
+  int at = 0;   // step % STAGES
   for (int step = 0; step < steps; ++step) {
     asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
-    __syncthreads();                                  // this stage has landed for all; the stage refilled below was read one step ago
+    // this step has landed for the whole group; the one refilled below was read a step ago
+    if constexpr (S::kGroup == 32)
+      __syncwarp();
+    else
+      asm volatile("bar.sync %0, %1;" ::"r"(1 + kg), "n"(S::kGroup) : "memory");
     if (step + STAGES - 1 < steps) {
       load_a(step + STAGES - 1);
       load_b(step + STAGES - 1);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
-    if (k_begin + step * KS + kg * 16 >= k_end) continue;   // past the range: zeros
-    const float* as = ring + (step % STAGES) * S::kStageFloats + (wm * MF * 16 + fr) * ROW + kg * 16 + fk;
-    const float* bs = ring + (step % STAGES) * S::kStageFloats + (BM + wn * NF * 8 + fr) * ROW + kg * 16 + fk;
+    const uint32_t stage = (uint32_t)(at * S::kStageFloats * 4), a_at = stage + (uint32_t)(wm * MF * 16 * 64), b_at = stage + (uint32_t)((BM + wn * NF * 8) * 64);
+    if (++at == STAGES) at = 0;
     double b[NF][4];
 #pragma unroll
     for (int j = 0; j < NF; ++j)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) b[j][e] = (double)bs[j * 8 * ROW + 4 * e];
+      for (int e = 0; e < 4; ++e) b[j][e] = lds_f64(chunk[e] + b_at + j * 8 * 64);
 #pragma unroll
     for (int i = 0; i < MF; ++i) {
       double a[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) a[e] = (double)as[(i * 16 + 8 * (e & 1)) * ROW + 4 * (e >> 1)];
+      for (int e = 0; e < 8; ++e) a[e] = lds_f64(chunk[e >> 1] + a_at + (i * 16 + 8 * (e & 1)) * 64);
 #pragma unroll
       for (int j = 0; j < NF; ++j) mma_f64(acc[i][j], a, b[j]);
     }
@@ -205,7 +223,7 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
   double* recv = reinterpret_cast<double*>(f32_smem + S::kMain);   // [Z][share]
   if (Z > 1) {
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");   // every CTA of the cluster runs
-    const uint32_t recv_s = ring_s + (uint32_t)S::kMain;
+    const uint32_t recv_s = smem_s + (uint32_t)S::kMain;
 #pragma unroll
     for (int i = 0; i < S::kOuts; ++i) {
       const int idx = tid + i * kF32Threads, q = idx / share;

@@ -10,10 +10,17 @@ struct F32Plan {
   int z = 1;       // CTAs of a cluster that share a tile's K
 };
 
+// K range of a CTA of the cluster: equal numbers of 16-wide steps, the unit the K groups take in turn, the last one shorter.  A ring
+// stage at a range's end may be short.  (In whole stages of 128 the cut of K = 1152 over four CTAs, or of 2304 over eight, was
+// three stages each and none for the last CTA, or the last two.)
+inline int f32_k_per(int k, int z) { return (int)f32_div(f32_div(k, 16), z) * 16; }
+
 // Tile and cluster size of a layer, from its geometry and max_batch.  Short K (stems on 3 channels): one K group, a ring
 // stage is 16 wide and nothing is padded to 128.  Grids of two waves of 64 x 64 tiles: that tile reads its operands least.
 // Everything else has idle SMs: small tiles (16 rows where the layer never has more than 32), eight K groups, and as many CTAs per tile (up to 8) as keep the grid within
-// two CTAs per SM while every CTA still has two ring stages of K.
+// two CTAs per SM while every CTA still has 64 of K, a 16-wide step for half its groups, and the last one any.  That line at 256 / 128 / 64 / 32, us a pass:
+// ResNet-50-shaped model at 33 px, batch 1 340 / 323 / 313 / 313, 64 px, batch 6 of which 30 % leave at every exit 448 / 436 / 436 / 436, tiny model
+// at 40 px, batch 8 with nobody leaving 75.7 / 73.4 / 77.1 / 76.5, at 24 px, batch 1 61 / 58 / 56 / 54.
 inline F32Plan f32_plan(long m_max, int n, int k, int sms) {
   F32Plan p;
   if (k < 128) return p;
@@ -23,13 +30,8 @@ inline F32Plan f32_plan(long m_max, int n, int k, int sms) {
   }
   p.tile = m_max <= 32 ? 3 : 2;   // 17 to 32 rows are two 16-row tiles: the same products, and half of them once samples have left
   const long tiles = f32_div(m_max, p.tile == 3 ? 16 : 32) * f32_div(n, 32);
-  while (p.z < 8 && tiles * p.z * 2 <= 2L * sms && k >= p.z * 2 * 256) p.z *= 2;
+  while (p.z < 8 && tiles * p.z * 2 <= 2L * sms && k >= p.z * 2 * 64 && f32_k_per(k, p.z * 2) * (p.z * 2L - 1) < k) p.z *= 2;
   return p;
 }
-
-// K range of a CTA of the cluster: equal numbers of 16-wide steps, the unit the K groups take in turn, the last one shorter.  A ring
-// stage at a range's end may be short.  (In whole stages of 128 the cut of K = 1152 over four CTAs, or of 2304 over eight, was
-// three stages each and none for the last CTA, or the last two.)
-inline int f32_k_per(int k, int z) { return (int)f32_div(f32_div(k, 16), z) * 16; }
 
 }  // namespace ee

@@ -287,6 +287,22 @@ def test_depthwise_layer_at_its_edges(C, stride, H, W, act):
         util.check_stage(spec, run.stage(0, x), util.oracle_stage(spec, 0, x), f"dw C={C} {H}x{W}/{stride} B={B}", elementwise=True)
 
 
+# fp32 convolutions at the lines of their plan (csrc/f32_plan.h): H, W, cin, cout, k, stride.  K of 64 a CTA of the cluster and just under it, steps that do not
+# divide among the CTAs or the K groups, groups without a step; 4-byte copies below and above K = 256, one K group and eight.
+F32_GEOMS = [(4, 4, 128, 32, 1, 1), (4, 4, 124, 32, 1, 1), (5, 3, 16, 40, 3, 1), (4, 4, 520, 64, 1, 1), (2, 2, 512, 512, 1, 1), (8, 8, 72, 96, 3, 2),
+             (33, 21, 3, 64, 7, 2), (9, 9, 6, 24, 5, 1), (7, 7, 30, 16, 3, 1)]
+
+
+@pytest.mark.parametrize("geom", F32_GEOMS)
+@pytest.mark.parametrize("max_batch", [1, 9])
+def test_fp32_layer_at_the_lines_of_its_plan(geom, max_batch):
+    H, W, cin, cout, k, stride = geom
+    spec = util.single_layer_model("f32", H, W, cin, cout, k, stride, k // 2, wl.ACT_RELU, False, seed=cin + k, max_batch=max_batch)
+    run = util.GpuRunner(spec)
+    x = wl.random_features((max_batch, H, W, cin), seed=max_batch, bf16=False, relu=False)
+    util.check_stage(spec, run.stage(0, x), util.oracle_stage(spec, 0, x), f"f32 {geom} of {max_batch}", elementwise=True)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_maxpool_layer(dtype):
     rng = wl._rng(5, 901)

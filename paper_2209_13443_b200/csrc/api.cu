@@ -1131,7 +1131,7 @@ ee_status_t ee_model_create(const ee_model_desc_t* desc, void* cuda_stream, ee_m
         L.tc.g_stride = d.stride, L.tc.g_pad = d.pad, L.tc.g_runp = runp;
       } else if (desc->dtype == EE_F32) {
         L.kind = KK_F32;
-        L.f32 = f32_plan((long)desc->max_batch * L.out_h * L.out_w, d.cout, d.kh * d.kw * d.cin, m->tc.sm_count);
+        L.f32 = f32_plan((long)desc->max_batch * L.out_h * L.out_w, d.cout, d.kh * d.kw * d.cin, m->tc.sm_count, d.cin % 4 == 0);
       } else {
         L.kind = KK_SIMT;
       }

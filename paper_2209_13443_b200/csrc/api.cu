@@ -271,7 +271,7 @@ ee_status_t launch_layer(ee_model* m, const LayerPlan& L, const void* src, const
     }
     case KK_F32: {
       if constexpr (sizeof(T) == 4)
-        EE_CUDA(f32_launch(L.f32, (const float*)src, (const float*)L.w_dev, L.scale_dev, L.bias_dev, (const float*)res, (float*)dst, g, st));
+        EE_CUDA(f32_launch(L.f32, (const float*)src, (const float*)L.w_dev, L.scale_dev, L.bias_dev, (const float*)res, (float*)dst, g, m->err_flag, st));
       else
         return EE_ERR_INTERNAL;
       break;

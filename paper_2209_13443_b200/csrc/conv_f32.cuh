@@ -18,11 +18,12 @@
 // What a small layer's time is (clocks of one CTA, 32 x 32 tile): 2050 of MMAs per 128 of K, which is the fp64 rate, and around
 // them first operands, reduction and epilogue.  So weights are requested before the wait for the layer in front, scale, bias
 // and residual come to registers during the K loop (fetched at the end they took 5000), tap positions are counted, not divided,
-// and one cluster barrier stands between the K loop and the result.  ResNet-50-shaped fp32 model at 64 x 64, batch 6:
+// and partial sums travel as asynchronous stores that the barrier of their receiver counts.  ResNet-50-shaped fp32 model at 64 x 64, batch 6:
 // 630 -> 567 us a pass with these; K cut in equal numbers of 16-wide steps instead of whole ring stages (f32_plan.h) 526 -> 513.
 #pragma once
 #include "common.cuh"
 #include "conv_simt.cuh"
+#include "conv_tc.cuh"
 #include "f32_plan.h"
 
 namespace ee {
@@ -41,7 +42,7 @@ struct F32Tile {   // WM x WN warps per K group, each MF x NF fragments of 16 x 
   static constexpr int kMain = kRing > kPart ? kRing : kPart;
   // a cluster's CTAs receive their share of the partial tiles behind the ring; the 64 x 64 tile is not cut further
   static constexpr int kRecv = KG == 8 ? kBM * kBN * 8 : 0;
-  static constexpr int kBytes = kMain + kRecv;
+  static constexpr int kBytes = kMain + kRecv + 16;        // and a barrier that counts it
   static_assert(WM * WN * KG == 8, "8 warps");
   static_assert(kBytes <= 227 * 1024, "exceeds the shared memory of an SM");
 };
@@ -64,17 +65,20 @@ __device__ __forceinline__ void cp_async_zfill(uint32_t dst, const void* src, bo
   else
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4 : 0) : "memory");
 }
-__device__ __forceinline__ void st_cluster_f64(uint32_t addr, uint32_t rank, double v) {
-  uint32_t a;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
-  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+// Two doubles into the shared memory of CTA `rank` of the cluster; its barrier `bar` counts them.  addr, bar: as in this CTA.
+__device__ __forceinline__ void st_async_f64x2(uint32_t addr, uint32_t bar, uint32_t rank, double v0, double v1) {
+  asm volatile(
+      "{\n .reg .b32 a, b;\n mapa.shared::cluster.u32 a, %0, %2;\n mapa.shared::cluster.u32 b, %1, %2;\n"
+      " st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [a], {%3, %4}, [b];\n}"
+      ::"r"(addr), "r"(bar), "r"(rank), "l"(__double_as_longlong(v0)), "l"(__double_as_longlong(v1))
+      : "memory");
 }
 
 // V: floats per copy (4 when Cin is a multiple of 4 and the pointers are 16-byte aligned, else 1).  k_per: K range of a CTA.
 template <int WM, int WN, int KG, int MF, int NF, int V>
 __global__ void __launch_bounds__(kF32Threads, KG == 1 || (KG == 8 && V == 4) ? 2 : 1)   // two CTAs an SM: 128 registers
 conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ w, const float* __restrict__ scale,
-                         const float* __restrict__ bias, const float* __restrict__ residual, float* __restrict__ y, ConvGeom g, int k_per) {
+                         const float* __restrict__ bias, const float* __restrict__ residual, float* __restrict__ y, ConvGeom g, int k_per, int* err_flag) {
   using S = F32Tile<WM, WN, KG, MF, NF>;
   constexpr int BM = S::kBM, BN = S::kBN, KS = S::kKS, STAGES = S::kStages;
   constexpr int UNITS = 16 / V;                       // copies per row and step
@@ -138,11 +142,22 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
 #pragma unroll
   for (int s = 0; s < STAGES - 1; ++s)
     if (s < steps) load_b(s);
-  if (Z > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  // outputs z * share + tid, + 256, ...: one channel per thread (256 is a multiple of every BN)
-  const int share = BM * BN / Z, out_first = z * share + tid;   // Z is 1, 2, 4 or 8: divides every tile
+  const uint32_t arrived = smem_s + (uint32_t)(S::kMain + S::kRecv);   // counts the partial sums that this CTA finishes
+  if (Z > 1) {
+    if (tid == 0) {
+      mbar_init(arrived, 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      mbar_expect_tx(arrived, (uint32_t)(BM * BN * 8));
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  }
+  // outputs z * share + 2 tid and its neighbour, + 512, ...: two channels per thread (512 is a multiple of every BN, Z is 1, 2, 4 or 8)
+  const int share = BM * BN / Z, out_first = z * share + 2 * tid;
   const int nc = n0 + out_first % BN;
-  const float sc = scale && nc < N ? scale[nc] : 1.f, bi = bias && nc < N ? bias[nc] : 0.f;
+  float sc[2], bi[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) sc[h] = scale && nc + h < N ? scale[nc + h] : 1.f, bi[h] = bias && nc + h < N ? bias[nc + h] : 0.f;
   // The next layer's CTAs may set up and fetch their weights while this layer still waits: they wait for its end themselves.  A layer's own
   // prologue is long here (copies of 4 to 16 bytes), and behind the wait it was not over when its turn came: 497 -> 485 us a pass (64 x 64, batch 6).
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -154,9 +169,10 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
   }
   float res[S::kOuts];
 #pragma unroll
-  for (int i = 0; i < S::kOuts; ++i) {
+  for (int i = 0; i < S::kOuts; i += 2) {
     const int m = m0 + (out_first + i * kF32Threads) / BN;
-    res[i] = residual && tid + i * kF32Threads < share && m < M && nc < N ? residual[(size_t)m * N + nc] : 0.f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) res[i + h] = residual && 2 * tid + i * kF32Threads < share && m < M && nc + h < N ? residual[(size_t)m * N + nc + h] : 0.f;
   }
   const int wmn = warp % (WM * WN), wm = wmn / WN, wn = wmn % WN;
   const int fr = lane >> 2, fk = lane & 3;            // fragment row (column of B) and K position of this lane
@@ -214,10 +230,13 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
           *reinterpret_cast<double2*>(p + (i * 16 + 8 * h) * S::kPRow + j * 8) = make_double2(acc[i][j][2 * h], acc[i][j][2 * h + 1]);
   }
   __syncthreads();
-  auto group_sum = [&](int o) {
-    double v = part[o];
+  auto group_sum = [&](int o) {   // of two outputs side by side
+    double2 v = *reinterpret_cast<const double2*>(part + o);
 #pragma unroll
-    for (int q = 1; q < KG; ++q) v += part[q * BM * S::kPRow + o];
+    for (int q = 1; q < KG; ++q) {
+      const double2 t = *reinterpret_cast<const double2*>(part + q * BM * S::kPRow + o);
+      v.x += t.x, v.y += t.y;
+    }
     return v;
   };
   double* recv = reinterpret_cast<double*>(f32_smem + S::kMain);   // [Z][share]
@@ -225,27 +244,38 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");   // every CTA of the cluster runs
     const uint32_t recv_s = smem_s + (uint32_t)S::kMain;
 #pragma unroll
-    for (int i = 0; i < S::kOuts; ++i) {
-      const int idx = tid + i * kF32Threads, q = idx / share;
-      st_cluster_f64(recv_s + (uint32_t)(z * share + idx - q * share) * 8u, (uint32_t)q, group_sum(idx / BN * S::kPRow + idx % BN));
+    for (int i = 0; i < S::kOuts; i += 2) {
+      const int idx = 2 * tid + i * kF32Threads, q = idx / share;
+      const double2 v = group_sum(idx / BN * S::kPRow + idx % BN);
+      st_async_f64x2(recv_s + (uint32_t)(z * share + idx - q * share) * 8u, arrived, (uint32_t)q, v.x, v.y);
     }
-    asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+    // Nothing but the data is waited for; a barrier of the cluster behind plain stores cost a pass of the ResNet-50-shaped model at 64 px 6 us of
+    // 427 at batch 6, 18 of 365 at batch 2.  Whoever waits here has been sent everything, so a CTA may leave while its own stores are on their way.
+    if (!mbar_wait(arrived, 0, err_flag)) return;
   }
 #pragma unroll
-  for (int i = 0; i < S::kOuts; ++i) {
-    const int rel = tid + i * kF32Threads, idx = z * share + rel, m = m0 + idx / BN;
-    if (rel >= share || m >= M || nc >= N) continue;
-    double v = 0.0;
+  for (int i = 0; i < S::kOuts; i += 2) {
+    const int rel = 2 * tid + i * kF32Threads, idx = z * share + rel, m = m0 + idx / BN;
+    if (rel >= share || m >= M) continue;
+    double v[2] = {0.0, 0.0};
     if (Z > 1) {
 #pragma unroll
       for (int q = 0; q < 8; ++q)
-        if (q < Z) v += recv[q * share + rel];
+        if (q < Z) {
+          const double2 t = *reinterpret_cast<const double2*>(recv + q * share + rel);
+          v[0] += t.x, v[1] += t.y;
+        }
     } else {
-      v = group_sum(idx / BN * S::kPRow + idx % BN);
+      const double2 t = group_sum(idx / BN * S::kPRow + idx % BN);
+      v[0] = t.x, v[1] = t.y;
     }
-    v = (double)sc * v + (double)bi;
-    if (residual) v += (double)res[i];
-    y[(size_t)m * N + nc] = (float)apply_act(v, g.act);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (nc + h >= N) continue;
+      double t = (double)sc[h] * v[h] + (double)bi[h];
+      if (residual) t += (double)res[i + h];
+      y[(size_t)m * N + nc + h] = (float)apply_act(t, g.act);
+    }
   }
 }
 
@@ -253,7 +283,7 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
 
 template <int WM, int WN, int KG, int MF, int NF, int V>
 inline cudaError_t f32_launch_t(const F32Plan& p, const float* x, const float* w, const float* scale, const float* bias, const float* residual,
-                                float* y, const ConvGeom& g, cudaStream_t st) {
+                                float* y, const ConvGeom& g, int* err_flag, cudaStream_t st) {
   using S = F32Tile<WM, WN, KG, MF, NF>;
   const int K = g.kh * g.kw * g.Cin;
   const int k_per = f32_k_per(K, p.z);
@@ -270,24 +300,24 @@ inline cudaError_t f32_launch_t(const F32Plan& p, const float* x, const float* w
   attr[1].val.clusterDim.z = p.z;
   cfg.attrs = attr;
   cfg.numAttrs = p.z > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, conv_igemm_f64mma_kernel<WM, WN, KG, MF, NF, V>, x, w, scale, bias, residual, y, g, k_per);
+  return cudaLaunchKernelEx(&cfg, conv_igemm_f64mma_kernel<WM, WN, KG, MF, NF, V>, x, w, scale, bias, residual, y, g, k_per, err_flag);
 }
 
 template <int V>
 inline cudaError_t f32_launch_v(const F32Plan& p, const float* x, const float* w, const float* scale, const float* bias, const float* residual,
-                                float* y, const ConvGeom& g, cudaStream_t st) {
+                                float* y, const ConvGeom& g, int* err_flag, cudaStream_t st) {
   switch (p.tile) {
-    case 1: return f32_launch_t<2, 2, 2, 2, 4, V>(p, x, w, scale, bias, residual, y, g, st);
-    case 2: return f32_launch_t<1, 1, 8, 2, 4, V>(p, x, w, scale, bias, residual, y, g, st);
-    case 3: return f32_launch_t<1, 1, 8, 1, 4, V>(p, x, w, scale, bias, residual, y, g, st);
-    default: return f32_launch_t<4, 2, 1, 1, 2, V>(p, x, w, scale, bias, residual, y, g, st);
+    case 1: return f32_launch_t<2, 2, 2, 2, 4, V>(p, x, w, scale, bias, residual, y, g, err_flag, st);
+    case 2: return f32_launch_t<1, 1, 8, 2, 4, V>(p, x, w, scale, bias, residual, y, g, err_flag, st);
+    case 3: return f32_launch_t<1, 1, 8, 1, 4, V>(p, x, w, scale, bias, residual, y, g, err_flag, st);
+    default: return f32_launch_t<4, 2, 1, 1, 2, V>(p, x, w, scale, bias, residual, y, g, err_flag, st);
   }
 }
 
 inline cudaError_t f32_launch(const F32Plan& p, const float* x, const float* w, const float* scale, const float* bias, const float* residual,
-                              float* y, const ConvGeom& g, cudaStream_t st) {
+                              float* y, const ConvGeom& g, int* err_flag, cudaStream_t st) {
   const bool vec = g.Cin % 4 == 0 && (((uintptr_t)x | (uintptr_t)w) & 15) == 0;
-  return vec ? f32_launch_v<4>(p, x, w, scale, bias, residual, y, g, st) : f32_launch_v<1>(p, x, w, scale, bias, residual, y, g, st);
+  return vec ? f32_launch_v<4>(p, x, w, scale, bias, residual, y, g, err_flag, st) : f32_launch_v<1>(p, x, w, scale, bias, residual, y, g, err_flag, st);
 }
 
 inline ee_status_t f32_context_init() {

@@ -411,13 +411,14 @@ ee_status_t launch_head(ee_model* m, StagePlan& sp, const void* x, int B, int hw
       EE_CUDA(launch_pdl(gap_blocks_kernel<float, 4, 1>, dim3(cdiv(C / 4, bl), B), dim3(kGapThreads), st, gap_part, nb, hw, C, bl, gap, cnt, n_zero, sb));
       pooled = true;
     } else if (vec) {
-      const int G = gap_block_rows(hw), nb = hw / G, bl = gap_block_lanes(nb);
-      const bool many = gap_many(G, nb, bl);
+      const int G = gap_block_rows(hw), nb = hw / G, lanes_all = gap_block_lanes(nb);
+      const bool many = gap_many(G, nb, lanes_all), halved = gap_halved(G, lanes_all, cdiv(C / V, lanes_all) * B, m->tc.sm_count);
+      const int bl = halved ? lanes_all / 2 : lanes_all;
       const dim3 bgrid(cdiv(C / V, bl), B);
       auto go = [&](auto kernel) { return launch_pdl(kernel, bgrid, dim3(kGapThreads), st, (const T*)x, nb, hw, C, bl, gap, cnt, n_zero, sb); };
       switch (G) {
-        case 32: EE_CUDA(go(gap_blocks_kernel<T, V, 32>)); break;
-        case 16: EE_CUDA(go(gap_blocks_kernel<T, V, 16>)); break;
+        case 32: EE_CUDA(halved ? go(gap_blocks_kernel<T, V, 32, false, true>) : go(gap_blocks_kernel<T, V, 32>)); break;
+        case 16: EE_CUDA(halved ? go(gap_blocks_kernel<T, V, 16, false, true>) : go(gap_blocks_kernel<T, V, 16>)); break;
         case 8: EE_CUDA(go(gap_blocks_kernel<T, V, 8>)); break;
         case 4: EE_CUDA(go(gap_blocks_kernel<T, V, 4>)); break;
         case 2: EE_CUDA(many ? go(gap_blocks_kernel<T, V, 2, true>) : go(gap_blocks_kernel<T, V, 2>)); break;

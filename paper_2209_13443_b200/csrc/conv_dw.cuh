@@ -1,8 +1,7 @@
 // Depthwise 3x3 pad-1 convolution on bf16 (stride 1 or 2) with the input staged in shared memory by TMA: the
-// bandwidth-bound layers of the inverted-residual blocks.
+// layers of the inverted-residual blocks that do 9 MACs per element.
 //
-// A depthwise layer does 9 MACs per element.  A kernel that loads through registers holds one item's inputs per thread and stalls on
-// every item.  Here
+// A kernel that loads through registers holds one item's inputs per thread and stalls on every item.  Here
 // one producer warp per persistent CTA asks the TMA unit for whole input tiles, a band of output rows x all columns x
 // one block of up to 64 channels, including the one-pixel frame of the padding (coordinates start at -1; the unit
 // zero-fills outside the image), into a ring of three slots: two or three tiles (up to 72 KB each) are in flight per

@@ -177,16 +177,47 @@ __device__ __forceinline__ void pool_blocks(const T* p, int nb, int C, int grp, 
 // CTAs side by side: 11 x 11 x 1024 at 64 19.8 -> 21.7.  Blocks of four rows and more have their loads in flight as it is.
 inline bool gap_many(int G, int nb, int lanes) { return G <= 2 && nb > 2 * (kGapThreads / lanes); }
 
-// T = bf16 (VEC 8, the feature map) or float (VEC 4, block sums written by a convolution's epilogue; G = 1).
-template <typename T, int VEC, int G, bool MANY = false>
+// The same for a thread that has half of every block's tree (gap_tree), rows h, h + 2, ...: the lane beside it has the other half, and both get the
+// sums.  Every lane of the warp calls it; take = false: without rows.
+template <int VP, int G, typename T>
+__device__ __forceinline__ void pool_blocks_halved(const T* p, int nb, int C, int grp, int groups, int h, bool take, float* acc) {
+  const int rounds = (nb + groups - 1) / groups;   // the same for every lane
+  for (int i = 0; i < rounds; ++i) {
+    const int j = grp + i * groups;
+    const bool in = take && j < nb;
+    float t[VP];
+#pragma unroll
+    for (int e = 0; e < VP; ++e) t[e] = 0.f;
+    if (in)
+      gap_tree<G / 2, VP>([&](int row, float* out) {
+        Vec16<T> x;
+        x.load(p + ((size_t)j * G + row) * C);
+#pragma unroll
+        for (int e = 0; e < VP; ++e) out[e] = x.v[e];
+      }, h, 2, t);
+#pragma unroll
+    for (int e = 0; e < VP; ++e) {
+      const float other = __shfl_xor_sync(0xffffffffu, t[e], 1);
+      if (in) acc[e] += t[e] + other;
+    }
+  }
+}
+// Few samples leave most SMs without a CTA: blocks of 16 and 32 rows are then halved, and a CTA has half as many channel vectors.  Pooling + FC, us, 56 x 56 x 256
+// at batch 1 / 4 / 7 whole 7.64 / 8.60 / 9.41, halved 7.19 / 8.46 / 9.52, 28 x 28 x 512 6.37 / 7.34 / 7.54 and 6.13 / 7.27 / 7.67: the line is
+// between 32 CTAs and 56.  A pass of the ResNet-50-shaped model at batch 1: 229.4 -> 227.2.
+inline bool gap_halved(int G, int lanes, int ctas, int sms) { return G >= 16 && lanes >= 2 && 4 * ctas <= sms; }
+
+// T = bf16 (VEC 8, the feature map) or float (VEC 4, block sums written by a convolution's epilogue; G = 1).  HALVED: `lanes` is half of what the
+// shape asks for, row groups are as many.
+template <typename T, int VEC, int G, bool MANY = false, bool HALVED = false>
 __global__ void __launch_bounds__(kGapThreads)
 gap_blocks_kernel(const T* __restrict__ x, int nb, int HW, int C, int lanes, float* __restrict__ gap, unsigned* __restrict__ zero_me,
                   int n_zero, int rev) {
   __shared__ float red[kGapThreads * VEC];
   const int tid = threadIdx.x, b = rev ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;
   const int cv = C / VEC;
-  const int groups = kGapThreads / lanes;
-  const int grp = tid / lanes, lv = tid - grp * lanes;
+  const int at = HALVED ? tid / 2 : tid, groups = kGapThreads / (HALVED ? 2 : 1) / lanes;
+  const int grp = at / lanes, lv = at - grp * lanes;
   const int v = blockIdx.x * lanes + lv;
   pdl_launch_dependents();
   pdl_wait();
@@ -195,9 +226,14 @@ gap_blocks_kernel(const T* __restrict__ x, int nb, int HW, int C, int lanes, flo
   float acc[VEC];
 #pragma unroll
   for (int e = 0; e < VEC; ++e) acc[e] = 0.f;
-  if (v < cv) pool_blocks<VEC, G, MANY>(x + (size_t)b * nb * G * C + (size_t)v * VEC, nb, C, grp, groups, acc);
+  const T* p = x + (size_t)b * nb * G * C + (size_t)v * VEC;
+  if constexpr (HALVED)
+    pool_blocks_halved<VEC, G>(p, nb, C, grp, groups, tid % 2, v < cv, acc);
+  else if (v < cv)
+    pool_blocks<VEC, G, MANY>(p, nb, C, grp, groups, acc);
+  if (!HALVED || tid % 2 == 0)
 #pragma unroll
-  for (int e = 0; e < VEC; ++e) red[(grp * lanes + lv) * VEC + e] = acc[e];
+    for (int e = 0; e < VEC; ++e) red[(grp * lanes + lv) * VEC + e] = acc[e];
   __syncthreads();
   if (tid < lanes * VEC) {
     const int c = blockIdx.x * lanes * VEC + tid;

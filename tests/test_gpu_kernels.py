@@ -450,8 +450,10 @@ def test_head_routes_against_the_oracle_and_alone(case):
     assert np.array_equal(out.logits[0].cpu().numpy(), z[B - 1]) and float(out.conf[0]) == float(conf[B - 1])
 
 
-# rows of a map, its blocks of G rows and row groups: one row a block with two, three and more than eight blocks a group, two rows likewise
-@pytest.mark.parametrize("HW,G,groups", [(63, 1, 32), (65, 1, 64), (127, 1, 64), (129, 1, 64), (513, 1, 64), (1681, 1, 64), (258, 2, 64), (1026, 2, 64), (98, 2, 32)])
+# rows of a map, its blocks of G rows and row groups: one row a block with two, three and more than eight blocks a group, two rows likewise; 16 and 32
+# rows, whose blocks two lanes share at few samples: fewer blocks than groups, as many, one more
+@pytest.mark.parametrize("HW,G,groups", [(63, 1, 32), (65, 1, 64), (127, 1, 64), (129, 1, 64), (513, 1, 64), (1681, 1, 64), (258, 2, 64), (1026, 2, 64), (98, 2, 32),
+                                         (48, 16, 8), (784, 16, 32), (1040, 16, 64), (96, 32, 8), (1056, 32, 32), (2048, 32, 64), (3136, 32, 64)])
 def test_pooling_adds_the_blocks_of_a_row_group_in_order(HW, G, groups):
     B, C = 2, 72
     spec = wl.Model("rows", "bf16", 1, HW, C, [wl.Stage([wl.Layer(wl.OP_MAXPOOL, C, C, 3, 3, 1, 1)], C, np.eye(C, dtype=np.float32), None, 0.5, False)], B)

@@ -41,8 +41,8 @@ constexpr int kDwMaxTileBytes = 72 * 1024;
 
 // What a thread does with its vector of eight channels, here and in conv_xdw.cuh, whose bits have to agree.  What bounds it is instructions:
 // nine FMAs an output are 4.5 packed ones (an SM does about 93 FMAs a clock, packed or not), so everything else has to be few.  Pairs of
-// channels stay packed from the unpacking to the rounding, columns are offsets from one address, and the activation is chosen once a strip.  (30
-// instructions an output before.)  us, batch 32 / 13 / 1: 112 x 112 x 32 18.2 / 8.6 / 2.7 -> 16.7 / 8.1 / 2.6, 112 x 112 x 96 at stride 2
+// channels stay packed from the unpacking to the rounding, columns are offsets from one address, and the activation is chosen once a strip.  (17
+// instructions an output, about 30 before.)  us, batch 32 / 13 / 1: 112 x 112 x 32 18.2 / 8.6 / 2.7 -> 16.7 / 8.1 / 2.6, 112 x 112 x 96 at stride 2
 // 22.9 / 9.2 / 3.1 -> 20.0 / 8.3 / 2.9.  A thread that walks down its columns, sums of three rows open in registers, reads every vector once
 // (13.7 and 17.5 at batch 32) but fills the register file, so that no neighbouring kernel sets up beside it: 9.3 and 9.4 at 13, 4.2 and 4.3 at 1.
 typedef unsigned long long f32x2;   // two floats

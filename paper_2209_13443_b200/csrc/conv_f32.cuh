@@ -130,7 +130,7 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
       if (BM % STEP == 0 || row < BM) {
         const int hi = a_h[i] + fr_, wi = a_w[i] + fs;
         const bool in = k < k_end && hi >= 0 && hi < g.H && wi >= 0 && wi < g.W;
-        cp_async_zfill<V * 4>(st + (uint32_t)(row * 64 + place(row)), in ? x + (size_t)((a_b[i] + hi) * g.W + wi) * g.Cin + ci : x, in);
+        cp_async_zfill<V * 4>(st + (uint32_t)(row * 64 + place(row)), in ? x + ((size_t)(a_b[i] + hi) * g.W + wi) * g.Cin + ci : x, in);
       }
     }
     k += KS, ci += dci, fs += dtap;

@@ -186,7 +186,7 @@ struct ee_model {
   bool proj_fusion = true;             // projection shortcuts computed inside the layer that adds them, where that applies
   int fc_room = 1;                     // clusters of the FC kernel that run side by side
   bool fused_head = false;             // bf16 models: pool + FC + decision + scan as one cluster kernel where the shape allows (an option)
-  long long wait_cycles = kTcWaitCycles;   // limit of the bounded device-side waits of the pair kernel and the self-test
+  long long wait_cycles = kTcWaitCycles;   // limit of the bounded device-side waits of the pair kernel, of the fp32 convolutions and of the self-test
   int device = -1;           // the GPU the model lives on
   bool timing = false;
   bool graphs = true;  // replay stages as CUDA graphs on capturable streams
@@ -271,7 +271,7 @@ ee_status_t launch_layer(ee_model* m, const LayerPlan& L, const void* src, const
     }
     case KK_F32: {
       if constexpr (sizeof(T) == 4)
-        EE_CUDA(f32_launch(L.f32, (const float*)src, (const float*)L.w_dev, L.scale_dev, L.bias_dev, (const float*)res, (float*)dst, g, m->err_flag, st));
+        EE_CUDA(f32_launch(L.f32, (const float*)src, (const float*)L.w_dev, L.scale_dev, L.bias_dev, (const float*)res, (float*)dst, g, m->err_flag, m->wait_cycles, st));
       else
         return EE_ERR_INTERNAL;
       break;

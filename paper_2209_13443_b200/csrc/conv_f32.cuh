@@ -78,7 +78,8 @@ __device__ __forceinline__ void st_async_f64x2(uint32_t addr, uint32_t bar, uint
 template <int WM, int WN, int KG, int MF, int NF, int V>
 __global__ void __launch_bounds__(kF32Threads, KG == 1 || (KG == 8 && V == 4) ? 2 : 1)   // two CTAs an SM: 128 registers
 conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ w, const float* __restrict__ scale,
-                         const float* __restrict__ bias, const float* __restrict__ residual, float* __restrict__ y, ConvGeom g, int k_per, int* err_flag) {
+                         const float* __restrict__ bias, const float* __restrict__ residual, float* __restrict__ y, ConvGeom g, int k_per,
+                         int* err_flag, long long wait_cycles) {
   using S = F32Tile<WM, WN, KG, MF, NF>;
   constexpr int BM = S::kBM, BN = S::kBN, KS = S::kKS, STAGES = S::kStages;
   constexpr int UNITS = 16 / V;                       // copies per row and step
@@ -250,8 +251,9 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
       st_async_f64x2(recv_s + (uint32_t)(z * share + idx - q * share) * 8u, arrived, (uint32_t)q, v.x, v.y);
     }
     // Nothing but the data is waited for; a barrier of the cluster behind plain stores cost a pass of the ResNet-50-shaped model at 64 px 6 us of
-    // 427 at batch 6, 18 of 365 at batch 2.  Whoever waits here has been sent everything, so a CTA may leave while its own stores are on their way.
-    if (!mbar_wait(arrived, 0, err_flag)) return;
+    // 427 at batch 6, 18 of 365 at batch 2.  Whoever waits here has been sent everything, so a CTA may leave while its own stores are on their way; one whose
+    // wait ran out stays until it has been.
+    if (!mbar_wait_cluster(arrived, 0, err_flag, wait_cycles) && !cluster_drain(arrived, 0, err_flag)) return;
   }
 #pragma unroll
   for (int i = 0; i < S::kOuts; i += 2) {
@@ -283,7 +285,7 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
 
 template <int WM, int WN, int KG, int MF, int NF, int V>
 inline cudaError_t f32_launch_t(const F32Plan& p, const float* x, const float* w, const float* scale, const float* bias, const float* residual,
-                                float* y, const ConvGeom& g, int* err_flag, cudaStream_t st) {
+                                float* y, const ConvGeom& g, int* err_flag, long long wait_cycles, cudaStream_t st) {
   using S = F32Tile<WM, WN, KG, MF, NF>;
   const int K = g.kh * g.kw * g.Cin;
   const int k_per = f32_k_per(K, p.z);
@@ -300,24 +302,24 @@ inline cudaError_t f32_launch_t(const F32Plan& p, const float* x, const float* w
   attr[1].val.clusterDim.z = p.z;
   cfg.attrs = attr;
   cfg.numAttrs = p.z > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, conv_igemm_f64mma_kernel<WM, WN, KG, MF, NF, V>, x, w, scale, bias, residual, y, g, k_per, err_flag);
+  return cudaLaunchKernelEx(&cfg, conv_igemm_f64mma_kernel<WM, WN, KG, MF, NF, V>, x, w, scale, bias, residual, y, g, k_per, err_flag, wait_cycles);
 }
 
 template <int V>
 inline cudaError_t f32_launch_v(const F32Plan& p, const float* x, const float* w, const float* scale, const float* bias, const float* residual,
-                                float* y, const ConvGeom& g, int* err_flag, cudaStream_t st) {
+                                float* y, const ConvGeom& g, int* err_flag, long long wait_cycles, cudaStream_t st) {
   switch (p.tile) {
-    case 1: return f32_launch_t<2, 2, 2, 2, 4, V>(p, x, w, scale, bias, residual, y, g, err_flag, st);
-    case 2: return f32_launch_t<1, 1, 8, 2, 4, V>(p, x, w, scale, bias, residual, y, g, err_flag, st);
-    case 3: return f32_launch_t<1, 1, 8, 1, 4, V>(p, x, w, scale, bias, residual, y, g, err_flag, st);
-    default: return f32_launch_t<4, 2, 1, 1, 2, V>(p, x, w, scale, bias, residual, y, g, err_flag, st);
+    case 1: return f32_launch_t<2, 2, 2, 2, 4, V>(p, x, w, scale, bias, residual, y, g, err_flag, wait_cycles, st);
+    case 2: return f32_launch_t<1, 1, 8, 2, 4, V>(p, x, w, scale, bias, residual, y, g, err_flag, wait_cycles, st);
+    case 3: return f32_launch_t<1, 1, 8, 1, 4, V>(p, x, w, scale, bias, residual, y, g, err_flag, wait_cycles, st);
+    default: return f32_launch_t<4, 2, 1, 1, 2, V>(p, x, w, scale, bias, residual, y, g, err_flag, wait_cycles, st);
   }
 }
 
 inline cudaError_t f32_launch(const F32Plan& p, const float* x, const float* w, const float* scale, const float* bias, const float* residual,
-                              float* y, const ConvGeom& g, int* err_flag, cudaStream_t st) {
+                              float* y, const ConvGeom& g, int* err_flag, long long wait_cycles, cudaStream_t st) {
   const bool vec = g.Cin % 4 == 0 && (((uintptr_t)x | (uintptr_t)w) & 15) == 0;
-  return vec ? f32_launch_v<4>(p, x, w, scale, bias, residual, y, g, err_flag, st) : f32_launch_v<1>(p, x, w, scale, bias, residual, y, g, err_flag, st);
+  return vec ? f32_launch_v<4>(p, x, w, scale, bias, residual, y, g, err_flag, wait_cycles, st) : f32_launch_v<1>(p, x, w, scale, bias, residual, y, g, err_flag, wait_cycles, st);
 }
 
 inline ee_status_t f32_context_init() {

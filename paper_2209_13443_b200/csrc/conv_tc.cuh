@@ -126,6 +126,26 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* er
   }
   return true;
 }
+// Bounded wait for what other CTAs of the cluster send into this one's shared memory (st.async, counted by the barrier).  A look that does not
+// suspend comes first, so the limit counts from there.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, int* err_flag, long long limit) {
+  if (mbar_test_wait(bar, parity)) return true;
+  const long long t0 = clock64();
+  do {
+    if (clock64() - t0 > limit) {
+      atomicExch(err_flag, (int)EE_ERR_TIMEOUT);
+      return false;
+    }
+  } while (!mbar_try_wait(bar, parity));
+  return true;
+}
+// For the threads of a CTA whose wait ran out, before they leave: what is on its way to a CTA must find its shared memory.  Other threads of the cluster
+// are past their sends when they exit (an exit counts as the arrival) or come here, and then the bytes have only to land.  Threads that neither
+// exit nor come here would be waited for.  Returns whether everything is here after all.
+__device__ __forceinline__ bool cluster_drain(uint32_t bar, uint32_t parity, int* err_flag) {
+  asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+  return mbar_wait_cluster(bar, parity, err_flag, kTcWaitCycles);
+}
 
 // One lane of a converged warp.  A feeding loop runs inside `if (elect_one())`, which tells the compiler that it has one
 // thread: addresses and descriptors live in uniform registers.  With the descriptors stepped instead of rebuilt, weights

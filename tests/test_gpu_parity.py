@@ -303,6 +303,32 @@ def test_fp32_layer_at_the_lines_of_its_plan(geom, max_batch):
     util.check_stage(spec, run.stage(0, x), util.oracle_stage(spec, 0, x), f"f32 {geom} of {max_batch}", elementwise=True)
 
 
+# 16- and 32-row tiles whose K a cluster shares, copies of 16 and of 4 bytes
+@pytest.mark.parametrize("geom,max_batch", [((2, 2, 512, 512, 1, 1), 2), ((8, 8, 72, 96, 3, 2), 9), ((4, 4, 520, 64, 1, 1), 1), ((7, 7, 62, 64, 3, 1), 2)])
+def test_fp32_exchange_that_runs_out_of_time_is_reported_and_stays_whole(geom, max_batch):
+    """With a limit of one clock the wait for the cluster's partial sums runs out in every CTA that is not its cluster's last.  Each then stays until
+    everything sent to it has landed, so the call ends, is reported once, and has even the right results."""
+    H, W, cin, cout, k, stride = geom
+    spec = util.single_layer_model("f32", H, W, cin, cout, k, stride, k // 2, wl.ACT_RELU, False, seed=cin + k, max_batch=max_batch)
+    m = eb.EEModel(spec)
+    ws, x = m.workspace(), eb.to_device("f32", wl.random_features((max_batch, H, W, cin), seed=3, bf16=False, relu=False))
+    shape = (max_batch,) + tuple(wl.stage_shapes(spec)[0]["layers"][0])
+    want, got = torch.full(shape, np.nan, device="cuda"), torch.full(shape, np.nan, device="cuda")
+    m.layer_run(0, 0, x, None, max_batch, want, ws)
+    m.check()
+    m.set_wait_limit(1)
+    m.layer_run(0, 0, x, None, max_batch, got, ws)
+    with pytest.raises(eb.EEError) as e:
+        m.check()
+    assert e.value.status == 7                                         # EE_ERR_TIMEOUT
+    assert torch.equal(got, want)
+    m.set_wait_limit(4_000_000_000)
+    got.fill_(np.nan)
+    m.layer_run(0, 0, x, None, max_batch, got, ws)
+    m.check()
+    assert torch.equal(got, want)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_maxpool_layer(dtype):
     rng = wl._rng(5, 901)

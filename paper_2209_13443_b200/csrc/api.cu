@@ -186,7 +186,7 @@ struct ee_model {
   bool proj_fusion = true;             // projection shortcuts computed inside the layer that adds them, where that applies
   int fc_room = 1;                     // clusters of the FC kernel that run side by side
   bool fused_head = false;             // bf16 models: pool + FC + decision + scan as one cluster kernel where the shape allows (an option)
-  long long wait_cycles = kTcWaitCycles;   // limit of the bounded device-side waits of the pair kernel, of the fp32 convolutions and of the self-test
+  long long wait_cycles = kTcWaitCycles;   // limit of the bounded device-side waits of the pair kernel, of the exchanges of fp32 convolutions and exit heads and of the self-test
   int device = -1;           // the GPU the model lives on
   bool timing = false;
   bool graphs = true;  // replay stages as CUDA graphs on capturable streams
@@ -397,7 +397,7 @@ ee_status_t launch_head(ee_model* m, StagePlan& sp, const void* x, int B, int hw
       unsigned* done = m->head_done + 2 * (&sp - m->stages.data());   // nothing in front of this kernel could zero the scratch's counters
       DecideArgs da{shift, shift_cls, sp.threshold, sp.always_exit, out->conf, out->pred, out->exit_mask,
                     in_ids ? in_ids->ids : nullptr, out->survivor_idx, out->ids_out, out->n_surv_dev, nullptr, done, (unsigned long long*)done, host_count, host_out};
-      EE_CUDA(fc_cluster_launch<T>(f, nullptr, &pa, sp.tm_fc, sp.fc_b, B, C, K, out->logits, nullptr, da, m->err_flag, st));
+      EE_CUDA(fc_cluster_launch<T>(f, nullptr, &pa, sp.tm_fc, sp.fc_b, B, C, K, out->logits, nullptr, da, m->err_flag, m->wait_cycles, st));
       return EE_OK;
     }
   }
@@ -438,7 +438,7 @@ ee_status_t launch_head(ee_model* m, StagePlan& sp, const void* x, int B, int hw
                 in_ids ? in_ids->ids : nullptr, out->survivor_idx, out->ids_out, out->n_surv_dev, cnt, cnt + m->max_batch,
                 f.cluster || f.CL == 1 ? (unsigned long long*)cnt : nullptr, host_count, host_out};
   if (sp.fc_cluster)
-    EE_CUDA(fc_cluster_launch<T>(f, gap, nullptr, sp.tm_fc, sp.fc_b, B, C, K, out->logits, (float4*)(scratch + h.off_z), da, m->err_flag, st));
+    EE_CUDA(fc_cluster_launch<T>(f, gap, nullptr, sp.tm_fc, sp.fc_b, B, C, K, out->logits, (float4*)(scratch + h.off_z), da, m->err_flag, m->wait_cycles, st));
   else
     EE_CUDA(launch_pdl(fc_kernel<T>, dim3(cdiv(K, kFcClasses), cdiv(B, kFcSamples)), dim3(kFcThreads), st, (const float*)gap, (const T*)sp.fc_w,
                        (const float*)sp.fc_b, B, C, K, z, da));

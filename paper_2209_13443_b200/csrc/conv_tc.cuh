@@ -141,8 +141,9 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
 }
 // For the threads of a CTA whose wait ran out, before they leave: what is on its way to a CTA must find its shared memory.  Other threads of the cluster
 // are past their sends when they exit (an exit counts as the arrival) or come here, and then the bytes have only to land.  Threads that neither
-// exit nor come here would be waited for.  Returns whether everything is here after all.
-__device__ __forceinline__ bool cluster_drain(uint32_t bar, uint32_t parity, int* err_flag) {
+// exit nor come here would be waited for.  Returns whether everything is here after all.  Out of line: between the decision and the scan of a bf16 head
+// of 37 samples it took 0.1 us of 11.4 without ever running.
+__device__ __noinline__ bool cluster_drain(uint32_t bar, uint32_t parity, int* err_flag) {
   asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
   return mbar_wait_cluster(bar, parity, err_flag, kTcWaitCycles);
 }

@@ -490,7 +490,7 @@ __device__ __forceinline__ void pool_tile(int samples, int C, int lanes, A* red,
 template <typename T, int S, bool POOL>
 __global__ void __launch_bounds__(kFcThreads)
 fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restrict__ gap, const float* __restrict__ bfc, int B, int C, int K,
-                  float* z, float4* exchange, DecideArgs d, FcShape f, PoolArgs pa, int* err_flag) {
+                  float* z, float4* exchange, DecideArgs d, FcShape f, PoolArgs pa, int* err_flag, long long wait_cycles) {
   typedef typename Accum<T>::type A;                        // fp64 sums for the fp32 model
   constexpr int VEC = 16 / (int)sizeof(T), CHUNK = 32 * VEC, NV = kFcRows * S, WARPS = kFcThreads / 32;
   extern __shared__ __align__(128) uint8_t fc_smem[];
@@ -712,9 +712,10 @@ fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restri
         __stcg(exchange + (size_t)tile * kFcBlocks * S + at, make_float4(m, __int_as_float(arg), sum, 0.f));
     }
   }
+  bool late = false;
   if (f.cluster) {
     if (rank != 0) return;
-    if (warp < S) mbar_wait(triples, 0, err_flag);   // every block's triple is here
+    if (warp < S && b0 + warp < B) late = !__all_sync(0xffffffffu, mbar_wait_cluster(triples, 0, err_flag, wait_cycles));   // else every block's triple is here
   } else {
     if (f.CL > 1) __threadfence();
     __syncthreads();
@@ -729,12 +730,14 @@ fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restri
       __syncthreads();
     }
   }
-  // ---- 3. decision: one warp per sample, lane r holds block r
+  // ---- 3. decision: one warp per sample, lane r holds block r.  A sample whose triples are late has confidence 0 and class 0, and the leader then stays,
+  // behind the barrier that follows, until what is sent to it has landed.
+  int* leave = reinterpret_cast<int*>(gs);   // [S] bit 0: leaves, bit 1: late.  Not where triples may still arrive; the pooled vectors have been read
   if (warp < S && b0 + warp < B) {
     const int s = warp, b = b0 + s;
     float mr = -INFINITY, sr = 0.f;
     int arg = 0x7fffffff;
-    if (lane < kFcBlocks) {
+    if (lane < kFcBlocks && !late) {
       const float* t3 = part + ((size_t)lane * S + s) * 4;
       mr = t3[0], arg = __float_as_int(t3[1]), sr = t3[2];
     }
@@ -744,12 +747,12 @@ fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restri
 #pragma unroll
     for (int o = kFcBlocks; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
     if (lane == 0) {
-      const float cf = 1.0f / tot;
+      const float cf = late ? 0.f : 1.0f / tot;
       if (d.conf) d.conf[b] = cf;
       if (d.pred) d.pred[b] = arg == 0x7fffffff ? 0 : arg;
       const int leaves = d.always_exit || cf >= d.thr ? 1 : 0;
       d.mask[b] = (uint8_t)leaves;
-      part[s * 4] = __int_as_float(leaves);   // nobody reads block 0's triple of this sample again
+      leave[s] = leaves | (late ? 2 : 0);
     }
   }
   if (packed) {
@@ -758,7 +761,8 @@ fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restri
     __syncthreads();
     if (tid == 0) {
       unsigned long long keep = 0;
-      for (int s = 0; s < S && b0 + s < B; ++s) keep |= (unsigned long long)(__float_as_int(part[s * 4]) ? 0 : 1) << (b0 + s);
+      int any = 0;
+      for (int s = 0; s < S && b0 + s < B; ++s) keep |= (unsigned long long)(~leave[s] & 1) << (b0 + s), any |= leave[s];
       unsigned long long last = 1;
       if (tiles > 1) {
         if (d.host_out) __threadfence();
@@ -767,11 +771,12 @@ fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restri
         keep = (before + keep) & ((1ull << kFcPackedBatch) - 1);
         if (last) *d.packed = 0;
       }
-      s_done[0] = keep, s_done[1] = last;
+      s_done[0] = keep, s_done[1] = last | (any & 2);
     }
     __syncthreads();
-    const unsigned long long keep = s_done[0];
-    if (!s_done[1]) return;
+    const unsigned long long keep = s_done[0], state = s_done[1];
+    if (state & 2) cluster_drain(triples, 0, err_flag);
+    if (!(state & 1)) return;
     if (tid < B && (keep >> tid & 1)) {
       const int pos = __popcll(keep & ((1ull << tid) - 1));
       d.surv_idx[pos] = tid;
@@ -788,6 +793,11 @@ fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restri
   }
   __threadfence();
   __syncthreads();
+  if (f.cluster) {
+    int any = 0;
+    for (int s = 0; s < S && b0 + s < B; ++s) any |= leave[s];
+    if (any & 2) cluster_drain(triples, 0, err_flag);
+  }
   if (tiles > 1) {         // the leader that finishes last scans
     int* flag = reinterpret_cast<int*>(part);
     if (tid == 0) *flag = atomicAdd(d.done, 1u) == (unsigned)(tiles - 1) ? 1 : 0;
@@ -802,7 +812,7 @@ fc_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const float* __restri
 // pool: null = `gap` holds the pooled vectors.
 template <typename T, int S>
 inline cudaError_t fc_cluster_launch_t(const float* gap, const PoolArgs* pool, const CUtensorMap& wfc, const float* bfc, int B, int C, int K, float* z,
-                                       float4* exchange, const DecideArgs& d, const FcShape& f, int* err_flag, cudaStream_t st) {
+                                       float4* exchange, const DecideArgs& d, const FcShape& f, int* err_flag, long long wait_cycles, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((B + S - 1) / S * f.CL));
   cfg.blockDim = dim3(kFcThreads);
@@ -817,21 +827,21 @@ inline cudaError_t fc_cluster_launch_t(const float* gap, const PoolArgs* pool, c
   cfg.attrs = attr;
   cfg.numAttrs = f.cluster ? 2 : 1;
   if constexpr (S == 1)   // fc_pools: tiles of one sample
-    if (pool) return cudaLaunchKernelEx(&cfg, fc_cluster_kernel<T, 1, true>, wfc, gap, bfc, B, C, K, z, exchange, d, f, *pool, err_flag);
+    if (pool) return cudaLaunchKernelEx(&cfg, fc_cluster_kernel<T, 1, true>, wfc, gap, bfc, B, C, K, z, exchange, d, f, *pool, err_flag, wait_cycles);
   if (pool) return cudaErrorInvalidValue;
-  return cudaLaunchKernelEx(&cfg, fc_cluster_kernel<T, S, false>, wfc, gap, bfc, B, C, K, z, exchange, d, f, PoolArgs{}, err_flag);
+  return cudaLaunchKernelEx(&cfg, fc_cluster_kernel<T, S, false>, wfc, gap, bfc, B, C, K, z, exchange, d, f, PoolArgs{}, err_flag, wait_cycles);
 }
 // d.done and d.tile_done must be zero when the kernel starts and are zero again when it ends.  exchange: 16 float4 per sample
 // of every tile, less than the batch's logits take wherever it is used (more than 512 classes).
 template <typename T>
 inline cudaError_t fc_cluster_launch(const FcShape& f, const float* gap, const PoolArgs* pool, const CUtensorMap& wfc, const float* bfc, int B, int C, int K, float* z,
-                                     float4* exchange, const DecideArgs& d, int* err_flag, cudaStream_t st) {
+                                     float4* exchange, const DecideArgs& d, int* err_flag, long long wait_cycles, cudaStream_t st) {
   switch (f.S) {
-    case 1: return fc_cluster_launch_t<T, 1>(gap, pool, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, st);
-    case 2: return fc_cluster_launch_t<T, 2>(gap, pool, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, st);
-    case 4: return fc_cluster_launch_t<T, 4>(gap, pool, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, st);
+    case 1: return fc_cluster_launch_t<T, 1>(gap, pool, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, wait_cycles, st);
+    case 2: return fc_cluster_launch_t<T, 2>(gap, pool, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, wait_cycles, st);
+    case 4: return fc_cluster_launch_t<T, 4>(gap, pool, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, wait_cycles, st);
   }
-  if constexpr (sizeof(T) == 2) return fc_cluster_launch_t<T, 8>(gap, pool, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, st);
+  if constexpr (sizeof(T) == 2) return fc_cluster_launch_t<T, 8>(gap, pool, wfc, bfc, B, C, K, z, exchange, d, f, err_flag, wait_cycles, st);
   return cudaErrorInvalidValue;
 }
 template <typename T, int S>

@@ -450,6 +450,50 @@ def test_head_routes_against_the_oracle_and_alone(case):
     assert np.array_equal(out.logits[0].cpu().numpy(), z[B - 1]) and float(out.conf[0]) == float(conf[B - 1])
 
 
+# heads whose tiles are clusters: 16 CTAs a tile, survivors in one word; two CTAs and the scan of more than 56 samples; eight CTAs whose warps share classes
+@pytest.mark.parametrize("case", [("bf16", 5, 64, 9, 64, 1000), ("bf16", 37, 64, 9, 64, 1000), ("f32", 60, 64, 16, 16, 100), ("f32", 6, 32, 4, 2048, 100)])
+def test_head_whose_exchange_runs_out_of_time_is_reported_and_keeps_its_samples(case):
+    """With a limit of one clock the wait for the tile's triples runs out.  The call ends all the same, the time-out is reported once, and a sample whose
+    triples were late stays in the batch, with confidence 0; one whose triples were there is decided as ever."""
+    dtype, B, most, HW, C, K = case
+    fw, fb = wl._head(wl._rng(B + C + K, 924), C, K, 4.0, dtype == "bf16")
+    spec = wl.Model("late", dtype, 1, HW, C, [wl.Stage([wl.Layer(wl.OP_MAXPOOL, C, C, 3, 3, 1, 1)], K, fw, fb, 0.5, False)], most)
+    m = eb.EEModel(spec)
+    scratch = torch.empty(m.exit_head_scratch_bytes(0) + 256, dtype=torch.uint8, device="cuda")
+    x = eb.to_device(dtype, wl.random_features((B, HW, C), seed=3, bf16=dtype == "bf16"))
+    shift = torch.as_tensor((np.arange(B) % 3 == 0).astype(np.float32) * 40.0, device="cuda")   # these leave
+    cls = torch.as_tensor((np.arange(B) * 7 % K).astype(np.int32), device="cuda")
+    right, late, again = (eb.StageBuffers(m, 0) for _ in range(3))
+
+    def call(out):
+        m.exit_head(0, x, B, HW, out, scratch, shift, cls)
+        torch.cuda.synchronize()
+        return out.conf[:B].cpu().numpy(), out.pred[:B].cpu().numpy(), out.exit_mask[:B].cpu().numpy(), out.logits[:B].cpu().numpy()
+
+    want = call(right)
+    m.check()
+    assert want[2][::3].all()
+    m.set_wait_limit(1)
+    for _ in range(20):   # a leader that happens to be its cluster's last has nothing to wait for
+        conf, pred, mask, z = call(late)
+        gone = conf == 0.0
+        if gone.any():
+            break
+    with pytest.raises(eb.EEError) as e:
+        m.check()
+    assert e.value.status == 7                                         # EE_ERR_TIMEOUT
+    assert gone.any() and not pred[gone].any() and not mask[gone].any()
+    for got, w in zip((conf, pred, mask), want):
+        assert np.array_equal(got[~gone], w[~gone])
+    assert np.array_equal(z, want[3])
+    n = int(late.n_surv_dev[0])
+    assert n == B - int(mask.sum()) and np.array_equal(late.survivor_idx[:n].cpu().numpy(), np.nonzero(mask == 0)[0])
+    m.set_wait_limit(4_000_000_000)
+    for got, w in zip(call(again), want):
+        assert np.array_equal(got, w)
+    m.check()
+
+
 # rows of a map, its blocks of G rows and row groups: one row a block with two, three and more than eight blocks a group, two rows likewise; 16 and 32
 # rows, whose blocks two lanes share at few samples: fewer blocks than groups, as many, one more
 @pytest.mark.parametrize("HW,G,groups", [(63, 1, 32), (65, 1, 64), (127, 1, 64), (129, 1, 64), (513, 1, 64), (1681, 1, 64), (258, 2, 64), (1026, 2, 64), (98, 2, 32),

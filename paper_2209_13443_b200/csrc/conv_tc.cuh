@@ -126,17 +126,23 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* er
   }
   return true;
 }
-// Bounded wait for what other CTAs of the cluster send into this one's shared memory (st.async, counted by the barrier).  A look that does not
-// suspend comes first, so the limit counts from there.
+// Bounded wait for what other CTAs of the cluster send into this one's shared memory (st.async, counted by the barrier): acquire at the scope of the
+// cluster, the one at which st.async releases (without a qualifier the waits are of the CTA's).  A look that does not suspend the thread comes first,
+// so the limit counts from there.
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, int* err_flag, long long limit) {
-  if (mbar_test_wait(bar, parity)) return true;
+  uint32_t ok;
+  asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+               : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  if (ok) return true;
   const long long t0 = clock64();
   do {
     if (clock64() - t0 > limit) {
       atomicExch(err_flag, (int)EE_ERR_TIMEOUT);
       return false;
     }
-  } while (!mbar_try_wait(bar, parity));
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  } while (!ok);
   return true;
 }
 // For the threads of a CTA whose wait ran out, before they leave: what is on its way to a CTA must find its shared memory.  Other threads of the cluster

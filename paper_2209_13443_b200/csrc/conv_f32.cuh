@@ -44,6 +44,7 @@ struct F32Tile {   // WM x WN warps per K group, each MF x NF fragments of 16 x 
   static constexpr int kRecv = KG == 8 ? kBM * kBN * 8 : 0;
   static constexpr int kBytes = kMain + kRecv + 16;        // and a barrier that counts it
   static_assert(WM * WN * KG == 8, "8 warps");
+  static_assert(KG != 8 || 2 * (kBytes + kBM * 16 + 1024) <= 228 * 1024, "the plan counts two CTAs of these tiles an SM");
   static_assert(kBytes <= 227 * 1024, "exceeds the shared memory of an SM");
 };
 
@@ -76,7 +77,7 @@ __device__ __forceinline__ void st_async_f64x2(uint32_t addr, uint32_t bar, uint
 
 // V: floats per copy (4 when Cin is a multiple of 4 and the pointers are 16-byte aligned, else 1).  k_per: K range of a CTA.
 template <int WM, int WN, int KG, int MF, int NF, int V>
-__global__ void __launch_bounds__(kF32Threads, KG == 1 || (KG == 8 && V == 4) ? 2 : 1)   // two CTAs an SM: 128 registers
+__global__ void __launch_bounds__(kF32Threads, KG == 1 || KG == 8 ? 2 : 1)   // two CTAs an SM, which the plan counts on: 128 registers
 conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ w, const float* __restrict__ scale,
                          const float* __restrict__ bias, const float* __restrict__ residual, float* __restrict__ y, ConvGeom g, int k_per,
                          int* err_flag, long long wait_cycles) {
@@ -96,16 +97,26 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
   const int k_mine = k_begin + kg * 16, steps = max(0, (k_end - k_mine + KS - 1) / KS);   // this group's steps: k_mine, k_mine + KS, ...
 
   const int ku = tid % UNITS, r0 = tid % S::kGroup / UNITS;   // this thread copies column ku of rows r0, r0 + STEP, ...
-  int a_b[RA], a_h[RA], a_w[RA];   // sample x image rows, row and column of the first tap
-#pragma unroll
-  for (int i = 0; i < RA; ++i) {
-    const int r = r0 + i * STEP, m = m0 + r;
+  // An output row's first tap: sample x image rows, row and column.  Each thread keeps those of its rows, but for the 32-row tile copied in 4 bytes: there
+  // they are 16, which with 16 addresses of weights took 254 registers and an SM to itself, half of what the plan counts on.  Read from shared
+  // memory, and weights eight at a time, 126.  us a layer, one CTA an SM / spilled / so: 3x3 on 8 x 8 x 126, batch 4 23.2 / 14.3 / 12.0, on 14 x 14 x 30, 6
+  // 12.5 / 9.0 / 7.5, 1x1 on 7 x 7 x 512 from an unaligned pointer, 6 24.8 / 24.7 / 19.4; where the grid never fills the chip, 3x3 on 7 x 7 x 62, 2, 6.8 / 8.4 / 7.3.
+  constexpr bool TABLE = KG == 8 && MF == 2 && V == 1;
+  auto row_at = [&](int r) {
+    const int m = m0 + r;
     const bool in = r < BM && m < M;
     const int mm = in ? m : 0;
     const int wo = mm % g.Wo, q = mm / g.Wo, ho = q % g.Ho, b = q / g.Ho;
-    a_b[i] = b * g.H;
-    a_h[i] = in ? ho * g.stride - g.pad : -(1 << 20);   // far outside the image: zeros
-    a_w[i] = wo * g.stride - g.pad_w;
+    return make_int4(b * g.H, in ? ho * g.stride - g.pad : -(1 << 20), wo * g.stride - g.pad_w, 0);   // far outside the image: zeros
+  };
+  __shared__ int4 s_rows[TABLE ? BM : 1];
+  int4 my_rows[TABLE ? 1 : RA];
+  if constexpr (TABLE) {
+    if (tid < BM) s_rows[tid] = row_at(tid);
+    __syncthreads();
+  } else {
+#pragma unroll
+    for (int i = 0; i < RA; ++i) my_rows[i] = row_at(r0 + i * STEP);
   }
   auto place = [&](int row) { return ((ku * V / 4 ^ (row >> 1 & 3)) << 4) + ku * V % 4 * 4; };   // byte of this thread's column in a row
   // position of this thread's column in a step: K index, channel, filter row and column, walked by counters
@@ -114,7 +125,7 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
   auto load_b = [&](int step) {   // weights
     const uint32_t st = ring_s + (uint32_t)((step % STAGES) * S::kStageFloats) * 4u;
     const int kb = k_mine + step * KS + ku * V;
-#pragma unroll
+#pragma unroll (TABLE ? RB / 2 : RB)
     for (int i = 0; i < RB; ++i) {
       const int row = r0 + i * STEP, n = n0 + row;
       if (BN % STEP == 0 || row < BN) {
@@ -129,9 +140,12 @@ conv_igemm_f64mma_kernel(const float* __restrict__ x, const float* __restrict__ 
     for (int i = 0; i < RA; ++i) {
       const int row = r0 + i * STEP;
       if (BM % STEP == 0 || row < BM) {
-        const int hi = a_h[i] + fr_, wi = a_w[i] + fs;
+        int4 at;
+        if constexpr (TABLE) at = s_rows[row];
+        else at = my_rows[i];
+        const int hi = at.y + fr_, wi = at.z + fs;
         const bool in = k < k_end && hi >= 0 && hi < g.H && wi >= 0 && wi < g.W;
-        cp_async_zfill<V * 4>(st + (uint32_t)(row * 64 + place(row)), in ? x + ((size_t)(a_b[i] + hi) * g.W + wi) * g.Cin + ci : x, in);
+        cp_async_zfill<V * 4>(st + (uint32_t)(row * 64 + place(row)), in ? x + ((size_t)(at.x + hi) * g.W + wi) * g.Cin + ci : x, in);
       }
     }
     k += KS, ci += dci, fs += dtap;

@@ -303,6 +303,28 @@ def test_fp32_layer_at_the_lines_of_its_plan(geom, max_batch):
     util.check_stage(spec, run.stage(0, x), util.oracle_stage(spec, 0, x), f"f32 {geom} of {max_batch}", elementwise=True)
 
 
+# copies of 4 bytes into tiles of 16 and of 32 rows, the last of them short, because of the channels or of the pointer alone: H, W, cin, cout, k, stride, max_batch
+@pytest.mark.parametrize("geom", [(8, 8, 126, 40, 3, 1, 4), (7, 7, 62, 64, 3, 2, 3), (9, 11, 29, 33, 3, 1, 1), (2, 2, 510, 64, 1, 1, 8), (7, 7, 65, 32, 5, 1, 6),
+                                  (8, 8, 128, 40, 3, 1, 4), (7, 7, 512, 96, 1, 1, 3), (9, 11, 32, 32, 3, 2, 1), (2, 2, 512, 64, 1, 1, 8)])
+def test_fp32_layer_copied_four_bytes_at_a_time(geom):
+    H, W, cin, cout, k, stride, B = geom
+    spec = util.single_layer_model("f32", H, W, cin, cout, k, stride, k // 2, wl.ACT_RELU, False, seed=cin + k, max_batch=B)
+    run = util.GpuRunner(spec)
+    x = wl.random_features((B, H, W, cin), seed=B, bf16=False, relu=False)
+    util.check_stage(spec, run.stage(0, x), util.oracle_stage(spec, 0, x), f"f32 {geom}", elementwise=True)
+    m, dev = eb.EEModel(spec), eb.to_device("f32", x)
+    ws, buf, outs = m.workspace(), eb.StageBuffers(m, 0), []
+    for off in range(4):    # floats past a 16-byte line
+        at = torch.empty(dev.numel() + off, device="cuda")[off:].view(dev.shape)
+        at.copy_(dev)
+        buf.features_out.fill_(np.nan)
+        m.stage_run(0, at, B, buf, ws)    # nobody leaves: the layer's whole output
+        torch.cuda.synchronize()
+        outs.append(buf.features_out[:B].clone())
+    m.check()
+    assert all(torch.equal(o, outs[0]) for o in outs[1:])   # the plan, and so the sums, do not depend on the pointer
+
+
 # 16- and 32-row tiles whose K a cluster shares, copies of 16 and of 4 bytes
 @pytest.mark.parametrize("geom,max_batch", [((2, 2, 512, 512, 1, 1), 2), ((8, 8, 72, 96, 3, 2), 9), ((4, 4, 520, 64, 1, 1), 1), ((7, 7, 62, 64, 3, 1), 2)])
 def test_fp32_exchange_that_runs_out_of_time_is_reported_and_stays_whole(geom, max_batch):

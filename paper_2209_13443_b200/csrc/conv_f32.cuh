@@ -301,6 +301,7 @@ template <int WM, int WN, int KG, int MF, int NF, int V>
 inline cudaError_t f32_launch_t(const F32Plan& p, const float* x, const float* w, const float* scale, const float* bias, const float* residual,
                                 float* y, const ConvGeom& g, int* err_flag, long long wait_cycles, cudaStream_t st) {
   using S = F32Tile<WM, WN, KG, MF, NF>;
+  if (p.z > 1 && S::kRecv == 0) return cudaErrorInvalidValue;   // no room for what a cluster's CTAs send
   const int K = g.kh * g.kw * g.Cin;
   const int k_per = f32_k_per(K, p.z);
   cudaLaunchConfig_t cfg = {};

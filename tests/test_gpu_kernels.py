@@ -519,6 +519,33 @@ def test_pooling_adds_the_blocks_of_a_row_group_in_order(HW, G, groups):
     assert np.array_equal(out.logits[:B].cpu().numpy(), want / np.float32(HW))   # the FC layer is the identity: the logits are the pooled vector
 
 
+# 16- and 32-row blocks at batches on both sides of the line up to which two lanes share them (a quarter of 148 SMs, in CTAs): rows, G, groups, channels, most samples
+@pytest.mark.parametrize("HW,G,groups,C,most", [(48, 16, 8, 72, 41), (784, 16, 32, 72, 41), (1040, 16, 64, 72, 41), (96, 32, 8, 72, 41), (1056, 32, 32, 72, 41), (3136, 32, 64, 72, 41),
+                                                (784, 16, 32, 512, 12), (3136, 32, 64, 256, 12)])
+def test_pooled_sums_do_not_depend_on_the_batch(HW, G, groups, C, most):
+    spec = wl.Model("rows", "bf16", 1, HW, C, [wl.Stage([wl.Layer(wl.OP_MAXPOOL, C, C, 3, 3, 1, 1)], C, np.eye(C, dtype=np.float32), None, 0.5, False)], most)
+    m = eb.EEModel(spec)
+    out = eb.StageBuffers(m, 0)
+    scratch = torch.empty(m.exit_head_scratch_bytes(0) + 256, dtype=torch.uint8, device="cuda")
+    x = wl.random_features((most, HW, C), seed=HW, bf16=True, relu=False)
+    xd = eb.to_device("bf16", x)
+    blocks = np.asarray(x, dtype=np.float32).reshape(most, HW // G, G, C)
+    while blocks.shape[2] > 1:      # the pairwise tree over a block's rows
+        blocks = blocks[:, :, :blocks.shape[2] // 2] + blocks[:, :, blocks.shape[2] // 2:]
+    blocks, want = blocks[:, :, 0], np.zeros((most, C), dtype=np.float32)
+    for q in range(groups):
+        part = np.zeros((most, C), dtype=np.float32)
+        for j in range(q, HW // G, groups):
+            part = part + blocks[:, j]
+        want = want + part
+    for B in (most, 13, 12, 1):
+        if B > most:
+            continue
+        m.exit_head(0, xd, B, HW, out, scratch)
+        torch.cuda.synchronize()
+        assert np.array_equal(out.logits[:B].cpu().numpy(), want[:B] / np.float32(HW)), B   # the FC layer is the identity
+
+
 # 1x1 layer + depthwise layer in one launch: H, W, cin, hidden, stride, batches: one to three K blocks, channel blocks that are short, odd
 # or not a multiple of 16, bands of one row and of the whole image, one pixel, the widest row, images smaller than a tile of positions
 XDW_GEOMS = [(14, 14, 64, 384, 1, (1, 5)), (7, 7, 160, 960, 1, (1, 9)), (20, 50, 16, 96, 2, (1, 4)), (9, 13, 24, 144, 1, (1, 3)), (5, 5, 96, 576, 2, (1, 40)),

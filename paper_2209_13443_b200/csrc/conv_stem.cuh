@@ -15,8 +15,9 @@
 // read by the up to (kh + 1) / 2 output rows P, P - 1, ...  Four gather warps, a thread per pixel pair, fetch three words of a row
 // with cp.async, eight pairs of rows ahead, and put them into the arrays; one thread issues the MMAs into four accumulators in turn;
 // eight epilogue warps, 32 channels of 32 pixels each, finish the rows.
-// What bounds it: the epilogue with the pool behind it, about 1500 clocks a row (sixteen warps of 16 channels take as long, and at 80
-// registers spill), against 780 of MMAs and 650 of gather (1430 to 1600 when every output pixel gathered its own runs).  A stage of the
+// What bounds it: none of its parts alone.  7x7 and pool on 64 images of 224 x 224 take 50 us, without the pooled rows' exchange 38, without any
+// epilogue 30: gather (650 clocks a row; 1430 to 1600 when every output pixel gathered its own runs), MMAs (780) and epilogue with the pool behind
+// it (1500; sixteen warps of 16 channels take as long, and at 80 registers spill) overlap only in part.  A stage of the
 // stem, the pool and an 8-channel 1x1 layer, gather per output pixel -> this, us: 7x7, batch 64 of 224 x 224 images 77.9 -> 74.9, batch 7
 // 30.8 -> 27.6, batch 21 of 161 x 161 41.1 -> 37.2; 3x3 without a pool, batch 32 of 224 x 224 74.3 -> 63.6.
 #pragma once

@@ -573,9 +573,9 @@ conv_igemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  // Programmatic dependent launch: everything above overlapped the tail of the previous kernel in the stream, and
-  // so do the weight tiles of the first ring slots, which no kernel writes.  From the wait on this kernel touches
-  // activations, so it needs that kernel's memory; the next kernel in the stream may begin its own prologue now.
+  // Programmatic dependent launch: from the line above on the next kernel in the stream may begin its own prologue.  This one's overlapped the
+  // tail of the previous kernel, and so do the weight tiles of the first ring slots, which no kernel writes.  From the wait on this kernel
+  // touches activations, so it needs that kernel's memory.
   const int w_ahead = min(num_kb, kStages);
   // ring walk of a producer: its K block (channel block x 64, position in the tap table), slot and phase
   struct Feed {

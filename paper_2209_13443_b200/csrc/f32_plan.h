@@ -19,9 +19,9 @@ inline int f32_k_per(int k, int z) { return (int)f32_div(f32_div(k, 16), z) * 16
 // channels are copied one by one (!vec: stems on 3 channels), where addresses and copies of a row are the cost and a 64 x 32 tile has the
 // fewest: 7x7 on 64 x 64 x 3, batch 6 24.3 us as 32 x 32 tiles, 11.9 so; a pass of that model 436 -> 422.  Grids of two waves of 64 x 64 tiles: that tile reads its operands least.
 // Everything else has idle SMs: small tiles (16 rows where the layer never has more than 32), eight K groups, and as many CTAs per tile (up to 8) as keep the grid within
-// two CTAs per SM while every CTA still has 64 of K, a 16-wide step for half its groups, and the last one any.  That line at 256 / 128 / 64 / 32, us a pass:
-// ResNet-50-shaped model at 33 px, batch 1 340 / 323 / 313 / 313, 64 px, batch 6 of which 30 % leave at every exit 448 / 436 / 436 / 436, tiny model
-// at 40 px, batch 8 with nobody leaving 75.7 / 73.4 / 77.1 / 76.5, at 24 px, batch 1 61 / 58 / 56 / 54.
+// two CTAs per SM while every CTA still has 64 of K, a 16-wide step for half its groups, and the last one any.  That line at 256 / 128 / 64 / 32, us a pass,
+// nobody leaving: tiny model at 32 px, batch 1 60.5 / 57.1 / 53.6 / 53.7, batch 8 64.1 / 61.6 / 58.0 / 58.1, at 40 px, batch 8 67.7 / 65.4 / 67.7 / 67.7; ResNet-50-shaped
+// model of batch 1 at 33 px 278 / 265 / 271 / 283, of 4 at 48 px 426 / 396 / 406 / 415, of 2 at 64 px 337 / 337 / 346 / 353, of 6 at 64 px 484 / 467 / 467 / 467.
 inline F32Plan f32_plan(long m_max, int n, int k, int sms, bool vec = true) {
   F32Plan p;
   if (k < (vec ? 128 : 256)) return p;
